@@ -130,14 +130,16 @@ def _check(rc, where):
         raise MtvError(rc, where)
 
 
+# Addresses and streams go over as plain integers (every function has its argument types declared): a decode loop makes
+# one attention call per layer, and wrapping each pointer and building a Stream object cost more than the kernel's launch.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def tree_gen_cartesian(topk: Sequence[int]):
@@ -216,7 +218,7 @@ def mtv_workspace_bytes(tree: Tree, B, H, V, Hq, Hkv, D, Lcap) -> int:
 
 
 def _ws(ws):
-    return C.c_void_p(ws.data_ptr()), ws.numel() * ws.element_size()
+    return ws.data_ptr(), ws.nbytes
 
 
 def medusa_heads_topk(tree, hidden, W1, b1, W2, root_tok, cand, cand_logit, tree_tok, ws, stream=None):
@@ -233,8 +235,8 @@ def tree_verify_attention(tree, q, k_cache, v_cache, seq_lens, out, ws, scale=0.
     B, T, Hq, D = q.shape
     Hkv = k_cache.shape[1]
     Lcap = k_cache.shape[2] if Lcap is None else Lcap
-    sb, sh, st = k_cache.stride(0), k_cache.stride(1), k_cache.stride(2)
-    assert (v_cache.stride(0), v_cache.stride(1), v_cache.stride(2)) == (sb, sh, st)
+    sb, sh, st = strides = k_cache.stride()[:3]
+    assert v_cache.stride()[:3] == strides
     p, n = _ws(ws)
     _check(lib().tree_verify_attention(tree.handle, B, Hq, Hkv, D, _ptr(q), _ptr(k_cache), _ptr(v_cache),
                                        sb, sh, st, Lcap, _ptr(seq_lens), scale, _ptr(out), _ptr(status), p, n,

@@ -1,4 +1,6 @@
-// Tree attention on the 5th-generation tensor cores (Section 3.2 / Fig. 2(b)), head_dim 128.
+// Tree attention on the 5th-generation tensor cores (Section 3.2 / Fig. 2(b)), head_dim 128, one layer per launch, on CTA
+// pairs.  It serves the single-layer calls where its short start and end count for more than an even division of the work
+// (see pair_kernel_is_better in attention.cu).
 //
 // A pair of CTAs (a cluster of two) owns up to 256 query rows — the (node, head-in-group) rows that
 // share one KV head: 128 / G whole tree nodes per CTA for a group of G <= 8 query heads (when G does not
@@ -39,16 +41,7 @@
 //
 // The running max of a stream moves only when a tile's max exceeds it by more than 8 (log2 units), so O is
 // rescaled rarely and P stays below 2^8.
-//
-// Build option -DMTV_TRACE: per-CTA cycle stamps of the phases through mtv_trace_set (development aid).
-#include <cuda.h>
-
-#include <cstring>
-#include <mutex>
-#include <type_traits>
-
-#include "common.cuh"
-#include "sm100_ptx.cuh"
+#include "attn_common.cuh"
 
 namespace mtv {
 
@@ -135,55 +128,8 @@ __device__ __forceinline__ uint64_t desc_nmajor(uint32_t saddr) { return smem_de
 __device__ __forceinline__ void cta_sync() { asm volatile("bar.sync 1, %0;" ::"n"(TC_THREADS) : "memory"); }
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 6, %0;" ::"n"(TC_SOFTMAX_WARPS * 32) : "memory"); }
 
-__device__ __forceinline__ float ex2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-// 2^x for two values on the FMA pipes: x = j + f with j the nearest integer (read off the low mantissa bits of
-// x + 1.5 * 2^23) and f in [-0.5, 0.5]; 2^f by a cubic (relative error 7.5e-5, far below the bf16 rounding of P);
-// 2^j by an add to the exponent field.  x is clamped at -126 (the result then underflows towards zero like ex2's).
-__device__ __forceinline__ float2 exp2_poly2(float2 x) {
-    const float magic = 12582912.f;
-    x.x = fmaxf(x.x, -126.f);
-    x.y = fmaxf(x.y, -126.f);
-    const float2 t = __fadd2_rn(x, make_float2(magic, magic));
-    const float2 jf = __fadd2_rn(t, make_float2(-magic, -magic));
-    const float2 f = __fadd2_rn(x, make_float2(-jf.x, -jf.y));
-    float2 q = __ffma2_rn(make_float2(0.055171650f, 0.055171650f), f, make_float2(0.24261113f, 0.24261113f));
-    q = __ffma2_rn(q, f, make_float2(0.69326097f, 0.69326097f));
-    q = __ffma2_rn(q, f, make_float2(0.99992806f, 0.99992806f));
-    return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23)),
-                       __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23)));
-}
-__device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
-__device__ __forceinline__ int ld_acquire(const int32_t *p) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-#ifdef MTV_TRACE
-__device__ long long *g_trace = nullptr;   // [ctas][64]
-// the buffer's address is read once per thread (TRACE_INIT); a stamp is then one clock read and one store
-#define TRACE_INIT                                                                                                  \
-    long long *trace_row = g_trace;                                                                                 \
-    if (trace_row) trace_row += ((size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * 64
-#define TRACE(id)                                                            \
-    do {                                                                     \
-        if (trace_row && (threadIdx.x % 32) == 0) trace_row[(id)] = clock64(); \
-    } while (0)
-#else
-#define TRACE_INIT
-#define TRACE(id)
-#endif
-
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TC_THREADS, 1)
-tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
+tree_attn_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                     const __grid_constant__ CUtensorMap v_map, const TcParams p) {
     extern __shared__ unsigned char smem_raw[];
     // Programmatic dependent launch: let the next kernel of the stream be set up while this one runs.
@@ -192,8 +138,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     const int split = blockIdx.x >> 1;
     const int g = blockIdx.y / p.n_blk, blk = blockIdx.y % p.n_blk;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    TRACE_INIT;
-    if (warp == 0) TRACE(0);
 
     // carve shared memory (tiles need 1024-byte alignment for the 128-byte swizzle); both CTAs of the pair
     // get the same offsets, which the pair MMAs and the remote barrier addresses rely on
@@ -243,7 +187,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     ptx::cluster_arrive();
     ptx::tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    if (warp == 0) TRACE(1);
 
     // Nothing above touched global memory.  From here on the previous kernel of the stream must be
     // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters).
@@ -350,7 +293,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
             const uint32_t par = (j / TC_STAGES) & 1;
             ok = ptx::mbar_wait(bar(BAR_KFULL + s), par);
             if (!ok) break;
-            if (j >= 2 && j < 7) TRACE(1 + j);   // K(j) landed
             if (lane == 0) ptx::mbar_arrive_remote(lead(BAR_KREADY + s));
             if (j == 0) {
                 ok = ptx::mbar_wait(bar(BAR_QFULL), 0);
@@ -406,8 +348,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                 ok = ptx::mbar_wait(bar(BAR_KREADY + j % TC_STAGES), (j / TC_STAGES) & 1) &&
                      (j < 2 || ptx::mbar_wait(bar(BAR_ODONE + (j & 1)), ((j >> 1) - 1) & 1));
                 if (!ok) break;
-                if (j == 0) TRACE(2);   // Q and K_0 of both CTAs landed
-                if (j >= 1 && j < 9) TRACE(55 + j);   // S(j) issued
                 ptx::tc_fence_after();
                 const uint64_t dk = dk0 + (uint64_t)(((j % TC_STAGES) * TC_K_BYTES) >> 4);
                 const uint32_t d = tmem + TM_S + (uint32_t)(j & 1) * 128;
@@ -436,7 +376,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                      ptx::mbar_wait(bar(BAR_PREADY + (j & 1)), (j >> 1) & 1);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                if (j < 8) TRACE(48 + j);   // O += P V of group j issued
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {   // stream t: keys [64 t, 64 t + 64) of the group
                     const uint64_t dv = dv0 + (uint64_t)(((j % TC_STAGES) * TC_V_BYTES + t * TC_HALF * 128) >> 4);
@@ -484,7 +423,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
         for (int j = 0; j < cnt; ++j) {
             if (!ok || !ptx::mbar_wait(bar(BAR_SREADY + (j & 1)), (j >> 1) & 1)) { if (ok && lane == 0) give_up(); ok = false; }
-            if (qd == 0 && j < 8) TRACE(8 + j * 4 + st * 2);       // S(j) ready
             ptx::tc_fence_after();
             uint32_t sr[64];
             ptx::tmem_ld32(t_s + (j & 1) * 128, *reinterpret_cast<uint32_t(*)[32]>(&sr[0]));
@@ -550,8 +488,8 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                 const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(sr[2 * e + 2]), __uint_as_float(sr[2 * e + 3])), sc2, nm2);
                 float2 p01, p23;
                 if (e % 8 == 6) {   // every fourth quadruple on the FMA pipes: the special-function unit is the bottleneck of a tile
-                    p01 = exp2_poly2(x01);
-                    p23 = exp2_poly2(x23);
+                    p01 = exp2_poly2<3>(x01);
+                    p23 = exp2_poly2<3>(x23);
                 } else {
                     p01 = make_float2(ex2(x01.x), ex2(x01.y));
                     p23 = make_float2(ex2(x23.x), ex2(x23.y));
@@ -567,23 +505,19 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
             ptx::tc_fence_before();
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_remote(lead(BAR_PREADY + (j & 1)));
-            if (qd == 0 && j < 8) TRACE(9 + j * 4 + st * 2);       // P(j) written by this warp
         }
         // ---- all tensor-core work of the pair is done
         if (cnt > 0) {
             if (*abort_flag) ok = false;
             if (ok && !ptx::mbar_wait(bar(BAR_FINAL), 0)) { ok = false; if (lane == 0) give_up(); }
-            if (warp == 0) TRACE(40);
             ptx::tc_fence_after();
         }
         __syncwarp();
         ptx::cluster_arrive_relaxed();   // nothing more goes to the peer from this thread
-        if (warp == 0) TRACE(3);
         // ---- the two streams of a row are merged: O = (w0 O0 + w1 O1) / (w0 l0 + w1 l1) with w_t = exp2(m_t - m);
         //      a stream that had no tile has (m, l) = (-inf, 0) and its accumulator is not read
         ml_x[st * 128 + row] = make_float2(m_used, l);
         pair_sync();
-        if (warp == 0) TRACE(4);
         const float2 other = ml_x[(st ^ 1) * 128 + row];
         const float m_all = fmaxf(m_used, other.x);
         const float w_own = m_used == -INFINITY ? 0.f : ex2(m_used - m_all);
@@ -635,9 +569,7 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
         const size_t slab0 = (size_t)grp * p.nsplit;     // first slab (256 rows) of this query block
         const int slab_row0 = (int)rank * 128;
         const int ch = lane & 15, hs = lane >> 4;
-        if (warp == 0) TRACE(5);
         pair_sync();   // the rows of this quarter of the tile are staged
-        if (warp == 0) TRACE(6);
         // what the merge below needs, computed while the stores are on their way
         const int rows_per = (128 + p.nsplit - 1) / p.nsplit;
         const int row_begin = split * rows_per;
@@ -662,23 +594,19 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                 for (int it = 0; it < 8; ++it) __stcg(dst + it * 2 * 16, v[it]);   // two rows of 16 chunks further each time
             }
         }
-        if (warp == 0) TRACE(7);
         if (p.nsplit > 1 && have_rows && !over) {
             // ---- publish this split's rows, then combine a slice of the rows of all splits
             if (st == 0) __stcg(p.ws_ml + (slab0 + split) * 256 + slab_row0 + row, make_float2(m_all, l_all));
             softmax_sync();   // every softmax thread's stores precede the release below
             int32_t *arrive = p.arrive + grp * 2 + rank, *depart = p.depart + grp * 2 + rank;
             if (threadIdx.x == 0) {
-                TRACE(44);   // partial written
                 __threadfence();
-                TRACE(41);   // fence done
                 asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(arrive) : "memory");
                 // relaxed polls (a round trip to L2 each), one acquire when the counter is full
                 const long long t0 = clock64();
                 while (*reinterpret_cast<volatile int32_t *>(arrive) < p.nsplit)
                     if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { atomicExch(p.dev_error, MTV_ERR_TIMEOUT); break; }
                 (void)ld_acquire(arrive);
-                TRACE(45);   // everybody arrived
             }
             softmax_sync();
             // This CTA has seen the counter full.  The last one to say so puts both counters back to zero at the end
@@ -706,7 +634,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                     for (int u = 0; u < 16; ++u)
                         v[u] = sp0 + u < p.nsplit ? __ldcg(reinterpret_cast<const uint4 *>(src + (size_t)(sp0 + u) * 256 * 128))
                                                   : make_uint4(0u, 0u, 0u, 0u);
-                    if (warp == 0 && sp0 == 0) TRACE(42);   // loads issued
                     // running maximum over the chunks of 16 splits (a second chunk rescales what has been summed)
                     float mc = ml.x;
 #pragma unroll
@@ -733,7 +660,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                     for (int o = 8; o > 0; o >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, o);
                     wsum = wsum * resc + ws;
                 }
-                if (warp == 0) TRACE(43);   // rows of all splits arrived and combined
                 const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
                 if (mine && valid_row(lrow))
                     *reinterpret_cast<uint4 *>(out_ptr(lrow) + ch * 8) =
@@ -745,7 +671,6 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
                 *depart = 0;
                 __threadfence();
             }
-            if (warp == 0) TRACE(46);   // merge done
         }
     }
 
@@ -757,77 +682,9 @@ tree_attn_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_cons
     ptx::cluster_wait();
     ptx::tc_fence_after();
     if (warp == TC_MMA_WARP) ptx::tmem_dealloc_pair(tmem, 512);
-    if (warp == 0) TRACE(47);
 }
 
 // ---------------------------------------------------------------------------------------- host
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                  const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void *ptr = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(ptr);
-    }
-    return fn;
-}
-
-// 4-D bf16 tensor map with a 128-byte-swizzled box whose innermost extent is 64 elements.  Encoding a map costs the host
-// a microsecond or two and an attention call needs three, so encoded maps are kept in a small direct-mapped table keyed by
-// everything that goes into them (a decode loop passes the same caches and strides step after step).
-namespace {
-struct MapKey {
-    const void *base;
-    cuuint64_t dims[4], strides[3];
-    cuuint32_t box[4];
-    int device;
-};
-struct MapSlot {
-    MapKey key;
-    CUtensorMap map;
-    bool valid = false;
-};
-constexpr int MAP_SLOTS = 512;
-MapSlot g_map_slots[MAP_SLOTS];
-std::mutex g_map_mutex;
-}  // namespace
-
-static bool encode_map(CUtensorMap *map, const void *base, const cuuint64_t dims[4], const cuuint64_t strides_bytes[3],
-                       const cuuint32_t box[4]) {
-    MapKey key;
-    memset(&key, 0, sizeof key);
-    key.base = base;
-    for (int i = 0; i < 4; ++i) { key.dims[i] = dims[i]; key.box[i] = box[i]; }
-    for (int i = 0; i < 3; ++i) key.strides[i] = strides_bytes[i];
-    if (cudaGetDevice(&key.device) != cudaSuccess) key.device = -1;
-    const uint64_t h = ((uint64_t)(uintptr_t)base >> 8) * 0x9E3779B97F4A7C15ull + dims[1] * 0xC2B2AE3D27D4EB4Full + box[1] * 0x165667B19E3779F9ull;
-    MapSlot &slot = g_map_slots[(h >> 40) % MAP_SLOTS];
-    {
-        std::lock_guard<std::mutex> lock(g_map_mutex);
-        if (slot.valid && memcmp(&slot.key, &key, sizeof key) == 0) {
-            *map = slot.map;
-            return true;
-        }
-    }
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    const cuuint32_t ones[4] = {1, 1, 1, 1};
-    if (fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides_bytes, box, ones,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return false;
-    std::lock_guard<std::mutex> lock(g_map_mutex);
-    slot.key = key;
-    slot.map = *map;
-    slot.valid = true;
-    return true;
-}
-
 // order[r] = the sequence with the r-th largest length (ties: lower index first).  B is small: every thread ranks one
 // sequence against all others.
 __global__ void attn_order_kernel(const int32_t *seq_lens, int B, int32_t *order) {
@@ -843,13 +700,13 @@ __global__ void attn_order_kernel(const int32_t *seq_lens, int B, int32_t *order
 }
 constexpr int TC_ORDER_MAX_B = 2048;
 
-bool attn_tc_eligible(int D, int G) { return D == 128 && G >= 1 && G <= 8; }
+bool attn_pair_eligible(int D, int G) { return D == 128 && G >= 1 && G <= 8; }
 
 static int tc_prepare() {
     static PerDeviceOnce once;
     bool *done = once.flag();
     if (!done || !*done) {
-        MTV_CUDA_CHECK(cudaFuncSetAttribute(tree_attn_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
+        MTV_CUDA_CHECK(cudaFuncSetAttribute(tree_attn_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM_BYTES));
         if (done) *done = true;
     }
     return MTV_OK;
@@ -858,7 +715,7 @@ static int tc_prepare() {
 // Number of key splits of a problem: as many as keep the whole grid within one wave of CTA pairs (one CTA
 // per SM), at most one per key tile, at most TC_MAX_SPLITS.  More than one split needs two merge counters
 // per query block.
-int attn_tc_plan(int T, int G, int B, int Hkv, int Lcap, int *n_blk_out) {
+int attn_pair_plan(int T, int G, int B, int Hkv, int Lcap, int *n_blk_out) {
     const int npc = 128 / G;                      // tree nodes per CTA; a pair takes 2 npc
     const int n_blk = (T + 2 * npc - 1) / (2 * npc);
     const long base = (long)B * Hkv * n_blk;
@@ -871,7 +728,7 @@ int attn_tc_plan(int T, int G, int B, int Hkv, int Lcap, int *n_blk_out) {
     return (int)ns;
 }
 
-int launch_tree_attn_tc(const mtv_tree *tree, int B, int Hq, int Hkv, const __nv_bfloat16 *q, const __nv_bfloat16 *k,
+int launch_tree_attn_pair(const mtv_tree *tree, int B, int Hq, int Hkv, const __nv_bfloat16 *q, const __nv_bfloat16 *k,
                         const __nv_bfloat16 *v, int64_t sb, int64_t sh, int64_t st, int Lcap, const int32_t *seq_lens,
                         float scale_log2, __nv_bfloat16 *out, int32_t *status, void *ws_o, float *ws_ml, int32_t *ws_order,
                         cudaStream_t stream) {
@@ -881,13 +738,13 @@ int launch_tree_attn_tc(const mtv_tree *tree, int B, int Hq, int Hkv, const __nv
         const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)Hq, (cuuint64_t)T, (cuuint64_t)B};
         const cuuint64_t str[3] = {(cuuint64_t)D * 2, (cuuint64_t)Hq * D * 2, (cuuint64_t)T * Hq * D * 2};
         const cuuint32_t box[4] = {64, (cuuint32_t)G, (cuuint32_t)(128 / G), 1};
-        if (!encode_map(&q_map, q, dims, str, box)) return MTV_ERR_CUDA;
+        if (!tensor_map_bf16(&q_map, q, 4, dims, str, box)) return MTV_ERR_CUDA;
     }
     {
         const cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)Lcap, (cuuint64_t)Hkv, (cuuint64_t)B};
         const cuuint64_t str[3] = {(cuuint64_t)st * 2, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
         const cuuint32_t kbox[4] = {64, TC_BN / 2, 1, 1}, vbox[4] = {64, TC_BN, 1, 1};
-        if (!encode_map(&k_map, k, dims, str, kbox) || !encode_map(&v_map, v, dims, str, vbox)) return MTV_ERR_CUDA;
+        if (!tensor_map_bf16(&k_map, k, 4, dims, str, kbox) || !tensor_map_bf16(&v_map, v, 4, dims, str, vbox)) return MTV_ERR_CUDA;
     }
     if (tc_prepare() != MTV_OK) return MTV_ERR_CUDA;
     TcParams p;
@@ -896,7 +753,7 @@ int launch_tree_attn_tc(const mtv_tree *tree, int B, int Hq, int Hkv, const __nv
     p.arrive = tree->d_counters; p.depart = tree->d_counters + TC_MAX_COUNTERS;
     p.scale_log2 = scale_log2;
     p.T = T; p.G = G; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
-    p.nsplit = attn_tc_plan(T, G, B, Hkv, Lcap, &p.n_blk);
+    p.nsplit = attn_pair_plan(T, G, B, Hkv, Lcap, &p.n_blk);
     p.npc = 128 / G;
     p.R = p.npc * G;
     p.order = nullptr;
@@ -916,14 +773,8 @@ int launch_tree_attn_tc(const mtv_tree *tree, int B, int Hq, int Hkv, const __nv
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    MTV_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tree_attn_tc_kernel, q_map, k_map, v_map, p));
+    MTV_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tree_attn_pair_kernel, q_map, k_map, v_map, p));
     return MTV_OK;
 }
 
 }  // namespace mtv
-
-#ifdef MTV_TRACE
-extern "C" int mtv_trace_set(long long *buf) {
-    return cudaMemcpyToSymbol(mtv::g_trace, &buf, sizeof buf) == cudaSuccess ? 0 : -1;
-}
-#endif

@@ -60,11 +60,13 @@ int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 
                     float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, cudaStream_t st);
 
 struct AttnWs {
-    size_t o_off, ml_off, order_off = 0, total;
-    int nsplit, m_rows;
-    bool use_tc;   // head_dim 128 path on the tcgen05 tensor cores
+    size_t o_off, ml_off, pair_ml_off = 0, order_off = 0, total;
 };
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap);
+int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, int n_layers, const mtv_bf16 *q,
+                          mtv_bf16 *const *k, mtv_bf16 *const *v, int64_t stride_b, int64_t stride_h, int64_t stride_t,
+                          int Lcap, const int32_t *seq_lens, float scale, mtv_bf16 *out, int32_t *status, void *ws,
+                          size_t ws_bytes, void *stream);
 
 struct AcceptWs {
     size_t part_off, total;

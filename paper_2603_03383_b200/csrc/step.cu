@@ -48,13 +48,10 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
                                         a->stride_h, a->stride_t, a->Lcap, a->seq_lens, ap->rope_theta, a->status, stream);
         if (rc != MTV_OK) return rc;
     }
-    const size_t per_layer = (size_t)a->B * tree->T * a->Hq * a->D;
-    for (int l = 0; l < a->n_layers; ++l) {
-        rc = tree_verify_attention(tree, a->B, a->Hq, a->Hkv, a->D, a->q_layers + l * per_layer, a->k_caches_host[l],
-                                   a->v_caches_host[l], a->stride_b, a->stride_h, a->stride_t, a->Lcap, a->seq_lens,
-                                   a->scale, a->out_layers + l * per_layer, a->status, a->ws, a->ws_bytes, stream);
-        if (rc != MTV_OK) return rc;
-    }
+    rc = mtv::tree_attention_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, a->q_layers, a->k_caches_host, a->v_caches_host,
+                                    a->stride_b, a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->scale, a->out_layers,
+                                    a->status, a->ws, a->ws_bytes, stream);
+    if (rc != MTV_OK) return rc;
     rc = step_accept(tree, a, stream);
     if (rc != MTV_OK) return rc;
     return kv_compact_accepted(tree, a->B, a->Hkv, a->D, a->n_layers, a->k_caches, a->v_caches, a->stride_b,
@@ -152,21 +149,19 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
     MTV_CUDA_CHECK(cudaMemcpyAsync(h->tree_tok, d->tree_tok, B * T * 4, cudaMemcpyDeviceToHost, st));
     // attention, its outputs leaving in groups of layers
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.q_up, 0));
-    const int per_group = (d->n_layers + 15) / 16;
-    int sent = 0, n_sent = 0;
-    for (int l = 0; l < d->n_layers; ++l) {
-        rc = tree_verify_attention(tree, d->B, d->Hq, d->Hkv, d->D, d->q_layers + l * per_layer, d->k_caches_host[l],
-                                   d->v_caches_host[l], d->stride_b, d->stride_h, d->stride_t, d->Lcap, d->seq_lens,
-                                   d->scale, d->out_layers + l * per_layer, d->status, d->ws, d->ws_bytes, stream);
+    const int per_group = (d->n_layers + 7) / 8;
+    int n_sent = 0;
+    for (int l = 0; l < d->n_layers; l += per_group) {
+        const int n = std::min(per_group, d->n_layers - l);
+        rc = mtv::tree_attention_layers(tree, d->B, d->Hq, d->Hkv, d->D, n, d->q_layers + l * per_layer, d->k_caches_host + l,
+                                        d->v_caches_host + l, d->stride_b, d->stride_h, d->stride_t, d->Lcap, d->seq_lens,
+                                        d->scale, d->out_layers + l * per_layer, d->status, d->ws, d->ws_bytes, stream);
         if (rc != MTV_OK) return rc;
-        if ((l + 1) % per_group == 0 || l + 1 == d->n_layers) {
-            cudaEvent_t ev = g_aux.chunk[n_sent++ % 8];
-            MTV_CUDA_CHECK(cudaEventRecord(ev, st));
-            MTV_CUDA_CHECK(cudaStreamWaitEvent(down, ev, 0));
-            MTV_CUDA_CHECK(cudaMemcpyAsync(h->out_layers + sent * per_layer, d->out_layers + sent * per_layer,
-                                           (size_t)(l + 1 - sent) * per_layer * 2, cudaMemcpyDeviceToHost, down));
-            sent = l + 1;
-        }
+        cudaEvent_t ev = g_aux.chunk[n_sent++];
+        MTV_CUDA_CHECK(cudaEventRecord(ev, st));
+        MTV_CUDA_CHECK(cudaStreamWaitEvent(down, ev, 0));
+        MTV_CUDA_CHECK(cudaMemcpyAsync(h->out_layers + l * per_layer, d->out_layers + l * per_layer, n * per_layer * 2,
+                                       cudaMemcpyDeviceToHost, down));
     }
     // acceptance and compaction
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.logits_up, 0));

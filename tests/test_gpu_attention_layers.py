@@ -1,0 +1,77 @@
+"""Tree attention of several layers in one launch, the two single-layer kernels on either side of their rule, and scores whose
+maximum grows along the cache (the reference of the exponentials has to move), against the fp64 checker."""
+
+import pytest
+import torch
+
+from oracle import reference as ref
+from paper_2603_03383_b200 import binding, synth
+from tests._cases import assert_close, make_tree, workspace
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,lens,n_layers", [
+    (64, 8, 2, 128, [63], 2),                  # one group and the tree across a group boundary
+    (64, 8, 2, 128, [64, 0, 129], 5),          # last group exactly full; an empty prefix; ragged
+    (29, 4, 1, 128, [700], 3),                 # one row tile: both streams on the same rows, pieces of one group
+    (128, 16, 2, 128, [1000, 1], 2),           # four row blocks
+    (64, 7, 1, 128, [300, 517], 9),            # rows that belong to nobody
+    (65, 8, 8, 64, [127, 128], 4),
+    (128, 8, 1, 64, [2500], 2),                # head size 64 with splits: fp32 partials
+])
+def test_layers_in_one_launch(T, Hq, Hkv, D, lens, n_layers):
+    K, H, V, B = 4, 64, 600, len(lens)
+    tb, tree = make_tree("rank_prior", K, (), T)
+    Lcap = max(lens) + T + 3
+    ks = [synth.normal_bf16(T, 10 + l, (B, Hkv, Lcap, D), device=DEV) for l in range(n_layers)]
+    vs = [synth.normal_bf16(T, 50 + l, (B, Hkv, Lcap, D), device=DEV) for l in range(n_layers)]
+    q = synth.normal_bf16(T, 90, (n_layers, B, T, Hq, D), device=DEV)
+    hidden, W1, b1, W2, root = synth.head_inputs(B, H, V, K, seed=3, device=DEV)
+    i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+    d = dict(hidden=hidden, W1=W1, b1=b1, W2=W2, root_tok=root, q_layers=q, out_layers=torch.full_like(q, 9.0),
+             logits=synth.normal_bf16(T, 91, (B, T, V), device=DEV), seq_lens=torch.tensor(lens, dtype=torch.int32, device=DEV),
+             cand=i32(B, tree.C), cand_logit=torch.zeros(B, tree.C - 1, device=DEV), tree_tok=i32(B, T), accept_len=i32(B),
+             best_path=i32(B), acc_nodes=i32(B, K + 1), acc_tok=i32(B, K + 1), next_root=i32(B), status=i32(B),
+             k_caches=binding.cache_pointer_array(ks, DEV), v_caches=binding.cache_pointer_array(vs, DEV),
+             k_caches_host=binding.cache_pointer_array(ks), v_caches_host=binding.cache_pointer_array(vs),
+             ws=workspace(tree, B, H, V, Hq, Hkv, D, Lcap))
+    a = binding.StepArgs()
+    a.B, a.H, a.V, a.Hq, a.Hkv, a.D, a.n_layers, a.Lcap = B, H, V, Hq, Hkv, D, n_layers, Lcap
+    a.stride_b, a.stride_h, a.stride_t = ks[0].stride()[:3]
+    for n, t in d.items():
+        setattr(a, n, t.data_ptr())
+    a.ws_bytes = d["ws"].numel()
+    want = [ref.tree_attention(q[l].cpu(), ks[l].cpu(), vs[l].cpu(), torch.tensor(lens, dtype=torch.int32), tb["mask"])
+            for l in range(n_layers)]
+    binding.mtv_verify_step(tree, a)
+    torch.cuda.synchronize()
+    assert binding.mtv_device_error(tree) == 0
+    for l in range(n_layers):
+        assert_close(d["out_layers"][l], want[l], "layer %d" % l)
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,lens,Lcap", [
+    (64, 8, 2, 128, [2000], 2200),             # key splits on CTA pairs
+    (64, 28, 4, 128, [40, 300, 1200, 900, 64, 0, 777], 8064),   # the even division: capacity says long
+    (128, 8, 4, 128, [600, 200], 33000),
+    (128, 8, 2, 64, [900, 17], 1030),
+])
+@pytest.mark.parametrize("gain", [1.0, 40.0])
+def test_single_layer_calls(T, Hq, Hkv, D, lens, Lcap, gain):
+    """gain 40: the scores' spread is about 60 in log2 units, so later groups exceed the first one's maximum by far."""
+    tb, tree = make_tree("rank_prior", 4, (), T)
+    B = len(lens)
+    q = (synth.normal_bf16(1, 1, (B, T, Hq, D), device=DEV) * gain).to(torch.bfloat16)
+    k, v = (synth.normal_bf16(1, i, (B, Hkv, Lcap, D), device=DEV) for i in (2, 3))
+    sl = torch.tensor(lens, dtype=torch.int32)
+    top = max(lens) + T
+    want = ref.tree_attention(q.cpu(), k[:, :, :top].cpu(), v[:, :, :top].cpu(), sl, tb["mask"])
+    out = torch.full_like(q, 9.0)
+    ws = workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap)
+    for _ in range(2):                          # the merge counters are back at zero after a call
+        binding.tree_verify_attention(tree, q, k, v, sl.to(DEV), out, ws)
+    torch.cuda.synchronize()
+    assert binding.mtv_device_error(tree) == 0
+    assert_close(out, want)
