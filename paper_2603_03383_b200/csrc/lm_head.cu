@@ -10,15 +10,16 @@
 // One persistent CTA per SM walks pairs of vocabulary tiles, so that a chunk of X fetched from L2
 // serves two weight tiles.  A tile holds R <= 128 rows, R chosen by the host so that every CTA gets
 // the same number of pairs (V = 32000 on 148 SMs: 112 rows); the MMA spans 128 rows all the same and
-// the rows past R, whatever the shared memory held, are left out of the maximum.  From 129 nodes up a
-// pass takes 256 nodes and one weight tile per stage: 128 x 256 x 16 is the MMA shape that runs at the
-// full tensor rate (128 x 128 x 16 reaches about 60 % of it), and the large batches are tensor-bound.
+// the rows past R, whatever the shared memory held, are left out of the maximum.  From 129 nodes up the
+// problem turns into a dense contraction, which lm_head_argmax_pair_kernel below does on CTA pairs.
 // Warp roles: TMA producer (ring of stages, one stage = 64
 // columns of the weight tiles and of the N node rows), MMA issuer (accumulators in tensor memory,
 // double-buffered: the epilogue of one pair overlaps the MMAs of the next), four epilogue warps
-// (one thread per vocabulary row: order-preserving (value, ~index) keys, butterfly max over the
+// (one thread per vocabulary row: order-preserving (value, ~index) keys, maximum over the
 // warp's 32 rows, shared-memory max across warps and pairs, one 64-bit atomic max per node at the end).
 #include <cuda.h>
+
+#include <climits>
 
 #include "common.cuh"
 #include "sm100_ptx.cuh"
@@ -37,55 +38,40 @@ constexpr uint32_t LM_IDESC_BASE = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >
 struct LmParams {
     unsigned long long *keys;   // [M] best (value, ~index) per node, zero before the launch
     int32_t *dev_error;
-    int M, H, V, N;             // N = nodes per pass (64, 128 or 256)
+    int M, H, V, N;             // N = nodes per pass
+    int passes;
     int R;                      // vocabulary rows per tile (<= 128, a multiple of 8), chosen so that the tiles
                                 // divide evenly among the CTAs; the MMA still spans 128 rows, the rest is ignored
-    int n_pairs;                // units (of two weight tiles, or of one when N = 256) over the vocabulary
+    int n_pairs;                // units of two weight tiles over the vocabulary
     int n_stages;
     uint32_t stage_bytes;
 };
 
-__device__ __forceinline__ uint64_t lm_desc(uint32_t saddr) {   // K-major, 128-byte swizzle
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= 1ull << 46;
-    d |= 2ull << 61;
-    return d;
-}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *map, uint32_t bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
-// larger fp32 first, equal values by lower index: one unsigned 64-bit max does both
-__device__ __forceinline__ unsigned long long lm_key(uint32_t fbits, uint32_t idx) {
-    uint32_t ord = (fbits & 0x80000000u) ? ~fbits : (fbits | 0x80000000u);
-    if ((fbits << 1) == 0) ord = 0x80000000u;   // -0.0 and +0.0 compare equal
-    return ((unsigned long long)ord << 32) | (0xffffffffu - idx);
-}
-__device__ __forceinline__ unsigned long long umax(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
-
-// Max over the 32 lanes of 32 per-lane keys at once: afterwards lane l holds the max of key number l.
-__device__ __forceinline__ unsigned long long warp_max_scatter32(unsigned long long (&v)[32], int lane) {
-    int n = 32;
+// Best key of 32 columns over the warp's 32 rows (row of lane l: v0 + l), acc[e] = this lane's row in column e: lane l gets
+// the key of column l — the order-preserving image of the value in the high word, 0xffffffff - row in the low one, so that a
+// 64-bit max finds the larger value and, among equals, the lower row; 0 if no row is valid.  The images are compared as
+// signed integers (-0.0 and +0.0 alike) by a warp-wide integer reduction per column: a butterfly of 64-bit keys took 1.9 k
+// cycles per 32 columns and set the pace up to H = 1000 (720 nodes, H = 768, V = 84034: 106 us).
+__device__ __forceinline__ unsigned long long warp_best32(const uint32_t (&acc)[32], bool valid, uint32_t v0, int lane) {
+    int best = INT_MIN;
+    uint32_t at = 0;
 #pragma unroll
-    for (int bit = 16; bit >= 1; bit >>= 1) {
-        n >>= 1;
-        const bool up = (lane & bit) != 0;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (i < n) {
-                const unsigned long long send = up ? v[i] : v[i + n];
-                const unsigned long long keep = up ? v[i + n] : v[i];
-                v[i] = umax(keep, __shfl_xor_sync(0xffffffffu, send, bit));
-            }
-        }
+    for (int e = 0; e < 32; ++e) {
+        const int bits = __float_as_int(__uint_as_float(acc[e]) + 0.f);
+        const int ord = valid ? bits ^ ((bits >> 31) & 0x7fffffff) : INT_MIN;
+        const int m = __reduce_max_sync(0xffffffffu, ord);
+        const uint32_t row = (uint32_t)__ffs(__ballot_sync(0xffffffffu, ord == m)) - 1u;
+        if (lane == e) { best = m; at = row; }
     }
-    return v[0];
+    if (best == INT_MIN) return 0ull;
+    return ((unsigned long long)((uint32_t)best ^ 0x80000000u) << 32) | (0xffffffffu - (v0 + at));
 }
 
-// N nodes per pass; TILES weight tiles per stage (2 for N <= 128, so that an X chunk serves two tiles; 1 for N = 256,
-// the MMA shape that runs at the full tensor rate, where two tiles' accumulators would not fit tensor memory twice)
+// N nodes (64 or 128) in one pass; two weight tiles per stage, so that an X chunk serves two tiles.
 template <int N>
 __global__ void __launch_bounds__(LM_THREADS, 1)
 lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map,
@@ -107,9 +93,9 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
     auto acc_empty = [&](int u) { return bars + (uint32_t)(2 * LM_MAX_STAGES + 2 + u) * 8u; };
     const uint32_t drain_bar = bars + (uint32_t)(2 * LM_MAX_STAGES + 4) * 8u;
     volatile int *abort_flag = &abort_flag_s;
-    constexpr int TILES = N <= 128 ? 2 : 1;
+    constexpr int TILES = 2;
     constexpr uint32_t W_BYTES = TILES * LM_TILE_BYTES;
-    constexpr uint32_t TMEM_COLS = 2 * TILES * N;   // 2 buffers x TILES x N columns (256 or 512)
+    constexpr uint32_t TMEM_COLS = 2 * TILES * N;   // 2 buffers x TILES x N columns
 
     for (int i = threadIdx.x; i < N; i += LM_THREADS) best[i] = 0ull;
     if (threadIdx.x == 0) {
@@ -131,10 +117,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
     ptx::tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    // grid = (passes, CTAs per pass): the CTAs that walk the same weight rows for different node
-    // passes are neighbours in launch order, so all but the first find those rows in L2
-    const int pass = blockIdx.x;                         // nodes [pass N, pass N + N)
-    const int cta = blockIdx.y, n_cta = gridDim.y;
+    const int cta = blockIdx.x, n_cta = gridDim.x;
     const int n_pairs = p.n_pairs, R = p.R;
     const int my_pairs = cta < n_pairs ? (n_pairs - cta + n_cta - 1) / n_cta : 0;
     const int n_kc = p.H / LM_KC;
@@ -153,7 +136,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                     ptx::mbar_arrive_expect_tx(full(s), (uint32_t)(TILES * R + N) * 128u);
                     tma_load_2d(base, &w_map, full(s), kc * LM_KC, row0);                 // rows past V arrive as zeros
                     if (TILES == 2) tma_load_2d(base + LM_TILE_BYTES, &w_map, full(s), kc * LM_KC, row0 + R);
-                    tma_load_2d(base + x_off, &x_map, full(s), kc * LM_KC, pass * N);      // rows past M arrive as zeros
+                    tma_load_2d(base + x_off, &x_map, full(s), kc * LM_KC, 0);             // rows past M arrive as zeros
                 }
                 __syncwarp();
             }
@@ -162,6 +145,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
     } else if (warp == 4) {
         // ---------------------------------------------------------------- MMA issuer
         constexpr uint32_t IDESC = LM_IDESC_BASE | ((uint32_t)(N >> 3) << 17);
+        const bool leader = ptx::elect_one();
         int it = 0;
         bool ok = true;
         for (int q = 0; ok && q < my_pairs && !*abort_flag; ++q) {
@@ -174,18 +158,16 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                 ok = ptx::mbar_wait(full(s), (it / NST) & 1);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t base = ring + s * p.stage_bytes;
+                // (the whole warp, one elected lane issues: operands stay in uniform registers)
+                const uint32_t w = ptx::desc_lo(ring + s * p.stage_bytes, 16);
 #pragma unroll
-                    for (int t = 0; t < TILES; ++t)
+                for (int t = 0; t < TILES; ++t)
 #pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            ptx::mma_ss(tmem + (u * TILES + t) * N, lm_desc(base + t * LM_TILE_BYTES + kk * 32),
-                                        lm_desc(base + x_off + kk * 32), IDESC, kc > 0 || kk > 0);
-                    ptx::tc_commit(empty(s));                         // the stage is free once these MMAs are done
-                    if (kc == n_kc - 1) ptx::tc_commit(acc_full(u));  // and so is the pair's accumulator
-                }
-                __syncwarp();
+                    for (int kk = 0; kk < 4; ++kk)
+                        ptx::mma_ss_elect(tmem + (u * TILES + t) * N, w + ((t * LM_TILE_BYTES) >> 4) + kk * 2, w + (x_off >> 4) + kk * 2,
+                                          ptx::DESC_HI, IDESC, kc > 0 || kk > 0, leader);
+                ptx::tc_commit_elect(empty(s), leader);                         // the stage is free once these MMAs are done
+                if (kc == n_kc - 1) ptx::tc_commit_elect(acc_full(u), leader);  // and so is the pair's accumulator
             }
         }
         if (!ok) *abort_flag = 1;
@@ -201,18 +183,15 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
             const int row0 = (cta + q * n_cta) * TILES * R;
 #pragma unroll 1
             for (int t = 0; t < TILES; ++t) {
-                const int r = warp * 32 + lane;
-                const int v = r < R ? row0 + t * R + r : p.V;          // this thread's vocabulary row (none past R)
+                const int r = warp * 32 + lane, v0 = row0 + t * R + warp * 32;
+                const bool valid = r < R && v0 + lane < p.V;           // this thread's vocabulary row (none past R)
+                if (warp * 32 >= R) continue;                          // none for the whole warp
 #pragma unroll 1
                 for (int c = 0; c < N / 32; ++c) {
                     uint32_t acc[32];
                     ptx::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (u * TILES + t) * N + c * 32, acc);
-                    ptx::tmem_ld_wait();
-                    unsigned long long key[32];
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) key[e] = v < p.V ? lm_key(acc[e], (uint32_t)v) : 0ull;
-                    const unsigned long long k = warp_max_scatter32(key, lane);   // node c * 32 + lane, this warp's 32 rows
-                    atomicMax(&best[c * 32 + lane], k);
+                    ptx::tmem_ld_wait_for(acc);
+                    atomicMax(&best[c * 32 + lane], warp_best32(acc, valid, (uint32_t)v0, lane));   // node c * 32 + lane
                 }
             }
             ptx::tc_fence_before();
@@ -239,13 +218,214 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
         __syncthreads();
     }
     for (int n = threadIdx.x; n < N; n += LM_THREADS) {
-        const int m = pass * N + n;
-        if (m < p.M && best[n] != 0ull) atomicMax(p.keys + m, best[n]);
+        if (n < p.M && best[n] != 0ull) atomicMax(p.keys + n, best[n]);
     }
     if (warp == 4) {
         ptx::tc_fence_after();
         ptx::tmem_dealloc(tmem, TMEM_COLS);
     }
+}
+
+// ---------------------------------------------------------------------------------------- more than 128 nodes
+// Bound by the tensor cores (512 MMA cycles per 64 columns of a 256 x 256 tile against 32 KB of operands per SM).  A cluster of
+// two CTAs forms a tcgen05 CTA pair: D[256 vocabulary rows][N <= 256 nodes], each CTA with 128 of the rows (its operand A and its
+// accumulator) and half of the nodes (operand B), so an operand byte is fetched by one SM of the pair only.  One CTA with
+// 128 x 256 tiles fetched 48 KB per 512 MMA cycles, more than L2 delivers, and its issuing lane paid for moving every operand
+// into uniform registers: 1029 us at 1024 nodes, V = 131072, H = 4096 (1.07 PFLOP/s).
+// The (vocabulary tile, node pass) items go round the pairs, passes of a tile next to each other (its rows are then read once from
+// memory); every CTA keeps the best key of all nodes in shared memory and hands them over at its end.  Per CTA: warps 0-3
+// epilogue, warp 4 (even CTA) MMA issuer, warp 5 TMA producer of the CTA's own halves, warp 6 (odd CTA) relay: tells
+// the issuer that the odd CTA's half of a stage has landed.
+constexpr int LP_THREADS = 224;
+constexpr int LP_STAGES = 6;
+constexpr uint32_t LP_STAGE_BYTES = 2 * LM_TILE_BYTES;
+constexpr int LP_MAX_NODES = 2048;                       // per launch: keys in shared memory
+constexpr uint32_t LP_SMEM_BYTES = 1024 + LP_STAGES * LP_STAGE_BYTES + LP_MAX_NODES * 8;
+static_assert(LP_SMEM_BYTES <= LM_SMEM_MAX, "shared memory");
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(LP_THREADS, 1)
+lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map, const LmParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag_s, issued_s;
+    __shared__ __align__(8) unsigned long long bar_mem[3 * LP_STAGES + 5];
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t rank = ptx::cluster_ctarank();
+    const uint32_t raw = ptx::smem_u32(smem_raw);
+    const uint32_t pad = (1024u - (raw & 1023u)) & 1023u, ring = raw + pad;     // the same offset in both CTAs
+    unsigned long long *best = reinterpret_cast<unsigned long long *>(smem_raw + pad + LP_STAGES * LP_STAGE_BYTES);
+    const uint32_t bars = ptx::smem_u32(bar_mem);
+    auto full = [&](int s) { return bars + (uint32_t)s * 8u; };
+    auto empty = [&](int s) { return bars + (uint32_t)(LP_STAGES + s) * 8u; };
+    auto ready = [&](int s) { return bars + (uint32_t)(2 * LP_STAGES + s) * 8u; };         // even CTA: the odd CTA's half is there
+    auto acc_full = [&](int u) { return bars + (uint32_t)(3 * LP_STAGES + u) * 8u; };
+    auto acc_empty = [&](int u) { return bars + (uint32_t)(3 * LP_STAGES + 2 + u) * 8u; }; // even CTA: both epilogues have read it
+    const uint32_t drain_bar = bars + (uint32_t)(3 * LP_STAGES + 4) * 8u;
+    volatile int *abort_flag = &abort_flag_s;
+    auto give_up = [&]() {
+        *abort_flag = 1;
+        ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&abort_flag_s), rank ^ 1), 1u);
+    };
+
+    for (int i = threadIdx.x; i < p.passes * p.N; i += LP_THREADS) best[i] = 0ull;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < LP_STAGES; ++s) { ptx::mbar_init(full(s), 1); ptx::mbar_init(empty(s), 1); ptx::mbar_init(ready(s), 1); }
+        for (int u = 0; u < 2; ++u) { ptx::mbar_init(acc_full(u), 1); ptx::mbar_init(acc_empty(u), 8); }
+        ptx::mbar_init(drain_bar, 1);
+        ptx::fence_mbar_init();
+        abort_flag_s = 0;
+        issued_s = 0;
+        ptx::prefetch_tensormap(&w_map);
+        ptx::prefetch_tensormap(&x_map);
+    }
+    if (warp == 4) {
+        ptx::tmem_alloc_pair(ptx::smem_u32(&tmem_slot), 512);
+        ptx::tmem_relinquish_pair();
+    }
+    ptx::tc_fence_before();
+    __syncthreads();
+    ptx::cluster_arrive();
+    ptx::cluster_wait();                                 // the peer's barriers and tensor memory exist
+    ptx::tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    const int n_pairs = (int)gridDim.x >> 1, pair = (int)blockIdx.x >> 1;
+    const int n_items = p.n_pairs * p.passes, half = p.N / 2;
+    const int my_items = pair < n_items ? (n_items - pair + n_pairs - 1) / n_pairs : 0;
+    const int n_kc = p.H / LM_KC, total = my_items * n_kc;
+
+    if (warp == 5) {
+        // ---------------------------------------------------------------- TMA producer
+        int it = 0;
+        for (int q = 0; q < my_items && !*abort_flag; ++q) {
+            const int item = pair + q * n_pairs;
+            const int row0 = item / p.passes * 2 * p.R + (int)rank * p.R, node0 = item % p.passes * p.N + (int)rank * half;
+            for (int kc = 0; kc < n_kc; ++kc, ++it) {
+                const int s = it % LP_STAGES;
+                if (it >= LP_STAGES && !ptx::mbar_wait(empty(s), (it / LP_STAGES - 1) & 1)) { give_up(); break; }
+                if (lane == 0) {
+                    const uint32_t base = ring + s * LP_STAGE_BYTES;
+                    ptx::mbar_arrive_expect_tx(full(s), (uint32_t)(p.R + half) * 128u);
+                    tma_load_2d(base, &w_map, full(s), kc * LM_KC, row0);                       // rows past V and
+                    tma_load_2d(base + LM_TILE_BYTES, &x_map, full(s), kc * LM_KC, node0);      // M arrive as zeros
+                }
+                __syncwarp();
+            }
+        }
+        if (lane == 0) issued_s = it;
+    } else if (warp == 6) {
+        // ---------------------------------------------------------------- relay (odd CTA)
+        if (rank == 1)
+            for (int it = 0; it < total && !*abort_flag; ++it) {
+                const int s = it % LP_STAGES;
+                if (!ptx::mbar_wait(full(s), (it / LP_STAGES) & 1)) { give_up(); break; }
+                if (lane == 0) ptx::mbar_arrive_remote(ptx::mapa(ready(s), 0));
+                __syncwarp();
+            }
+    } else if (warp == 4) {
+        // ---------------------------------------------------------------- MMA issuer (even CTA)
+        if (rank == 0) {
+            const bool leader = ptx::elect_one();
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 4) << 24) | ((uint32_t)(p.N >> 3) << 17);
+            int it = 0;
+            bool ok = true;
+            for (int q = 0; ok && q < my_items && !*abort_flag; ++q) {
+                const int u = q & 1;
+                if (q >= 2) ok = ptx::mbar_wait(acc_empty(u), ((q >> 1) - 1) & 1);
+                if (!ok) break;
+                ptx::tc_fence_after();
+                for (int kc = 0; kc < n_kc; ++kc, ++it) {
+                    const int s = it % LP_STAGES;
+                    const uint32_t ph = (uint32_t)(it / LP_STAGES) & 1;
+                    ok = ptx::mbar_wait(full(s), ph) && ptx::mbar_wait(ready(s), ph);
+                    if (!ok) break;
+                    ptx::tc_fence_after();
+                    const uint32_t w = ptx::desc_lo(ring + s * LP_STAGE_BYTES, 16);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        ptx::mma_pair_ss_elect(tmem + u * 256, w + kk * 2, w + (LM_TILE_BYTES >> 4) + kk * 2, ptx::DESC_HI, idesc,
+                                               kc > 0 || kk > 0, leader);
+                    ptx::tc_commit_pair_mask_elect(empty(s), 3, leader);                        // the stage is free in both CTAs
+                    if (kc == n_kc - 1) ptx::tc_commit_pair_mask_elect(acc_full(u), 3, leader);
+                }
+            }
+            if (!ok) give_up();
+            __syncwarp();
+            if (*abort_flag) {                           // issued tensor-core work gets one more bounded wait
+                ptx::tc_commit_pair_mask_elect(drain_bar, 1, leader);
+                ptx::mbar_wait(drain_bar, 0);
+            }
+        }
+    } else {
+        // ---------------------------------------------------------------- epilogue: thread = vocabulary row
+        bool ok = true;
+        for (int q = 0; q < my_items && ok; ++q) {
+            const int u = q & 1, item = pair + q * n_pairs;
+            ok = !*abort_flag && ptx::mbar_wait(acc_full(u), (q >> 1) & 1);
+            ok = __all_sync(0xffffffffu, ok);            // (the tensor-memory loads below need the whole warp)
+            if (!ok) break;
+            ptx::tc_fence_after();
+            const int r = warp * 32 + lane, v0 = item / p.passes * 2 * p.R + (int)rank * p.R + warp * 32;
+            const bool valid = r < p.R && v0 + lane < p.V;
+            unsigned long long *b = best + item % p.passes * p.N;
+#pragma unroll 1
+            for (int c = 0; c < (warp * 32 < p.R ? p.N / 32 : 0); ++c) {
+                uint32_t acc[32];
+                ptx::tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + u * 256 + c * 32, acc);
+                ptx::tmem_ld_wait_for(acc);
+                atomicMax(&b[c * 32 + lane], warp_best32(acc, valid, (uint32_t)v0, lane));   // node c * 32 + lane
+            }
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_remote(ptx::mapa(acc_empty(u), 0));
+        }
+        if (!ok) give_up();
+    }
+    __syncwarp();
+    ptx::tc_fence_before();
+    __syncthreads();
+    if (*abort_flag) {
+        if (threadIdx.x == 0) atomicExch(p.dev_error, MTV_ERR_TIMEOUT);
+        // copies in flight get one more bounded wait before the shared memory is given back
+        if (warp == 5 && lane == 0)
+            for (int s = 0; s < LP_STAGES; ++s) {
+                const int uses = (issued_s - s + LP_STAGES - 1) / LP_STAGES;
+                if (issued_s > s) ptx::mbar_wait(full(s), (uses - 1) & 1);
+            }
+    }
+    for (int n = threadIdx.x; n < p.passes * p.N; n += LP_THREADS)
+        if (n < p.M && best[n] != 0ull) atomicMax(p.keys + n, best[n]);
+    // nobody leaves while the pair's MMAs may still read its shared memory or its barriers may be signalled
+    ptx::cluster_arrive();
+    ptx::cluster_wait();
+    ptx::tc_fence_after();
+    if (warp == 4) ptx::tmem_dealloc_pair(tmem, 512);
+}
+
+static int launch_lm_head_pair(const mtv_tree_t *tree, int M, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W,
+                               unsigned long long *keys, cudaStream_t st) {
+    for (int m0 = 0; m0 < M; m0 += LP_MAX_NODES) {
+        const int m = M - m0 < LP_MAX_NODES ? M - m0 : LP_MAX_NODES;
+        CUtensorMap w_map, x_map;
+        LmParams p;
+        p.keys = keys + m0; p.dev_error = tree->d_error; p.M = m; p.H = H; p.V = V;
+        p.passes = (m + 255) / 256;
+        p.N = ((m + p.passes - 1) / p.passes + 31) / 32 * 32;       // passes of equal width: no columns of an MMA for nothing
+        const int pairs = sm_count() / 2;
+        // as many rows per tile as make all pairs walk the same number of items
+        const long rounds = ((long)((V + 255) / 256) * p.passes + pairs - 1) / pairs;
+        const long tiles = rounds * pairs / p.passes;                // vocabulary tiles that fit those rounds
+        p.R = (int)(((V + 2 * tiles - 1) / (2 * tiles) + 7) / 8 * 8);
+        if (p.R < 32) p.R = 32;                                     // one warp's worth
+        if (p.R > 128) p.R = 128;
+        p.n_pairs = (V + 2 * p.R - 1) / (2 * p.R);
+        p.n_stages = LP_STAGES; p.stage_bytes = LP_STAGE_BYTES;
+        if (!tma_map_2d_bf16(&w_map, W, V, H, p.R) || !tma_map_2d_bf16(&x_map, x + (size_t)m0 * H, m, H, p.N / 2)) return MTV_ERR_CUDA;
+        const long items = (long)p.n_pairs * p.passes;
+        const int grid = 2 * (int)(items < pairs ? items : pairs);
+        lm_head_argmax_pair_kernel<<<grid, LP_THREADS, LP_SMEM_BYTES, st>>>(w_map, x_map, p);
+    }
+    return MTV_OK;
 }
 
 // keys -> (argmax, value)
@@ -271,39 +451,41 @@ extern "C" int lm_head_argmax(const mtv_tree_t *tree, int B, int H, int V, const
     if (H < 64 || H % 64 != 0) return MTV_ERR_UNSUPPORTED_SHAPE;
     if (((uintptr_t)x | (uintptr_t)W) & 15) return MTV_ERR_INVALID_ARG;
     const int M = B * tree->T;
-    const int N = M <= 64 ? 64 : M <= 128 ? 128 : 256;
-    const int tiles = N <= 128 ? 2 : 1;                  // weight tiles per stage (see the kernel)
-    const int passes = (M + N - 1) / N;
     cudaStream_t st = (cudaStream_t)stream;
-    CUtensorMap w_map, x_map;
-    LmParams p;
-    p.keys = keys; p.dev_error = tree->d_error; p.M = M; p.H = H; p.V = V; p.N = N;
-    p.stage_bytes = tiles * LM_TILE_BYTES + N * 128;
-    p.n_stages = (int)((LM_SMEM_MAX - 1024) / p.stage_bytes);
-    if (p.n_stages > LM_MAX_STAGES) p.n_stages = LM_MAX_STAGES;
-    const size_t smem = 1024 + (size_t)p.n_stages * p.stage_bytes;
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
         MTV_CUDA_CHECK(cudaFuncSetAttribute(lm_head_argmax_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, LM_SMEM_MAX));
         MTV_CUDA_CHECK(cudaFuncSetAttribute(lm_head_argmax_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, LM_SMEM_MAX));
-        MTV_CUDA_CHECK(cudaFuncSetAttribute(lm_head_argmax_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, LM_SMEM_MAX));
+        MTV_CUDA_CHECK(cudaFuncSetAttribute(lm_head_argmax_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LP_SMEM_BYTES));
         if (attr_done) *attr_done = true;
     }
     MTV_CUDA_CHECK(cudaMemsetAsync(keys, 0, (size_t)M * 8, st));
-    int ctas = sm_count() / passes;                      // per pass; one CTA per SM in all
-    const int min_pairs = (V + tiles * 128 - 1) / (tiles * 128);   // units of `tiles` weight tiles
-    if (ctas > (V + 63) / 64) ctas = (V + 63) / 64;      // no tile below 32 rows
-    if (ctas < 1) ctas = 1;
-    // every CTA walks the same number of tile pairs; the tile height shrinks until they just cover V
-    const int rounds = (min_pairs + ctas - 1) / ctas;
-    p.n_pairs = ctas * rounds;
-    p.R = ((V + tiles * p.n_pairs - 1) / (tiles * p.n_pairs) + 7) / 8 * 8;
-    if (!tma_map_2d_bf16(&w_map, W, V, H, p.R) || !tma_map_2d_bf16(&x_map, x, M, H, N)) return MTV_ERR_CUDA;
-    const dim3 grid(passes, ctas);
-    if (N == 64) lm_head_argmax_kernel<64><<<grid, LM_THREADS, smem, st>>>(w_map, x_map, p);
-    else if (N == 128) lm_head_argmax_kernel<128><<<grid, LM_THREADS, smem, st>>>(w_map, x_map, p);
-    else lm_head_argmax_kernel<256><<<grid, LM_THREADS, smem, st>>>(w_map, x_map, p);
+    if (M > 128) {
+        const int rc = launch_lm_head_pair(tree, M, H, V, x, W, keys, st);
+        if (rc != MTV_OK) return rc;
+    } else {
+        const int N = M <= 64 ? 64 : 128;
+        constexpr int tiles = 2;                             // weight tiles per stage (see the kernel)
+        CUtensorMap w_map, x_map;
+        LmParams p;
+        p.keys = keys; p.dev_error = tree->d_error; p.M = M; p.H = H; p.V = V; p.N = N; p.passes = 1;
+        p.stage_bytes = tiles * LM_TILE_BYTES + N * 128;
+        p.n_stages = (int)((LM_SMEM_MAX - 1024) / p.stage_bytes);
+        if (p.n_stages > LM_MAX_STAGES) p.n_stages = LM_MAX_STAGES;
+        const size_t smem = 1024 + (size_t)p.n_stages * p.stage_bytes;
+        int ctas = sm_count();                               // one CTA per SM
+        const int min_pairs = (V + tiles * 128 - 1) / (tiles * 128);   // units of `tiles` weight tiles
+        if (ctas > (V + 63) / 64) ctas = (V + 63) / 64;      // no tile below 32 rows
+        if (ctas < 1) ctas = 1;
+        // every CTA walks the same number of tile pairs; the tile height shrinks until they just cover V
+        const int rounds = (min_pairs + ctas - 1) / ctas;
+        p.n_pairs = ctas * rounds;
+        p.R = ((V + tiles * p.n_pairs - 1) / (tiles * p.n_pairs) + 7) / 8 * 8;
+        if (!tma_map_2d_bf16(&w_map, W, V, H, p.R) || !tma_map_2d_bf16(&x_map, x, M, H, N)) return MTV_ERR_CUDA;
+        if (N == 64) lm_head_argmax_kernel<64><<<ctas, LM_THREADS, smem, st>>>(w_map, x_map, p);
+        else lm_head_argmax_kernel<128><<<ctas, LM_THREADS, smem, st>>>(w_map, x_map, p);
+    }
     if (am) lm_head_finish_kernel<<<(M + 127) / 128, 128, 0, st>>>(M, keys, am, am_val);
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;

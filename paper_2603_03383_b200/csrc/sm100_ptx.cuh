@@ -103,6 +103,14 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
         "}\n"
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
 }
+// Shared-memory operand descriptors with 128-byte swizzle and 8-row (8-key) groups 1024 bytes apart, as lower and upper
+// word.  The upper word is the same for all of them; the start address in the lower one counts 16-byte units and never
+// carries (shared-memory addresses stay below 256 KB), so that moving along an operand is one 32-bit add.  lbo_bytes: 16
+// for a K-major operand, the distance of the next 64 columns for an N-major one.
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
+    return ((saddr & 0x3FFFFu) >> 4) | (lbo_bytes >> 4) << 16;
+}
+constexpr uint32_t DESC_HI = (1024u >> 4) | 1u << 14 /* descriptor version */ | 2u << 29 /* 128-byte swizzle */;
 // The forms below are executed by a whole (converged) warp and issued by the one lane whose `leader` is set: the operands
 // then stay in uniform registers.  Descriptors as lower and upper word.
 __device__ __forceinline__ bool elect_one() {
@@ -138,6 +146,30 @@ __device__ __forceinline__ void mma_ss_elect(uint32_t d_tmem, uint32_t a_lo, uin
         "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %4, p;\n"
         "}\n"
         ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"((uint32_t)accumulate), "r"((uint32_t)leader) : "memory");
+}
+// The same over a CTA pair, and its commit to the barriers at the same offset in the CTAs of `mask`.
+__device__ __forceinline__ void mma_pair_ss_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
+                                                  bool accumulate, bool leader) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        ".reg .b64 a, b;\n"
+        "setp.ne.b32 p, %5, 0;\n"
+        "setp.ne.b32 q, %6, 0;\n"
+        "mov.b64 a, {%1, %3};\n"
+        "mov.b64 b, {%2, %3};\n"
+        "@q tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %4, p;\n"
+        "}\n"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(desc_hi), "r"(idesc), "r"((uint32_t)accumulate), "r"((uint32_t)leader) : "memory");
+}
+__device__ __forceinline__ void tc_commit_pair_mask_elect(uint32_t bar, uint16_t mask, bool leader) {
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "setp.ne.b32 q, %2, 0;\n"
+        "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n"
+        "}\n"
+        ::"r"(bar), "h"(mask), "r"((uint32_t)leader) : "memory");
 }
 // A in tensor memory
 __device__ __forceinline__ void mma_ts_elect(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
