@@ -39,7 +39,10 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
 
 // grid = (nsplit, B*T).  Partial argmax of one chunk of one row.
 __global__ void __launch_bounds__(ARGMAX_THREADS)
-node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsigned long long *__restrict__ part) {
+node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsigned long long *__restrict__ part, int alongside) {
+    // alongside: the logits were complete before the previous kernel started, which is then only waited for at the end
+    let_next_start();
+    if (!alongside) previous_done();
     const int row = blockIdx.y, ns = gridDim.x;
     // chunk boundaries on multiples of 8 elements so that 16-byte loads stay aligned
     const int per = ((V + ns - 1) / ns + 7) / 8 * 8;
@@ -97,6 +100,7 @@ node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsi
         for (int w = 1; w < ARGMAX_THREADS / 32; ++w) best = umax64(best, sm[w]);
         part[(size_t)row * ns + blockIdx.x] = best;
     }
+    if (alongside) previous_done();
 }
 
 // grid = B, block = 128.  Finish the argmax, score every path, pick the best, gather.
@@ -110,6 +114,8 @@ accept_finish_kernel(int T, int K, int P, int ns, const unsigned long long *__re
     __shared__ int32_t tok[MTV_MAX_T];
     __shared__ unsigned int best_key;
     const int b = blockIdx.x;
+    let_next_start();
+    previous_done();
     for (int i = threadIdx.x; i < T; i += blockDim.x) {
         unsigned long long best = 0;
         for (int s = 0; s < ns; ++s) best = umax64(best, part[((size_t)b * T + i) * ns + s]);
@@ -146,11 +152,25 @@ accept_finish_kernel(int T, int K, int P, int ns, const unsigned long long *__re
 
 }  // namespace mtv
 
-extern "C" int tree_accept(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok,
-                           int32_t *accept_len, int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok,
-                           int32_t *next_root, void *ws, size_t ws_bytes, void *stream) {
-    using namespace mtv;
-    MTV_RANGE("tree_accept");
+namespace mtv {
+static int launch_argmax(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const AcceptWs &L, unsigned long long *part,
+                         int alongside, cudaStream_t st) {
+    TapScope tap(MTV_KERNEL_ARGMAX_PARTIAL, st);
+    MTV_CUDA_CHECK(launch_dependent(node_argmax_partial_kernel, dim3(L.nsplit, B * tree->T), ARGMAX_THREADS, 0, st, V,
+                                    reinterpret_cast<const __nv_bfloat16 *>(logits), part, alongside));
+    return MTV_OK;
+}
+static int launch_finish(const mtv_tree_t *tree, int B, int ns, const unsigned long long *part, const int32_t *tree_tok,
+                         int32_t *accept_len, int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root,
+                         cudaStream_t st) {
+    MTV_CUDA_CHECK(launch_dependent(accept_finish_kernel, dim3(B), 128, 0, st, tree->T, tree->K, tree->P, ns, part, tree_tok,
+                                    tree->d_retrieve, accept_len, best_path, acc_nodes, acc_tok, next_root, tree->d_error));
+    return MTV_OK;
+}
+
+int accept_logits(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
+                  int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
+                  void *stream, bool alongside) {
     if (!tree || !tree->on_device || !logits || !tree_tok || !accept_len || !best_path || !acc_nodes ||
         !acc_tok || !next_root || !ws || B < 1 || V < 1)
         return MTV_ERR_INVALID_ARG;
@@ -160,16 +180,19 @@ extern "C" int tree_accept(const mtv_tree_t *tree, int B, int V, const mtv_bf16 
     if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     auto *part = reinterpret_cast<unsigned long long *>((char *)ws + L.part_off);
-    {
-        TapScope tap(MTV_KERNEL_ARGMAX_PARTIAL, st);
-        node_argmax_partial_kernel<<<dim3(L.nsplit, B * tree->T), ARGMAX_THREADS, 0, st>>>(
-            V, reinterpret_cast<const __nv_bfloat16 *>(logits), part);
-    }
+    const int rc = launch_argmax(tree, B, V, logits, L, part, alongside, st);
+    if (rc != MTV_OK) return rc;
     TapScope tap(MTV_KERNEL_ACCEPT_FINISH, st);
-    accept_finish_kernel<<<B, 128, 0, st>>>(tree->T, tree->K, tree->P, L.nsplit, part, tree_tok, tree->d_retrieve,
-                                            accept_len, best_path, acc_nodes, acc_tok, next_root, tree->d_error);
-    MTV_CUDA_CHECK(cudaGetLastError());
-    return MTV_OK;
+    return launch_finish(tree, B, L.nsplit, part, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, st);
+}
+}  // namespace mtv
+
+extern "C" int tree_accept(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok,
+                           int32_t *accept_len, int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok,
+                           int32_t *next_root, void *ws, size_t ws_bytes, void *stream) {
+    MTV_RANGE("tree_accept");
+    return mtv::accept_logits(tree, B, V, logits, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, ws, ws_bytes,
+                              stream, false);
 }
 
 // Per-node argmax keys of stored logits, in the form tree_accept_keys reads: what tree_accept computes before its path
@@ -197,11 +220,8 @@ extern "C" int node_argmax_keys(const mtv_tree_t *tree, int B, int V, const mtv_
     cudaStream_t st = (cudaStream_t)stream;
     auto *part = reinterpret_cast<unsigned long long *>((char *)ws + L.part_off);
     const int rows = B * tree->T;
-    {
-        TapScope tap(MTV_KERNEL_ARGMAX_PARTIAL, st);
-        node_argmax_partial_kernel<<<dim3(L.nsplit, rows), ARGMAX_THREADS, 0, st>>>(
-            V, reinterpret_cast<const __nv_bfloat16 *>(logits), part);
-    }
+    const int rc = launch_argmax(tree, B, V, logits, L, part, 0, st);
+    if (rc != MTV_OK) return rc;
     argmax_keys_reduce_kernel<<<(rows + 127) / 128, 128, 0, st>>>(rows, L.nsplit, part, keys);
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
@@ -218,11 +238,7 @@ extern "C" int tree_accept_keys(const mtv_tree_t *tree, int B, const unsigned lo
         !next_root || B < 1)
         return MTV_ERR_INVALID_ARG;
     if (tree->P > 255) return MTV_ERR_UNSUPPORTED_SHAPE;
-    accept_finish_kernel<<<B, 128, 0, (cudaStream_t)stream>>>(tree->T, tree->K, tree->P, 1, keys, tree_tok,
-                                                              tree->d_retrieve, accept_len, best_path, acc_nodes,
-                                                              acc_tok, next_root, tree->d_error);
-    MTV_CUDA_CHECK(cudaGetLastError());
-    return MTV_OK;
+    return launch_finish(tree, B, 1, keys, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, (cudaStream_t)stream);
 }
 
 // ---------------------------------------------------------------------------
@@ -282,10 +298,7 @@ extern "C" int tree_accept_static_scratch(const mtv_tree_t *tree, int B, int V, 
     if (rc != MTV_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     // every entry of `part` that the second kernel reads is written by the first one: nothing to clear
-    node_argmax_partial_kernel<<<dim3(L.nsplit, B * tree->T), ARGMAX_THREADS, 0, st>>>(
-        V, reinterpret_cast<const __nv_bfloat16 *>(logits), part);
-    accept_finish_kernel<<<B, 128, 0, st>>>(tree->T, tree->K, tree->P, L.nsplit, part, tree_tok, tree->d_retrieve,
-                                            accept_len, best_path, acc_nodes, acc_tok, next_root, tree->d_error);
-    MTV_CUDA_CHECK(cudaGetLastError());
-    return MTV_OK;
+    const int rc2 = launch_argmax(tree, B, V, logits, L, part, 0, st);
+    if (rc2 != MTV_OK) return rc2;
+    return launch_finish(tree, B, L.nsplit, part, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, st);
 }

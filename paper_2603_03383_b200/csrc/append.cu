@@ -39,6 +39,8 @@ tree_kv_append_rope_kernel(int T, int Hq, int Hkv, int D, int Lcap, int n_layers
                            const int32_t *__restrict__ depth, double log2_theta, int32_t *__restrict__ status) {
     __shared__ __align__(16) float cs[64], sn[64];   // D / 2 <= 64
     const int i = blockIdx.x, b = blockIdx.y, B = gridDim.y;
+    previous_done();
+    let_next_start();
     const int L = seq_lens[b];
     if (L + T > Lcap) {
         if (status && i == 0 && threadIdx.x == 0) status[b] = MTV_ERR_CAPACITY;
@@ -123,11 +125,11 @@ extern "C" int tree_kv_append_rope(const mtv_tree_t *tree, int B, int Hq, int Hk
     const double theta = rope_theta == 0.f ? 10000.0 : (double)rope_theta;
     int per = 1;
     const dim3 grid = rope_grid(tree->T, B, 1, &per);
-    tree_kv_append_rope_kernel<<<grid, ROPE_THREADS, 0, (cudaStream_t)stream>>>(
-        tree->T, Hq, Hkv, D, Lcap, 1, per, reinterpret_cast<__nv_bfloat16 *>(q), reinterpret_cast<const __nv_bfloat16 *>(k_new),
+    MTV_CUDA_CHECK(launch_dependent(
+        tree_kv_append_rope_kernel, grid, ROPE_THREADS, 0, (cudaStream_t)stream, tree->T, Hq, Hkv, D, Lcap, 1, per, reinterpret_cast<__nv_bfloat16 *>(q), reinterpret_cast<const __nv_bfloat16 *>(k_new),
         reinterpret_cast<const __nv_bfloat16 *>(v_new), reinterpret_cast<__nv_bfloat16 *>(k_cache),
         reinterpret_cast<__nv_bfloat16 *>(v_cache), nullptr, nullptr, stride_b, stride_h, stride_t, seq_lens,
-        tree->d_depth, log2(theta), status);
+        tree->d_depth, log2(theta), status));
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
 }
@@ -146,12 +148,12 @@ extern "C" int tree_kv_append_rope_layers(const mtv_tree_t *tree, int B, int Hq,
     const double theta = rope_theta == 0.f ? 10000.0 : (double)rope_theta;
     int per = 1;
     const dim3 grid = rope_grid(tree->T, B, n_layers, &per);
-    tree_kv_append_rope_kernel<<<grid, ROPE_THREADS, 0, (cudaStream_t)stream>>>(
-        tree->T, Hq, Hkv, D, Lcap, n_layers, per, reinterpret_cast<__nv_bfloat16 *>(q_layers),
+    MTV_CUDA_CHECK(launch_dependent(
+        tree_kv_append_rope_kernel, grid, ROPE_THREADS, 0, (cudaStream_t)stream, tree->T, Hq, Hkv, D, Lcap, n_layers, per, reinterpret_cast<__nv_bfloat16 *>(q_layers),
         reinterpret_cast<const __nv_bfloat16 *>(k_new_layers), reinterpret_cast<const __nv_bfloat16 *>(v_new_layers),
         nullptr, nullptr, reinterpret_cast<__nv_bfloat16 *const *>(k_caches),
         reinterpret_cast<__nv_bfloat16 *const *>(v_caches), stride_b, stride_h, stride_t, seq_lens, tree->d_depth,
-        log2(theta), status);
+        log2(theta), status));
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
 }

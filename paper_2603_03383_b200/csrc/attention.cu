@@ -133,16 +133,10 @@ struct AttnParams {
     int npc, R;              // tree nodes per tile (128 / G) and the rows they fill
     unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
     int n_tiles, n_blk, teams;
+    int alongside;           // nothing of the previous kernel is needed: it is waited for at the end
 };
 
-// 128-byte-swizzled shared-memory operand descriptors.  K-major: rows 128 bytes apart, 8-row groups 1024 bytes apart;
-// N-major (V): 8-key groups 1024 bytes apart, the next 64 columns one half tile further.
-// The upper word is the same for all of them; the start address in the lower one counts 16-byte units and never carries
-// (shared-memory addresses stay below 256 KB), so that moving along an operand is one 32-bit add.
-__device__ __forceinline__ uint32_t at_desc_lo(uint32_t saddr, uint32_t lbo_bytes) {
-    return ((saddr & 0x3FFFFu) >> 4) | (lbo_bytes >> 4) << 16;
-}
-constexpr uint32_t AT_DESC_HI = (1024u >> 4) | 1u << 14 /* descriptor version */ | 2u << 29 /* 128-byte swizzle */;
+// Operands: queries and keys K-major; V N-major, its next 64 columns one half tile further.
 // bf16 x bf16 -> fp32, M = 128
 constexpr uint32_t AT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
 constexpr uint32_t AT_B_NMAJOR = 1u << 16;
@@ -223,7 +217,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     constexpr int ST = SM::STAGES;
     extern __shared__ __align__(1024) unsigned char smem[];
     // Programmatic dependent launch: let the next kernel of the stream be set up while this one runs.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    let_next_start();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const uint32_t sbase = ptx::smem_u32(smem);
     auto bar = [&](int i) { return sbase + SM::OFF_BAR + (uint32_t)i * 8u; };
@@ -276,11 +270,11 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     }
     ptx::tc_fence_before();
     // Ends the set-up; nothing in front of it touches global memory.  Behind it the previous kernel of the stream is
-    // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters).
+    // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters), or it does not matter.
     auto begin = [&]() -> uint32_t {
         asm volatile("bar.sync 0, %0;" ::"n"(AT_THREADS) : "memory");
         ptx::tc_fence_after();
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!p.alongside) previous_done();
         return *tmem_slot;                    // tensor-memory base
     };
 
@@ -534,8 +528,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         const bool leader = ptx::elect_one();
         const int st = warp == AT_MMA_WARP ? 0 : 1, qt = one ? 0 : st;
         const int first = one ? st : 0, step = one ? 2 : 1;
-        const uint32_t ring_lo = at_desc_lo(sbase + SM::OFF_RING, 16), ring_v_lo = at_desc_lo(sbase + SM::OFF_RING, SM::HALF);
-        const uint32_t dq = at_desc_lo(sbase + qt * SM::TILE, 16);
+        const uint32_t ring_lo = ptx::desc_lo(sbase + SM::OFF_RING, 16), ring_v_lo = ptx::desc_lo(sbase + SM::OFF_RING, SM::HALF);
+        const uint32_t dq = ptx::desc_lo(sbase + qt * SM::TILE, 16);
         const uint32_t tmem = begin();
         const uint32_t t_s = tmem + TM_S + st * 128, t_o = tmem + TM_O + st * 128;
         AttnPiece d;
@@ -573,7 +567,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 for (int kk = 0; kk < D / 16; ++kk) {
                     constexpr uint32_t half = SM::HALF >> 4;
                     const uint32_t o = (kk / 4) * half + (kk % 4) * 2;
-                    ptx::mma_ss_elect(t_s, dq + o, dk + o, AT_DESC_HI, idesc, kk > 0, leader);
+                    ptx::mma_ss_elect(t_s, dq + o, dk + o, ptx::DESC_HI, idesc, kk > 0, leader);
                     if (kk == D / 16 - 3) pass_turn();
                 }
                 ptx::tc_commit_elect(bar(SM::BAR_S + st), leader);
@@ -610,11 +604,11 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 if (steps == 8) {
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk)
-                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, AT_DESC_HI, idesc, j > first || kk > 0, leader);
+                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, ptx::DESC_HI, idesc, j > first || kk > 0, leader);
                 } else {
 #pragma unroll 1
                     for (int kk = 0; kk < steps; ++kk)
-                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, AT_DESC_HI, idesc, j > first || kk > 0, leader);
+                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, ptx::DESC_HI, idesc, j > first || kk > 0, leader);
                 }
                 p_ph ^= 1;
                 TRACE();
@@ -1012,6 +1006,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     __syncthreads();
     ptx::tc_fence_after();
     if (warp == AT_MMA_WARP) ptx::tmem_dealloc(*tmem_slot, 512);
+    if (p.alongside) previous_done();
 }
 
 // ---------------------------------------------------------------------------------------- host
@@ -1164,20 +1159,8 @@ static int launch_attn(const mtv_tree *tree, const AttnPlan &a, AttnParams &p, c
         MTV_CUDA_CHECK(cudaFuncSetAttribute(tree_attn_kernel<D, ML, NEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D>::TOTAL));
         if (done) *done = true;
     }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.teams * a.n_blk, 1, 1);
-    cfg.blockDim = dim3(AT_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = AttnSmem<D>::TOTAL;
-    cfg.stream = stream;
-    // Launched as a programmatic dependent of the previous kernel in the stream (the kernel itself
-    // waits for that kernel before it reads anything), which hides most of the launch latency when
-    // attention calls follow each other.
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
     TapScope tap(MTV_KERNEL_ATTN_PARTIAL, stream);
-    MTV_CUDA_CHECK(cudaLaunchKernelEx(&cfg, tree_attn_kernel<D, ML, NEG>, maps, p));
+    MTV_CUDA_CHECK(launch_dependent(tree_attn_kernel<D, ML, NEG>, dim3(a.teams * a.n_blk), AT_THREADS, AttnSmem<D>::TOTAL, stream, maps, p));
     return MTV_OK;
 }
 
@@ -1188,7 +1171,7 @@ static int launch_attn(const mtv_tree *tree, const AttnPlan &a, AttnParams &p, c
 int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, int n_layers, const mtv_bf16 *q,
                           mtv_bf16 *const *k, mtv_bf16 *const *v, int64_t stride_b, int64_t stride_h, int64_t stride_t,
                           int Lcap, const int32_t *seq_lens, float scale, mtv_bf16 *out, int32_t *status, void *ws,
-                          size_t ws_bytes, void *stream) {
+                          size_t ws_bytes, void *stream, bool alongside) {
     if (!tree || !tree->on_device || !q || !k || !v || !seq_lens || !out || !ws) return MTV_ERR_INVALID_ARG;
     if (B < 1 || Hq < 1 || Hkv < 1 || n_layers < 1 || Lcap < tree->T) return MTV_ERR_INVALID_ARG;
     if ((D != 64 && D != 128) || Hq % Hkv != 0 || Hq / Hkv > 8 || B > 65535) return MTV_ERR_UNSUPPORTED_SHAPE;
@@ -1220,6 +1203,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
     p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_tiles = a.n_tiles; p.n_blk = a.n_blk; p.teams = a.teams;
+    p.alongside = alongside;
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;
     // positions in the common address space of a launch's groups are 32 bits wide
@@ -1227,6 +1211,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     int per_launch = n_layers == 1 ? 1 : AT_MAX_LAYERS;
     while (per_launch > 1 && per_launch * layer_len > 4e9) per_launch /= 2;
     for (int l = 0; l < n_layers; l += per_launch) {
+        if (l > 0) p.alongside = 0;          // (it shares the counters and the workspace with the launch before)
         p.n_layers = n_layers - l < per_launch ? n_layers - l : per_launch;
         p.out = reinterpret_cast<__nv_bfloat16 *>(out) + l * per_layer;
         const __nv_bfloat16 *ql = reinterpret_cast<const __nv_bfloat16 *>(q) + l * per_layer;

@@ -63,16 +63,22 @@ struct AttnWs {
     size_t o_off, ml_off, pair_ml_off = 0, order_off = 0, total;
 };
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap);
+// alongside: nothing that the previous kernel in the stream writes is needed, nor its workspace touched (everything before
+// that kernel is complete, see launch_dependent): the attention starts beside that kernel's end.
 int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, int n_layers, const mtv_bf16 *q,
                           mtv_bf16 *const *k, mtv_bf16 *const *v, int64_t stride_b, int64_t stride_h, int64_t stride_t,
                           int Lcap, const int32_t *seq_lens, float scale, mtv_bf16 *out, int32_t *status, void *ws,
-                          size_t ws_bytes, void *stream);
+                          size_t ws_bytes, void *stream, bool alongside = false);
 
 struct AcceptWs {
     size_t part_off, total;
     int nsplit;
 };
 AcceptWs accept_ws_layout(const mtv_tree *t, int B, int V);
+// tree_accept; alongside: the logits were complete before the previous kernel in the stream started (as above).
+int accept_logits(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
+                  int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
+                  void *stream, bool alongside);
 
 int sm_count();   // of the current device
 
@@ -88,6 +94,30 @@ struct PerDeviceOnce {
         return &done[dev];
     }
 };
+
+// Programmatic dependent launch: the kernel may be set up while the previous kernel of the stream runs, from the moment all
+// of that kernel's blocks have executed let_next_start() or ended.  Rules of the kernels launched so:
+//   - whatever the previous kernel (or one before it) writes is touched only behind previous_done();
+//   - every block executes previous_done() before it ends, early or late: a kernel that is complete then implies that
+//     all before it are;
+//   - a kernel that calls previous_done() in FRONT of let_next_start() makes everything enqueued before it complete for
+//     whoever follows; what follows may then read what was ready at that point without waiting (weights, logits).
+template <typename... P, typename... A>
+static inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Index checks of the -DMTV_DEBUG_BOUNDS build: MTV_INDEX_OK(i, n, err) is true when 0 <= i < n; otherwise it
 // records MTV_ERR_BOUNDS in the device error word and is false, and the caller skips the access.  In normal builds

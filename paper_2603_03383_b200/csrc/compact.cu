@@ -15,6 +15,8 @@ kv_compact_kernel(int T, int K, int D, int Lcap, __nv_bfloat16 *const *__restric
                   const int32_t *__restrict__ acc_nodes, int32_t *__restrict__ dev_error) {
     __shared__ uint4 stage[2 * MTV_MAX_K * 16];  // [k|v][j][D/8 <= 16]
     const int g = blockIdx.x, b = blockIdx.y, layer = blockIdx.z;
+    let_next_start();
+    previous_done();
     const int L = seq_lens[b];
     const int n = accept_len[b];
     if (L + T > Lcap || n <= 0) return;
@@ -44,6 +46,8 @@ kv_compact_kernel(int T, int K, int D, int Lcap, __nv_bfloat16 *const *__restric
 __global__ void seq_lens_advance_kernel(int B, int T, int Lcap, int32_t *seq_lens, const int32_t *accept_len,
                                         int32_t *status, int K, int32_t *dev_error) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    let_next_start();
+    previous_done();
     if (b >= B) return;
     const int L = seq_lens[b];
     if (L + T > Lcap) {
@@ -73,14 +77,14 @@ extern "C" int kv_compact_accepted(const mtv_tree_t *tree, int B, int Hkv, int D
     cudaStream_t st = (cudaStream_t)stream;
     {
         TapScope tap(MTV_KERNEL_KV_COMPACT, st);
-        kv_compact_kernel<<<dim3(Hkv, B, n_layers), 256, 0, st>>>(
-        tree->T, tree->K, D, Lcap, reinterpret_cast<__nv_bfloat16 *const *>(k_caches),
-        reinterpret_cast<__nv_bfloat16 *const *>(v_caches), stride_b, stride_h, stride_t, seq_lens, accept_len,
-            acc_nodes, tree->d_error);
+        MTV_CUDA_CHECK(launch_dependent(kv_compact_kernel, dim3(Hkv, B, n_layers), 256, 0, st, tree->T, tree->K, D, Lcap,
+                                        reinterpret_cast<__nv_bfloat16 *const *>(k_caches),
+                                        reinterpret_cast<__nv_bfloat16 *const *>(v_caches), stride_b, stride_h, stride_t, seq_lens,
+                                        accept_len, acc_nodes, tree->d_error));
     }
     TapScope tap(MTV_KERNEL_SEQ_ADVANCE, st);
-    seq_lens_advance_kernel<<<(B + 127) / 128, 128, 0, st>>>(B, tree->T, Lcap, seq_lens, accept_len, status, tree->K,
-                                                                   tree->d_error);
+    MTV_CUDA_CHECK(launch_dependent(seq_lens_advance_kernel, dim3((B + 127) / 128), 128, 0, st, B, tree->T, Lcap, seq_lens, accept_len,
+                                    status, tree->K, tree->d_error));
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
 }

@@ -142,6 +142,8 @@ heads_resblock_kernel(int B, int H, int K, const __nv_bfloat16 *__restrict__ hid
                       float *__restrict__ hprime, int32_t *__restrict__ counters, int n_counters) {
     extern __shared__ float sh[];  // [NB][H]
     const int b0 = blockIdx.y * NB;
+    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at once
+    let_next_start();
     // tickets of the vocabulary kernel (the next launch on the stream) start at zero
     if (blockIdx.x == 0 && blockIdx.y == 0)
         for (int i = threadIdx.x; i < n_counters; i += HEADS_THREADS) counters[i] = 0;
@@ -216,19 +218,7 @@ heads_vocab_topk_kernel(const VocabParams p) {
     const uint32_t row_bytes = (uint32_t)H * 2;
     const int n_chunk16 = H / 8;
 
-    // activations: chunk c = it*32 + lane of row b lives at xs4[((b*n_it + it)*2 + half)*32 + lane]
-    for (int i = threadIdx.x; i < NB * p.n_it * 64; i += VT_THREADS) {
-        const int ln = i % 32, half = (i / 32) % 2, it = (i / 64) % p.n_it, b = i / (64 * p.n_it);
-        const int c = it * 32 + ln;
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c < n_chunk16 && b0 + b < p.B)
-            v = *reinterpret_cast<const float4 *>(p.hprime + ((size_t)k * p.B + b0 + b) * H + c * 8 + half * 4);
-        xs4[i] = v;
-    }
-    for (int i = threadIdx.x; i < VT_CONS_WARPS * NB * MTV_MAX_TOPK; i += VT_THREADS) {
-        lval[i] = -INFINITY;
-        lidx[i] = 0x7fffffff;
-    }
+    let_next_start();
     if (threadIdx.x == 0) {
         for (int s = 0; s < NST; ++s) {
             ptx::mbar_init(bars + s * 8, 1);                               // full: the producer's expect_tx arrival
@@ -236,6 +226,10 @@ heads_vocab_topk_kernel(const VocabParams p) {
         }
         ptx::fence_mbar_init();
         s_abort = 0;
+    }
+    for (int i = threadIdx.x; i < VT_CONS_WARPS * NB * MTV_MAX_TOPK; i += VT_THREADS) {
+        lval[i] = -INFINITY;
+        lidx[i] = 0x7fffffff;
     }
     __syncthreads();
 
@@ -247,19 +241,37 @@ heads_vocab_topk_kernel(const VocabParams p) {
     const __nv_bfloat16 *Wk = p.W2 + (size_t)k * p.V * H;
     const uint32_t ring = ptx::smem_u32(smem);
     volatile int *abort_flag = &s_abort;
+    // chunk t of the slab into its stage (the producer warp)
+    auto request = [&](int t) {
+        const int s = t % NST, v0 = v_begin + t * RS, rows = min(RS, v_end - v0);
+        if (lane == 0) ptx::mbar_arrive_expect_tx(bars + s * 8, rows * row_bytes);
+        __syncwarp();
+        if (lane < rows)
+            ptx::bulk_g2s(ring + s * p.stage_bytes + lane * row_bytes, Wk + (size_t)(v0 + lane) * H, row_bytes, bars + s * 8);
+    };
+    // The weights do not depend on the residual block: the ring is filled while that kernel ends.
+    const int n_early = min(NST, n_chunks);
+    if (warp == VT_CONS_WARPS)
+        for (int t = 0; t < n_early; ++t) request(t);
+    previous_done();
+
+    // activations: chunk c = it*32 + lane of row b lives at xs4[((b*n_it + it)*2 + half)*32 + lane]
+    for (int i = threadIdx.x; i < NB * p.n_it * 64; i += VT_THREADS) {
+        const int ln = i % 32, half = (i / 32) % 2, it = (i / 64) % p.n_it, b = i / (64 * p.n_it);
+        const int c = it * 32 + ln;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (c < n_chunk16 && b0 + b < p.B)
+            v = *reinterpret_cast<const float4 *>(p.hprime + ((size_t)k * p.B + b0 + b) * H + c * 8 + half * 4);
+        xs4[i] = v;
+    }
+    __syncthreads();
 
     if (warp == VT_CONS_WARPS) {
         // ---- producer
-        for (int t = 0; t < n_chunks && !*abort_flag; ++t) {
+        for (int t = n_early; t < n_chunks && !*abort_flag; ++t) {
             const int s = t % NST, use = t / NST;
-            if (use > 0 && !ptx::mbar_wait(bars + (NST + s) * 8, (use - 1) & 1)) { *abort_flag = 1; break; }
-            const int v0 = v_begin + t * RS;
-            const int rows = min(RS, v_end - v0);
-            if (lane == 0) ptx::mbar_arrive_expect_tx(bars + s * 8, rows * row_bytes);
-            __syncwarp();
-            if (lane < rows)
-                ptx::bulk_g2s(ring + s * p.stage_bytes + lane * row_bytes, Wk + (size_t)(v0 + lane) * H, row_bytes,
-                              bars + s * 8);
+            if (!ptx::mbar_wait(bars + (NST + s) * 8, (use - 1) & 1)) { *abort_flag = 1; break; }
+            request(t);
         }
     } else {
         // ---- consumers
@@ -463,8 +475,8 @@ static int launch_heads(const mtv_tree *t, int B, int H, int V, const __nv_bfloa
     int32_t *counters = reinterpret_cast<int32_t *>(ws + L.counters_off);
     {
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
-        heads_resblock_kernel<NB><<<dim3(g1, btiles), HEADS_THREADS, sm1, st>>>(B, H, t->K, hidden, W1, b1, hprime,
-                                                                               counters, L.n_counters);
+        MTV_CUDA_CHECK(launch_dependent(heads_resblock_kernel<NB>, dim3(g1, btiles), HEADS_THREADS, sm1, st, B, H, t->K, hidden, W1,
+                                        b1, hprime, counters, L.n_counters));
     }
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = t->K; p.T = t->T; p.C = t->C;
@@ -479,7 +491,7 @@ static int launch_heads(const mtv_tree *t, int B, int H, int V, const __nv_bfloa
     p.stage_bytes = S.stage_bytes; p.xs_off = S.xs_off; p.lists_off = S.lists_off; p.zbuf_off = S.zbuf_off; p.bars_off = S.bars_off;
     {
         TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
-        heads_vocab_topk_kernel<NB><<<dim3(L.ctas_per_head, t->K, btiles), VT_THREADS, S.total, st>>>(p);
+        MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_kernel<NB>, dim3(L.ctas_per_head, t->K, btiles), VT_THREADS, S.total, st, p));
     }
     return MTV_OK;
 }

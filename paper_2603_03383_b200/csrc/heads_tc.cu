@@ -39,14 +39,6 @@ static_assert(HT_SMEM_BYTES <= 220 * 1024, "shared memory");
 
 constexpr uint32_t HT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HT_N >> 3) << 17) | ((128u >> 4) << 24);
 
-__device__ __forceinline__ uint64_t ht_desc(uint32_t saddr) {   // K-major, 128-byte swizzle
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(16u >> 4) << 16;
-    d |= (uint64_t)(1024u >> 4) << 32;
-    d |= 1ull << 46;
-    d |= 2ull << 61;
-    return d;
-}
 __device__ __forceinline__ void ht_tma_2d(uint32_t dst, const void *map, uint32_t bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
@@ -96,6 +88,8 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
     volatile int *abort_flag = &abort_flag_s;
     constexpr uint32_t TMEM_COLS = 2 * HT_NACC * HT_NB;   // 128
 
+    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at once
+    let_next_start();
     // tickets of the vocabulary kernel (the next launch on the stream) start at zero
     if (blockIdx.x == 0)
         for (int i = threadIdx.x; i < p.n_counters; i += HT_THREADS) p.counters[i] = 0;
@@ -143,6 +137,7 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
         if (lane == 0) issued_s = it;
     } else if (warp == 4) {
         // ---------------------------------------------------------------- MMA issuer
+        const bool leader = ptx::elect_one();
         int it = 0;
         bool ok = true;
         for (int q = 0; ok && q < my_tiles && !*abort_flag; ++q) {
@@ -155,17 +150,14 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
                 ok = ptx::mbar_wait(full(s), (it / RT_STAGES) & 1);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t base = ring + s * RT_STAGE_BYTES;
-                    const uint32_t d = tmem + (u * HT_NACC + kc % HT_NACC) * HT_NB;
+                // (the whole warp, one elected lane issues: operands stay in uniform registers)
+                const uint32_t w = ptx::desc_lo(ring + s * RT_STAGE_BYTES, 16);
+                const uint32_t d = tmem + (u * HT_NACC + kc % HT_NACC) * HT_NB;
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        ptx::mma_ss(d, ht_desc(base + kk * 32), ht_desc(base + HT_W_BYTES + kk * 32), RT_IDESC,
-                                    kc >= HT_NACC || kk > 0);
-                    ptx::tc_commit(empty(s));
-                    if (kc == n_kc - 1) ptx::tc_commit(acc_full(u));
-                }
-                __syncwarp();
+                for (int kk = 0; kk < 4; ++kk)
+                    ptx::mma_ss_elect(d, w + kk * 2, w + (HT_W_BYTES >> 4) + kk * 2, ptx::DESC_HI, RT_IDESC, kc >= HT_NACC || kk > 0, leader);
+                ptx::tc_commit_elect(empty(s), leader);
+                if (kc == n_kc - 1) ptx::tc_commit_elect(acc_full(u), leader);
             }
         }
         if (!ok) *abort_flag = 1;
@@ -258,6 +250,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     const uint32_t drain_bar = bars + (uint32_t)(2 * HT_STAGES + 4) * 8u;
     volatile int *abort_flag = &abort_flag_s;
 
+    let_next_start();
     const int k = blockIdx.y, per = gridDim.x;
     const int kd = p.kd_arr[k];
     for (int i = threadIdx.x; i < HT_EPI_WARPS * HT_NB * MTV_MAX_TOPK; i += HT_THREADS) {
@@ -292,6 +285,15 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
 
     if (warp == 5) {
         // ---------------------------------------------------------------- TMA producer
+        // The weights do not depend on the residual block: their part of the first stages is requested while that kernel ends.
+        const int n_early = min(HT_STAGES, n_tiles * n_kc);
+        if (lane == 0)
+            for (int t = 0; t < n_early; ++t) {
+                ptx::mbar_arrive_expect_tx(full(t), HT_STAGE_BYTES);
+                ht_tma_2d(ring + t * HT_STAGE_BYTES, &w_map, full(t), t % n_kc * 64, k * p.V + v_begin + t / n_kc * 128);
+            }
+        __syncwarp();
+        previous_done();
         int it = 0;
         for (int q = 0; q < n_tiles && !*abort_flag; ++q) {
             const int row0 = k * p.V + v_begin + q * 128;     // rows past the slab are loaded and ignored
@@ -300,8 +302,10 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 if (use > 0 && !ptx::mbar_wait(empty(s), (use - 1) & 1)) { *abort_flag = 1; break; }
                 if (lane == 0) {
                     const uint32_t base = ring + s * HT_STAGE_BYTES;
-                    ptx::mbar_arrive_expect_tx(full(s), HT_STAGE_BYTES);
-                    ht_tma_2d(base, &w_map, full(s), kc * 64, row0);
+                    if (it >= n_early) {
+                        ptx::mbar_arrive_expect_tx(full(s), HT_STAGE_BYTES);
+                        ht_tma_2d(base, &w_map, full(s), kc * 64, row0);
+                    }
                     ht_tma_2d(base + HT_W_BYTES, &x_map, full(s), kc * 64, k * HT_N);
                 }
                 __syncwarp();
@@ -310,6 +314,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         if (lane == 0) issued_s = it;
     } else if (warp == 4) {
         // ---------------------------------------------------------------- MMA issuer
+        const bool leader = ptx::elect_one();
         int it = 0;
         bool ok = true;
         for (int q = 0; ok && q < n_tiles && !*abort_flag; ++q) {
@@ -322,17 +327,13 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 ok = ptx::mbar_wait(full(s), (it / HT_STAGES) & 1);
                 if (!ok) break;
                 ptx::tc_fence_after();
-                if (lane == 0) {
-                    const uint32_t base = ring + s * HT_STAGE_BYTES;
-                    const uint32_t d = tmem + (u * HT_NACC + kc % HT_NACC) * HT_ACC_COLS;
+                const uint32_t w = ptx::desc_lo(ring + s * HT_STAGE_BYTES, 16);
+                const uint32_t d = tmem + (u * HT_NACC + kc % HT_NACC) * HT_ACC_COLS;
 #pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        ptx::mma_ss(d, ht_desc(base + kk * 32), ht_desc(base + HT_W_BYTES + kk * 32), HT_IDESC,
-                                    kc >= HT_NACC || kk > 0);
-                    ptx::tc_commit(empty(s));
-                    if (kc == n_kc - 1) ptx::tc_commit(acc_full(u));
-                }
-                __syncwarp();
+                for (int kk = 0; kk < 4; ++kk)
+                    ptx::mma_ss_elect(d, w + kk * 2, w + (HT_W_BYTES >> 4) + kk * 2, ptx::DESC_HI, HT_IDESC, kc >= HT_NACC || kk > 0, leader);
+                ptx::tc_commit_elect(empty(s), leader);
+                if (kc == n_kc - 1) ptx::tc_commit_elect(acc_full(u), leader);
             }
         }
         if (!ok) *abort_flag = 1;
@@ -393,6 +394,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         }
         if (!ok) *abort_flag = 1;
     }
+    previous_done();                 // (the tickets and lists of the tail, for the warps that did not wait above)
     ptx::tc_fence_before();
     __syncthreads();
     if (warp == 4) {
@@ -444,7 +446,7 @@ int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 
         int ctas = (t->K * H + 127) / 128;
         if (ctas > sm_count()) ctas = sm_count();
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
-        heads_resblock_tc_kernel<<<ctas, HT_THREADS, RT_SMEM_BYTES, st>>>(w1_map, h_map, r);
+        MTV_CUDA_CHECK(launch_dependent(heads_resblock_tc_kernel, dim3(ctas), HT_THREADS, RT_SMEM_BYTES, st, w1_map, h_map, r));
     }
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = t->K; p.T = t->T; p.C = t->C;
@@ -458,7 +460,7 @@ int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 
     p.rows_per_stage = 0; p.n_stages = 0; p.n_it = 0;
     p.stage_bytes = 0; p.xs_off = 0; p.lists_off = 0; p.zbuf_off = 0; p.bars_off = 0;
     TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
-    heads_vocab_topk_tc_kernel<<<dim3(L.ctas_per_head, t->K), HT_THREADS, HT_SMEM_BYTES, st>>>(w2_map, x_map, p);
+    MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_tc_kernel, dim3(L.ctas_per_head, t->K), HT_THREADS, HT_SMEM_BYTES, st, w2_map, x_map, p));
     return MTV_OK;
 }
 

@@ -7,19 +7,42 @@
 extern "C" size_t mtv_workspace_bytes(const mtv_tree_t *tree, int B, int H, int V, int Hq, int Hkv, int D, int Lcap) {
     using namespace mtv;
     if (!tree || B < 1) return 0;
+    // side by side: the parts of a step overlap in time
     size_t need = 256;
-    if (H > 0 && V > 0) {
-        need = std::max(need, heads_ws_layout(tree, B, H, V).total);
-        need = std::max(need, accept_ws_layout(tree, B, V).total);
-    }
-    if (Hq > 0 && Hkv > 0 && D > 0 && Lcap > 0 && Hq % Hkv == 0)
-        need = std::max(need, attn_ws_layout(tree, B, Hq, Hkv, D, Lcap).total);
+    if (H > 0 && V > 0) need += heads_ws_layout(tree, B, H, V).total + accept_ws_layout(tree, B, V).total;
+    if (Hq > 0 && Hkv > 0 && D > 0 && Lcap > 0 && Hq % Hkv == 0) need += attn_ws_layout(tree, B, Hq, Hkv, D, Lcap).total;
     return need;
 }
 
+namespace {
+// The workspace of a step: heads | acceptance | attention, each with a region of its own if the buffer is large enough
+// (mtv_workspace_bytes); otherwise all start at the beginning, as successive calls on one stream may, and wait for each other.
+struct StepWs {
+    char *accept, *attn;
+    size_t accept_bytes, attn_bytes;
+    bool apart;
+};
+StepWs step_ws(const mtv_tree_t *tree, const mtv_step_args *a) {
+    StepWs w;
+    char *ws = static_cast<char *>(a->ws);
+    w.accept = w.attn = ws;
+    w.accept_bytes = w.attn_bytes = a->ws_bytes;
+    w.apart = false;
+    if (!ws || a->B < 1 || a->H < 1 || a->V < 1 || a->Hq < 1 || a->Hkv < 1 || a->Hq % a->Hkv != 0 || a->D < 1 || a->Lcap < 1) return w;
+    const size_t heads = mtv::heads_ws_layout(tree, a->B, a->H, a->V).total, accept = mtv::accept_ws_layout(tree, a->B, a->V).total;
+    if (a->ws_bytes < heads + accept + mtv::attn_ws_layout(tree, a->B, a->Hq, a->Hkv, a->D, a->Lcap).total) return w;
+    w.accept = ws + heads;
+    w.attn = w.accept + accept;
+    w.accept_bytes = accept;
+    w.attn_bytes = a->ws_bytes - heads - accept;
+    w.apart = true;
+    return w;
+}
+}  // namespace
+
 // Acceptance of a step: from stored logits, or from the fused LM head when the caller gave its operands
 // (the per-node keys then sit at the start of the workspace, which no other kernel uses at that point).
-static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, void *stream) {
+static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, const StepWs &w, bool alongside, void *stream) {
     if (a->x_final && a->W_lm) {
         if (!a->ws || a->ws_bytes < (size_t)a->B * tree->T * sizeof(unsigned long long)) return MTV_ERR_WORKSPACE;
         unsigned long long *keys = static_cast<unsigned long long *>(a->ws);
@@ -28,8 +51,8 @@ static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, void *str
         return tree_accept_keys(tree, a->B, keys, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
                                 a->next_root, stream);
     }
-    return tree_accept(tree, a->B, a->V, a->logits, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
-                       a->next_root, a->ws, a->ws_bytes, stream);
+    return mtv::accept_logits(tree, a->B, a->V, a->logits, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
+                              a->next_root, w.accept, w.accept_bytes, stream, alongside);
 }
 
 // One step; root_tok and the optional append are given separately so that a chain of steps can feed a step's root
@@ -37,22 +60,26 @@ static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, void *str
 static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int32_t *root_tok,
                        const mtv_append_args *ap, void *stream) {
     if (!tree || !a || !a->k_caches_host || !a->v_caches_host || !root_tok) return MTV_ERR_INVALID_ARG;
-    int rc = medusa_heads_topk(tree, a->B, a->H, a->V, a->hidden, a->W1, a->b1, a->W2, root_tok, a->cand,
-                               a->cand_logit, a->tree_tok, a->ws, a->ws_bytes, stream);
-    if (rc != MTV_OK) return rc;
+    // The attention needs nothing of the heads, and the scan of stored logits nothing of either: the heads' first kernel
+    // makes everything in front of it complete (see launch_dependent), so each starts where SMs fall free at the end
+    // of the one before.  The append, which the attention does need, goes in front of the heads.
+    const StepWs w = step_ws(tree, a);
+    int rc = MTV_OK;
     if (ap && (ap->k_new_layers || ap->v_new_layers)) {
-        // the tree nodes' K/V rows of every layer, in one launch in front of the first attention (which starts its
-        // set-up under this kernel's tail: programmatic dependent launch)
+        // the tree nodes' K/V rows of every layer, in one launch
         rc = tree_kv_append_rope_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, const_cast<mtv_bf16 *>(a->q_layers),
                                         ap->k_new_layers, ap->v_new_layers, a->k_caches, a->v_caches, a->stride_b,
                                         a->stride_h, a->stride_t, a->Lcap, a->seq_lens, ap->rope_theta, a->status, stream);
         if (rc != MTV_OK) return rc;
     }
+    rc = medusa_heads_topk(tree, a->B, a->H, a->V, a->hidden, a->W1, a->b1, a->W2, root_tok, a->cand, a->cand_logit, a->tree_tok,
+                           a->ws, a->ws_bytes, stream);
+    if (rc != MTV_OK) return rc;
     rc = mtv::tree_attention_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, a->q_layers, a->k_caches_host, a->v_caches_host,
                                     a->stride_b, a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->scale, a->out_layers,
-                                    a->status, a->ws, a->ws_bytes, stream);
+                                    a->status, w.attn, w.attn_bytes, stream, w.apart);
     if (rc != MTV_OK) return rc;
-    rc = step_accept(tree, a, stream);
+    rc = step_accept(tree, a, w, w.apart, stream);
     if (rc != MTV_OK) return rc;
     return kv_compact_accepted(tree, a->B, a->Hkv, a->D, a->n_layers, a->k_caches, a->v_caches, a->stride_b,
                                a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->accept_len, a->acc_nodes, a->status,
@@ -165,7 +192,8 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
     }
     // acceptance and compaction
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.logits_up, 0));
-    rc = step_accept(tree, d, stream);
+    const StepWs w = step_ws(tree, d);
+    rc = step_accept(tree, d, w, false, stream);
     if (rc != MTV_OK) return rc;
     rc = kv_compact_accepted(tree, d->B, d->Hkv, d->D, d->n_layers, d->k_caches, d->v_caches, d->stride_b, d->stride_h,
                              d->stride_t, d->Lcap, d->seq_lens, d->accept_len, d->acc_nodes, d->status, stream);
