@@ -353,7 +353,7 @@ int mtv_verify_steps(const mtv_tree_t *tree, const mtv_step_args *steps, const m
  * and the tree stay resident on the device.  `host` uses the same struct: only
  * the fields listed above are read from it.
  * The transfers overlap the compute on two copy streams that the library creates
- * on first use: queries and logits go up while the heads run, the attention
+ * on first use: queries and logits go up while the heads run (half of them before the attention, half behind it), the attention
  * outputs come down in groups of layers while later layers run.  Unlike the other
  * step calls this one is therefore neither allocation-free on its first call nor
  * capturable; use pinned host buffers, or the copies serialise. */

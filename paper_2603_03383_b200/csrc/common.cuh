@@ -52,10 +52,18 @@ struct HeadsWs {
     int ctas_per_head, n_counters;
     bool use_tc;   // several batch rows: vocabulary projection on the tcgen05 tensor cores
 };
-HeadsWs heads_ws_layout(const mtv_tree *t, int B, int H, int V);
+HeadsWs heads_ws_layout(int K, int B, int H, int V);
+// Heads [k0, k0 + n) of a call; expand: the tree's tokens follow (the other heads' candidates are already there).
+struct HeadsRange {
+    int k0, n;
+    bool expand;
+};
+int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
+                     const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
+                     int32_t *tree_tok, void *ws, size_t ws_bytes, void *stream);
 bool heads_tc_eligible(int B, int H);
 size_t heads_tc_xsplit_bytes(int K, int H);
-int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
+int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
                     const __nv_bfloat16 *b1, const __nv_bfloat16 *W2, const int32_t *root_tok, int32_t *cand,
                     float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, cudaStream_t st);
 

@@ -63,24 +63,24 @@ static VocabSmem vocab_smem_plan(int NB, int H, int ctas_per_head) {
     return s;
 }
 
-HeadsWs heads_ws_layout(const mtv_tree *t, int B, int H, int V) {
+HeadsWs heads_ws_layout(int K, int B, int H, int V) {
     HeadsWs w;
     // one persistent CTA per SM, the SMs divided evenly among the heads
-    int per_head = sm_count() / t->K;
+    int per_head = sm_count() / K;
     const int max_useful = (V + VT_GROUP_WARPS - 1) / VT_GROUP_WARPS;
     if (per_head > max_useful) per_head = max_useful;
     if (per_head < 1) per_head = 1;
     w.ctas_per_head = per_head;
     const int btiles = (B + nb_for(B) - 1) / nb_for(B);
     size_t off = 0;
-    w.hprime_off = off;   off = align_up(off + (size_t)t->K * B * H * sizeof(float), 256);
-    w.part_val_off = off; off = align_up(off + (size_t)t->K * B * per_head * MTV_MAX_TOPK * sizeof(float), 256);
-    w.part_idx_off = off; off = align_up(off + (size_t)t->K * B * per_head * MTV_MAX_TOPK * sizeof(int32_t), 256);
-    w.counters_off = off; off = align_up(off + (size_t)(t->K + 1) * btiles * sizeof(int32_t), 256);
-    w.n_counters = (t->K + 1) * btiles;
+    w.hprime_off = off;   off = align_up(off + (size_t)K * B * H * sizeof(float), 256);
+    w.part_val_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(float), 256);
+    w.part_idx_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(int32_t), 256);
+    w.counters_off = off; off = align_up(off + (size_t)(K + 1) * btiles * sizeof(int32_t), 256);
+    w.n_counters = (K + 1) * btiles;
     w.use_tc = heads_tc_eligible(B, H);
     w.xsplit_off = off;
-    if (w.use_tc) off = align_up(off + heads_tc_xsplit_bytes(t->K, H), 256);
+    if (w.use_tc) off = align_up(off + heads_tc_xsplit_bytes(K, H), 256);
     w.total = off;
     return w;
 }
@@ -452,7 +452,7 @@ heads_vocab_topk_kernel(const VocabParams p) {
 }
 
 template <int NB>
-static int launch_heads(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 *hidden,
+static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, int V, const __nv_bfloat16 *hidden,
                         const __nv_bfloat16 *W1, const __nv_bfloat16 *b1, const __nv_bfloat16 *W2,
                         const int32_t *root_tok, int32_t *cand, float *cand_logit, int32_t *tree_tok,
                         const HeadsWs &L, char *ws, cudaStream_t st) {
@@ -469,19 +469,19 @@ static int launch_heads(const mtv_tree *t, int B, int H, int V, const __nv_bfloa
         MTV_CUDA_CHECK(cudaFuncSetAttribute(heads_vocab_topk_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM_MAX));
         if (attr_done) *attr_done = true;
     }
-    int g1 = (t->K * H + HEADS_WARPS - 1) / HEADS_WARPS;
+    int g1 = (r.n * H + HEADS_WARPS - 1) / HEADS_WARPS;
     const int cap = 4 * sm_count();
     if (g1 > cap) g1 = cap;
     int32_t *counters = reinterpret_cast<int32_t *>(ws + L.counters_off);
     {
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
-        MTV_CUDA_CHECK(launch_dependent(heads_resblock_kernel<NB>, dim3(g1, btiles), HEADS_THREADS, sm1, st, B, H, t->K, hidden, W1,
+        MTV_CUDA_CHECK(launch_dependent(heads_resblock_kernel<NB>, dim3(g1, btiles), HEADS_THREADS, sm1, st, B, H, r.n, hidden, W1,
                                         b1, hprime, counters, L.n_counters));
     }
     VocabParams p;
-    p.B = B; p.H = H; p.V = V; p.K = t->K; p.T = t->T; p.C = t->C;
+    p.B = B; p.H = H; p.V = V; p.K = r.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = hprime;
-    p.kd_arr = t->d_kd; p.off_arr = t->d_cand_offset; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
+    p.kd_arr = t->d_kd + r.k0; p.off_arr = t->d_cand_offset + r.k0; p.expand = r.expand; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
     p.part_idx = reinterpret_cast<int32_t *>(ws + L.part_idx_off);
     p.counters = counters;
@@ -491,8 +491,32 @@ static int launch_heads(const mtv_tree *t, int B, int H, int V, const __nv_bfloa
     p.stage_bytes = S.stage_bytes; p.xs_off = S.xs_off; p.lists_off = S.lists_off; p.zbuf_off = S.zbuf_off; p.bars_off = S.bars_off;
     {
         TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
-        MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_kernel<NB>, dim3(L.ctas_per_head, t->K, btiles), VT_THREADS, S.total, st, p));
+        MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_kernel<NB>, dim3(L.ctas_per_head, r.n, btiles), VT_THREADS, S.total, st, p));
     }
+    return MTV_OK;
+}
+
+int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
+                     const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
+                     int32_t *tree_tok, void *ws, size_t ws_bytes, void *stream) {
+    if (!tree || !tree->on_device || !hidden || !W1 || !W2 || !root_tok || !cand || !tree_tok || !ws)
+        return MTV_ERR_INVALID_ARG;
+    if (B < 1 || H < 8 || V < 1) return MTV_ERR_INVALID_ARG;
+    if (B > 16 || H % 8 != 0) return MTV_ERR_UNSUPPORTED_SHAPE;
+    if (((uintptr_t)W2 | (uintptr_t)W1 | (uintptr_t)hidden | (uintptr_t)ws) & 15) return MTV_ERR_INVALID_ARG;
+    for (int d = 0; d < tree->K; ++d)
+        if (tree->k_d[d] > V) return MTV_ERR_INVALID_ARG;
+    const HeadsWs L = heads_ws_layout(r.n, B, H, V);
+    if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
+    cudaStream_t st = (cudaStream_t)stream;
+    auto *h = reinterpret_cast<const __nv_bfloat16 *>(hidden);
+    auto *w1 = reinterpret_cast<const __nv_bfloat16 *>(W1) + (size_t)r.k0 * H * H;
+    auto *bb = b1 ? reinterpret_cast<const __nv_bfloat16 *>(b1) + (size_t)r.k0 * H : nullptr;
+    auto *w2 = reinterpret_cast<const __nv_bfloat16 *>(W2) + (size_t)r.k0 * V * H;
+    auto launch = L.use_tc ? launch_heads_tc : B == 1 ? launch_heads<1> : B == 2 ? launch_heads<2> : B <= 4 ? launch_heads<4> : launch_heads<8>;
+    const int rc = launch(tree, r, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
+    if (rc != MTV_OK) return rc;
+    MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
 }
 
@@ -503,29 +527,8 @@ extern "C" int medusa_heads_topk(const mtv_tree_t *tree, int B, int H, int V,
                                  const mtv_bf16 *W2, const int32_t *root_tok,
                                  int32_t *cand, float *cand_logit, int32_t *tree_tok,
                                  void *ws, size_t ws_bytes, void *stream) {
-    using namespace mtv;
     MTV_RANGE("medusa_heads_topk");
-    if (!tree || !tree->on_device || !hidden || !W1 || !W2 || !root_tok || !cand || !tree_tok || !ws)
-        return MTV_ERR_INVALID_ARG;
-    if (B < 1 || H < 8 || V < 1) return MTV_ERR_INVALID_ARG;
-    if (B > 16 || H % 8 != 0) return MTV_ERR_UNSUPPORTED_SHAPE;
-    if (((uintptr_t)W2 | (uintptr_t)W1 | (uintptr_t)hidden | (uintptr_t)ws) & 15) return MTV_ERR_INVALID_ARG;
-    for (int d = 0; d < tree->K; ++d)
-        if (tree->k_d[d] > V) return MTV_ERR_INVALID_ARG;
-    const HeadsWs L = heads_ws_layout(tree, B, H, V);
-    if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
-    cudaStream_t st = (cudaStream_t)stream;
-    auto *h = reinterpret_cast<const __nv_bfloat16 *>(hidden);
-    auto *w1 = reinterpret_cast<const __nv_bfloat16 *>(W1);
-    auto *bb = reinterpret_cast<const __nv_bfloat16 *>(b1);
-    auto *w2 = reinterpret_cast<const __nv_bfloat16 *>(W2);
-    int rc;
-    if (L.use_tc) rc = launch_heads_tc(tree, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
-    else if (B == 1) rc = launch_heads<1>(tree, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
-    else if (B == 2) rc = launch_heads<2>(tree, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
-    else if (B <= 4) rc = launch_heads<4>(tree, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
-    else rc = launch_heads<8>(tree, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
-    if (rc != MTV_OK) return rc;
-    MTV_CUDA_CHECK(cudaGetLastError());
-    return MTV_OK;
+    if (!tree) return MTV_ERR_INVALID_ARG;
+    return mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true}, B, H, V, hidden, W1, b1, W2, root_tok, cand, cand_logit,
+                                 tree_tok, ws, ws_bytes, stream);
 }

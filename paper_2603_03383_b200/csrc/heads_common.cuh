@@ -26,6 +26,7 @@ struct VocabParams {
     float *cand_logit;
     int32_t *tree_tok;
     int32_t *dev_error;
+    int expand;          // the last head to finish expands all heads' candidates into the tree tokens
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, xs_off, lists_off, zbuf_off, bars_off;
 };
@@ -131,6 +132,7 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
         }
     }
     // ---- last head of this batch tile expands the candidates into the tree tokens
+    if (!p.expand) return;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) s_flag = atomicAdd(&counters[p.K], 1) == p.K - 1;

@@ -423,7 +423,7 @@ bool heads_tc_eligible(int B, int H) { return B >= 2 && B <= HT_NB && H >= 64 &&
 size_t heads_tc_xsplit_bytes(int K, int H) { return (size_t)K * HT_N * H * sizeof(__nv_bfloat16); }
 
 // Residual block, then projection, top-k, merges and tree expansion: the whole medusa_heads_topk for 2..16 rows.
-int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
+int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
                     const __nv_bfloat16 *b1, const __nv_bfloat16 *W2, const int32_t *root_tok, int32_t *cand,
                     float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, cudaStream_t st) {
     static PerDeviceOnce attr_once;
@@ -435,23 +435,23 @@ int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 
     }
     __nv_bfloat16 *xsplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.xsplit_off);
     CUtensorMap w1_map, h_map, w2_map, x_map;
-    if (!tma_map_2d_bf16(&w1_map, W1, t->K * H, H, 128) || !tma_map_2d_bf16(&h_map, hidden, B, H, HT_NB) ||
-        !tma_map_2d_bf16(&w2_map, W2, t->K * V, H, 128) || !tma_map_2d_bf16(&x_map, xsplit, t->K * HT_N, H, HT_N))
+    if (!tma_map_2d_bf16(&w1_map, W1, range.n * H, H, 128) || !tma_map_2d_bf16(&h_map, hidden, B, H, HT_NB) ||
+        !tma_map_2d_bf16(&w2_map, W2, range.n * V, H, 128) || !tma_map_2d_bf16(&x_map, xsplit, range.n * HT_N, H, HT_N))
         return MTV_ERR_CUDA;
     {
         ResblockTcParams r;
-        r.B = B; r.H = H; r.K = t->K; r.hidden = hidden; r.b1 = b1; r.xsplit = xsplit;
+        r.B = B; r.H = H; r.K = range.n; r.hidden = hidden; r.b1 = b1; r.xsplit = xsplit;
         r.counters = reinterpret_cast<int32_t *>(ws + L.counters_off); r.n_counters = L.n_counters;
         r.dev_error = t->d_error;
-        int ctas = (t->K * H + 127) / 128;
+        int ctas = (range.n * H + 127) / 128;
         if (ctas > sm_count()) ctas = sm_count();
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
         MTV_CUDA_CHECK(launch_dependent(heads_resblock_tc_kernel, dim3(ctas), HT_THREADS, RT_SMEM_BYTES, st, w1_map, h_map, r));
     }
     VocabParams p;
-    p.B = B; p.H = H; p.V = V; p.K = t->K; p.T = t->T; p.C = t->C;
+    p.B = B; p.H = H; p.V = V; p.K = range.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = nullptr;
-    p.kd_arr = t->d_kd; p.off_arr = t->d_cand_offset; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
+    p.kd_arr = t->d_kd + range.k0; p.off_arr = t->d_cand_offset + range.k0; p.expand = range.expand; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
     p.part_idx = reinterpret_cast<int32_t *>(ws + L.part_idx_off);
     p.counters = reinterpret_cast<int32_t *>(ws + L.counters_off);
@@ -460,7 +460,7 @@ int launch_heads_tc(const mtv_tree *t, int B, int H, int V, const __nv_bfloat16 
     p.rows_per_stage = 0; p.n_stages = 0; p.n_it = 0;
     p.stage_bytes = 0; p.xs_off = 0; p.lists_off = 0; p.zbuf_off = 0; p.bars_off = 0;
     TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
-    MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_tc_kernel, dim3(L.ctas_per_head, t->K), HT_THREADS, HT_SMEM_BYTES, st, w2_map, x_map, p));
+    MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_tc_kernel, dim3(L.ctas_per_head, range.n), HT_THREADS, HT_SMEM_BYTES, st, w2_map, x_map, p));
     return MTV_OK;
 }
 

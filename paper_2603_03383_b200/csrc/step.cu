@@ -1,4 +1,5 @@
 // Whole verification step on one stream, and its host-buffer variant.
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -9,7 +10,11 @@ extern "C" size_t mtv_workspace_bytes(const mtv_tree_t *tree, int B, int H, int 
     if (!tree || B < 1) return 0;
     // side by side: the parts of a step overlap in time
     size_t need = 256;
-    if (H > 0 && V > 0) need += heads_ws_layout(tree, B, H, V).total + accept_ws_layout(tree, B, V).total;
+    if (H > 0 && V > 0) {
+        size_t heads = 0;
+        for (int k = 1; k <= tree->K; ++k) heads = std::max(heads, heads_ws_layout(k, B, H, V).total);   // (a part of them at a time)
+        need += heads + accept_ws_layout(tree, B, V).total;
+    }
     if (Hq > 0 && Hkv > 0 && D > 0 && Lcap > 0 && Hq % Hkv == 0) need += attn_ws_layout(tree, B, Hq, Hkv, D, Lcap).total;
     return need;
 }
@@ -29,7 +34,7 @@ StepWs step_ws(const mtv_tree_t *tree, const mtv_step_args *a) {
     w.accept_bytes = w.attn_bytes = a->ws_bytes;
     w.apart = false;
     if (!ws || a->B < 1 || a->H < 1 || a->V < 1 || a->Hq < 1 || a->Hkv < 1 || a->Hq % a->Hkv != 0 || a->D < 1 || a->Lcap < 1) return w;
-    const size_t heads = mtv::heads_ws_layout(tree, a->B, a->H, a->V).total, accept = mtv::accept_ws_layout(tree, a->B, a->V).total;
+    const size_t heads = mtv::heads_ws_layout(tree->K, a->B, a->H, a->V).total, accept = mtv::accept_ws_layout(tree, a->B, a->V).total;
     if (a->ws_bytes < heads + accept + mtv::attn_ws_layout(tree, a->B, a->Hq, a->Hkv, a->D, a->Lcap).total) return w;
     w.accept = ws + heads;
     w.attn = w.accept + accept;
@@ -115,10 +120,11 @@ extern "C" int mtv_verify_steps(const mtv_tree_t *tree, const mtv_step_args *ste
 namespace {
 // Copy streams and events of the host-buffer variant, created on first use, one set per device (the variant
 // synchronises anyway, so it is not one of the allocation-free hot calls).  Calls on one device take turns.
+constexpr int HOST_GROUPS = 8;   // most groups of layers in which queries go up and attention outputs come down
 struct HostStepAux {
     cudaStream_t up = nullptr, down = nullptr;
-    cudaEvent_t start = nullptr, q_up = nullptr, logits_up = nullptr, down_done = nullptr;
-    cudaEvent_t chunk[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t start = nullptr, logits_up = nullptr, down_done = nullptr;
+    cudaEvent_t q_up[HOST_GROUPS] = {}, done[HOST_GROUPS] = {};   // a group's queries are up / its attention is done
     bool ready = false;
     std::mutex busy;
 };
@@ -133,17 +139,55 @@ int host_step_aux(HostStepAux **out) {
     if (g_aux.ready) return MTV_OK;
     MTV_CUDA_CHECK(cudaStreamCreateWithFlags(&g_aux.up, cudaStreamNonBlocking));
     MTV_CUDA_CHECK(cudaStreamCreateWithFlags(&g_aux.down, cudaStreamNonBlocking));
-    cudaEvent_t *ev[] = {&g_aux.start, &g_aux.q_up, &g_aux.logits_up, &g_aux.down_done, &g_aux.chunk[0], &g_aux.chunk[1],
-                         &g_aux.chunk[2], &g_aux.chunk[3], &g_aux.chunk[4], &g_aux.chunk[5], &g_aux.chunk[6], &g_aux.chunk[7]};
-    for (cudaEvent_t *e : ev) MTV_CUDA_CHECK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    for (cudaEvent_t *e : {&g_aux.start, &g_aux.logits_up, &g_aux.down_done}) MTV_CUDA_CHECK(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    for (int i = 0; i < HOST_GROUPS; ++i) {
+        MTV_CUDA_CHECK(cudaEventCreateWithFlags(&g_aux.q_up[i], cudaEventDisableTiming));
+        MTV_CUDA_CHECK(cudaEventCreateWithFlags(&g_aux.done[i], cudaEventDisableTiming));
+    }
     g_aux.ready = true;
+    return MTV_OK;
+}
+
+// A step's small results (tokens, lengths, paths) written straight into mapped host buffers: one launch instead of a copy
+// of 3 us and a gap as long for each of them.
+struct HostResults {
+    static constexpr int N = 7;
+    const int32_t *src[N];
+    int32_t *dst[N];
+    int n[N];
+};
+__global__ void __launch_bounds__(256) host_results_kernel(const HostResults r) {
+    mtv::previous_done();
+#pragma unroll 1
+    for (int k = 0; k < HostResults::N; ++k)
+        for (int i = threadIdx.x; i < r.n[k]; i += blockDim.x) r.dst[k][i] = r.src[k][i];
+}
+int send_results(HostResults r, cudaStream_t st) {
+    HostResults m = r;
+    bool mapped = true;
+    for (int k = 0; k < HostResults::N && mapped; ++k) {
+        cudaPointerAttributes a;
+        mapped = cudaPointerGetAttributes(&a, r.dst[k]) == cudaSuccess && a.type == cudaMemoryTypeHost && a.devicePointer;
+        if (mapped) m.dst[k] = static_cast<int32_t *>(a.devicePointer);
+    }
+    (void)cudaGetLastError();
+    if (mapped) {
+        MTV_CUDA_CHECK(mtv::launch_dependent(host_results_kernel, dim3(1), 256, 0, st, m));
+        return MTV_OK;
+    }
+    for (int k = 0; k < HostResults::N; ++k)     // pageable buffers
+        MTV_CUDA_CHECK(cudaMemcpyAsync(r.dst[k], r.src[k], (size_t)r.n[k] * 4, cudaMemcpyDeviceToHost, st));
     return MTV_OK;
 }
 }  // namespace
 
-// The transfers overlap the compute: the queries and the base-model logits go up on a copy stream while the
-// heads run (attention waits for the queries, acceptance for the logits), and the attention outputs come
-// down on a second copy stream in up to sixteen groups of layers while later layers are still running.
+// The transfers overlap the compute.  At the 7B shape with L = 8192 the queries (17 MB) take 330 us to come up, the logits as
+// much again and the attention outputs to go down, against 640 us of heads and 270 us of attention.  Nothing orders the
+// heads and the attention, so half of the heads run while the queries come up, then the attention in groups of layers as
+// their queries arrive, its outputs leaving at once, and the other heads while the last outputs go down and the logits
+// come up.  (With all heads first the outputs' way down was waited for at the end: 1173 us.)  A launch of the attention
+// costs about 15 us beside its work, so there are no more groups than it takes for the first group's queries and the
+// last group's outputs to hide behind half of the heads.
 extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args *d, const mtv_step_args *h,
                                     void *stream) {
     MTV_RANGE("mtv_verify_step_host");
@@ -155,41 +199,52 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
     cudaStream_t st = (cudaStream_t)stream, up = g_aux.up, down = g_aux.down;
     const size_t B = d->B, T = tree->T, K = tree->K;
     const size_t per_layer = B * T * d->Hq * d->D;           // elements
-    const size_t q_bytes = (size_t)d->n_layers * per_layer * 2;
+    const double copy_us = (double)d->n_layers * per_layer * 2 / 50e3, heads_us = 0.5 * tree->K * d->V * (double)d->H * 2 / 6.5e6;
+    const int groups = std::max(1, std::min({HOST_GROUPS, d->n_layers, std::max(2, (int)(copy_us / (heads_us + 1.0)) + 1)}));
+    auto first_layer = [&](int g) { return (int)((int64_t)d->n_layers * g / groups); };
     // uploads
     MTV_CUDA_CHECK(cudaEventRecord(g_aux.start, st));         // the copy streams start where the caller's stream is
     MTV_CUDA_CHECK(cudaStreamWaitEvent(up, g_aux.start, 0));
     MTV_CUDA_CHECK(cudaStreamWaitEvent(down, g_aux.start, 0));
     MTV_CUDA_CHECK(cudaMemcpyAsync((void *)d->hidden, h->hidden, B * d->H * 2, cudaMemcpyHostToDevice, st));
     MTV_CUDA_CHECK(cudaMemcpyAsync((void *)d->root_tok, h->root_tok, B * 4, cudaMemcpyHostToDevice, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync((void *)d->q_layers, h->q_layers, q_bytes, cudaMemcpyHostToDevice, up));
-    MTV_CUDA_CHECK(cudaEventRecord(g_aux.q_up, up));
+    auto upload_q = [&](int g) {
+        const size_t l0 = first_layer(g), n = first_layer(g + 1) - l0;
+        MTV_CUDA_CHECK(cudaMemcpyAsync((void *)(d->q_layers + l0 * per_layer), h->q_layers + l0 * per_layer, n * per_layer * 2,
+                                       cudaMemcpyHostToDevice, up));
+        MTV_CUDA_CHECK(cudaEventRecord(g_aux.q_up[g], up));
+        return MTV_OK;
+    };
+    auto heads = [&](int k0, int n, bool expand) {
+        return mtv::heads_topk_range(tree, mtv::HeadsRange{k0, n, expand}, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok,
+                                     d->cand, d->cand_logit, d->tree_tok, d->ws, d->ws_bytes, stream);
+    };
+    const int before = tree->K / 2;
+    int rc = upload_q(0);
+    if (rc == MTV_OK && before > 0) rc = heads(0, before, false);   // (enqueued before the other copies: each costs the host 4 us)
+    for (int g = 1; g < groups && rc == MTV_OK; ++g) rc = upload_q(g);
+    if (rc != MTV_OK) return rc;
     if (d->x_final && d->W_lm)
         MTV_CUDA_CHECK(cudaMemcpyAsync((void *)d->x_final, h->x_final, B * T * d->H * 2, cudaMemcpyHostToDevice, up));
     else
         MTV_CUDA_CHECK(cudaMemcpyAsync((void *)d->logits, h->logits, B * T * d->V * 2, cudaMemcpyHostToDevice, up));
     MTV_CUDA_CHECK(cudaEventRecord(g_aux.logits_up, up));
-    // heads
-    int rc = medusa_heads_topk(tree, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok, d->cand, d->cand_logit,
-                               d->tree_tok, d->ws, d->ws_bytes, stream);
-    if (rc != MTV_OK) return rc;
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->tree_tok, d->tree_tok, B * T * 4, cudaMemcpyDeviceToHost, st));
-    // attention, its outputs leaving in groups of layers
-    MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.q_up, 0));
-    const int per_group = (d->n_layers + 7) / 8;
-    int n_sent = 0;
-    for (int l = 0; l < d->n_layers; l += per_group) {
-        const int n = std::min(per_group, d->n_layers - l);
-        rc = mtv::tree_attention_layers(tree, d->B, d->Hq, d->Hkv, d->D, n, d->q_layers + l * per_layer, d->k_caches_host + l,
-                                        d->v_caches_host + l, d->stride_b, d->stride_h, d->stride_t, d->Lcap, d->seq_lens,
-                                        d->scale, d->out_layers + l * per_layer, d->status, d->ws, d->ws_bytes, stream);
+    // attention, a group of layers at a time
+    for (int g = 0; g < groups; ++g) {
+        const size_t l0 = first_layer(g);
+        const int n = first_layer(g + 1) - (int)l0;
+        MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.q_up[g], 0));
+        rc = mtv::tree_attention_layers(tree, d->B, d->Hq, d->Hkv, d->D, n, d->q_layers + l0 * per_layer, d->k_caches_host + l0,
+                                        d->v_caches_host + l0, d->stride_b, d->stride_h, d->stride_t, d->Lcap, d->seq_lens,
+                                        d->scale, d->out_layers + l0 * per_layer, d->status, d->ws, d->ws_bytes, stream);
         if (rc != MTV_OK) return rc;
-        cudaEvent_t ev = g_aux.chunk[n_sent++];
-        MTV_CUDA_CHECK(cudaEventRecord(ev, st));
-        MTV_CUDA_CHECK(cudaStreamWaitEvent(down, ev, 0));
-        MTV_CUDA_CHECK(cudaMemcpyAsync(h->out_layers + l * per_layer, d->out_layers + l * per_layer, n * per_layer * 2,
+        MTV_CUDA_CHECK(cudaEventRecord(g_aux.done[g], st));
+        MTV_CUDA_CHECK(cudaStreamWaitEvent(down, g_aux.done[g], 0));
+        MTV_CUDA_CHECK(cudaMemcpyAsync(h->out_layers + l0 * per_layer, d->out_layers + l0 * per_layer, n * per_layer * 2,
                                        cudaMemcpyDeviceToHost, down));
     }
+    rc = heads(before, tree->K - before, true);
+    if (rc != MTV_OK) return rc;
     // acceptance and compaction
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.logits_up, 0));
     const StepWs w = step_ws(tree, d);
@@ -198,12 +253,11 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
     rc = kv_compact_accepted(tree, d->B, d->Hkv, d->D, d->n_layers, d->k_caches, d->v_caches, d->stride_b, d->stride_h,
                              d->stride_t, d->Lcap, d->seq_lens, d->accept_len, d->acc_nodes, d->status, stream);
     if (rc != MTV_OK) return rc;
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->accept_len, d->accept_len, B * 4, cudaMemcpyDeviceToHost, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->best_path, d->best_path, B * 4, cudaMemcpyDeviceToHost, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->acc_nodes, d->acc_nodes, B * (K + 1) * 4, cudaMemcpyDeviceToHost, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->acc_tok, d->acc_tok, B * (K + 1) * 4, cudaMemcpyDeviceToHost, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->next_root, d->next_root, B * 4, cudaMemcpyDeviceToHost, st));
-    MTV_CUDA_CHECK(cudaMemcpyAsync(h->seq_lens, d->seq_lens, B * 4, cudaMemcpyDeviceToHost, st));
+    rc = send_results({{d->tree_tok, d->accept_len, d->best_path, d->acc_nodes, d->acc_tok, d->next_root, d->seq_lens},
+                       {h->tree_tok, h->accept_len, h->best_path, h->acc_nodes, h->acc_tok, h->next_root, h->seq_lens},
+                       {(int)(B * T), (int)B, (int)B, (int)(B * (K + 1)), (int)(B * (K + 1)), (int)B, (int)B}},
+                      st);
+    if (rc != MTV_OK) return rc;
     MTV_CUDA_CHECK(cudaEventRecord(g_aux.down_done, down));
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.down_done, 0));
     MTV_CUDA_CHECK(cudaStreamSynchronize(st));
