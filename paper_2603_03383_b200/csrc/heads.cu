@@ -32,7 +32,7 @@ struct VocabSmem {
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, ring_bytes, xs_off, lists_off, zbuf_off, bars_off, total;
 };
-static VocabSmem vocab_smem_plan(int NB, int H, int ctas_per_head) {
+static VocabSmem vocab_smem_plan(int NB, int MR, int H, int ctas_per_head) {
     VocabSmem s;
     s.n_it = (H / 8 + 31) / 32;                       // 16-byte chunks per lane and row
     const uint32_t row_bytes = (uint32_t)H * 2;
@@ -42,7 +42,7 @@ static VocabSmem vocab_smem_plan(int NB, int H, int ctas_per_head) {
     const uint32_t zbuf_bytes = NB > 1 ? VT_GROUPS * 2 * VT_GROUP_WARPS * 32 * 4 : 0;   // partial logits of the column parts
     const uint32_t fixed = xs_bytes + lists_bytes + zbuf_bytes + 256;
     s.rows_per_stage = 0;
-    for (int rs = VT_GROUP_WARPS; rs >= 1; rs /= 2) {
+    for (int rs = VT_GROUP_WARPS * MR; rs >= 1; rs /= 2) {
         const uint32_t sb = rs * row_bytes;
         if (fixed + 2 * sb > VT_SMEM_MAX) continue;
         int n = (int)((VT_SMEM_MAX - fixed) / sb);
@@ -191,8 +191,8 @@ heads_resblock_kernel(int B, int H, int K, const __nv_bfloat16 *__restrict__ hid
 //
 // grid = (ctas_per_head, K, ceil(B/NB)): one persistent CTA per SM, each owning a
 // contiguous slab of one head's vocabulary rows.  A producer warp streams the slab
-// through a ring of shared-memory stages with bulk (TMA) copies, one copy per weight
-// row, completion counted on an mbarrier per stage, so that the bytes in flight per SM
+// through a ring of shared-memory stages with bulk (TMA) copies, one per stage, completion
+// counted on an mbarrier per stage, so that the bytes in flight per SM
 // do not depend on how many registers the consumers have.  Two groups of eight consumer
 // warps take alternate stages; a warp computes the dot products of one weight row with
 // NB activation rows (fp32 activations in shared memory, laid out so that a warp's
@@ -200,7 +200,9 @@ heads_resblock_kernel(int B, int H, int K, const __nv_bfloat16 *__restrict__ hid
 // when it beats the list's last entry.  Afterwards the warps' lists are merged per CTA;
 // the last CTA of a head (atomic ticket, no waiting) merges the CTAs' lists into the
 // candidate buffer, and the last head to finish expands the candidates into tree tokens.
-template <int NB>
+// MR: (one batch row) weight rows per warp and stage, so that short rows, too, come in stages of tens of kilobytes and pay
+// for waits, activation reads and reductions together: H = 1152, V = 91936, two heads took 124 us.
+template <int NB, int MR>
 __global__ void __launch_bounds__(VT_THREADS, 1)
 heads_vocab_topk_kernel(const VocabParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -244,10 +246,11 @@ heads_vocab_topk_kernel(const VocabParams p) {
     // chunk t of the slab into its stage (the producer warp)
     auto request = [&](int t) {
         const int s = t % NST, v0 = v_begin + t * RS, rows = min(RS, v_end - v0);
-        if (lane == 0) ptx::mbar_arrive_expect_tx(bars + s * 8, rows * row_bytes);
+        if (lane == 0) {       // rows of a slab follow one another in memory: one copy
+            ptx::mbar_arrive_expect_tx(bars + s * 8, rows * row_bytes);
+            ptx::bulk_g2s(ring + s * p.stage_bytes, Wk + (size_t)v0 * H, rows * row_bytes, bars + s * 8);
+        }
         __syncwarp();
-        if (lane < rows)
-            ptx::bulk_g2s(ring + s * p.stage_bytes + lane * row_bytes, Wk + (size_t)(v0 + lane) * H, row_bytes, bars + s * 8);
     };
     // The weights do not depend on the residual block: the ring is filled while that kernel ends.
     const int n_early = min(NST, n_chunks);
@@ -279,10 +282,8 @@ heads_vocab_topk_kernel(const VocabParams p) {
         const int group = warp / VT_GROUP_WARPS, wr = warp % VT_GROUP_WARPS;
         float *my_val = lval + (warp * NB) * MTV_MAX_TOPK;
         int32_t *my_idx = lidx + (warp * NB) * MTV_MAX_TOPK;
-        float thr_v[NB];
-        int thr_i[NB];
-#pragma unroll
-        for (int b = 0; b < NB; ++b) { thr_v[b] = -INFINITY; thr_i[b] = 0x7fffffff; }
+        float thr_v = -INFINITY, ev = -INFINITY;        // the last entry of the warp's list; this lane's entry (lane s: entry s)
+        int thr_i = 0x7fffffff, ei = 0x7fffffff;
         for (int t = group; t < n_chunks; t += VT_GROUPS) {
             const int s = t % NST, use = t / NST;
             if (*abort_flag) break;
@@ -294,65 +295,46 @@ heads_vocab_topk_kernel(const VocabParams p) {
             if (!ptx::mbar_wait(bars + s * 8, use & 1)) { *abort_flag = 1; break; }
             const int v0 = v_begin + t * RS;
             const int rows = min(RS, v_end - v0);
-            float acc[NB];
+            // this warp's rows of the stage: wr, wr + 8, ... (long rows: a stage may hold fewer than eight)
+            const int n_mine = (rows - wr + VT_GROUP_WARPS - 1) / VT_GROUP_WARPS;
+            const unsigned char *wrow = smem + s * p.stage_bytes + wr * row_bytes + lane * 16;
+            float acc[MR], acc2[MR];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) acc[b] = 0.f;
-            if (wr < rows) {
-                const uint4 *wrow = reinterpret_cast<const uint4 *>(smem + s * p.stage_bytes + wr * row_bytes);
-                float acc2[NB];
-#pragma unroll
-                for (int b = 0; b < NB; ++b) acc2[b] = 0.f;
+            for (int r = 0; r < MR; ++r) acc[r] = acc2[r] = 0.f;
 #pragma unroll 4
-                for (int it = 0; it < p.n_it; ++it) {
-                    const int c = it * 32 + lane;
-                    if (c < n_chunk16) {
-                        float wf[8];
-                        bf16x8_to_float(wrow[c], wf);
+            for (int it = 0; it < p.n_it; ++it) {
+                if (it * 32 + lane < n_chunk16) {
+                    const float4 x0 = xs4[(it * 2) * 32 + lane], x1 = xs4[(it * 2 + 1) * 32 + lane];
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) {
-                            const float4 x0 = xs4[((b * p.n_it + it) * 2) * 32 + lane];
-                            const float4 x1 = xs4[((b * p.n_it + it) * 2 + 1) * 32 + lane];
-                            float a = acc[b], a2 = acc2[b];
-                            a = fmaf(wf[0], x0.x, a); a2 = fmaf(wf[1], x0.y, a2);
-                            a = fmaf(wf[2], x0.z, a); a2 = fmaf(wf[3], x0.w, a2);
-                            a = fmaf(wf[4], x1.x, a); a2 = fmaf(wf[5], x1.y, a2);
-                            a = fmaf(wf[6], x1.z, a); a2 = fmaf(wf[7], x1.w, a2);
-                            acc[b] = a; acc2[b] = a2;
-                        }
+                    for (int r = 0; r < MR; ++r) {
+                        if (r >= n_mine) break;
+                        float wf[8];
+                        bf16x8_to_float(*reinterpret_cast<const uint4 *>(wrow + r * VT_GROUP_WARPS * row_bytes + it * 512), wf);
+                        float a = acc[r], a2 = acc2[r];
+                        a = fmaf(wf[0], x0.x, a); a2 = fmaf(wf[1], x0.y, a2);
+                        a = fmaf(wf[2], x0.z, a); a2 = fmaf(wf[3], x0.w, a2);
+                        a = fmaf(wf[4], x1.x, a); a2 = fmaf(wf[5], x1.y, a2);
+                        a = fmaf(wf[6], x1.z, a); a2 = fmaf(wf[7], x1.w, a2);
+                        acc[r] = a; acc2[r] = a2;
                     }
                 }
-#pragma unroll
-                for (int b = 0; b < NB; ++b) acc[b] += acc2[b];
             }
-            float z[NB];
+            float z[MR];
 #pragma unroll
-            for (int b = 0; b < NB; ++b) z[b] = warp_sum(acc[b]);     // identical in every lane
+            for (int r = 0; r < MR; ++r) z[r] = warp_sum(acc[r] + acc2[r]);     // identical in every lane
             // every lane's reads of the stage are complete (their values fed the sums): release it
             if (lane == 0) ptx::mbar_arrive(bars + (NST + s) * 8);
-            if (wr < rows) {
-                const int v = v0 + wr;
 #pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    if (cand_before(z[b], v, thr_v[b], thr_i[b])) {
-                        if (lane == 0) {
-                            // insertion into the sorted list of kd entries
-                            int pos = kd - 1;
-                            while (pos > 0 && cand_before(z[b], v, my_val[b * MTV_MAX_TOPK + pos - 1],
-                                                          my_idx[b * MTV_MAX_TOPK + pos - 1])) {
-                                my_val[b * MTV_MAX_TOPK + pos] = my_val[b * MTV_MAX_TOPK + pos - 1];
-                                my_idx[b * MTV_MAX_TOPK + pos] = my_idx[b * MTV_MAX_TOPK + pos - 1];
-                                --pos;
-                            }
-                            my_val[b * MTV_MAX_TOPK + pos] = z[b];
-                            my_idx[b * MTV_MAX_TOPK + pos] = v;
-                        }
-                        __syncwarp();
-                        thr_v[b] = my_val[b * MTV_MAX_TOPK + kd - 1];
-                        thr_i[b] = my_idx[b * MTV_MAX_TOPK + kd - 1];
-                    }
+            for (int r = 0; r < MR; ++r) {
+                const int row = wr + r * VT_GROUP_WARPS, v = v0 + row;
+                if (row < rows && cand_before(z[r], v, thr_v, thr_i)) {
+                    list_insert(ev, ei, z[r], v, kd, lane);
+                    thr_v = __shfl_sync(0xffffffffu, ev, kd - 1);
+                    thr_i = __shfl_sync(0xffffffffu, ei, kd - 1);
                 }
             }
         }
+        if (lane < kd) { my_val[lane] = ev; my_idx[lane] = ei; }
             } else {
         // Several batch rows: every activation chunk read from shared memory must serve several weight
         // rows, or shared-memory bandwidth, not HBM, sets the pace.  A group's eight warps split a stage
@@ -451,7 +433,7 @@ heads_vocab_topk_kernel(const VocabParams p) {
     vocab_tail(p, NB, VT_CONS_WARPS, lval, lidx, smem, k, bz, b0, per, kd, p.xs_off);
 }
 
-template <int NB>
+template <int NB, int MR>
 static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, int V, const __nv_bfloat16 *hidden,
                         const __nv_bfloat16 *W1, const __nv_bfloat16 *b1, const __nv_bfloat16 *W2,
                         const int32_t *root_tok, int32_t *cand, float *cand_logit, int32_t *tree_tok,
@@ -459,14 +441,14 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     float *hprime = reinterpret_cast<float *>(ws + L.hprime_off);
     const int btiles = (B + NB - 1) / NB;
     const size_t sm1 = (size_t)NB * H * sizeof(float);
-    const VocabSmem S = vocab_smem_plan(NB, H, L.ctas_per_head);
+    const VocabSmem S = vocab_smem_plan(NB, MR, H, L.ctas_per_head);
     if (sm1 > VT_SMEM_MAX || S.total == 0) return MTV_ERR_UNSUPPORTED_SHAPE;
     if (NB > 1 && S.rows_per_stage < (NB >= 4 ? 4 : 2)) return MTV_ERR_UNSUPPORTED_SHAPE;   // rows too long for a block of rows per stage
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
         MTV_CUDA_CHECK(cudaFuncSetAttribute(heads_resblock_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM_MAX));
-        MTV_CUDA_CHECK(cudaFuncSetAttribute(heads_vocab_topk_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM_MAX));
+        MTV_CUDA_CHECK(cudaFuncSetAttribute(heads_vocab_topk_kernel<NB, MR>, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM_MAX));
         if (attr_done) *attr_done = true;
     }
     int g1 = (r.n * H + HEADS_WARPS - 1) / HEADS_WARPS;
@@ -491,7 +473,7 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     p.stage_bytes = S.stage_bytes; p.xs_off = S.xs_off; p.lists_off = S.lists_off; p.zbuf_off = S.zbuf_off; p.bars_off = S.bars_off;
     {
         TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
-        MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_kernel<NB>, dim3(L.ctas_per_head, r.n, btiles), VT_THREADS, S.total, st, p));
+        MTV_CUDA_CHECK(launch_dependent(heads_vocab_topk_kernel<NB, MR>, dim3(L.ctas_per_head, r.n, btiles), VT_THREADS, S.total, st, p));
     }
     return MTV_OK;
 }
@@ -513,7 +495,11 @@ int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, in
     auto *w1 = reinterpret_cast<const __nv_bfloat16 *>(W1) + (size_t)r.k0 * H * H;
     auto *bb = b1 ? reinterpret_cast<const __nv_bfloat16 *>(b1) + (size_t)r.k0 * H : nullptr;
     auto *w2 = reinterpret_cast<const __nv_bfloat16 *>(W2) + (size_t)r.k0 * V * H;
-    auto launch = L.use_tc ? launch_heads_tc : B == 1 ? launch_heads<1> : B == 2 ? launch_heads<2> : B <= 4 ? launch_heads<4> : launch_heads<8>;
+    // one batch row: stages of 32 KB or more, but at least four to a CTA's slab
+    const int slab = (V + L.ctas_per_head - 1) / L.ctas_per_head;
+    const int mr = H < 1024 && slab >= 128 ? 4 : H < 2048 && slab >= 64 ? 2 : 1;
+    auto launch = L.use_tc ? launch_heads_tc : B == 1 ? (mr == 4 ? launch_heads<1, 4> : mr == 2 ? launch_heads<1, 2> : launch_heads<1, 1>)
+                  : B == 2 ? launch_heads<2, 1> : B <= 4 ? launch_heads<4, 1> : launch_heads<8, 1>;
     const int rc = launch(tree, r, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
     if (rc != MTV_OK) return rc;
     MTV_CUDA_CHECK(cudaGetLastError());

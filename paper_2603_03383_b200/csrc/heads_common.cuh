@@ -14,6 +14,58 @@ __device__ __forceinline__ bool cand_before(float va, int ia, float vb, int ib) 
     return va > vb || (va == vb && ia < ib);
 }
 
+// A sorted list of candidates held by a warp: lane s has entry s.  Insertion of one candidate (the same in all lanes) into a
+// list of kd entries: the entries ahead of it stay, the others move down by one.
+__device__ __forceinline__ void list_insert(float &ev, int &ei, float z, int v, int kd, int lane) {
+    const int pos = __popc(__ballot_sync(0xffffffffu, lane < kd && cand_before(ev, ei, z, v)));
+    const float uv = __shfl_up_sync(0xffffffffu, ev, 1);
+    const int ui = __shfl_up_sync(0xffffffffu, ei, 1);
+    if (lane < kd && lane > pos) { ev = uv; ei = ui; }
+    if (lane == pos && pos < kd) { ev = z; ei = v; }
+}
+// lanes l and l ^ o: the better one goes to the lower lane if `down`, else to the upper
+__device__ __forceinline__ void cand_exchange(float &v, int &i, int o, bool down, int lane) {
+    const float ov = __shfl_xor_sync(0xffffffffu, v, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, i, o);
+    const bool lower = (lane & o) == 0, mine_better = cand_before(v, i, ov, oi);
+    if ((lower == down) != mine_better) { v = ov; i = oi; }
+}
+// One candidate per lane (cand: it has one) against a list of kd <= 16 entries in shared memory.  A few are inserted one
+// after the other (about 100 cycles each); many, as when a list is still empty, are sorted over the lanes and merged (about
+// 900 cycles).  s_thr: the best kd-th entry of any list of this batch row in the CTA, as an order-preserving integer.
+static __device__ __noinline__ void list_update(float z, int v, bool cand, float *lv, int32_t *li, int kd, int *s_thr, int lane) {
+    unsigned m = __ballot_sync(0xffffffffu, cand);
+    float ev = lane < kd ? lv[lane] : -INFINITY;
+    int ei = lane < kd ? li[lane] : 0x7fffffff;
+    if (__popc(m) < 8) {
+        while (m) {
+            const int src = __ffs(m) - 1;
+            m &= m - 1;
+            list_insert(ev, ei, __shfl_sync(0xffffffffu, z, src), __shfl_sync(0xffffffffu, v, src), kd, lane);
+        }
+    } else {
+        float x = cand ? z : -INFINITY;
+        int xi = cand ? v : 0x7fffffff;
+#pragma unroll 1
+        for (int k = 2; k <= 32; k <<= 1)          // bitonic sort, best first
+#pragma unroll 1
+            for (int o = k >> 1; o > 0; o >>= 1) cand_exchange(x, xi, o, (lane & k) == 0, lane);
+        // the better of entry s and candidate 15 - s: the sixteen best of both, bitonic
+        const float rv = __shfl_sync(0xffffffffu, x, 15 - (lane & 15));
+        const int ri = __shfl_sync(0xffffffffu, xi, 15 - (lane & 15));
+        if (!cand_before(ev, ei, rv, ri)) { ev = rv; ei = ri; }
+#pragma unroll 1
+        for (int o = 8; o > 0; o >>= 1) cand_exchange(ev, ei, o, true, lane);
+    }
+    if (lane < kd) { lv[lane] = ev; li[lane] = ei; }
+    if (lane == kd - 1) {
+        const int bits = __float_as_int(ev);
+        atomicMax(s_thr, bits ^ ((bits >> 31) & 0x7fffffff));
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ float thr_value(int ord) { return __int_as_float(ord ^ ((ord >> 31) & 0x7fffffff)); }
+
 struct VocabParams {
     int B, H, V, K, T, C;
     const __nv_bfloat16 *W2;
@@ -27,6 +79,7 @@ struct VocabParams {
     int32_t *tree_tok;
     int32_t *dev_error;
     int expand;          // the last head to finish expands all heads' candidates into the tree tokens
+    int tile_rows;       // (tensor cores) vocabulary rows per tile
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, xs_off, lists_off, zbuf_off, bars_off;
 };
@@ -85,10 +138,23 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
             for (int b = warp; b < NB && b0 + b < p.B; b += n_w) {
                 const size_t base = ((size_t)k * p.B + b0 + b) * per * MTV_MAX_TOPK;
                 __syncwarp();
-                for (int e = lane; e < per * MTV_MAX_TOPK; e += 32) {
-                    const bool used = e % MTV_MAX_TOPK < kd;
-                    mval[e] = used ? __ldcg(p.part_val + base + e) : -INFINITY;
-                    midx[e] = used ? __ldcg(p.part_idx + base + e) : 0x7fffffff;
+                // the kd entries of each list, many loads in flight (all sixteen slots of every list, one round trip to L2
+                // at a time, took 8 us at the end of every call)
+                const unsigned n_e = (unsigned)(per * kd), inv = (1u << 20) / (unsigned)kd + 1u;   // e / kd for e < 4096
+#pragma unroll 1
+                for (unsigned e0 = lane; e0 < n_e; e0 += 32 * 8) {
+                    float v[8];
+                    int id[8];
+                    unsigned at[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const unsigned e = min(e0 + 32 * q, n_e - 1), c = (e * inv) >> 20;
+                        at[q] = c * MTV_MAX_TOPK + (e - c * (unsigned)kd);
+                        v[q] = __ldcg(p.part_val + base + at[q]);
+                        id[q] = __ldcg(p.part_idx + base + at[q]);
+                    }
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) { mval[at[q]] = v[q]; midx[at[q]] = id[q]; }
                 }
                 __syncwarp();
                 int head[MAXL];

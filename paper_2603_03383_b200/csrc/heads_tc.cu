@@ -11,9 +11,11 @@
 // Layout of the work as in the fused LM head: persistent CTAs (a contiguous slab of one head's vocabulary
 // rows each), TMA producer warp -> ring of stages (64 columns of 128 weight rows + the 48 activation
 // rows) -> MMA issuer, accumulators double-buffered in tensor memory -> four epilogue warps, one thread
-// per vocabulary row, that keep per-warp sorted candidate lists (a logit is inserted only if it beats
-// the list's last entry).  What follows the projection is shared with the single-row kernel.
+// per vocabulary row, that keep per-warp sorted candidate lists (a logit is looked at only if it beats
+// the last entry of the warp's list and those of the CTA's other warps).  What follows the projection is shared with the single-row kernel.
 #include <cuda.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "heads_common.cuh"
@@ -60,6 +62,7 @@ static_assert(RT_STAGE_BYTES % 1024 == 0, "stages must keep the 1024-byte alignm
 
 struct ResblockTcParams {
     int B, H, K;
+    int R;               // rows per tile (<= 128): as many as give all CTAs the same number of tiles; the MMA spans 128
     const __nv_bfloat16 *hidden, *b1;
     __nv_bfloat16 *xsplit;
     int32_t *counters;
@@ -113,7 +116,7 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
     const uint32_t tmem = tmem_slot;
 
     const int rows = p.K * p.H;
-    const int n_tiles_all = (rows + 127) / 128;
+    const int n_tiles_all = (rows + p.R - 1) / p.R;
     const int my_tiles = (int)blockIdx.x < n_tiles_all ? (n_tiles_all - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int n_kc = p.H / 64;
 
@@ -121,13 +124,13 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
         // ---------------------------------------------------------------- TMA producer
         int it = 0;
         for (int q = 0; q < my_tiles && !*abort_flag; ++q) {
-            const int row0 = ((int)blockIdx.x + q * (int)gridDim.x) * 128;
+            const int row0 = ((int)blockIdx.x + q * (int)gridDim.x) * p.R;
             for (int kc = 0; kc < n_kc; ++kc, ++it) {
                 const int s = it % RT_STAGES, use = it / RT_STAGES;
                 if (use > 0 && !ptx::mbar_wait(empty(s), (use - 1) & 1)) { *abort_flag = 1; break; }
                 if (lane == 0) {
                     const uint32_t base = ring + s * RT_STAGE_BYTES;
-                    ptx::mbar_arrive_expect_tx(full(s), RT_STAGE_BYTES);
+                    ptx::mbar_arrive_expect_tx(full(s), (uint32_t)p.R * 128u + RT_X_BYTES);
                     ht_tma_2d(base, &w_map, full(s), kc * 64, row0);
                     ht_tma_2d(base + HT_W_BYTES, &h_map, full(s), kc * 64, 0);
                 }
@@ -183,8 +186,8 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(acc_empty(u));
-            const int r = ((int)blockIdx.x + q * (int)gridDim.x) * 128 + warp * 32 + lane;
-            if (ok && r < rows) {
+            const int r = ((int)blockIdx.x + q * (int)gridDim.x) * p.R + warp * 32 + lane;
+            if (ok && warp * 32 + lane < p.R && r < rows) {
                 const int k = r / p.H, o = r % p.H;
                 const float bias = p.b1 ? __bfloat162float(p.b1[(size_t)k * p.H + o]) : 0.f;
 #pragma unroll
@@ -234,6 +237,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag_s;
     __shared__ int issued_s;
+    __shared__ int s_thr[HT_NB];
     __shared__ __align__(8) unsigned long long bar_mem[2 * HT_STAGES + 5];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const uint32_t raw = ptx::smem_u32(smem_raw);
@@ -257,6 +261,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         lval[i] = -INFINITY;
         lidx[i] = 0x7fffffff;
     }
+    if (threadIdx.x < HT_NB) s_thr[threadIdx.x] = (int)0x807fffff;      // -inf
     if (threadIdx.x == 0) {
         for (int s = 0; s < HT_STAGES; ++s) { ptx::mbar_init(full(s), 1); ptx::mbar_init(empty(s), 1); }
         for (int u = 0; u < 2; ++u) { ptx::mbar_init(acc_full(u), 1); ptx::mbar_init(acc_empty(u), 128); }
@@ -276,11 +281,12 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     ptx::tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    // slab of this CTA: vocabulary rows [v_begin, v_end) of head k, in tiles of 128 rows
+    // slab of this CTA: vocabulary rows [v_begin, v_end) of head k, in tiles of R rows (the MMA spans 128, the rest is ignored)
+    const int R = p.tile_rows;
     const int rows_per = (p.V + per - 1) / per;
     const int v_begin = min(p.V, (int)blockIdx.x * rows_per);
     const int v_end = kd > 0 ? min(p.V, v_begin + rows_per) : v_begin;
-    const int n_tiles = (v_end - v_begin + 127) / 128;
+    const int n_tiles = (v_end - v_begin + R - 1) / R;
     const int n_kc = p.H / 64;
 
     if (warp == 5) {
@@ -289,21 +295,21 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         const int n_early = min(HT_STAGES, n_tiles * n_kc);
         if (lane == 0)
             for (int t = 0; t < n_early; ++t) {
-                ptx::mbar_arrive_expect_tx(full(t), HT_STAGE_BYTES);
-                ht_tma_2d(ring + t * HT_STAGE_BYTES, &w_map, full(t), t % n_kc * 64, k * p.V + v_begin + t / n_kc * 128);
+                ptx::mbar_arrive_expect_tx(full(t), (uint32_t)R * 128u + HT_X_BYTES);
+                ht_tma_2d(ring + t * HT_STAGE_BYTES, &w_map, full(t), t % n_kc * 64, k * p.V + v_begin + t / n_kc * R);
             }
         __syncwarp();
         previous_done();
         int it = 0;
         for (int q = 0; q < n_tiles && !*abort_flag; ++q) {
-            const int row0 = k * p.V + v_begin + q * 128;     // rows past the slab are loaded and ignored
+            const int row0 = k * p.V + v_begin + q * R;       // rows past the slab are loaded and ignored
             for (int kc = 0; kc < n_kc; ++kc, ++it) {
                 const int s = it % HT_STAGES, use = it / HT_STAGES;
                 if (use > 0 && !ptx::mbar_wait(empty(s), (use - 1) & 1)) { *abort_flag = 1; break; }
                 if (lane == 0) {
                     const uint32_t base = ring + s * HT_STAGE_BYTES;
                     if (it >= n_early) {
-                        ptx::mbar_arrive_expect_tx(full(s), HT_STAGE_BYTES);
+                        ptx::mbar_arrive_expect_tx(full(s), (uint32_t)R * 128u + HT_X_BYTES);
                         ht_tma_2d(base, &w_map, full(s), kc * 64, row0);
                     }
                     ht_tma_2d(base + HT_W_BYTES, &x_map, full(s), kc * 64, k * HT_N);
@@ -365,31 +371,16 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             }
             ptx::tc_fence_before();
             ptx::mbar_arrive(acc_empty(u));
-            const int v = v_begin + q * 128 + warp * 32 + lane;
-            const bool valid = ok && v < v_end;
+            const int r = warp * 32 + lane, v = v_begin + q * R + r;
+            const bool valid = ok && r < R && v < v_end;
 #pragma unroll
             for (int b = 0; b < HT_NB; ++b) {
                 if (b >= p.B) break;
                 float *bv = my_val + b * MTV_MAX_TOPK;
                 int32_t *bi = my_idx + b * MTV_MAX_TOPK;
-                unsigned m = __ballot_sync(0xffffffffu, valid && cand_before(z[b], v, bv[kd - 1], bi[kd - 1]));
-                while (m) {
-                    // the whole warp inserts the candidate of lane src: lane s holds entry s, the entries ahead
-                    // of the candidate stay, the others move down by one
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1;
-                    const float zc = __shfl_sync(0xffffffffu, z[b], src);
-                    const int vc = __shfl_sync(0xffffffffu, v, src);
-                    const float ev = lane < kd ? bv[lane] : 0.f;
-                    const int ei = lane < kd ? bi[lane] : 0;
-                    const int pos = __popc(__ballot_sync(0xffffffffu, lane < kd && cand_before(ev, ei, zc, vc)));
-                    __syncwarp();
-                    if (pos < kd) {          // else the list has moved on since the ballot
-                        if (lane >= pos && lane < kd - 1) { bv[lane + 1] = ev; bi[lane + 1] = ei; }
-                        if (lane == pos) { bv[pos] = zc; bi[pos] = vc; }
-                    }
-                    __syncwarp();
-                }
+                // not behind this warp's list nor behind any list of the CTA
+                const bool cand = valid && z[b] >= thr_value(s_thr[b]) && cand_before(z[b], v, bv[kd - 1], bi[kd - 1]);
+                if (__any_sync(0xffffffffu, cand)) list_update(z[b], v, cand, bv, bi, kd, &s_thr[b], lane);
             }
         }
         if (!ok) *abort_flag = 1;
@@ -435,16 +426,22 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     }
     __nv_bfloat16 *xsplit = reinterpret_cast<__nv_bfloat16 *>(ws + L.xsplit_off);
     CUtensorMap w1_map, h_map, w2_map, x_map;
-    if (!tma_map_2d_bf16(&w1_map, W1, range.n * H, H, 128) || !tma_map_2d_bf16(&h_map, hidden, B, H, HT_NB) ||
-        !tma_map_2d_bf16(&w2_map, W2, range.n * V, H, 128) || !tma_map_2d_bf16(&x_map, xsplit, range.n * HT_N, H, HT_N))
+    // tiles of equal height over equally many tiles per CTA: whole tiles of 128 rows loaded up to 60 % of padding
+    const int w1_rows = range.n * H, sms = sm_count();
+    const int w1_rounds = (w1_rows + 128 * sms - 1) / (128 * sms);
+    const int w1_R = std::max(8, (w1_rows + sms * w1_rounds - 1) / (sms * w1_rounds));
+    const int slab = (V + L.ctas_per_head - 1) / L.ctas_per_head, slab_tiles = (slab + 127) / 128;
+    const int w2_R = (slab + slab_tiles - 1) / slab_tiles;
+    if (!tma_map_2d_bf16(&w1_map, W1, w1_rows, H, w1_R) || !tma_map_2d_bf16(&h_map, hidden, B, H, HT_NB) ||
+        !tma_map_2d_bf16(&w2_map, W2, range.n * V, H, w2_R) || !tma_map_2d_bf16(&x_map, xsplit, range.n * HT_N, H, HT_N))
         return MTV_ERR_CUDA;
     {
         ResblockTcParams r;
         r.B = B; r.H = H; r.K = range.n; r.hidden = hidden; r.b1 = b1; r.xsplit = xsplit;
         r.counters = reinterpret_cast<int32_t *>(ws + L.counters_off); r.n_counters = L.n_counters;
         r.dev_error = t->d_error;
-        int ctas = (range.n * H + 127) / 128;
-        if (ctas > sm_count()) ctas = sm_count();
+        r.R = w1_R;
+        const int ctas = std::min(sms, (w1_rows + w1_R - 1) / w1_R);
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
         MTV_CUDA_CHECK(launch_dependent(heads_resblock_tc_kernel, dim3(ctas), HT_THREADS, RT_SMEM_BYTES, st, w1_map, h_map, r));
     }
@@ -457,6 +454,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     p.counters = reinterpret_cast<int32_t *>(ws + L.counters_off);
     p.cand = cand; p.cand_logit = cand_logit; p.tree_tok = tree_tok;
     p.dev_error = t->d_error;
+    p.tile_rows = w2_R;
     p.rows_per_stage = 0; p.n_stages = 0; p.n_it = 0;
     p.stage_bytes = 0; p.xs_off = 0; p.lists_off = 0; p.zbuf_off = 0; p.bars_off = 0;
     TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
