@@ -907,7 +907,6 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 // this warp's part is written: tell those that share the item (each warp counts for itself)
                 __syncwarp();
                 if (lane == 0) {
-                    __threadfence();
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrive + d.first * p.n_blk + blk) : "memory");
                 }
             }
@@ -923,6 +922,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         for (int i = 0; i < n_m; ++i) {
             const AttnMerge m = merges[i];
             const int ctr = m.first * p.n_blk + blk, all = m.n * AT_SOFTMAX_WARPS;
+            int departed = 0;
             if (lane == 0) {
                 // relaxed polls (a round trip to L2 each), one acquire when the counter is full
                 int32_t *c = p.arrive + ctr;
@@ -930,12 +930,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 while (*reinterpret_cast<volatile int32_t *>(c) < all)
                     if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { give_up(); break; }
                 (void)ld_acquire(c);
-                // The last warp to have seen the counter full puts both counters back to zero (nobody polls them any
-                // more; the next call cannot start before this kernel has ended).
-                if (atomicAdd(p.depart + ctr, 1) == all - 1) {
-                    p.arrive[ctr] = 0;
-                    p.depart[ctr] = 0;
-                }
+                departed = atomicAdd(p.depart + ctr, 1);         // (its round trip overlaps the merge)
             }
             __syncwarp();
             // rows of the item: tile 0's, then tile 1's; this CTA combines its share of them, a thread per 16-byte chunk of the
@@ -999,6 +994,12 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                     dst[o * (D / 8) + c] =
                         make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
                                    pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
+            }
+            // The last warp to have seen the counter full puts both counters back to zero (nobody polls them any more; the
+            // next call cannot start before this kernel has ended).
+            if (lane == 0 && departed == all - 1) {
+                p.arrive[ctr] = 0;
+                p.depart[ctr] = 0;
             }
         }
     }
