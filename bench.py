@@ -204,7 +204,7 @@ def build_problem(w, n_layers, device, seed=None):
     return d
 
 
-LAUNCHES_PER_STEP = lambda n_layers: 2 + (n_layers + 63) // 64 + 2 + 2    # attention: up to 64 layers per launch
+LAUNCHES_PER_STEP = lambda n_layers: 2 + (n_layers + 63) // 64 + 2    # heads 2, attention: up to 64 layers per launch, scan of the logits, acceptance with compaction
 
 
 def workload_string(w, T, n_layers):
@@ -646,7 +646,7 @@ def run_sharded(args):
             "clocks": clocks,
             "e2e": {"value": 1.0 / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                     "steps": e2e_steps},
-            "gpu_launches": K_steps * (LAUNCHES_PER_STEP(0) + 2 + 2 * n_layers),   # one attention call per layer
+            "gpu_launches": K_steps * (LAUNCHES_PER_STEP(0) + 2 + 2 + 2 * n_layers),   # one attention call per layer
             "device_error": binding.mtv_device_error(tree, clear=False),
             "parity_gate": dict(gate or {}, split="integers bit-exact, attention max |diff| %.2e <= %.2e against the unsplit "
                                 "step" % (err, tol)) if gate is not None else "skipped",

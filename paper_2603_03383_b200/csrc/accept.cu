@@ -168,6 +168,12 @@ static int launch_finish(const mtv_tree_t *tree, int B, int ns, const unsigned l
     return MTV_OK;
 }
 
+int argmax_keys_partial(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, bool alongside,
+                        cudaStream_t st) {
+    if (!logits || V < 1 || ((uintptr_t)logits & 15)) return MTV_ERR_INVALID_ARG;
+    return launch_argmax(tree, B, V, logits, accept_ws_layout(tree, B, V), part, alongside, st);
+}
+
 int accept_logits(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
                   int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
                   void *stream, bool alongside) {

@@ -48,7 +48,7 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 // Workspace carving shared by the entry points (all offsets 256-byte aligned).
 struct HeadsWs {
-    size_t hprime_off, part_val_off, part_idx_off, counters_off, xsplit_off, total;
+    size_t hprime_off, part_val_off, part_idx_off, counters_off, tickets_off, xsplit_off, total;
     int ctas_per_head, n_counters;
     bool use_tc;   // several batch rows: vocabulary projection on the tcgen05 tensor cores
 };
@@ -87,6 +87,9 @@ AcceptWs accept_ws_layout(const mtv_tree *t, int B, int V);
 int accept_logits(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
                   int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
                   void *stream, bool alongside);
+// its scan alone: per-chunk keys into part (accept_ws_layout(...).nsplit per node)
+int argmax_keys_partial(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, bool alongside,
+                        cudaStream_t stream);
 
 int sm_count();   // of the current device
 
@@ -126,6 +129,11 @@ static inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int 
 }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The end of a step in one launch: acceptance from `ns` argmax keys per node (part [B][T][ns]), compaction, seq_lens.
+// tickets [B]: zero before the call.
+int accept_compact(const mtv_tree *tree, const mtv_step_args *a, int ns, const unsigned long long *part, int32_t *tickets,
+                   cudaStream_t stream);
 
 // Index checks of the -DMTV_DEBUG_BOUNDS build: MTV_INDEX_OK(i, n, err) is true when 0 <= i < n; otherwise it
 // records MTV_ERR_BOUNDS in the device error word and is false, and the caller skips the access.  In normal builds

@@ -76,8 +76,9 @@ HeadsWs heads_ws_layout(int K, int B, int H, int V) {
     w.hprime_off = off;   off = align_up(off + (size_t)K * B * H * sizeof(float), 256);
     w.part_val_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(float), 256);
     w.part_idx_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(int32_t), 256);
-    w.counters_off = off; off = align_up(off + (size_t)(K + 1) * btiles * sizeof(int32_t), 256);
-    w.n_counters = (K + 1) * btiles;
+    w.n_counters = (K + 1) * btiles + B;    // and one per sequence for the end of a step
+    w.counters_off = off; w.tickets_off = off + (size_t)(K + 1) * btiles * sizeof(int32_t);
+    off = align_up(off + (size_t)w.n_counters * sizeof(int32_t), 256);
     w.use_tc = heads_tc_eligible(B, H);
     w.xsplit_off = off;
     if (w.use_tc) off = align_up(off + heads_tc_xsplit_bytes(K, H), 256);

@@ -84,7 +84,20 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
                                     a->stride_b, a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->scale, a->out_layers,
                                     a->status, w.attn, w.attn_bytes, stream, w.apart);
     if (rc != MTV_OK) return rc;
-    rc = step_accept(tree, a, w, w.apart, stream);
+    if (w.apart) {       // acceptance and compaction in one launch behind the scan of the logits or the LM head
+        unsigned long long *keys = reinterpret_cast<unsigned long long *>(w.accept);
+        int ns = 1;
+        if (a->x_final && a->W_lm) {
+            rc = lm_head_argmax(tree, a->B, a->H, a->V, a->x_final, a->W_lm, nullptr, nullptr, keys, stream);
+        } else {
+            ns = mtv::accept_ws_layout(tree, a->B, a->V).nsplit;
+            rc = mtv::argmax_keys_partial(tree, a->B, a->V, a->logits, keys, true, (cudaStream_t)stream);
+        }
+        if (rc != MTV_OK) return rc;
+        return mtv::accept_compact(tree, a, ns, keys, reinterpret_cast<int32_t *>((char *)a->ws + mtv::heads_ws_layout(tree->K, a->B, a->H, a->V).tickets_off),
+                                   (cudaStream_t)stream);
+    }
+    rc = step_accept(tree, a, w, false, stream);
     if (rc != MTV_OK) return rc;
     return kv_compact_accepted(tree, a->B, a->Hkv, a->D, a->n_layers, a->k_caches, a->v_caches, a->stride_b,
                                a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->accept_len, a->acc_nodes, a->status,

@@ -21,7 +21,9 @@ DEV = "cuda"
     (65, 8, 8, 64, [127, 128], 4),
     (128, 8, 1, 64, [2500], 2),                # head size 64 with splits: fp32 partials
 ])
-def test_layers_in_one_launch(T, Hq, Hkv, D, lens, n_layers):
+@pytest.mark.parametrize("apart", [True, False])
+def test_layers_in_one_launch(T, Hq, Hkv, D, lens, n_layers, apart):
+    """apart = False: a workspace too small for the parts of the step side by side, which then wait for each other."""
     K, H, V, B = 4, 64, 600, len(lens)
     tb, tree = make_tree("rank_prior", K, (), T)
     Lcap = max(lens) + T + 3
@@ -42,7 +44,7 @@ def test_layers_in_one_launch(T, Hq, Hkv, D, lens, n_layers):
     a.stride_b, a.stride_h, a.stride_t = ks[0].stride()[:3]
     for n, t in d.items():
         setattr(a, n, t.data_ptr())
-    a.ws_bytes = d["ws"].numel()
+    a.ws_bytes = d["ws"].numel() if apart else workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap).numel()
     want = [ref.tree_attention(q[l].cpu(), ks[l].cpu(), vs[l].cpu(), torch.tensor(lens, dtype=torch.int32), tb["mask"])
             for l in range(n_layers)]
     binding.mtv_verify_step(tree, a)
@@ -50,6 +52,9 @@ def test_layers_in_one_launch(T, Hq, Hkv, D, lens, n_layers):
     assert binding.mtv_device_error(tree) == 0
     for l in range(n_layers):
         assert_close(d["out_layers"][l], want[l], "layer %d" % l)
+    acc = ref.tree_accept(ref.node_argmax(d["logits"].cpu()), d["tree_tok"].cpu(), tb)
+    assert d["accept_len"].tolist() == acc["accept_len"].tolist() and d["next_root"].tolist() == acc["next_root"].tolist()
+    assert d["seq_lens"].tolist() == [L + n + 1 for L, n in zip(lens, d["accept_len"].tolist())]
 
 
 @pytest.mark.parametrize("T,Hq,Hkv,D,lens,Lcap", [
