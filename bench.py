@@ -430,8 +430,7 @@ def run_ours(args):
         per_step = {k: (sum(v) / tap_steps if v else 0.0) for k, v in tm.items()}
         out["kernel_ms_per_step"] = per_step
         dom = max(per_step, key=per_step.get)
-        bytes_of = {"heads_vocab_topk": alg["heads_vocab"], "attn_partial": alg["attn_per_layer"] * n_layers,    # all layers of a step in one launch
-                   
+        bytes_of = {"heads_vocab_topk": alg["heads_vocab"], "attn_partial": alg["attn_per_layer"] * n_layers,    # one launch
                     "argmax_partial": alg["accept"], "heads_resblock": alg["heads"] - alg["heads_vocab"]}
         ach = bytes_of.get(dom, 0) / avg[dom] / 1e6
         out["roofline"] = {"kernel": dom, "bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
