@@ -65,8 +65,8 @@ def peaks():
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu captures summarised under
 # profiles/, keyed by tap name, with the hash of the kernel's source at capture time: a changed kernel reports null.
 NCU_TRAFFIC = {
-    "heads_vocab_topk": ("heads.cu", "914e411d83fc386f", 4.2995e9),
-    "lm_head_argmax": ("lm_head.cu", "8eac35b20edf1166", 1.0795e9),
+    "heads_vocab_topk": ("heads.cu", "b59857872e55bb9a", 4.2960e9),
+    "lm_head_argmax": ("lm_head.cu", "58bde0fae376055d", 1.0769e9),
 }
 
 
