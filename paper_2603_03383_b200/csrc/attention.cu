@@ -11,9 +11,9 @@
 //   * More items than teams: an item counts its groups plus AT_ITEM_COST (what starting and ending an item costs beside
 //     its groups) and the cuts fall anywhere.
 //   * Fewer: no CTA gets two pieces; the piece length is the smallest for which the pieces of all items fit the teams.
-// Pieces that are not whole items leave O / l (bf16; fp32 at head size 64) and (m, l) in the workspace; at the end of the launch the CTAs that
-// share an item meet at a counter and each combines a slice of its rows.  That needs all CTAs resident together: the
-// grid never exceeds one CTA per SM; the wait is bounded all the same.
+// Pieces that are not whole items leave O / l (fp32: where an item is cut must not show in its precision) and (m, l) in the
+// workspace; at the end of the launch the CTAs that share an item meet at a counter and each combines a slice of its rows.
+// That needs all CTAs resident together: the grid never exceeds one CTA per SM; the wait is bounded all the same.
 //
 // One piece.  Two STREAMS of 128 query rows by 128 keys share the tensor core: with two row tiles stream t owns tile t and
 // both see every key group; with one row tile both use it and take alternate groups (merged at the end).  A stream runs
@@ -123,7 +123,7 @@ struct AttnParams {
     const int32_t *seq_lens;
     const uint64_t *anc;     // [T][2]
     __nv_bfloat16 *out;      // [layers][B][T][Hq][D]
-    uint4 *ws_o;             // [CTA][2 slabs][2 tiles][16 chunks][128 rows] 16-byte chunks of O / l: bf16 at D = 128, fp32 at D = 64
+    uint4 *ws_o;             // [CTA][2 slabs][2 tiles][D / 4 chunks][128 rows] 16-byte chunks of O / l, fp32
     float2 *ws_ml;           // [CTA][2 slabs][2 tiles][128 rows] (m, l)
     int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls
     int32_t *status;         // [B] or null
@@ -665,10 +665,9 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         auto item_out = [&](int layer, int b, int hd) {      // first row of an item's output
             return reinterpret_cast<uint4 *>(p.out + (((size_t)layer * p.B + b) * p.T * p.Hq + hd * p.G) * D);
         };
-        // slabs of the workspace: 16-byte chunk c of row r of tile t (8 columns in bf16 at D = 128, 4 in fp32 at D = 64); the
-        // row's (m, l)
+        // slabs of the workspace: 16-byte chunk c (4 columns) of row r of tile t; the row's (m, l)
         auto slab_o = [&](int cta, int slab, int t, int r, int c) {
-            return p.ws_o + ((((unsigned)cta * 2 + slab) * 2 + t) * 16 + c) * 128 + r;
+            return p.ws_o + ((((unsigned)cta * 2 + slab) * 2 + t) * (D / 4) + c) * 128 + r;
         };
         auto slab_ml = [&](int cta, int slab, int t, int r) { return p.ws_ml + (((unsigned)cta * 2 + slab) * 2 + t) * 128 + r; };
         constexpr uint32_t hidden = NEG ? 0x7f800000u : 0xff800000u;   // times the scale: -inf
@@ -875,18 +874,18 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 }
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    const uint4 x = make_uint4(pack2_bf16(v[8 * e], v[8 * e + 1]), pack2_bf16(v[8 * e + 2], v[8 * e + 3]),
-                                               pack2_bf16(v[8 * e + 4], v[8 * e + 5]), pack2_bf16(v[8 * e + 6], v[8 * e + 7]));
                     const uint32_t ch = (uint32_t)c0 / 8 + e;
-                    if (partial && mine && D == 64) {
+                    if (!partial) {
+                        *reinterpret_cast<uint4 *>(stage + lane * rowb + ((ch ^ (lane & (n_ch - 1))) << 4)) =
+                            make_uint4(pack2_bf16(v[8 * e], v[8 * e + 1]), pack2_bf16(v[8 * e + 2], v[8 * e + 3]),
+                                       pack2_bf16(v[8 * e + 4], v[8 * e + 5]), pack2_bf16(v[8 * e + 6], v[8 * e + 7]));
+                    } else if (mine) {
 #pragma unroll
                         for (int q = 0; q < 2; ++q)
                             *slab_o(blockIdx.x, slab, tile, row, c_begin / 4 + 2 * ch + q) =
                                 make_uint4(__float_as_uint(v[8 * e + 4 * q]), __float_as_uint(v[8 * e + 4 * q + 1]),
                                            __float_as_uint(v[8 * e + 4 * q + 2]), __float_as_uint(v[8 * e + 4 * q + 3]));
                     }
-                    if (!partial) *reinterpret_cast<uint4 *>(stage + lane * rowb + ((ch ^ (lane & (n_ch - 1))) << 4)) = x;
-                    else if (mine && D == 128) *slab_o(blockIdx.x, slab, tile, row, c_begin / 8 + ch) = x;
                 }
             }
             if (!partial) {
@@ -935,7 +934,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             __syncwarp();
             // rows of the item: tile 0's, then tile 1's; this CTA combines its share of them, a thread per 16-byte chunk of the
             // output, with the loads of several contributors in flight
-            constexpr int VC = D == 128 ? 1 : 2, NS = 6 / VC;    // chunks per thread and contributor; contributors at a time
+            constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
             const int rows = one ? p.R : 2 * p.R;
             const int per = (rows + m.n - 1) / m.n, r_begin = (team - m.first) * per;
             const int n_my = max(0, min(rows, r_begin + per) - r_begin);
@@ -977,14 +976,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                         for (int q = 0; q < VC; ++q) {
                             const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
 #pragma unroll
-                            for (int i = 0; i < 4; ++i) {
-                                if (D == 128) {
-                                    acc[2 * i] = fmaf(w, bf16_lo(vw[i]), acc[2 * i]);
-                                    acc[2 * i + 1] = fmaf(w, bf16_hi(vw[i]), acc[2 * i + 1]);
-                                } else {
-                                    acc[4 * q + i] = fmaf(w, __uint_as_float(vw[i]), acc[4 * q + i]);
-                                }
-                            }
+                            for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(w, __uint_as_float(vw[i]), acc[4 * q + i]);
                         }
                     }
                 }
@@ -1100,7 +1092,7 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
     const AttnPlan a = attn_plan(t->T, Hq / Hkv);
     const size_t slabs = (size_t)a.teams * a.n_blk * 2;
     w.o_off = 0;
-    w.ml_off = align_up(slabs * 2 * 16 * 128 * sizeof(uint4), 256);
+    w.ml_off = align_up(slabs * 2 * 128 * D * sizeof(float), 256);
     w.total = align_up(w.ml_off + slabs * 2 * 128 * sizeof(float2), 256);
     if (attn_pair_eligible(D, Hq / Hkv)) {
         int n_blk = 1;
