@@ -69,10 +69,21 @@ constexpr int AT_MAX_LAYERS = 64;     // layers per launch (two tensor maps each
 // registers per thread: 96 at launch, moved from the four auxiliary warps to the sixteen softmax warps
 constexpr int AT_LAUNCH_REGS = 96, AT_SOFTMAX_REGS = 104, AT_AUX_REGS = 64;
 static_assert(512 * AT_SOFTMAX_REGS + 128 * AT_AUX_REGS <= AT_THREADS * AT_LAUNCH_REGS, "register split");
+// P goes to the tensor core as bf16, whose rounding is the largest error beside the output's own.  Where a reference that
+// follows the row's maximum made the largest weights exact (they were 1), a fixed reference does not: P then has a second bf16
+// term, what the rounding of the first left.  At head size 64 in every group (O += P V is short there); at 128 in a piece's
+// first group, whose maximum alone used to be the reference.  Rel. error against 64 bits with one term / two / the kernels that
+// this one replaced: D = 64, L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 / .00210; D = 128, L = 512:
+// .00235 / .00204 / .00268.  Cost: eight one-layer calls at head size 64 171 -> 198 us, steps at 128 1 to 2 %.
+template <int D>
+__host__ __device__ constexpr bool two_terms(int group) { return D == 64 || group == 0; }   // of the stream's groups of a piece
 constexpr float AT_SUM_LIMIT = 4294967296.f;   // 2^32: a thread's sum of P over a group beyond it moves the reference
 constexpr float LOG2E = 1.4426950408889634f;
 
-constexpr uint32_t TM_S = 0, TM_O = 256;   // tensor-memory columns: S of stream t at 128 t (P over its first half), O at 256 + 128 t
+// tensor-memory columns: S of stream t at 128 t, O at 256 + 128 t.  P lies over S, each half of the keys over its own scores:
+// keys 0-63 at columns 0-31, keys 64-127 at 64-95; in two terms each quarter over its own: keys 0-31 at columns 0-15, their
+// second terms at 16-31, and so on.
+constexpr uint32_t TM_S = 0, TM_O = 256;
 
 // Shared memory: two query tiles, the K/V ring, the (m, l) exchange of the two streams, barriers, descriptors.
 template <int D>
@@ -141,11 +152,14 @@ struct AttnParams {
 constexpr uint32_t AT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
 constexpr uint32_t AT_B_NMAJOR = 1u << 16;
 
-// P = 2^(scale S - m) of 32 scores (two values per instruction where the instruction set has packed forms): bf16 pairs and
-// their contribution to the row sum.  Every fourth quadruple runs on the FMA pipes: the special-function unit is the
-// bottleneck of a group.
-template <int DEGREE>
-__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t (&pk)[16]) {
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+__device__ __forceinline__ float trunc_bf16(float x) { return bf16_hi(__float_as_uint(x)); }
+// P = 2^(scale S - m) of 32 scores (two values per instruction where the instruction set has packed forms) and its
+// contribution to the row sum.  Every fourth quadruple runs on the FMA pipes: the special-function unit is the bottleneck of
+// a group.  pk: bf16 pairs; TWO: rest has what their rounding left, as bf16 pairs.
+template <int DEGREE, bool TWO>
+__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t *pk, uint32_t *rest) {
 #pragma unroll
     for (int e = 0; e < 16; e += 2) {
         const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2);
@@ -160,8 +174,17 @@ __device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2,
         }
         la = __fadd2_rn(la, p01);
         lb = __fadd2_rn(lb, p23);
-        pk[e] = pack2_bf16(p01.x, p01.y);
-        pk[e + 1] = pack2_bf16(p23.x, p23.y);
+        if (TWO) {
+            pk[e] = pack2_bf16(p01.x, p01.y);
+            pk[e + 1] = pack2_bf16(p23.x, p23.y);
+            const float2 r01 = __fadd2_rn(p01, make_float2(-bf16_lo(pk[e]), -bf16_hi(pk[e])));
+            const float2 r23 = __fadd2_rn(p23, make_float2(-bf16_lo(pk[e + 1]), -bf16_hi(pk[e + 1])));
+            rest[e] = pack2_bf16(r01.x, r01.y);
+            rest[e + 1] = pack2_bf16(r23.x, r23.y);
+        } else {
+            pk[e] = pack2_bf16(p01.x, p01.y);
+            pk[e + 1] = pack2_bf16(p23.x, p23.y);
+        }
     }
 }
 // the largest scale * s of 32 scores; NEG: the scale is negative
@@ -176,8 +199,6 @@ __device__ __forceinline__ float max_quarter(const uint32_t (&s)[32], float scal
     }
     return fmaxf(a, b) * fabsf(scale);
 }
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
 // Build option -DMTV_TRACE: cycle stamps of one CTA's phases into a buffer given by mtv_trace_set (development aid).
 #ifdef MTV_TRACE
 __device__ long long *g_trace = nullptr;   // [ctas][8 rows][512]
@@ -600,15 +621,28 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 const uint32_t dv = ring_v_lo + s * (SM::TILE >> 4);
                 constexpr uint32_t idesc = AT_IDESC | AT_B_NMAJOR | ((uint32_t)(D / 8) << 17);
                 const int steps = j == cnt - 1 ? last_steps : 8;
-                // P of keys 0-63 lies at columns 0-31, that of keys 64-127 at 64-95
-                if (steps == 8) {
+                // the A operand of sixteen keys: where P lies (see TM_S)
+                auto issue_pv = [&](int kk, uint32_t col, bool accumulate) {
+                    ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + col, dv + kk * 128, ptx::DESC_HI, idesc, accumulate, leader);
+                };
+                if (two_terms<D>(i - 1)) {
+                    if (steps == 8 && D == 64) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk)
-                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, ptx::DESC_HI, idesc, j > first || kk > 0, leader);
+                        for (int kk = 0; kk < 16; ++kk)
+                            issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > first || kk > 0);
+                    } else {
+#pragma unroll 1
+                        for (int kk = 0; kk < 2 * steps; ++kk) {
+                            const int k = kk >> 1;
+                            issue_pv(k, k / 2 % 2 * 32 + k % 2 * 8 + kk % 2 * 16, j > first || kk > 0);
+                        }
+                    }
+                } else if (steps == 8) {
+#pragma unroll
+                    for (int kk = 0; kk < 8; ++kk) issue_pv(kk, kk % 4 * 8, true);
                 } else {
 #pragma unroll 1
-                    for (int kk = 0; kk < steps; ++kk)
-                        ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + (kk % 4) * 8, dv + kk * 128, ptx::DESC_HI, idesc, j > first || kk > 0, leader);
+                    for (int kk = 0; kk < steps; ++kk) issue_pv(kk, kk % 4 * 8, true);
                 }
                 p_ph ^= 1;
                 TRACE();
@@ -694,7 +728,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 const float alpha = need ? ex2(m_used - m_new) : 1.f;
                 uint32_t x[16];
 #pragma unroll 1
-                for (int c = 0; p_written && c < 2; ++c) {       // (a power of two: exact)
+                for (int c = 0; p_written && c < 4; ++c) {       // both terms (a power of two: exact)
                     ptx::tmem_ld16(t_s + c * 16, x);
                     ptx::tmem_ld_wait_for16(x);
 #pragma unroll
@@ -741,25 +775,74 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             begun = false;
             const bool releases = qd == 0 && hf == 0 && lane == 0;
             if (first >= cnt && releases) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + tile));
-            for (int j = first; j < cnt; j += step) {
-                uint32_t pk[32];
+            // These scores are complete: this stream is done with their K tile and, the MMAs before them being complete too, with
+            // the V tile of its previous group.
+            auto scores_done = [&](int j) {
+                s_ph ^= 1;
+                TRACE();
+                ptx::tc_fence_after();
+                if (releases) {
+                    ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)k_pos(one, j)) % ST));
+                    if (j >= step) ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)v_pos(one, j - step, cnt)) % ST));
+                    if (j + step >= cnt) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + tile));
+                }
+            };
+            auto p_done = [&]() {
+                ptx::tmem_st_wait();
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar_p);
+                begun = true;
+                TRACE();
+            };
+            constexpr int DEGREE = D == 128 ? 3 : 4;
+            const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+            // ---- the first group: its maximum, then its P in two terms, a quarter at a time (the scores are loaded twice, which
+            //      costs less than the registers of all of them in two terms)
+            if (first < cnt) {
+                if (!ptx::mbar_wait(bar_s, s_ph)) { ok = false; break; }
+                scores_done(first);
+                const int a0 = a_first + first * AT_BN;      // tree row of this half's first column
+                auto quarter = [&](uint32_t (&q)[32], int c) {
+                    ptx::tmem_ld32(t_s + 32 * c, q);
+                    ptx::tmem_ld_wait_for(q);
+                    if (a0 + 64 > 0) {       // bit e of vis is column e (see below)
+                        const uint32_t vis = __funnelshift_r(anc_word((a0 >> 5) + c), anc_word((a0 >> 5) + c + 1), a0 & 31);
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (!((vis >> e) & 1u)) q[e] = hidden;
+                    }
+                };
+                uint32_t q[32], pk[16], rest[16];
+                float mx = -INFINITY;
+#pragma unroll 1
+                for (int c = 0; c < 2; ++c) {
+                    quarter(q, c);
+                    mx = fmaxf(mx, max_quarter<NEG>(q, p.scale_log2));
+                }
+                move_reference(mx, true, false);
+                if (!ok) break;
+                const float m_eff = m_used == -INFINITY ? 0.f : m_used;
+                float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int c = 0; c < 2; ++c) {
+                    quarter(q, c);
+                    exp_quarter<DEGREE, true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, rest);
+                    ptx::tmem_st16(t_s + 32 * c, pk);
+                    ptx::tmem_st16(t_s + 32 * c + 16, rest);
+                }
+                l = (la.x + la.y) + (lb.x + lb.y);
+                p_done();
+            }
+            for (int j = first + step; j < cnt; j += step) {
                 float sum;
-                bool moves = j == first, asked = false;
+                bool asked = false;
 #pragma unroll 1
                 for (;;) {
                     if (!asked) {
                         wait_tc(bar_s, s_ph);
                         if (!ok) break;
-                        s_ph ^= 1;
-                        TRACE();
-                        ptx::tc_fence_after();
-                        // These scores are complete: this stream is done with their K tile and, the MMAs before them being
-                        // complete too, with the V tile of its previous group.
-                        if (releases) {
-                            ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)k_pos(one, j)) % ST));
-                            if (j >= step) ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)v_pos(one, j - step, cnt)) % ST));
-                            if (j + step >= cnt) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + tile));
-                        }
+                        scores_done(j);
                     }
                     uint32_t qa[32], qb[32];
                     ptx::tmem_ld32(t_s, qa);
@@ -778,31 +861,45 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                             if (!((vb >> e) & 1u)) qb[e] = hidden;
                         }
                     }
-                    if (moves) {
+                    if (asked) {
                         const float mx = fmaxf(max_quarter<NEG>(qa, p.scale_log2), max_quarter<NEG>(qb, p.scale_log2));
-                        move_reference(asked && !(mx > m_used + 16.f) ? -INFINITY : mx, !asked, false);
-                        moves = false;
+                        move_reference(mx > m_used + 16.f ? mx : -INFINITY, false, false);
                     }
                     const float m_eff = m_used == -INFINITY ? 0.f : m_used;
-                    const float2 sc2 = make_float2(p.scale_log2, p.scale_log2), nm2 = make_float2(-m_eff, -m_eff);
+                    const float2 nm2 = make_float2(-m_eff, -m_eff);
                     float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-                    exp_quarter<D == 128 ? 3 : 4>(qa, sc2, nm2, la, lb, *reinterpret_cast<uint32_t(*)[16]>(&pk[0]));
-                    exp_quarter<D == 128 ? 3 : 4>(qb, sc2, nm2, la, lb, *reinterpret_cast<uint32_t(*)[16]>(&pk[16]));
-                    sum = (la.x + la.y) + (lb.x + lb.y);
-                    if (asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT)) break;   // (rows that belong to nobody may hold anything)
+                    // (rows that belong to nobody may hold anything)
+                    auto fits = [&]() {
+                        sum = (la.x + la.y) + (lb.x + lb.y);
+                        return asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT);
+                    };
+                    if constexpr (two_terms<D>(1)) {
+                        uint32_t pa[16], pb[16], ra[16], rb[16];
+                        exp_quarter<DEGREE, true>(qa, sc2, nm2, la, lb, pa, ra);
+                        exp_quarter<DEGREE, true>(qb, sc2, nm2, la, lb, pb, rb);
+                        if (fits()) {
+                            ptx::tmem_st16(t_s, pa);
+                            ptx::tmem_st16(t_s + 16, ra);
+                            ptx::tmem_st16(t_s + 32, pb);
+                            ptx::tmem_st16(t_s + 48, rb);
+                            break;
+                        }
+                    } else {
+                        uint32_t pk[32];
+                        exp_quarter<DEGREE, false>(qa, sc2, nm2, la, lb, pk, nullptr);
+                        exp_quarter<DEGREE, false>(qb, sc2, nm2, la, lb, pk + 16, nullptr);
+                        if (fits()) {
+                            ptx::tmem_st32(t_s, pk);
+                            break;
+                        }
+                    }
                     // rare: ask the other warp of these rows to come and move the reference, start over
-                    asked = moves = true;
+                    asked = true;
                     if (lane == 0) beyond[st * 4 + qd] = 1;
                 }
                 if (!ok) break;
                 l += sum;
-                ptx::tmem_st32(t_s, pk);
-                ptx::tmem_st_wait();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_p);
-                begun = true;
-                TRACE();
+                p_done();
             }
             // ---- the stream's O of this piece
             const bool ran = first < cnt;       // (a one-tile piece of a single group has no second stream)

@@ -44,6 +44,10 @@ def _step_attention(tree, q, ks, vs, lens, Hkv, D, Lcap):
 @pytest.mark.parametrize("T,Hq,Hkv,D,lens,n_layers,roundings", [
     (64, 32, 8, 128, [1500] * 6, 2, 2),        # items cut anywhere: 96 of 13 groups on 148 SMs
     (64, 8, 2, 128, [3000], 4, 2),             # one item over many SMs
+    (64, 8, 2, 128, [50, 64], 6, 1),           # a single group: two-term weights
+    (29, 8, 2, 64, [128], 8, 1),               # head size 64: two-term weights in every group; one row tile
+    (128, 16, 2, 64, [97, 2000], 2, 1),        # several row blocks, last groups of every length
+    (65, 7, 1, 64, [1000], 3, 1),              # rows that belong to nobody
 ])
 def test_error_of_a_step(T, Hq, Hkv, D, lens, n_layers, roundings):
     tb, tree = make_tree("rank_prior", 4, (), T)
