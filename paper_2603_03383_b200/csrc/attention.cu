@@ -38,9 +38,10 @@
 // two shorten that chain: a warp's exponentials take 1.2 k cycles for 128 columns, most of it latency.
 //
 // The reference of a row's exponentials is the maximum of its first group, rounded up to a whole number; it moves only when
-// the sum of a thread's P in some later group exceeds 2^32.  P and O are floating-point numbers, so a reference that is not
-// the maximum costs no precision, only range; in return no maximum is formed and nothing is exchanged between the two
-// threads of a row in an ordinary group.
+// the sum of a thread's P in some later group exceeds 2^32, or one of its exponents 32 where a polynomial would not show it in
+// the sum (from 128 on its result is meaningless).  P and O are floating-point numbers, so a reference that is not the maximum
+// costs range, and the exactness of the largest weights, which a second term of P makes up for (see two_terms); in return no
+// maximum is formed and nothing is exchanged between the two threads of a row in an ordinary group.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -157,15 +158,19 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 __device__ __forceinline__ float trunc_bf16(float x) { return bf16_hi(__float_as_uint(x)); }
 // P = 2^(scale S - m) of 32 scores (two values per instruction where the instruction set has packed forms) and its
 // contribution to the row sum.  Every fourth quadruple runs on the FMA pipes: the special-function unit is the bottleneck of
-// a group.  pk: bf16 pairs; TWO: rest has what their rounding left, as bf16 pairs.
+// a group.  pk: bf16 pairs; TWO: rest has what their rounding left, as bf16 pairs.  top: the largest exponent among those of
+// the polynomials, which go wrong silently where ex2 gives +inf or NaN.
 template <int DEGREE, bool TWO>
-__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t *pk, uint32_t *rest) {
+__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t *pk, uint32_t *rest,
+                                            float &top) {
 #pragma unroll
     for (int e = 0; e < 16; e += 2) {
         const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2);
         const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e + 2]), __uint_as_float(s[2 * e + 3])), sc2, nm2);
         float2 p01, p23;
         if (e % 8 == 6) {
+            top = ptx::fmax3_nan(top, x01.x, x01.y);
+            top = ptx::fmax3_nan(top, x23.x, x23.y);
             p01 = exp2_poly2<DEGREE>(x01);
             p23 = exp2_poly2<DEGREE>(x23);
         } else {
@@ -824,14 +829,15 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 if (!ok) break;
                 const float m_eff = m_used == -INFINITY ? 0.f : m_used;
                 float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+                float top = -INFINITY;
 #pragma unroll 1
                 for (int c = 0; c < 2; ++c) {
                     quarter(q, c);
-                    exp_quarter<DEGREE, true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, rest);
+                    exp_quarter<DEGREE, true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, rest, top);
                     ptx::tmem_st16(t_s + 32 * c, pk);
                     ptx::tmem_st16(t_s + 32 * c + 16, rest);
                 }
-                l = (la.x + la.y) + (lb.x + lb.y);
+                l = top != top ? top : (la.x + la.y) + (lb.x + lb.y);      // (no exponent is above 0 here)
                 p_done();
             }
             for (int j = first + step; j < cnt; j += step) {
@@ -861,22 +867,24 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                             if (!((vb >> e) & 1u)) qb[e] = hidden;
                         }
                     }
-                    if (asked) {
+                    if (asked) {      // (by a NaN, too, which the row's sum then has to show)
                         const float mx = fmaxf(max_quarter<NEG>(qa, p.scale_log2), max_quarter<NEG>(qb, p.scale_log2));
                         move_reference(mx > m_used + 16.f ? mx : -INFINITY, false, false);
                     }
                     const float m_eff = m_used == -INFINITY ? 0.f : m_used;
                     const float2 nm2 = make_float2(-m_eff, -m_eff);
                     float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
+                    float top = -INFINITY;
                     // (rows that belong to nobody may hold anything)
                     auto fits = [&]() {
                         sum = (la.x + la.y) + (lb.x + lb.y);
-                        return asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT);
+                        if (asked && top != top) sum = top;
+                        return asked || !__any_sync(0xffffffffu, mine && (sum > AT_SUM_LIMIT || !(top <= 32.f)));
                     };
                     if constexpr (two_terms<D>(1)) {
                         uint32_t pa[16], pb[16], ra[16], rb[16];
-                        exp_quarter<DEGREE, true>(qa, sc2, nm2, la, lb, pa, ra);
-                        exp_quarter<DEGREE, true>(qb, sc2, nm2, la, lb, pb, rb);
+                        exp_quarter<DEGREE, true>(qa, sc2, nm2, la, lb, pa, ra, top);
+                        exp_quarter<DEGREE, true>(qb, sc2, nm2, la, lb, pb, rb, top);
                         if (fits()) {
                             ptx::tmem_st16(t_s, pa);
                             ptx::tmem_st16(t_s + 16, ra);
@@ -886,8 +894,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                         }
                     } else {
                         uint32_t pk[32];
-                        exp_quarter<DEGREE, false>(qa, sc2, nm2, la, lb, pk, nullptr);
-                        exp_quarter<DEGREE, false>(qb, sc2, nm2, la, lb, pk + 16, nullptr);
+                        exp_quarter<DEGREE, false>(qa, sc2, nm2, la, lb, pk, nullptr, top);
+                        exp_quarter<DEGREE, false>(qb, sc2, nm2, la, lb, pk + 16, nullptr, top);
                         if (fits()) {
                             ptx::tmem_st32(t_s, pk);
                             break;
@@ -939,7 +947,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 l_all = w_own * l_all + w_oth * l_oth;
             }
             if (!ok) break;
-            const float inv_l = l_all > 0.f ? 1.f / l_all : 0.f;
+            const float inv_l = l_all == 0.f ? 0.f : 1.f / l_all;     // (NaN stays NaN)
             w_own *= inv_l;
             w_oth *= inv_l;
             // this thread's columns: a half of them, a quarter in a one-tile piece.  Partial results go to the workspace, whose
@@ -1077,7 +1085,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                         }
                     }
                 }
-                const float inv = wsum > 0.f ? 1.f / wsum : 0.f;
+                const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
                 const int o = out_row(t, r);
                 if (o >= 0)
                     dst[o * (D / 8) + c] =

@@ -15,7 +15,8 @@ __device__ __forceinline__ float ex2(float x) {
 // 2^x for two values on the FMA pipes: x = j + f with j the nearest integer (read off the low mantissa bits of
 // x + 1.5 * 2^23) and f in [-0.5, 0.5]; 2^f by a polynomial with the smallest largest relative error over that interval
 // (degree 3: 7.5e-5, far below the bf16 rounding of P; degree 4: 3.7e-6); 2^j by an add to the exponent field.  x is
-// clamped at -126 (the result then underflows towards zero like ex2's).
+// clamped at -126 (the result then underflows towards zero like ex2's).  From x = 128 on the exponent field overflows (the
+// result may be negative, NaN or small) and a NaN counts as -126: the caller sees to it that neither is used.
 template <int DEGREE>
 __device__ __forceinline__ float2 exp2_poly2(float2 x) {
     const float magic = 12582912.f;
