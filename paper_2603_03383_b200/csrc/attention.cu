@@ -758,12 +758,16 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             meet();
             ptx::tc_fence_after();
         };
-        // Waits for the tensor core; meanwhile the other warp of these rows may ask to move the reference.
+        // Waits for the tensor core; meanwhile the other warp of these rows may ask to move the reference.  If it asks for the
+        // very group that is waited for (complete between the two tests), this warp's P of that group does not exist yet: the
+        // barrier, tested again behind the flag, then says so, the group is taken first, and the question is met at the next
+        // wait.  Otherwise the asked-for group is the one whose P this warp has written, and the barrier cannot complete
+        // before they have met.
         auto wait_tc = [&](uint32_t b, uint32_t parity) {
             const long long t0 = clock64();
             while (!ptx::mbar_try_wait(b, parity)) {
                 if (beyond[st * 4 + qd]) {
-                    move_reference(-INFINITY, false, true);
+                    if (!ptx::mbar_try_wait(b, parity)) move_reference(-INFINITY, false, true);
                     continue;
                 }
                 if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { ok = false; return; }
