@@ -1007,6 +1007,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                     const int o = out_row(tile, qd * 32 + r);
                     if (o >= 0) dst[o * (D / 8)] = x;
                 }
+                ptx::fence_proxy_async();         // (the next tile comes into the slot through the async proxy)
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_STAGED + slot));
             }
