@@ -1199,9 +1199,10 @@ AttnPlan attn_plan(int T, int G) {
 // pairs keeps a slab per key split of a query block and the order of the sequences.
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap) {
     AttnWs w;
+    w.o_off = w.ml_off = w.total = 0;
+    if (Hq / Hkv > 8) return w;          // the call itself refuses such a group; sizes are asked for before that
     const AttnPlan a = attn_plan(t->T, Hq / Hkv);
     const size_t slabs = (size_t)a.teams * a.n_blk * 2;
-    w.o_off = 0;
     w.ml_off = align_up(slabs * 2 * 128 * D * sizeof(float), 256);
     w.total = align_up(w.ml_off + slabs * 2 * 128 * sizeof(float2), 256);
     if (attn_pair_eligible(D, Hq / Hkv)) {

@@ -106,3 +106,10 @@ def test_hot_calls_validate_before_touching_the_device():
     assert lib.kv_compact_accepted(t.handle, 1, 2, 64, 1, one, one, 8, 8, 7, 16, one, one, one, None, None) == -1
     assert lib.mtv_workspace_bytes(None, 1, 8, 8, 4, 2, 64, 16) == 0
     assert lib.mtv_last_error() is not None
+
+
+@pytest.mark.parametrize("Hq,Hkv,D", [(9, 1, 128), (64, 1, 64), (129, 1, 128), (256, 1, 64), (4096, 2, 128)])
+def test_sizes_of_a_group_that_no_call_takes(Hq, Hkv, D):
+    """More query heads per KV head than a call takes: asking for a size answers, as the refusing call does."""
+    t = binding.Tree(3, binding.tree_gen_cartesian([4, 2, 2]), upload=False)
+    assert binding.mtv_workspace_bytes(t, 2, 64, 1000, Hq, Hkv, D, 500) >= binding.mtv_workspace_bytes(t, 2, 64, 1000, 0, 0, 0, 0) > 0
