@@ -39,10 +39,15 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
 
 // grid = (nsplit, B*T).  Partial argmax of one chunk of one row.
 __global__ void __launch_bounds__(ARGMAX_THREADS)
-node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsigned long long *__restrict__ part, int alongside) {
-    // alongside: the logits were complete before the previous kernel started, which is then only waited for at the end
+node_argmax_partial_kernel(int V, const __nv_bfloat16 *logits, unsigned long long *part, const Gate gate) {
+    // with a gate the logits are complete behind it, and the previous kernel is only waited for at the end
     let_next_start();
-    if (!alongside) previous_done();
+    if (!gate.word) {
+        previous_done();
+    } else {
+        if (threadIdx.x == 0) wait_gate(gate);
+        __syncthreads();
+    }
     const int row = blockIdx.y, ns = gridDim.x;
     // chunk boundaries on multiples of 8 elements so that 16-byte loads stay aligned
     const int per = ((V + ns - 1) / ns + 7) / 8 * 8;
@@ -65,7 +70,7 @@ node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsi
                 const int i = i0 + k * ARGMAX_THREADS * 8;
                 u[k] = make_uint4(0u, 0u, 0u, 0u);
                 if (i + 8 <= end)
-                    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+                    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                                  : "=r"(u[k].x), "=r"(u[k].y), "=r"(u[k].z), "=r"(u[k].w) : "l"(p + i));
             }
 #pragma unroll
@@ -100,7 +105,7 @@ node_argmax_partial_kernel(int V, const __nv_bfloat16 *__restrict__ logits, unsi
         for (int w = 1; w < ARGMAX_THREADS / 32; ++w) best = umax64(best, sm[w]);
         part[(size_t)row * ns + blockIdx.x] = best;
     }
-    if (alongside) previous_done();
+    if (gate.word) previous_done();
 }
 
 // grid = B, block = 128.  Finish the argmax, score every path, pick the best, gather.
@@ -154,10 +159,10 @@ accept_finish_kernel(int T, int K, int P, int ns, const unsigned long long *__re
 
 namespace mtv {
 static int launch_argmax(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const AcceptWs &L, unsigned long long *part,
-                         int alongside, cudaStream_t st) {
+                         const Gate &gate, cudaStream_t st) {
     TapScope tap(MTV_KERNEL_ARGMAX_PARTIAL, st);
     MTV_CUDA_CHECK(launch_dependent(node_argmax_partial_kernel, dim3(L.nsplit, B * tree->T), ARGMAX_THREADS, 0, st, V,
-                                    reinterpret_cast<const __nv_bfloat16 *>(logits), part, alongside));
+                                    reinterpret_cast<const __nv_bfloat16 *>(logits), part, gate));
     return MTV_OK;
 }
 static int launch_finish(const mtv_tree_t *tree, int B, int ns, const unsigned long long *part, const int32_t *tree_tok,
@@ -168,15 +173,19 @@ static int launch_finish(const mtv_tree_t *tree, int B, int ns, const unsigned l
     return MTV_OK;
 }
 
-int argmax_keys_partial(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, bool alongside,
+int argmax_keys_partial(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, const Gate &alongside,
                         cudaStream_t st) {
     if (!logits || V < 1 || ((uintptr_t)logits & 15)) return MTV_ERR_INVALID_ARG;
     return launch_argmax(tree, B, V, logits, accept_ws_layout(tree, B, V), part, alongside, st);
 }
 
-int accept_logits(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
-                  int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
-                  void *stream, bool alongside) {
+}  // namespace mtv
+
+extern "C" int tree_accept(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok,
+                           int32_t *accept_len, int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok,
+                           int32_t *next_root, void *ws, size_t ws_bytes, void *stream) {
+    using namespace mtv;
+    MTV_RANGE("tree_accept");
     if (!tree || !tree->on_device || !logits || !tree_tok || !accept_len || !best_path || !acc_nodes ||
         !acc_tok || !next_root || !ws || B < 1 || V < 1)
         return MTV_ERR_INVALID_ARG;
@@ -186,19 +195,10 @@ int accept_logits(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, 
     if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
     cudaStream_t st = (cudaStream_t)stream;
     auto *part = reinterpret_cast<unsigned long long *>((char *)ws + L.part_off);
-    const int rc = launch_argmax(tree, B, V, logits, L, part, alongside, st);
+    const int rc = launch_argmax(tree, B, V, logits, L, part, Gate{}, st);
     if (rc != MTV_OK) return rc;
     TapScope tap(MTV_KERNEL_ACCEPT_FINISH, st);
     return launch_finish(tree, B, L.nsplit, part, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, st);
-}
-}  // namespace mtv
-
-extern "C" int tree_accept(const mtv_tree_t *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok,
-                           int32_t *accept_len, int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok,
-                           int32_t *next_root, void *ws, size_t ws_bytes, void *stream) {
-    MTV_RANGE("tree_accept");
-    return mtv::accept_logits(tree, B, V, logits, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, ws, ws_bytes,
-                              stream, false);
 }
 
 // Per-node argmax keys of stored logits, in the form tree_accept_keys reads: what tree_accept computes before its path
@@ -226,7 +226,7 @@ extern "C" int node_argmax_keys(const mtv_tree_t *tree, int B, int V, const mtv_
     cudaStream_t st = (cudaStream_t)stream;
     auto *part = reinterpret_cast<unsigned long long *>((char *)ws + L.part_off);
     const int rows = B * tree->T;
-    const int rc = launch_argmax(tree, B, V, logits, L, part, 0, st);
+    const int rc = launch_argmax(tree, B, V, logits, L, part, Gate{}, st);
     if (rc != MTV_OK) return rc;
     argmax_keys_reduce_kernel<<<(rows + 127) / 128, 128, 0, st>>>(rows, L.nsplit, part, keys);
     MTV_CUDA_CHECK(cudaGetLastError());
@@ -304,7 +304,7 @@ extern "C" int tree_accept_static_scratch(const mtv_tree_t *tree, int B, int V, 
     if (rc != MTV_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     // every entry of `part` that the second kernel reads is written by the first one: nothing to clear
-    const int rc2 = launch_argmax(tree, B, V, logits, L, part, 0, st);
+    const int rc2 = launch_argmax(tree, B, V, logits, L, part, Gate{}, st);
     if (rc2 != MTV_OK) return rc2;
     return launch_finish(tree, B, L.nsplit, part, tree_tok, accept_len, best_path, acc_nodes, acc_tok, next_root, st);
 }

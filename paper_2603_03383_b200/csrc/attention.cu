@@ -145,7 +145,7 @@ struct AttnParams {
     int npc, R;              // tree nodes per tile (128 / G) and the rows they fill
     unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
     int n_tiles, n_blk, teams;
-    int alongside;           // nothing of the previous kernel is needed: it is waited for at the end
+    Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
 };
 
 // Operands: queries and keys K-major; V N-major, its next 64 columns one half tile further.
@@ -296,11 +296,14 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     }
     ptx::tc_fence_before();
     // Ends the set-up; nothing in front of it touches global memory.  Behind it the previous kernel of the stream is
-    // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters), or it does not matter.
+    // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters), or what this kernel reads
+    // was written before the gate's call.
     auto begin = [&]() -> uint32_t {
+        if (p.gate.word && threadIdx.x == 0) wait_gate(p.gate);
         asm volatile("bar.sync 0, %0;" ::"n"(AT_THREADS) : "memory");
         ptx::tc_fence_after();
-        if (!p.alongside) previous_done();
+        if (p.gate.word) ptx::fence_proxy_async_global();      // (for the TMA loads that follow)
+        else previous_done();
         return *tmem_slot;                    // tensor-memory base
     };
 
@@ -1109,7 +1112,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     __syncthreads();
     ptx::tc_fence_after();
     if (warp == AT_MMA_WARP) ptx::tmem_dealloc(*tmem_slot, 512);
-    if (p.alongside) previous_done();
+    if (p.gate.word) previous_done();
 }
 
 // ---------------------------------------------------------------------------------------- host
@@ -1275,7 +1278,7 @@ static int launch_attn(const mtv_tree *tree, const AttnPlan &a, AttnParams &p, c
 int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, int n_layers, const mtv_bf16 *q,
                           mtv_bf16 *const *k, mtv_bf16 *const *v, int64_t stride_b, int64_t stride_h, int64_t stride_t,
                           int Lcap, const int32_t *seq_lens, float scale, mtv_bf16 *out, int32_t *status, void *ws,
-                          size_t ws_bytes, void *stream, bool alongside) {
+                          size_t ws_bytes, void *stream, const Gate *alongside) {
     if (!tree || !tree->on_device || !q || !k || !v || !seq_lens || !out || !ws) return MTV_ERR_INVALID_ARG;
     if (B < 1 || Hq < 1 || Hkv < 1 || n_layers < 1 || Lcap < tree->T) return MTV_ERR_INVALID_ARG;
     if ((D != 64 && D != 128) || Hq % Hkv != 0 || Hq / Hkv > 8 || B > 65535) return MTV_ERR_UNSUPPORTED_SHAPE;
@@ -1307,7 +1310,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
     p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_tiles = a.n_tiles; p.n_blk = a.n_blk; p.teams = a.teams;
-    p.alongside = alongside;
+    p.gate = alongside ? *alongside : Gate{};
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;
     // positions in the common address space of a launch's groups are 32 bits wide
@@ -1315,7 +1318,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     int per_launch = n_layers == 1 ? 1 : AT_MAX_LAYERS;
     while (per_launch > 1 && per_launch * layer_len > 4e9) per_launch /= 2;
     for (int l = 0; l < n_layers; l += per_launch) {
-        if (l > 0) p.alongside = 0;          // (it shares the counters and the workspace with the launch before)
+        if (l > 0) p.gate = Gate{};          // (it shares the counters and the workspace with the launch before)
         p.n_layers = n_layers - l < per_launch ? n_layers - l : per_launch;
         p.out = reinterpret_cast<__nv_bfloat16 *>(out) + l * per_layer;
         const __nv_bfloat16 *ql = reinterpret_cast<const __nv_bfloat16 *>(q) + l * per_layer;

@@ -48,15 +48,23 @@ static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; 
 
 // Workspace carving shared by the entry points (all offsets 256-byte aligned).
 struct HeadsWs {
-    size_t hprime_off, part_val_off, part_idx_off, counters_off, tickets_off, xsplit_off, total;
+    size_t hprime_off, part_val_off, part_idx_off, counters_off, tickets_off, gate_off, xsplit_off, total;
     int ctas_per_head, n_counters;
     bool use_tc;   // several batch rows: vocabulary projection on the tcgen05 tensor cores
 };
 HeadsWs heads_ws_layout(int K, int B, int H, int V);
+// "Everything enqueued in front of the heads is complete": the word takes the call's number once that is so (see
+// launch_dependent), and is cleared at the end of what may wait for it.  word null: nothing to wait for.
+struct Gate {
+    int32_t *word = nullptr;
+    int32_t number = 0;
+};
 // Heads [k0, k0 + n) of a call; expand: the tree's tokens follow (the other heads' candidates are already there).
+// gate_stays: later kernels of the step wait at the gate, too, and the last of them clears it (null: the heads do).
 struct HeadsRange {
     int k0, n;
     bool expand;
+    Gate *gate_stays = nullptr;
 };
 int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
                      const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
@@ -65,30 +73,27 @@ bool heads_tc_eligible(int B, int H);
 size_t heads_tc_xsplit_bytes(int K, int H);
 int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
                     const __nv_bfloat16 *b1, const __nv_bfloat16 *W2, const int32_t *root_tok, int32_t *cand,
-                    float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, cudaStream_t st);
+                    float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, const Gate &gate, cudaStream_t st);
 
 struct AttnWs {
     size_t o_off, ml_off, pair_ml_off = 0, order_off = 0, total;
 };
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap);
-// alongside: nothing that the previous kernel in the stream writes is needed, nor its workspace touched (everything before
-// that kernel is complete, see launch_dependent): the attention starts beside that kernel's end.
+// alongside: nothing that the previous kernels in the stream back to the heads write is needed, nor their workspace touched,
+// and everything before the heads is complete at this gate: the attention starts beside the previous kernel's end.
 int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, int n_layers, const mtv_bf16 *q,
                           mtv_bf16 *const *k, mtv_bf16 *const *v, int64_t stride_b, int64_t stride_h, int64_t stride_t,
                           int Lcap, const int32_t *seq_lens, float scale, mtv_bf16 *out, int32_t *status, void *ws,
-                          size_t ws_bytes, void *stream, bool alongside = false);
+                          size_t ws_bytes, void *stream, const Gate *alongside = nullptr);
 
 struct AcceptWs {
     size_t part_off, total;
     int nsplit;
 };
 AcceptWs accept_ws_layout(const mtv_tree *t, int B, int V);
-// tree_accept; alongside: the logits were complete before the previous kernel in the stream started (as above).
-int accept_logits(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, const int32_t *tree_tok, int32_t *accept_len,
-                  int32_t *best_path, int32_t *acc_nodes, int32_t *acc_tok, int32_t *next_root, void *ws, size_t ws_bytes,
-                  void *stream, bool alongside);
-// its scan alone: per-chunk keys into part (accept_ws_layout(...).nsplit per node)
-int argmax_keys_partial(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, bool alongside,
+// tree_accept's scan alone: per-chunk keys into part (accept_ws_layout(...).nsplit per node); alongside: the logits are complete
+// at this gate (as above).
+int argmax_keys_partial(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, const Gate &alongside,
                         cudaStream_t stream);
 
 int sm_count();   // of the current device
@@ -107,12 +112,15 @@ struct PerDeviceOnce {
 };
 
 // Programmatic dependent launch: the kernel may be set up while the previous kernel of the stream runs, from the moment all
-// of that kernel's blocks have executed let_next_start() or ended.  Rules of the kernels launched so:
+// of that kernel's blocks have executed let_next_start() or ended.  What is guaranteed is that previous_done() returns when
+// the previous kernel is complete and its writes are visible.  Rules of the kernels launched so:
 //   - whatever the previous kernel (or one before it) writes is touched only behind previous_done();
 //   - every block executes previous_done() before it ends, early or late: a kernel that is complete then implies that
 //     all before it are;
-//   - a kernel that calls previous_done() in FRONT of let_next_start() makes everything enqueued before it complete for
-//     whoever follows; what follows may then read what was ready at that point without waiting (weights, logits).
+//   - what was written before the heads (weights, queries, caches, lengths, logits) may be read by the heads' second kernel
+//     and the kernels behind it without previous_done(), but behind a gate: the heads' first kernel executes previous_done(),
+//     then stores the call's number to the gate's word with release; a reader acquires it.  (That a kernel which waited has
+//     let the reader start orders nothing by itself.)  Bulk and TMA loads need the proxy fence behind the acquire.
 template <typename... P, typename... A>
 static inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, A... args) {
     cudaLaunchConfig_t cfg = {};
@@ -129,11 +137,25 @@ static inline cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, int 
 }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void open_gate(const Gate &g) {
+    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(g.word), "r"(g.number) : "memory");
+}
+// One thread; others read behind a barrier with it.  The word was stored before this kernel could start: a poll or two.
+// (Should it not come within a millisecond, waiting for the previous kernel does as well.)
+__device__ __forceinline__ void wait_gate(const Gate &g) {
+    const long long t0 = clock64();
+    int v;
+    for (;;) {
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(g.word) : "memory");
+        if (v == g.number) break;
+        if (clock64() - t0 > 2000000ll) { previous_done(); break; }
+    }
+}
 
 // The end of a step in one launch: acceptance from `ns` argmax keys per node (part [B][T][ns]), compaction, seq_lens.
-// tickets [B]: zero before the call.
+// tickets [B]: zero before the call.  gate: the step's, cleared here.
 int accept_compact(const mtv_tree *tree, const mtv_step_args *a, int ns, const unsigned long long *part, int32_t *tickets,
-                   cudaStream_t stream);
+                   const Gate &gate, cudaStream_t stream);
 
 // Index checks of the -DMTV_DEBUG_BOUNDS build: MTV_INDEX_OK(i, n, err) is true when 0 <= i < n; otherwise it
 // records MTV_ERR_BOUNDS in the device error word and is false, and the caller skips the access.  In normal builds

@@ -53,7 +53,7 @@ accept_compact_kernel(int T, int K, int P, int ns, int D, int Lcap, int n_layers
                       __nv_bfloat16 *const *__restrict__ v_caches, int64_t sb, int64_t sh, int64_t st, int32_t *seq_lens,
                       int32_t *__restrict__ accept_len, int32_t *__restrict__ best_path, int32_t *__restrict__ acc_nodes,
                       int32_t *__restrict__ acc_tok, int32_t *__restrict__ next_root, int32_t *__restrict__ status,
-                      int32_t *tickets, int32_t *__restrict__ dev_error) {
+                      int32_t *tickets, int32_t *gate, int32_t *__restrict__ dev_error) {
     __shared__ int32_t am[MTV_MAX_T], tok[MTV_MAX_T], node_of[MTV_MAX_K + 1];
     __shared__ unsigned int best_key;
     __shared__ uint4 stage[2 * MTV_MAX_K * 16];  // [k|v][j][D/8 <= 16]
@@ -61,6 +61,7 @@ accept_compact_kernel(int T, int K, int P, int ns, int D, int Lcap, int n_layers
     const int g = blockIdx.x, b = blockIdx.y, tid = threadIdx.x;
     if (tid == 0) best_key = 0;
     previous_done();
+    if (tid == 0 && g == 0 && b == 0 && blockIdx.z == 0) *gate = 0;      // every kernel that waits at it is complete
     const int L = seq_lens[b];
     // two threads per node take turns over its keys
     const int i = tid >> 1;
@@ -126,7 +127,7 @@ accept_compact_kernel(int T, int K, int P, int ns, int D, int Lcap, int n_layers
 }
 
 int accept_compact(const mtv_tree *tree, const mtv_step_args *a, int ns, const unsigned long long *part, int32_t *tickets,
-                   cudaStream_t stream) {
+                   const Gate &gate, cudaStream_t stream) {
     if (!a->tree_tok || !a->accept_len || !a->best_path || !a->acc_nodes || !a->acc_tok || !a->next_root || !a->k_caches || !a->v_caches ||
         !a->seq_lens || a->B < 1 || a->Hkv < 1 || a->n_layers < 1 || a->Lcap < 1)
         return MTV_ERR_INVALID_ARG;
@@ -141,7 +142,7 @@ int accept_compact(const mtv_tree *tree, const mtv_step_args *a, int ns, const u
                                     reinterpret_cast<__nv_bfloat16 *const *>(a->k_caches),
                                     reinterpret_cast<__nv_bfloat16 *const *>(a->v_caches), a->stride_b, a->stride_h, a->stride_t,
                                     a->seq_lens, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok, a->next_root, a->status,
-                                    tickets, tree->d_error));
+                                    tickets, gate.word, tree->d_error));
     return MTV_OK;
 }
 

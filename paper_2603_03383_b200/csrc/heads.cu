@@ -6,6 +6,8 @@
 // multiply-adds, so the kernels are organised around 16-byte coalesced weight loads
 // with many loads in flight; activations stay in shared memory in fp32 so that no
 // intermediate is rounded.
+#include <atomic>
+
 #include "common.cuh"
 #include "heads_common.cuh"
 #include "sm100_ptx.cuh"
@@ -78,7 +80,8 @@ HeadsWs heads_ws_layout(int K, int B, int H, int V) {
     w.part_idx_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(int32_t), 256);
     w.n_counters = (K + 1) * btiles + B;    // and one per sequence for the end of a step
     w.counters_off = off; w.tickets_off = off + (size_t)(K + 1) * btiles * sizeof(int32_t);
-    off = align_up(off + (size_t)w.n_counters * sizeof(int32_t), 256);
+    w.gate_off = off + (size_t)w.n_counters * sizeof(int32_t);
+    off = align_up(w.gate_off + sizeof(int32_t), 256);
     w.use_tc = heads_tc_eligible(B, H);
     w.xsplit_off = off;
     if (w.use_tc) off = align_up(off + heads_tc_xsplit_bytes(K, H), 256);
@@ -140,10 +143,11 @@ template <int NB>
 __global__ void __launch_bounds__(HEADS_THREADS)
 heads_resblock_kernel(int B, int H, int K, const __nv_bfloat16 *__restrict__ hidden,
                       const __nv_bfloat16 *__restrict__ W1, const __nv_bfloat16 *__restrict__ b1,
-                      float *__restrict__ hprime, int32_t *__restrict__ counters, int n_counters) {
+                      float *__restrict__ hprime, int32_t *__restrict__ counters, int n_counters, const Gate gate) {
     extern __shared__ float sh[];  // [NB][H]
     const int b0 = blockIdx.y * NB;
-    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at once
+    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at the gate
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) open_gate(gate);
     let_next_start();
     // tickets of the vocabulary kernel (the next launch on the stream) start at zero
     if (blockIdx.x == 0 && blockIdx.y == 0)
@@ -254,9 +258,15 @@ heads_vocab_topk_kernel(const VocabParams p) {
         __syncwarp();
     };
     // The weights do not depend on the residual block: the ring is filled while that kernel ends.
-    const int n_early = min(NST, n_chunks);
-    if (warp == VT_CONS_WARPS)
+    const int n_early = p.gate.word ? min(NST, n_chunks) : 0;
+    if (warp == VT_CONS_WARPS && n_early > 0) {
+        if (lane == 0) {
+            wait_gate(p.gate);
+            ptx::fence_proxy_async_global();
+        }
+        __syncwarp();
         for (int t = 0; t < n_early; ++t) request(t);
+    }
     previous_done();
 
     // activations: chunk c = it*32 + lane of row b lives at xs4[((b*n_it + it)*2 + half)*32 + lane]
@@ -274,7 +284,7 @@ heads_vocab_topk_kernel(const VocabParams p) {
         // ---- producer
         for (int t = n_early; t < n_chunks && !*abort_flag; ++t) {
             const int s = t % NST, use = t / NST;
-            if (!ptx::mbar_wait(bars + (NST + s) * 8, (use - 1) & 1)) { *abort_flag = 1; break; }
+            if (use > 0 && !ptx::mbar_wait(bars + (NST + s) * 8, (use - 1) & 1)) { *abort_flag = 1; break; }
             request(t);
         }
     } else {
@@ -438,7 +448,7 @@ template <int NB, int MR>
 static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, int V, const __nv_bfloat16 *hidden,
                         const __nv_bfloat16 *W1, const __nv_bfloat16 *b1, const __nv_bfloat16 *W2,
                         const int32_t *root_tok, int32_t *cand, float *cand_logit, int32_t *tree_tok,
-                        const HeadsWs &L, char *ws, cudaStream_t st) {
+                        const HeadsWs &L, char *ws, const Gate &gate, cudaStream_t st) {
     float *hprime = reinterpret_cast<float *>(ws + L.hprime_off);
     const int btiles = (B + NB - 1) / NB;
     const size_t sm1 = (size_t)NB * H * sizeof(float);
@@ -459,12 +469,14 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     {
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
         MTV_CUDA_CHECK(launch_dependent(heads_resblock_kernel<NB>, dim3(g1, btiles), HEADS_THREADS, sm1, st, B, H, r.n, hidden, W1,
-                                        b1, hprime, counters, L.n_counters));
+                                        b1, hprime, counters, L.n_counters, gate));
     }
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = r.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = hprime;
-    p.kd_arr = t->d_kd + r.k0; p.off_arr = t->d_cand_offset + r.k0; p.expand = r.expand; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
+    p.kd_arr = t->d_kd + r.k0; p.off_arr = t->d_cand_offset + r.k0; p.expand = r.expand;
+    p.gate = btiles == 1 ? gate : Gate{}; p.gate_clear = btiles == 1 && !r.gate_stays;   // (a second batch tile would meet it cleared)
+    p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
     p.part_idx = reinterpret_cast<int32_t *>(ws + L.part_idx_off);
     p.counters = counters;
@@ -501,7 +513,12 @@ int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, in
     const int mr = H < 1024 && slab >= 128 ? 4 : H < 2048 && slab >= 64 ? 2 : 1;
     auto launch = L.use_tc ? launch_heads_tc : B == 1 ? (mr == 4 ? launch_heads<1, 4> : mr == 2 ? launch_heads<1, 2> : launch_heads<1, 1>)
                   : B == 2 ? launch_heads<2, 1> : B <= 4 ? launch_heads<4, 1> : launch_heads<8, 1>;
-    const int rc = launch(tree, r, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, st);
+    static std::atomic<uint32_t> calls{0};
+    Gate gate;
+    gate.word = reinterpret_cast<int32_t *>((char *)ws + L.gate_off);
+    gate.number = (int32_t)(calls.fetch_add(1, std::memory_order_relaxed) & 0x3fffffffu) + 1;
+    if (r.gate_stays) *r.gate_stays = gate;
+    const int rc = launch(tree, r, B, H, V, h, w1, bb, w2, root_tok, cand, cand_logit, tree_tok, L, (char *)ws, gate, st);
     if (rc != MTV_OK) return rc;
     MTV_CUDA_CHECK(cudaGetLastError());
     return MTV_OK;
@@ -516,6 +533,6 @@ extern "C" int medusa_heads_topk(const mtv_tree_t *tree, int B, int H, int V,
                                  void *ws, size_t ws_bytes, void *stream) {
     MTV_RANGE("medusa_heads_topk");
     if (!tree) return MTV_ERR_INVALID_ARG;
-    return mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true}, B, H, V, hidden, W1, b1, W2, root_tok, cand, cand_logit,
+    return mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true, nullptr}, B, H, V, hidden, W1, b1, W2, root_tok, cand, cand_logit,
                                  tree_tok, ws, ws_bytes, stream);
 }

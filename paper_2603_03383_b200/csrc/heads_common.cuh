@@ -78,6 +78,8 @@ struct VocabParams {
     float *cand_logit;
     int32_t *tree_tok;
     int32_t *dev_error;
+    Gate gate;           // the weights are complete behind it (no word: behind the previous kernel)
+    int gate_clear;      // the last CTA of all clears it
     int expand;          // the last head to finish expands all heads' candidates into the tree tokens
     int tile_rows;       // (tensor cores) vocabulary rows per tile
     int rows_per_stage, n_stages, n_it;
@@ -198,12 +200,14 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
         }
     }
     // ---- last head of this batch tile expands the candidates into the tree tokens
-    if (!p.expand) return;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_flag = atomicAdd(&counters[p.K], 1) == p.K - 1;
+    if (threadIdx.x == 0) {
+        s_flag = atomicAdd(&counters[p.K], 1) == p.K - 1;
+        if (s_flag && p.gate_clear) *p.gate.word = 0;
+    }
     __syncthreads();
-    if (!s_flag) return;
+    if (!s_flag || !p.expand) return;
     __threadfence();
     for (int e = threadIdx.x; e < NB * p.T; e += (int)blockDim.x) {
         const int b = b0 + e / p.T, i = e % p.T;

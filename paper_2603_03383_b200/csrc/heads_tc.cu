@@ -67,6 +67,7 @@ struct ResblockTcParams {
     __nv_bfloat16 *xsplit;
     int32_t *counters;
     int n_counters;
+    Gate gate;
     int32_t *dev_error;
 };
 
@@ -91,7 +92,8 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
     volatile int *abort_flag = &abort_flag_s;
     constexpr uint32_t TMEM_COLS = 2 * HT_NACC * HT_NB;   // 128
 
-    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at once
+    previous_done();      // in this order: whoever follows may read what was ready before this call (W2) at the gate
+    if (blockIdx.x == 0 && threadIdx.x == 0) open_gate(p.gate);
     let_next_start();
     // tickets of the vocabulary kernel (the next launch on the stream) start at zero
     if (blockIdx.x == 0)
@@ -293,11 +295,14 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         // ---------------------------------------------------------------- TMA producer
         // The weights do not depend on the residual block: their part of the first stages is requested while that kernel ends.
         const int n_early = min(HT_STAGES, n_tiles * n_kc);
-        if (lane == 0)
+        if (lane == 0 && n_early > 0) {
+            wait_gate(p.gate);
+            ptx::fence_proxy_async_global();
             for (int t = 0; t < n_early; ++t) {
                 ptx::mbar_arrive_expect_tx(full(t), (uint32_t)R * 128u + HT_X_BYTES);
                 ht_tma_2d(ring + t * HT_STAGE_BYTES, &w_map, full(t), t % n_kc * 64, k * p.V + v_begin + t / n_kc * R);
             }
+        }
         __syncwarp();
         previous_done();
         int it = 0;
@@ -416,7 +421,7 @@ size_t heads_tc_xsplit_bytes(int K, int H) { return (size_t)K * HT_N * H * sizeo
 // Residual block, then projection, top-k, merges and tree expansion: the whole medusa_heads_topk for 2..16 rows.
 int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, int V, const __nv_bfloat16 *hidden, const __nv_bfloat16 *W1,
                     const __nv_bfloat16 *b1, const __nv_bfloat16 *W2, const int32_t *root_tok, int32_t *cand,
-                    float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, cudaStream_t st) {
+                    float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, const Gate &gate, cudaStream_t st) {
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
@@ -441,6 +446,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
         r.counters = reinterpret_cast<int32_t *>(ws + L.counters_off); r.n_counters = L.n_counters;
         r.dev_error = t->d_error;
         r.R = w1_R;
+        r.gate = gate;
         const int ctas = std::min(sms, (w1_rows + w1_R - 1) / w1_R);
         TapScope tap(MTV_KERNEL_HEADS_RESBLOCK, st);
         MTV_CUDA_CHECK(launch_dependent(heads_resblock_tc_kernel, dim3(ctas), HT_THREADS, RT_SMEM_BYTES, st, w1_map, h_map, r));
@@ -448,7 +454,8 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = range.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = nullptr;
-    p.kd_arr = t->d_kd + range.k0; p.off_arr = t->d_cand_offset + range.k0; p.expand = range.expand; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
+    p.kd_arr = t->d_kd + range.k0; p.off_arr = t->d_cand_offset + range.k0; p.expand = range.expand;
+    p.gate = gate; p.gate_clear = !range.gate_stays; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
     p.part_idx = reinterpret_cast<int32_t *>(ws + L.part_idx_off);
     p.counters = reinterpret_cast<int32_t *>(ws + L.counters_off);

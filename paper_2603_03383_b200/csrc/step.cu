@@ -47,7 +47,7 @@ StepWs step_ws(const mtv_tree_t *tree, const mtv_step_args *a) {
 
 // Acceptance of a step: from stored logits, or from the fused LM head when the caller gave its operands
 // (the per-node keys then sit at the start of the workspace, which no other kernel uses at that point).
-static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, const StepWs &w, bool alongside, void *stream) {
+static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, const StepWs &w, void *stream) {
     if (a->x_final && a->W_lm) {
         if (!a->ws || a->ws_bytes < (size_t)a->B * tree->T * sizeof(unsigned long long)) return MTV_ERR_WORKSPACE;
         unsigned long long *keys = static_cast<unsigned long long *>(a->ws);
@@ -56,8 +56,8 @@ static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, const Ste
         return tree_accept_keys(tree, a->B, keys, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
                                 a->next_root, stream);
     }
-    return mtv::accept_logits(tree, a->B, a->V, a->logits, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
-                              a->next_root, w.accept, w.accept_bytes, stream, alongside);
+    return tree_accept(tree, a->B, a->V, a->logits, a->tree_tok, a->accept_len, a->best_path, a->acc_nodes, a->acc_tok,
+                       a->next_root, w.accept, w.accept_bytes, stream);
 }
 
 // One step; root_tok and the optional append are given separately so that a chain of steps can feed a step's root
@@ -65,9 +65,9 @@ static int step_accept(const mtv_tree_t *tree, const mtv_step_args *a, const Ste
 static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int32_t *root_tok,
                        const mtv_append_args *ap, void *stream) {
     if (!tree || !a || !a->k_caches_host || !a->v_caches_host || !root_tok) return MTV_ERR_INVALID_ARG;
-    // The attention needs nothing of the heads, and the scan of stored logits nothing of either: the heads' first kernel
-    // makes everything in front of it complete (see launch_dependent), so each starts where SMs fall free at the end
-    // of the one before.  The append, which the attention does need, goes in front of the heads.
+    // The attention needs nothing of the heads, and the scan of stored logits nothing of either: what was enqueued in front of
+    // the heads is complete at the heads' gate (see launch_dependent), so each starts where SMs fall free at the end of the one
+    // before.  The append, which the attention does need, goes in front of the heads.
     const StepWs w = step_ws(tree, a);
     int rc = MTV_OK;
     if (ap && (ap->k_new_layers || ap->v_new_layers)) {
@@ -77,12 +77,13 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
                                         a->stride_h, a->stride_t, a->Lcap, a->seq_lens, ap->rope_theta, a->status, stream);
         if (rc != MTV_OK) return rc;
     }
-    rc = medusa_heads_topk(tree, a->B, a->H, a->V, a->hidden, a->W1, a->b1, a->W2, root_tok, a->cand, a->cand_logit, a->tree_tok,
-                           a->ws, a->ws_bytes, stream);
+    mtv::Gate gate;
+    rc = mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true, w.apart ? &gate : nullptr}, a->B, a->H, a->V, a->hidden, a->W1, a->b1,
+                               a->W2, root_tok, a->cand, a->cand_logit, a->tree_tok, a->ws, a->ws_bytes, stream);
     if (rc != MTV_OK) return rc;
     rc = mtv::tree_attention_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, a->q_layers, a->k_caches_host, a->v_caches_host,
                                     a->stride_b, a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->scale, a->out_layers,
-                                    a->status, w.attn, w.attn_bytes, stream, w.apart);
+                                    a->status, w.attn, w.attn_bytes, stream, w.apart ? &gate : nullptr);
     if (rc != MTV_OK) return rc;
     if (w.apart) {       // acceptance and compaction in one launch behind the scan of the logits or the LM head
         unsigned long long *keys = reinterpret_cast<unsigned long long *>(w.accept);
@@ -91,13 +92,13 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
             rc = lm_head_argmax(tree, a->B, a->H, a->V, a->x_final, a->W_lm, nullptr, nullptr, keys, stream);
         } else {
             ns = mtv::accept_ws_layout(tree, a->B, a->V).nsplit;
-            rc = mtv::argmax_keys_partial(tree, a->B, a->V, a->logits, keys, true, (cudaStream_t)stream);
+            rc = mtv::argmax_keys_partial(tree, a->B, a->V, a->logits, keys, gate, (cudaStream_t)stream);
         }
         if (rc != MTV_OK) return rc;
         return mtv::accept_compact(tree, a, ns, keys, reinterpret_cast<int32_t *>((char *)a->ws + mtv::heads_ws_layout(tree->K, a->B, a->H, a->V).tickets_off),
-                                   (cudaStream_t)stream);
+                                   gate, (cudaStream_t)stream);
     }
-    rc = step_accept(tree, a, w, false, stream);
+    rc = step_accept(tree, a, w, stream);
     if (rc != MTV_OK) return rc;
     return kv_compact_accepted(tree, a->B, a->Hkv, a->D, a->n_layers, a->k_caches, a->v_caches, a->stride_b,
                                a->stride_h, a->stride_t, a->Lcap, a->seq_lens, a->accept_len, a->acc_nodes, a->status,
@@ -229,7 +230,7 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
         return MTV_OK;
     };
     auto heads = [&](int k0, int n, bool expand) {
-        return mtv::heads_topk_range(tree, mtv::HeadsRange{k0, n, expand}, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok,
+        return mtv::heads_topk_range(tree, mtv::HeadsRange{k0, n, expand, nullptr}, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok,
                                      d->cand, d->cand_logit, d->tree_tok, d->ws, d->ws_bytes, stream);
     };
     const int before = tree->K / 2;
@@ -261,7 +262,7 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
     // acceptance and compaction
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.logits_up, 0));
     const StepWs w = step_ws(tree, d);
-    rc = step_accept(tree, d, w, false, stream);
+    rc = step_accept(tree, d, w, stream);
     if (rc != MTV_OK) return rc;
     rc = kv_compact_accepted(tree, d->B, d->Hkv, d->D, d->n_layers, d->k_caches, d->v_caches, d->stride_b, d->stride_h,
                              d->stride_t, d->Lcap, d->seq_lens, d->accept_len, d->acc_nodes, d->status, stream);
