@@ -177,12 +177,14 @@ int tree_kv_append_rope_layers(const mtv_tree_t *tree, int B, int Hq, int Hkv, i
  * multiples of 8; base 16-byte aligned); the caller has already written the tree
  * nodes' K/V to rows seq_lens[b] + i.  seq_lens [B] device int32 (0 is legal).
  * scale == 0 means 1/sqrt(D).  status[b] = MTV_ERR_CAPACITY if seq_lens[b] + T > Lcap.
- * Precondition: the thread blocks that share an item (a sequence's KV head) meet inside the launch through
- * counters of the tree, so all blocks of the launch must be resident at once.  The grid is sized to fit an
- * idle device (one block per SM); do not run the call while another long-running kernel occupies
- * SMs of the same device (other streams, other processes under MPS).  If the blocks cannot
- * meet, the bounded waits run out after about a second, the tree's device error word reads
- * MTV_ERR_TIMEOUT and the output is undefined — the call never hangs.  Calls that share a
+ * Precondition of a one-layer call at head size 128 whose keys are split over several thread-block pairs (few, long
+ * sequences: B * Hkv * ceil(T*Hq/Hkv / 256) at most half the pairs the device holds): the splits of a query block
+ * meet inside the launch through counters of the tree, so all blocks of the launch must be resident at once.  The
+ * grid is sized to fit an idle device (one block per SM); do not run such a call while another long-running kernel
+ * occupies SMs of the same device (other streams, other processes under MPS).  If the blocks cannot meet, the bounded
+ * waits run out after about a second, the tree's device error word reads MTV_ERR_TIMEOUT and the output is
+ * undefined — the call never hangs.  All other calls, the step calls among them, need no such thing: their blocks wait
+ * for each other a millisecond at most and then leave the work to the last one.  Calls that share a
  * tree or a workspace must not overlap on the device.  The encoded tensor maps of (pointer,
  * shape, strides) are kept in a process-wide table; a mutex guards it, so calls from several
  * host threads are safe.

@@ -13,7 +13,8 @@
 //   * Fewer: no CTA gets two pieces; the piece length is the smallest for which the pieces of all items fit the teams.
 // Pieces that are not whole items leave O / l (fp32: where an item is cut must not show in its precision) and (m, l) in the
 // workspace; at the end of the launch the CTAs that share an item meet at a counter and each combines a slice of its rows.
-// That needs all CTAs resident together: the grid never exceeds one CTA per SM; the wait is bounded all the same.
+// They all do so when the device is this launch's alone (the grid never exceeds one CTA per SM), but nothing depends on it:
+// a warp that has waited for a millisecond leaves its slice to the last one to leave and makes room.
 //
 // One piece.  Two STREAMS of 128 query rows by 128 keys share the tensor core: with two row tiles stream t owns tile t and
 // both see every key group; with one row tile both use it and take alternate groups (merged at the end).  A stream runs
@@ -65,6 +66,13 @@ constexpr int AT_SOFTMAX_WARPS = 16;
 constexpr int AT_MMA_WARP = 16, AT_TMA_WARP = 17, AT_Q_WARP = 19;   // warp 18: MMAs of stream 1
 constexpr int AT_PIECES = 4;          // piece descriptors in flight
 constexpr int AT_ITEM_COST = 1;       // what an item costs beside its key groups, in groups
+// How long a warp waits for the others of an item, in cycles.  In the bounds-checking build it looks once: nearly all slices
+// are then left to the last warp.
+#ifdef MTV_DEBUG_BOUNDS
+constexpr long long AT_MERGE_WAIT = 0;
+#else
+constexpr long long AT_MERGE_WAIT = 2000000;
+#endif
 constexpr int AT_MAX_CTAS = 256;      // merge counters in the tree object: one pair per CTA
 constexpr int AT_MAX_LAYERS = 64;     // layers per launch (two tensor maps each in the kernel's parameters)
 // registers per thread: 96 at launch, moved from the four auxiliary warps to the sixteen softmax warps
@@ -137,7 +145,8 @@ struct AttnParams {
     __nv_bfloat16 *out;      // [layers][B][T][Hq][D]
     uint4 *ws_o;             // [CTA][2 slabs][2 tiles][D / 4 chunks][128 rows] 16-byte chunks of O / l, fp32
     float2 *ws_ml;           // [CTA][2 slabs][2 tiles][128 rows] (m, l)
-    int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls
+    int32_t *left;           // [CTA][2 slabs][16 warps] 1: the warp's slice of the item is left to the last one
+    int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls; depart counts slices left in its upper half
     int32_t *status;         // [B] or null
     int32_t *dev_error;
     float scale_log2;
@@ -231,14 +240,103 @@ __device__ __forceinline__ void tile_at(bool one, int pos, int cnt, bool &is_v, 
     is_v = true; idx = (pos - 2) >> 1;
 }
 
-// NEG: the scale is negative (only taken at head size 64, and kept apart so that the usual case pays nothing for it)
 __device__ __forceinline__ int ring_slots(const AttnPiece &d, bool one) {
     return 2 * d.cnt + (d.flags & PIECE_PARTIAL ? 0 : one ? 1 : 2);
 }
 
+// Output row of row r of tile t of a row block (in units of D elements from the item's first row), or -1 if it belongs to nobody.
+// With a group size that does not divide 128 the last 128 - R rows of a tile do (whatever the tile's shared memory held is
+// computed and never written out).
+__device__ __forceinline__ int node_in_tile(const AttnParams &p, int r) { return (int)(((unsigned)r * p.inv_g) >> 16); }
+__device__ __forceinline__ int out_row(const AttnParams &p, int blk, int t, int r) {
+    const int n = node_in_tile(p, r), node = (blk * 2 + t) * p.npc + n;
+    return r < p.R && node < p.T ? node * p.Hq + (r - n * p.G) : -1;
+}
+template <int D>
+__device__ __forceinline__ uint4 *item_out(const AttnParams &p, int layer, int b, int hd) {      // first row of an item's output
+    return reinterpret_cast<uint4 *>(p.out + (((size_t)layer * p.B + b) * p.T * p.Hq + hd * p.G) * D);
+}
+// slabs of the workspace: 16-byte chunk c (4 columns) of row r of tile t; the row's (m, l)
+template <int D>
+__device__ __forceinline__ uint4 *slab_o(const AttnParams &p, int cta, int slab, int t, int r, int c) {
+    return p.ws_o + ((((unsigned)cta * 2 + slab) * 2 + t) * (D / 4) + c) * 128 + r;
+}
+__device__ __forceinline__ float2 *slab_ml(const AttnParams &p, int cta, int slab, int t, int r) {
+    return p.ws_ml + (((unsigned)cta * 2 + slab) * 2 + t) * 128 + r;
+}
+
+// Rows of an item that is shared between CTAs: tile 0's, then tile 1's; contributor c0 combines its share of them, a thread per
+// 16-byte chunk of the output, with the loads of several contributors in flight.  This is warp w's part of it.
+template <int D>
+__device__ __forceinline__ void merge_slice(const AttnParams &p, const AttnMerge &m, int c0, int w, int blk, bool one, int lane) {
+    constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
+    const int rows = one ? p.R : 2 * p.R;
+    const int per = (rows + m.n - 1) / m.n, r_begin = c0 * per;
+    const int n_my = max(0, min(rows, r_begin + per) - r_begin);
+    const unsigned inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;    // e / n_my for e < 4096, n_my <= 256
+    uint4 *dst = item_out<D>(p, m.layer, m.b, m.head);
+#pragma unroll 1
+    for (int e = w * 32 + lane; e < n_my * (D / 8); e += AT_SOFTMAX_WARPS * 32) {
+        const int c = (int)(((unsigned)e * inv_n) >> 20), rr = r_begin + e - c * n_my;
+        const int t = rr >= p.R, r = rr - t * p.R;
+        float acc[8], mm = -INFINITY, wsum = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+#pragma unroll 1
+        for (int s0 = 0; s0 < m.n; s0 += NS) {
+            float2 ml[NS];
+            uint4 v[NS][VC];
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const int s = min(s0 + k, m.n - 1), cta = (m.first + s) * p.n_blk + blk;
+                const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
+                ml[k] = __ldcg(slab_ml(p, cta, sl, t, r));
+#pragma unroll
+                for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, t, r, c * VC + q));
+                if (s0 + k >= m.n) ml[k] = make_float2(-INFINITY, 0.f);
+            }
+            float mc = mm;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
+            const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
+            mm = mc;
+            wsum *= resc;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k] *= resc;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
+                wsum += wt;
+#pragma unroll
+                for (int q = 0; q < VC; ++q) {
+                    const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
+                }
+            }
+        }
+        const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
+        const int o = out_row(p, blk, t, r);
+        if (o >= 0)
+            dst[o * (D / 8) + c] =
+                make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
+                           pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
+    }
+}
+// The slices that warps left, of one item, by the softmax warps of the CTA whose warp was the last to leave it.  (Out of the way of the
+// usual case: as part of the merge below it cost the softmax loop, of all things, 4 %.)
+template <int D>
+static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, bool one, int warp, int lane) {
+    for (int u = warp; u < m.n * AT_SOFTMAX_WARPS; u += AT_SOFTMAX_WARPS) {
+        const int c = u / AT_SOFTMAX_WARPS, w = u % AT_SOFTMAX_WARPS, cta = (m.first + c) * p.n_blk + blk;
+        if (__ldcg(p.left + ((unsigned)cta * 2 + (c == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + w)) merge_slice<D>(p, m, c, w, blk, one, lane);
+    }
+}
+
+// NEG: the scale is negative (only taken at head size 64, and kept apart so that the usual case pays nothing for it)
 template <int D, int ML, bool NEG>
 __global__ void __launch_bounds__(AT_THREADS, 1)
-tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) {
+tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constant__ AttnParams p) {
     using SM = AttnSmem<D>;
     constexpr int ST = SM::STAGES;
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -252,6 +350,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + SM::OFF_MISC + 64);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 68);
     volatile int *n_merge = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 72);     // partial pieces of this CTA
+    int *left_items = reinterpret_cast<int *>(smem + SM::OFF_MISC + 108);                   // of this CTA's: bit i, merges[i]
     volatile int *beyond = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 76);      // [2 streams][4] a sum beyond AT_SUM_LIMIT
 
     const int team = (int)blockIdx.x / p.n_blk, blk = (int)blockIdx.x % p.n_blk;
@@ -289,6 +388,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         ptx::fence_mbar_init();
         *abort_flag = 0;
         *n_merge = 0;
+        *left_items = 0;
     }
     if (warp == AT_MMA_WARP) {
         ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), 512);
@@ -681,18 +781,9 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         const int row = qd * 32 + lane;
         const int tile = one ? 0 : st;
         const int step = one ? 2 : 1, first = one ? st : 0;
-        // With a group size that does not divide 128 the last 128 - R rows of a tile belong to nobody (whatever the
-        // tile's shared memory held is computed and never written out).
-        const int node_of_blk = blk * 2 * p.npc;
-        auto node_in_tile = [&](int r) { return (int)(((unsigned)r * p.inv_g) >> 16); };
-        // output row of row r of tile t (in units of D elements from the item's first row), or -1
-        auto out_row = [&](int t, int r) {
-            const int n = node_in_tile(r), node = node_of_blk + t * p.npc + n;
-            return r < p.R && node < p.T ? node * p.Hq + (r - n * p.G) : -1;
-        };
         // 128 bits: the row's node sees tree row i
-        const uint32_t *anc = reinterpret_cast<const uint32_t *>(p.anc + (node_of_blk + tile * p.npc + node_in_tile(row)) * 2);
-        const bool mine = out_row(tile, row) >= 0;
+        const uint32_t *anc = reinterpret_cast<const uint32_t *>(p.anc + ((blk * 2 + tile) * p.npc + node_in_tile(p, row)) * 2);
+        const bool mine = out_row(p, blk, tile, row) >= 0;
         auto anc_word = [&](int w) -> uint32_t {
             if (w < 0) return 0xffffffffu;     // prefix rows are visible to every node
             return w < 4 && mine ? anc[w] : 0u;    // past the tree rows: nothing
@@ -700,36 +791,30 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         const uint32_t tmem = begin();
         const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16);
         const uint32_t t_s = lane_base + TM_S + st * 128 + hf * 64, t_o = lane_base + TM_O + st * 128;
-        const uint32_t bar_s = bar(SM::BAR_S + st), bar_p = bar(SM::BAR_P + st), bar_xm = bar(SM::BAR_XM + st * 4 + qd),
-                       bar_xo = bar(SM::BAR_XO + (one ? qd : st * 4 + qd));
-        volatile float *xch = reinterpret_cast<volatile float *>(smem + SM::OFF_ML);      // [stream][half][row]
-        volatile float *x_mine = xch + (st * 2 + hf) * 128 + row, *x_other = xch + (st * 2 + (hf ^ 1)) * 128 + row;
-        auto item_out = [&](int layer, int b, int hd) {      // first row of an item's output
-            return reinterpret_cast<uint4 *>(p.out + (((size_t)layer * p.B + b) * p.T * p.Hq + hd * p.G) * D);
-        };
-        // slabs of the workspace: 16-byte chunk c (4 columns) of row r of tile t; the row's (m, l)
-        auto slab_o = [&](int cta, int slab, int t, int r, int c) {
-            return p.ws_o + ((((unsigned)cta * 2 + slab) * 2 + t) * (D / 4) + c) * 128 + r;
-        };
-        auto slab_ml = [&](int cta, int slab, int t, int r) { return p.ws_ml + (((unsigned)cta * 2 + slab) * 2 + t) * 128 + r; };
+        // (addresses in 32 bits and formed where they are used, phases in one word: the loop below has no register to spare)
+        auto bar_s = [&]() { return bar(SM::BAR_S + st); };
+        auto x_at = [&](int s, int h) { return sbase + SM::OFF_ML + (uint32_t)((s * 2 + h) * 128 + row) * 4u; };   // [stream][half][row]
+        const uint32_t beyond_at = sbase + SM::OFF_MISC + 76u + (uint32_t)(st * 4 + qd) * 4u;
+        if (lane < 2) p.left[((unsigned)blockIdx.x * 2 + lane) * AT_SOFTMAX_WARPS + warp] = 0;      // (released with the arrivals)
         constexpr uint32_t hidden = NEG ? 0x7f800000u : 0xff800000u;   // times the scale: -inf
-        uint32_t s_ph = 0, o_ph = 0, xm_ph = 0, xo_ph = 0, seq = 0;
+        uint32_t phases = 0, seq = 0;             // bit 0: scores, 1: O, 2 and 3: the two exchanges
+        auto phase = [&](int i) { return (phases >> i) & 1u; };
         bool ok = true;
         TRACE_INIT(1 + st, qd == 0 && hf == 0 && lane == 0);
         float m_used = -INFINITY, l = 0.f;
         bool begun = false;                    // the stream's O holds something of this piece
         auto meet = [&]() {                    // the two warps of these rows
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar_xm);
-            if (!ptx::mbar_wait(bar_xm, xm_ph)) ok = false;
-            xm_ph ^= 1;
+            if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XM + st * 4 + qd));
+            if (!ptx::mbar_wait(bar(SM::BAR_XM + st * 4 + qd), phase(2))) ok = false;
+            phases ^= 4;
         };
         // The reference becomes max(both halves' mx) where `is_first` or that exceeds it; O and l (and P, if already written
         // against the old one) follow.  The two warps of the rows do this together.
         auto move_reference = [&](float mx, bool is_first, bool p_written) {
-            *x_mine = mx;
+            ptx::sts_f32(x_at(st, hf), mx);
             meet();
-            const float both = ceilf(fmaxf(mx, *x_other));
+            const float both = ceilf(fmaxf(mx, ptx::lds_f32(x_at(st, hf ^ 1))));
             const float m_new = is_first ? both : fmaxf(m_used, both);
             const bool need = !is_first && m_new != m_used && m_used != -INFINITY;
             if (__any_sync(0xffffffffu, need)) {
@@ -756,7 +841,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             }
             m_used = m_new;
             if (is_first) return;                  // (the values exchanged are not written again before both warps' P is used)
-            if (lane == 0) beyond[st * 4 + qd] = 0;
+            if (lane == 0) ptx::sts_u32(beyond_at, 0u);
             ptx::tc_fence_before();
             meet();
             ptx::tc_fence_after();
@@ -769,7 +854,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
         auto wait_tc = [&](uint32_t b, uint32_t parity) {
             const long long t0 = clock64();
             while (!ptx::mbar_try_wait(b, parity)) {
-                if (beyond[st * 4 + qd]) {
+                if (ptx::lds_u32(beyond_at)) {
                     if (!ptx::mbar_try_wait(b, parity)) move_reference(-INFINITY, false, true);
                     continue;
                 }
@@ -790,7 +875,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             // These scores are complete: this stream is done with their K tile and, the MMAs before them being complete too, with
             // the V tile of its previous group.
             auto scores_done = [&](int j) {
-                s_ph ^= 1;
+                phases ^= 1;
                 TRACE();
                 ptx::tc_fence_after();
                 if (releases) {
@@ -803,7 +888,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_p);
+                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_P + st));
                 begun = true;
                 TRACE();
             };
@@ -812,7 +897,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             // ---- the first group: its maximum, then its P in two terms, a quarter at a time (the scores are loaded twice, which
             //      costs less than the registers of all of them in two terms)
             if (first < cnt) {
-                if (!ptx::mbar_wait(bar_s, s_ph)) { ok = false; break; }
+                if (!ptx::mbar_wait(bar_s(), phase(0))) { ok = false; break; }
                 scores_done(first);
                 const int a0 = a_first + first * AT_BN;      // tree row of this half's first column
                 auto quarter = [&](uint32_t (&q)[32], int c) {
@@ -853,7 +938,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
 #pragma unroll 1
                 for (;;) {
                     if (!asked) {
-                        wait_tc(bar_s, s_ph);
+                        wait_tc(bar_s(), phase(0));
                         if (!ok) break;
                         scores_done(j);
                     }
@@ -910,7 +995,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                     }
                     // rare: ask the other warp of these rows to come and move the reference, start over
                     asked = true;
-                    if (lane == 0) beyond[st * 4 + qd] = 1;
+                    if (lane == 0) ptx::sts_u32(beyond_at, 1u);
                 }
                 if (!ok) break;
                 l += sum;
@@ -919,8 +1004,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             // ---- the stream's O of this piece
             const bool ran = first < cnt;       // (a one-tile piece of a single group has no second stream)
             if (ok && ran) {
-                wait_tc(bar(SM::BAR_O + st), o_ph);
-                o_ph ^= 1;
+                wait_tc(bar(SM::BAR_O + st), phase(1));
+                phases ^= 2;
                 if (releases) {
                     const int jl = one ? cnt - 1 - ((cnt - 1 - st) & 1) : cnt - 1;    // the stream's last group
                     ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)v_pos(one, jl, cnt)) % ST));
@@ -935,18 +1020,19 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             auto gather = [&]() {
                 ptx::tc_fence_before();
                 __syncwarp();
+                const uint32_t bar_xo = bar(SM::BAR_XO + (one ? qd : st * 4 + qd));
                 if (lane == 0) ptx::mbar_arrive(bar_xo);
-                if (!ptx::mbar_wait(bar_xo, xo_ph)) ok = false;
-                xo_ph ^= 1;
+                if (!ptx::mbar_wait(bar_xo, phase(3))) ok = false;
+                phases ^= 8;
                 ptx::tc_fence_after();
             };
             volatile float *x_m = reinterpret_cast<volatile float *>(smem + SM::TILE);   // [stream][row]: the unused query tile
-            *x_mine = l;
+            ptx::sts_f32(x_at(st, hf), l);
             if (one && hf == 0) x_m[st * 128 + row] = m_used;
             gather();
-            float l_all = l + *x_other, m_all = m_used, w_own = 1.f, w_oth = 0.f;
+            float l_all = l + ptx::lds_f32(x_at(st, hf ^ 1)), m_all = m_used, w_own = 1.f, w_oth = 0.f;
             if (one) {
-                const float l_oth = xch[((st ^ 1) * 2) * 128 + row] + xch[((st ^ 1) * 2 + 1) * 128 + row];
+                const float l_oth = ptx::lds_f32(x_at(st ^ 1, 0)) + ptx::lds_f32(x_at(st ^ 1, 1));
                 const float m_oth = x_m[(st ^ 1) * 128 + row];
                 m_all = fmaxf(m_used, m_oth);
                 w_own = m_used == -INFINITY ? 0.f : ex2(m_used - m_all);
@@ -994,7 +1080,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                     } else if (mine) {
 #pragma unroll
                         for (int q = 0; q < 2; ++q)
-                            *slab_o(blockIdx.x, slab, tile, row, c_begin / 4 + 2 * ch + q) =
+                            *slab_o<D>(p, blockIdx.x, slab, tile, row, c_begin / 4 + 2 * ch + q) =
                                 make_uint4(__float_as_uint(v[8 * e + 4 * q]), __float_as_uint(v[8 * e + 4 * q + 1]),
                                            __float_as_uint(v[8 * e + 4 * q + 2]), __float_as_uint(v[8 * e + 4 * q + 3]));
                     }
@@ -1003,11 +1089,11 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
             if (!partial) {
                 __syncwarp();
                 const uint32_t sh = n_ch == 8 ? 3 : n_ch == 4 ? 2 : 1, ch = lane & (n_ch - 1);     // n_ch lanes store a row's part
-                uint4 *dst = item_out(d.layer, d.b, d.head) + c_begin / 8 + ch;
+                uint4 *dst = item_out<D>(p, d.layer, d.b, d.head) + c_begin / 8 + ch;
 #pragma unroll 2
                 for (uint32_t r = lane >> sh; r < 32; r += 32u >> sh) {
                     const uint4 x = *reinterpret_cast<const uint4 *>(stage + r * rowb + ((ch ^ (r & (n_ch - 1))) << 4));
-                    const int o = out_row(tile, qd * 32 + r);
+                    const int o = out_row(p, blk, tile, qd * 32 + r);
                     if (o >= 0) dst[o * (D / 8)] = x;
                 }
                 ptx::fence_proxy_async();         // (the next tile comes into the slot through the async proxy)
@@ -1015,7 +1101,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
                 if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_STAGED + slot));
             }
             if (partial) {
-                if (mine && hf == 0 && (!one || st == 0)) *slab_ml(blockIdx.x, slab, tile, row) = make_float2(m_all, l_all);
+                if (mine && hf == 0 && (!one || st == 0)) *slab_ml(p, blockIdx.x, slab, tile, row) = make_float2(m_all, l_all);
                 // this warp's part is written: tell those that share the item (each warp counts for itself)
                 __syncwarp();
                 if (lane == 0) {
@@ -1033,76 +1119,32 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
 #pragma unroll 1
         for (int i = 0; i < n_m; ++i) {
             const AttnMerge m = merges[i];
-            const int ctr = m.first * p.n_blk + blk, all = m.n * AT_SOFTMAX_WARPS;
-            int departed = 0;
+            const int ctr = m.first * p.n_blk + blk, all = m.n * AT_SOFTMAX_WARPS, c0 = team - m.first;
+            int departed = 0, full = 0;
             if (lane == 0) {
                 // relaxed polls (a round trip to L2 each), one acquire when the counter is full
                 int32_t *c = p.arrive + ctr;
                 const long long t0 = clock64();
-                while (*reinterpret_cast<volatile int32_t *>(c) < all)
-                    if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { give_up(); break; }
-                (void)ld_acquire(c);
-                departed = atomicAdd(p.depart + ctr, 1);         // (its round trip overlaps the merge)
-            }
-            __syncwarp();
-            // rows of the item: tile 0's, then tile 1's; this CTA combines its share of them, a thread per 16-byte chunk of the
-            // output, with the loads of several contributors in flight
-            constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
-            const int rows = one ? p.R : 2 * p.R;
-            const int per = (rows + m.n - 1) / m.n, r_begin = (team - m.first) * per;
-            const int n_my = max(0, min(rows, r_begin + per) - r_begin);
-            const unsigned inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;    // e / n_my for e < 4096, n_my <= 256
-            uint4 *dst = item_out(m.layer, m.b, m.head);
-#pragma unroll 1
-            for (int e = threadIdx.x; e < n_my * (D / 8); e += AT_SOFTMAX_WARPS * 32) {
-                const int c = (int)(((unsigned)e * inv_n) >> 20), rr = r_begin + e - c * n_my;
-                const int t = rr >= p.R, r = rr - t * p.R;
-                float acc[8], mm = -INFINITY, wsum = 0.f;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) acc[k] = 0.f;
-#pragma unroll 1
-                for (int s0 = 0; s0 < m.n; s0 += NS) {
-                    float2 ml[NS];
-                    uint4 v[NS][VC];
-#pragma unroll
-                    for (int k = 0; k < NS; ++k) {
-                        const int s = min(s0 + k, m.n - 1), cta = (m.first + s) * p.n_blk + blk;
-                        const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
-                        ml[k] = __ldcg(slab_ml(cta, sl, t, r));
-#pragma unroll
-                        for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o(cta, sl, t, r, c * VC + q));
-                        if (s0 + k >= m.n) ml[k] = make_float2(-INFINITY, 0.f);
-                    }
-                    float mc = mm;
-#pragma unroll
-                    for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
-                    const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
-                    mm = mc;
-                    wsum *= resc;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) acc[k] *= resc;
-#pragma unroll
-                    for (int k = 0; k < NS; ++k) {
-                        const float w = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
-                        wsum += w;
-#pragma unroll
-                        for (int q = 0; q < VC; ++q) {
-                            const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
-#pragma unroll
-                            for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(w, __uint_as_float(vw[i]), acc[4 * q + i]);
-                        }
-                    }
+                while (!(full = *reinterpret_cast<volatile int32_t *>(c) >= all))
+                    if (clock64() - t0 > AT_MERGE_WAIT) break;
+                if (full) {
+                    (void)ld_acquire(c);
+                    departed = atomicAdd(p.depart + ctr, 1);         // (its round trip overlaps the merge)
+                } else {
+                    p.left[((unsigned)blockIdx.x * 2 + (c0 == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + warp] = 1;
+                    __threadfence();
+                    departed = atomicAdd(p.depart + ctr, 0x10001) + 0x10000;
                 }
-                const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
-                const int o = out_row(t, r);
-                if (o >= 0)
-                    dst[o * (D / 8) + c] =
-                        make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
-                                   pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
             }
-            // The last warp to have seen the counter full puts both counters back to zero (nobody polls them any more; the
-            // next call cannot start before this kernel has ended).
-            if (lane == 0 && departed == all - 1) {
+            if (__shfl_sync(0xffffffffu, full, 0)) merge_slice<D>(p, m, c0, warp, blk, one, lane);
+            // The last warp to leave: its CTA does what others left, all parts and all marks being complete, and the counters go
+            // back to zero (nobody polls them any more; the next call cannot start before this kernel has ended).
+            if (lane == 0 && (departed & 0xffff) == all - 1) {
+                if (departed >> 16) {
+                    (void)ld_acquire(p.arrive + ctr);
+                    (void)ld_acquire(p.depart + ctr);
+                    atomicOr(left_items, 1 << i);
+                }
                 p.arrive[ctr] = 0;
                 p.depart[ctr] = 0;
             }
@@ -1112,6 +1154,9 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const AttnParams p) 
     __syncthreads();
     ptx::tc_fence_after();
     if (warp == AT_MMA_WARP) ptx::tmem_dealloc(*tmem_slot, 512);
+    if (warp < AT_SOFTMAX_WARPS && *left_items)       // (the other warps have too few registers for it)
+        for (int i = 0; i < 2; ++i)
+            if ((*left_items >> i) & 1) merge_left<D>(p, merges[i], blk, one, warp, lane);
     if (p.gate.word) previous_done();
 }
 
@@ -1202,12 +1247,13 @@ AttnPlan attn_plan(int T, int G) {
 // pairs keeps a slab per key split of a query block and the order of the sequences.
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap) {
     AttnWs w;
-    w.o_off = w.ml_off = w.total = 0;
+    w.o_off = w.ml_off = w.left_off = w.total = 0;
     if (Hq / Hkv > 8) return w;          // the call itself refuses such a group; sizes are asked for before that
     const AttnPlan a = attn_plan(t->T, Hq / Hkv);
     const size_t slabs = (size_t)a.teams * a.n_blk * 2;
     w.ml_off = align_up(slabs * 2 * 128 * D * sizeof(float), 256);
-    w.total = align_up(w.ml_off + slabs * 2 * 128 * sizeof(float2), 256);
+    w.left_off = align_up(w.ml_off + slabs * 2 * 128 * sizeof(float2), 256);
+    w.total = align_up(w.left_off + slabs * AT_SOFTMAX_WARPS * sizeof(int32_t), 256);
     if (attn_pair_eligible(D, Hq / Hkv)) {
         int n_blk = 1;
         const int ns = attn_pair_plan(t->T, Hq / Hkv, B, Hkv, Lcap, &n_blk);
@@ -1306,6 +1352,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.seq_lens = seq_lens; p.anc = tree->d_anc; p.status = status; p.dev_error = tree->d_error;
     p.ws_o = reinterpret_cast<uint4 *>((char *)ws + Lw.o_off);
     p.ws_ml = reinterpret_cast<float2 *>((char *)ws + Lw.ml_off);
+    p.left = reinterpret_cast<int32_t *>((char *)ws + Lw.left_off);
     p.arrive = tree->d_counters; p.depart = tree->d_counters + AT_MAX_CTAS;
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;

@@ -76,7 +76,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
                     float *cand_logit, int32_t *tree_tok, const HeadsWs &L, char *ws, const Gate &gate, cudaStream_t st);
 
 struct AttnWs {
-    size_t o_off, ml_off, pair_ml_off = 0, order_off = 0, total;
+    size_t o_off, ml_off, left_off, pair_ml_off = 0, order_off = 0, total;
 };
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap);
 // alongside: nothing that the previous kernels in the stream back to the heads write is needed, nor their workspace touched,

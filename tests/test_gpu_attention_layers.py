@@ -80,3 +80,55 @@ def test_single_layer_calls(T, Hq, Hkv, D, lens, Lcap, gain):
     torch.cuda.synchronize()
     assert binding.mtv_device_error(tree) == 0
     assert_close(out, want)
+
+
+@pytest.mark.parametrize("D,n_layers", [(64, 1), (64, 4), (128, 4)])
+def test_two_trees_on_two_streams(D, n_layers):
+    """Launches that share the device: neither needs all its blocks resident at once."""
+    T, Hq, Hkv, L = 64, 8, 2, 1500
+    K, H, V, B = 4, 64, 600, 2
+    sides = []
+    for i in range(2):
+        tb, tree = make_tree("rank_prior", K, (), T)
+        Lcap = L + T
+        ks, vs = ([synth.normal_bf16(i, s + l, (B, Hkv, Lcap, D), device=DEV) for l in range(n_layers)] for s in (10, 50))
+        q = synth.normal_bf16(i, 90, (n_layers, B, T, Hq, D), device=DEV)
+        lens = torch.tensor([L, 700 + 100 * i], dtype=torch.int32, device=DEV)
+        out = torch.zeros_like(q)
+        ws = workspace(tree, B, H, V, Hq, Hkv, D, Lcap)
+        hidden, W1, b1, W2, root = (t.to(DEV) for t in synth.head_inputs(B, H, V, K, seed=3))
+        i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+        d = dict(hidden=hidden, W1=W1, b1=b1, W2=W2, root_tok=root, q_layers=q, out_layers=out, seq_lens=lens.clone(),
+                 logits=synth.normal_bf16(T, 91, (B, T, V), device=DEV), cand=i32(B, tree.C), tree_tok=i32(B, T), accept_len=i32(B),
+                 best_path=i32(B), acc_nodes=i32(B, K + 1), acc_tok=i32(B, K + 1), next_root=i32(B),
+                 k_caches=binding.cache_pointer_array(ks, DEV), v_caches=binding.cache_pointer_array(vs, DEV),
+                 k_caches_host=binding.cache_pointer_array(ks), v_caches_host=binding.cache_pointer_array(vs), ws=ws)
+        a = binding.StepArgs()
+        a.B, a.H, a.V, a.Hq, a.Hkv, a.D, a.n_layers, a.Lcap = B, H, V, Hq, Hkv, D, n_layers, Lcap
+        a.stride_b, a.stride_h, a.stride_t = ks[0].stride()[:3]
+        for n, t in d.items():
+            setattr(a, n, t.data_ptr())
+        a.ws_bytes = ws.numel()
+        st = torch.cuda.Stream()
+
+        def call(tree=tree, a=a, d=d, lens=lens, q=q, ks=ks, vs=vs, out=out, ws=ws, st=st):
+            with torch.cuda.stream(st):
+                if n_layers == 1:
+                    binding.tree_verify_attention(tree, q[0], ks[0], vs[0], lens, out[0], ws)
+                else:
+                    d["seq_lens"].copy_(lens)
+                    binding.mtv_verify_step(tree, a)
+        torch.cuda.synchronize()
+        call()
+        torch.cuda.synchronize()
+        assert d["accept_len"].sum().item() == 0           # nothing accepted: the step moves no cache rows, calls repeat
+        sides.append((tree, call, out, out.clone()))
+        out.zero_()
+    torch.cuda.synchronize()
+    for _ in range(60):
+        for _, call, _, _ in sides:
+            call()
+    torch.cuda.synchronize()
+    for tree, _, out, want in sides:
+        assert binding.mtv_device_error(tree) == 0
+        assert torch.equal(out, want)

@@ -30,6 +30,7 @@ def test_steps_under_the_bounds_checking_build():
              "tests/test_gpu_parity.py::test_full_step_with_fused_lm_head",
              "tests/test_gpu_parity.py::test_verify_steps_chain_in_one_call",
              "tests/test_gpu_parity.py::test_attention_large_ragged_batch",
+             "tests/test_gpu_attention_layers.py",          # in that build most of a merge is left to its last warp
              "tests/test_gpu_debug_bounds.py::test_indices_out_of_range_are_reported_not_followed"]
     r = subprocess.run([sys.executable, "-m", "pytest", "-x", "-q", "-m", "gpu", "-rs"] + cases, cwd=ROOT, env=env,
                        capture_output=True, text=True, timeout=900)
