@@ -6,6 +6,7 @@
 // multiply-adds, so the kernels are organised around 16-byte coalesced weight loads
 // with many loads in flight; activations stay in shared memory in fp32 so that no
 // intermediate is rounded.
+#include <algorithm>
 #include <atomic>
 
 #include "common.cuh"
@@ -78,6 +79,7 @@ HeadsWs heads_ws_layout(int K, int B, int H, int V) {
     w.hprime_off = off;   off = align_up(off + (size_t)K * B * H * sizeof(float), 256);
     w.part_val_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(float), 256);
     w.part_idx_off = off; off = align_up(off + (size_t)K * B * per_head * MTV_MAX_TOPK * sizeof(int32_t), 256);
+    off = std::max(off, align_up((size_t)B * MTV_MAX_T * sizeof(unsigned long long), 256));   // (a step's LM-head keys begin the workspace)
     w.n_counters = (K + 1) * btiles + B;    // and one per sequence for the end of a step
     w.counters_off = off; w.tickets_off = off + (size_t)(K + 1) * btiles * sizeof(int32_t);
     w.gate_off = off + (size_t)w.n_counters * sizeof(int32_t);

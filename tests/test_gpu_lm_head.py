@@ -4,7 +4,7 @@ import torch
 
 from oracle import reference as ref
 from paper_2603_03383_b200 import binding, synth
-from tests._cases import make_tree
+from tests._cases import make_tree, workspace
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -130,3 +130,33 @@ def test_lm_head_full_size_7b(V):
         _check(x, W, am, val)
     keys2, am2, val2 = _run(tree, x, W)
     assert torch.equal(keys, keys2)                          # bitwise repeatable
+
+
+def test_keys_of_a_step_begin_the_workspace():
+    """A step fed by the fused LM head leaves the per-node keys at the start of its workspace, as the call alone gives them."""
+    B, T, K, H, V, Hq, Hkv, D, L, n_layers = 2, 64, 4, 64, 1000, 4, 1, 64, 100, 2
+    tb, tree = make_tree("rank_prior", K, (), T)
+    Lcap = L + T
+    hidden, W1, b1, W2, root = (t.to(DEV) for t in synth.head_inputs(B, H, V, K, seed=5))
+    i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+    ks, vs = ([synth.normal_bf16(1, s + l, (B, Hkv, Lcap, D), device=DEV) for l in range(n_layers)] for s in (10, 50))
+    x, W = synth.normal_bf16(1, 7, (B, T, H), device=DEV), synth.normal_bf16(1, 8, (V, H), device=DEV)
+    want = torch.zeros(B * T, dtype=torch.int64, device=DEV)
+    binding.lm_head_argmax(tree, x, W, want)
+    q = synth.normal_bf16(1, 90, (n_layers, B, T, Hq, D), device=DEV)
+    d = dict(hidden=hidden, W1=W1, b1=b1, W2=W2, root_tok=root, q_layers=q, out_layers=torch.zeros_like(q), x_final=x, W_lm=W,
+             seq_lens=torch.full((B,), L, dtype=torch.int32, device=DEV), cand=i32(B, tree.C), tree_tok=i32(B, T), accept_len=i32(B),
+             best_path=i32(B), acc_nodes=i32(B, K + 1), acc_tok=i32(B, K + 1), next_root=i32(B),
+             k_caches=binding.cache_pointer_array(ks, DEV), v_caches=binding.cache_pointer_array(vs, DEV),
+             k_caches_host=binding.cache_pointer_array(ks), v_caches_host=binding.cache_pointer_array(vs),
+             ws=workspace(tree, B, H, V, Hq, Hkv, D, Lcap))
+    a = binding.StepArgs()
+    a.B, a.H, a.V, a.Hq, a.Hkv, a.D, a.n_layers, a.Lcap = B, H, V, Hq, Hkv, D, n_layers, Lcap
+    a.stride_b, a.stride_h, a.stride_t = ks[0].stride()[:3]
+    for n, t in d.items():
+        setattr(a, n, t.data_ptr())
+    a.ws_bytes = d["ws"].numel()
+    binding.mtv_verify_step(tree, a)
+    torch.cuda.synchronize()
+    assert binding.mtv_device_error(tree) == 0
+    assert torch.equal(d["ws"][:B * T * 8].view(torch.int64), want)
