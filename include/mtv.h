@@ -330,8 +330,7 @@ int mtv_verify_step(const mtv_tree_t *tree, const mtv_step_args *args, void *str
  *   - all steps share one seq_lens array, advanced on the device by every step's compaction.
  * appends (NULL, or n_steps entries): where appends[s].k_new_layers / v_new_layers are given,
  * step s first writes its tree nodes' K/V rows into the caches — all layers in one launch of
- * tree_kv_append_rope's kernel, directly in front of the step's first attention call, which
- * starts its set-up under that kernel's tail (programmatic dependent launch) — and rotates
+ * tree_kv_append_rope's kernel, in front of the step's heads (whose arguments are checked before it) — and rotates
  * steps[s].q_layers in place (so that buffer must be writable although the struct says const).
  * k_new_layers, v_new_layers: [n_layers][B][T][Hkv][D] device, un-rotated K rows and V rows;
  * rope_theta == 0 means 10000.  Per-step inputs that a backbone would compute from the previous

@@ -66,6 +66,9 @@ struct HeadsRange {
     bool expand;
     Gate *gate_stays = nullptr;
 };
+// MTV_OK, or what such a call is refused with
+int heads_check(const mtv_tree *tree, int n_heads, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1, const mtv_bf16 *W2,
+                const int32_t *root_tok, const int32_t *cand, const int32_t *tree_tok, const void *ws, size_t ws_bytes);
 int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
                      const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
                      int32_t *tree_tok, void *ws, size_t ws_bytes, void *stream);

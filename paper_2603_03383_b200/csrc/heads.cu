@@ -455,8 +455,6 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     const int btiles = (B + NB - 1) / NB;
     const size_t sm1 = (size_t)NB * H * sizeof(float);
     const VocabSmem S = vocab_smem_plan(NB, MR, H, L.ctas_per_head);
-    if (sm1 > VT_SMEM_MAX || S.total == 0) return MTV_ERR_UNSUPPORTED_SHAPE;
-    if (NB > 1 && S.rows_per_stage < (NB >= 4 ? 4 : 2)) return MTV_ERR_UNSUPPORTED_SHAPE;   // rows too long for a block of rows per stage
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
@@ -493,9 +491,14 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     return MTV_OK;
 }
 
-int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
-                     const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
-                     int32_t *tree_tok, void *ws, size_t ws_bytes, void *stream) {
+// one batch row: stages of 32 KB or more, but at least four to a CTA's slab
+static int rows_per_warp(int H, int V, const HeadsWs &L) {
+    const int slab = (V + L.ctas_per_head - 1) / L.ctas_per_head;
+    return H < 1024 && slab >= 128 ? 4 : H < 2048 && slab >= 64 ? 2 : 1;
+}
+
+int heads_check(const mtv_tree *tree, int n_heads, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1, const mtv_bf16 *W2,
+                const int32_t *root_tok, const int32_t *cand, const int32_t *tree_tok, const void *ws, size_t ws_bytes) {
     if (!tree || !tree->on_device || !hidden || !W1 || !W2 || !root_tok || !cand || !tree_tok || !ws)
         return MTV_ERR_INVALID_ARG;
     if (B < 1 || H < 8 || V < 1) return MTV_ERR_INVALID_ARG;
@@ -503,16 +506,29 @@ int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, in
     if (((uintptr_t)W2 | (uintptr_t)W1 | (uintptr_t)hidden | (uintptr_t)ws) & 15) return MTV_ERR_INVALID_ARG;
     for (int d = 0; d < tree->K; ++d)
         if (tree->k_d[d] > V) return MTV_ERR_INVALID_ARG;
-    const HeadsWs L = heads_ws_layout(r.n, B, H, V);
+    const HeadsWs L = heads_ws_layout(n_heads, B, H, V);
     if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
+    if (!L.use_tc) {
+        const int NB = nb_for(B);
+        const VocabSmem S = vocab_smem_plan(NB, B == 1 ? rows_per_warp(H, V, L) : 1, H, L.ctas_per_head);
+        if ((size_t)NB * H * sizeof(float) > VT_SMEM_MAX || S.total == 0) return MTV_ERR_UNSUPPORTED_SHAPE;
+        if (NB > 1 && S.rows_per_stage < (NB >= 4 ? 4 : 2)) return MTV_ERR_UNSUPPORTED_SHAPE;   // rows too long for a block of rows per stage
+    }
+    return MTV_OK;
+}
+
+int heads_topk_range(const mtv_tree *tree, const HeadsRange &r, int B, int H, int V, const mtv_bf16 *hidden, const mtv_bf16 *W1,
+                     const mtv_bf16 *b1, const mtv_bf16 *W2, const int32_t *root_tok, int32_t *cand, float *cand_logit,
+                     int32_t *tree_tok, void *ws, size_t ws_bytes, void *stream) {
+    const int refused = heads_check(tree, r.n, B, H, V, hidden, W1, W2, root_tok, cand, tree_tok, ws, ws_bytes);
+    if (refused != MTV_OK) return refused;
+    const HeadsWs L = heads_ws_layout(r.n, B, H, V);
     cudaStream_t st = (cudaStream_t)stream;
     auto *h = reinterpret_cast<const __nv_bfloat16 *>(hidden);
     auto *w1 = reinterpret_cast<const __nv_bfloat16 *>(W1) + (size_t)r.k0 * H * H;
     auto *bb = b1 ? reinterpret_cast<const __nv_bfloat16 *>(b1) + (size_t)r.k0 * H : nullptr;
     auto *w2 = reinterpret_cast<const __nv_bfloat16 *>(W2) + (size_t)r.k0 * V * H;
-    // one batch row: stages of 32 KB or more, but at least four to a CTA's slab
-    const int slab = (V + L.ctas_per_head - 1) / L.ctas_per_head;
-    const int mr = H < 1024 && slab >= 128 ? 4 : H < 2048 && slab >= 64 ? 2 : 1;
+    const int mr = rows_per_warp(H, V, L);
     auto launch = L.use_tc ? launch_heads_tc : B == 1 ? (mr == 4 ? launch_heads<1, 4> : mr == 2 ? launch_heads<1, 2> : launch_heads<1, 1>)
                   : B == 2 ? launch_heads<2, 1> : B <= 4 ? launch_heads<4, 1> : launch_heads<8, 1>;
     static std::atomic<uint32_t> calls{0};

@@ -69,7 +69,9 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
     // the heads is complete at the heads' gate (see launch_dependent), so each starts where SMs fall free at the end of the one
     // before.  The append, which the attention does need, goes in front of the heads.
     const StepWs w = step_ws(tree, a);
-    int rc = MTV_OK;
+    // (in front of the append, which rotates the queries in place: a refused call can be repeated)
+    int rc = mtv::heads_check(tree, tree->K, a->B, a->H, a->V, a->hidden, a->W1, a->W2, root_tok, a->cand, a->tree_tok, a->ws, a->ws_bytes);
+    if (rc != MTV_OK) return rc;
     if (ap && (ap->k_new_layers || ap->v_new_layers)) {
         // the tree nodes' K/V rows of every layer, in one launch
         rc = tree_kv_append_rope_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, const_cast<mtv_bf16 *>(a->q_layers),

@@ -102,3 +102,33 @@ def test_step(D, B, lm_head, graph):
     assert binding.mtv_device_error(tree) == 0
     for i, r in enumerate(got):
         assert all(torch.equal(x, y) for x, y in zip(r, want[i % 3])), i
+
+
+def test_a_refused_chain_changes_nothing():
+    """Heads that are refused (here: a workspace too small for them) leave the queries unrotated and the caches as they were."""
+    K, H, V, Hq, Hkv, T, L, n_layers, B, D = 4, 64, 600, 4, 1, 64, 50, 2, 1, 64
+    tb, tree = make_tree("rank_prior", K, (), T)
+    hidden, W1, b1, W2, root = (t.to(DEV) for t in synth.head_inputs(B, H, V, K, seed=5))
+    i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+    kc, vc = (synth.normal_bf16(1, i, (n_layers, B, Hkv, L + T, D), device=DEV) for i in (2, 3))
+    q = synth.normal_bf16(1, 4, (n_layers, B, T, Hq, D), device=DEV)
+    kn, vn = (synth.normal_bf16(1, i, (n_layers, B, T, Hkv, D), device=DEV) for i in (5, 6))
+    d = dict(hidden=hidden, W1=W1, b1=b1, W2=W2, root_tok=root, q_layers=q, out_layers=torch.zeros_like(q), logits=synth.normal_bf16(1, 7, (B, T, V), device=DEV),
+             seq_lens=torch.full((B,), L, dtype=torch.int32, device=DEV), cand=i32(B, tree.C), tree_tok=i32(B, T), accept_len=i32(B), best_path=i32(B),
+             acc_nodes=i32(B, K + 1), acc_tok=i32(B, K + 1), next_root=i32(B), k_caches=binding.cache_pointer_array(list(kc), DEV),
+             v_caches=binding.cache_pointer_array(list(vc), DEV), k_caches_host=binding.cache_pointer_array(list(kc)),
+             v_caches_host=binding.cache_pointer_array(list(vc)), ws=workspace(tree, B, H, V, Hq, Hkv, D, L + T))
+    a = binding.StepArgs()
+    a.B, a.H, a.V, a.Hq, a.Hkv, a.D, a.n_layers, a.Lcap = B, H, V, Hq, Hkv, D, n_layers, L + T
+    a.stride_b, a.stride_h, a.stride_t = kc.stride()[1:4]
+    for n, t in d.items():
+        setattr(a, n, t.data_ptr())
+    a.ws_bytes = 256
+    ap = binding.AppendArgs()
+    ap.k_new_layers, ap.v_new_layers, ap.rope_theta = kn.data_ptr(), vn.data_ptr(), 0.0
+    before = [t.clone() for t in (q, kc, vc)]
+    with pytest.raises(binding.MtvError) as e:
+        binding.mtv_verify_steps(tree, [a], [ap])
+    torch.cuda.synchronize()
+    assert e.value.code == -3
+    assert all(torch.equal(x, y) for x, y in zip(before, (q, kc, vc)))
