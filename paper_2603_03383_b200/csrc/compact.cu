@@ -120,7 +120,10 @@ accept_compact_kernel(int T, int K, int P, int ns, int D, int Lcap, int n_layers
         }
         __syncthreads();
     }
-    if (tid == 0 && atomicAdd(&tickets[b], 1) == (int)(gridDim.x * gridDim.z) - 1) {
+    if (tid != 0) return;
+    __threadfence();             // this block has read the length: before its ticket says so
+    if (atomicAdd(&tickets[b], 1) == (int)(gridDim.x * gridDim.z) - 1) {
+        __threadfence();
         if (status) status[b] = fits ? MTV_OK : MTV_ERR_CAPACITY;
         if (fits) seq_lens[b] = L + n + 1;
     }
