@@ -322,6 +322,9 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 __syncwarp();
             }
         }
+        // (given up early: the other half of the early stages, so that their barriers complete when their copies have landed)
+        for (; it < n_early; ++it)
+            if (lane == 0) ht_tma_2d(ring + it * HT_STAGE_BYTES + HT_W_BYTES, &x_map, full(it), it % n_kc * 64, k * HT_N);
         if (lane == 0) issued_s = it;
     } else if (warp == 4) {
         // ---------------------------------------------------------------- MMA issuer
