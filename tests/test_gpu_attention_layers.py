@@ -132,3 +132,48 @@ def test_two_trees_on_two_streams(D, n_layers):
     for tree, _, out, want in sides:
         assert binding.mtv_device_error(tree) == 0
         assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,lens,n_layers,scale", [
+    (29, 4, 1, 128, [70], 70, 0.0),                              # a second launch behind the first 64 layers
+    (16, 2, 2, 64, [40, 129], 65, 0.0),
+    (29, 8, 2, 128, [5 * i % 301 for i in range(70)], 2, 0.0),   # lengths in three lots of 32
+    (64, 2, 1, 64, [7 * i % 401 for i in range(33)], 3, 0.0),
+    (64, 8, 2, 64, [300, 0, 63], 3, -0.11),                      # a negative scale, hidden tree columns
+])
+@pytest.mark.parametrize("apart", [True, False])
+def test_many_layers_many_sequences_negative_scale(T, Hq, Hkv, D, lens, n_layers, scale, apart):
+    tb, tree = make_tree("rank_prior", 4, (), T)
+    B, Lcap, H, V, K = len(lens), max(lens) + T + 3, 64, 600, 4
+    ks, vs = ([synth.normal_bf16(T, s + l, (B, Hkv, Lcap, D), device=DEV) for l in range(n_layers)] for s in (100, 300))
+    q = synth.normal_bf16(T, 90, (n_layers, B, T, Hq, D), device=DEV)
+    sl = torch.tensor(lens, dtype=torch.int32)
+    want = [ref.tree_attention(q[l].cpu(), ks[l].cpu(), vs[l].cpu(), sl, tb["mask"], scale=scale) for l in range(n_layers)]
+    if B > 16:          # more sequences than the heads take: one-layer calls
+        out = torch.full_like(q, 9.0)
+        ws = workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap)
+        for l in range(n_layers):
+            binding.tree_verify_attention(tree, q[l], ks[l], vs[l], sl.to(DEV), out[l], ws, scale=scale)
+        torch.cuda.synchronize()
+    else:
+        hidden, W1, b1, W2, root = synth.head_inputs(B, H, V, K, seed=3, device=DEV)
+        i32 = lambda *s: torch.zeros(s, dtype=torch.int32, device=DEV)
+        d = dict(hidden=hidden, W1=W1, b1=b1, W2=W2, root_tok=root, q_layers=q, out_layers=torch.full_like(q, 9.0),
+                 logits=synth.normal_bf16(T, 91, (B, T, V), device=DEV), seq_lens=sl.to(DEV), cand=i32(B, tree.C), tree_tok=i32(B, T),
+                 accept_len=i32(B), best_path=i32(B), acc_nodes=i32(B, K + 1), acc_tok=i32(B, K + 1), next_root=i32(B),
+                 k_caches=binding.cache_pointer_array(ks, DEV), v_caches=binding.cache_pointer_array(vs, DEV),
+                 k_caches_host=binding.cache_pointer_array(ks), v_caches_host=binding.cache_pointer_array(vs),
+                 ws=workspace(tree, B, H, V, Hq, Hkv, D, Lcap))
+        a = binding.StepArgs()
+        a.B, a.H, a.V, a.Hq, a.Hkv, a.D, a.n_layers, a.Lcap = B, H, V, Hq, Hkv, D, n_layers, Lcap
+        a.stride_b, a.stride_h, a.stride_t = ks[0].stride()[:3]
+        a.scale = scale
+        for n, t in d.items():
+            setattr(a, n, t.data_ptr())
+        a.ws_bytes = d["ws"].numel() if apart else workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap).numel()
+        binding.mtv_verify_step(tree, a)
+        torch.cuda.synchronize()
+        out = d["out_layers"]
+    assert binding.mtv_device_error(tree) == 0
+    for l in range(n_layers):
+        assert_close(out[l], want[l], "layer %d" % l)
