@@ -1266,20 +1266,25 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
 }
 
 // Which kernel a call for ONE layer takes at head size 128 (several layers always take the one of this file: 32 layers at
-// L = 512 take 60 us instead of 320, at L = 8192 265 instead of 570).  The kernel on CTA pairs starts and ends faster but
-// needs 0.97 us per key group on a pair of SMs and leaves pairs idle where blocks and splits do not fill the 74; this
-// one needs 1.55 us on one SM, divides the groups evenly, and costs 4.5 us per further item.  In us per call:
-//     L (one sequence, 8 KV heads, T = 64)   512: 10 / 15   8192: 17 / 24   32768: 39 / 48
-//     7 sequences, 28 / 4 heads, L <= 6000, capacity 8000: 55 / 46;    4 sequences, T = 128, L = 32768: 262 / 166
-//     16 sequences, L <= 4096: 60 / 69
-// Only the capacity is known here, not the lengths; this kernel is taken where the estimate is better by a tenth.
+// L = 512 take 60 us instead of 320, at L = 8192 290 instead of 570).  The kernel on CTA pairs starts and ends faster but
+// leaves pairs idle where blocks and splits do not fill the 74; this one divides the groups evenly.  Only the capacity is known
+// here, not the lengths.  us per call, lengths uniform in [h / 4, h] with h = all, a half, a quarter, an eighth of the
+// capacity (pairs / even division):
+//      7 sequences, 28 / 4 heads, capacity  8112:   72 / 60    41 / 38    26 / 30    18 / 25
+//     12 sequences, 16 / 4 heads, capacity  8192:   71 / 58    40 / 35    25 / 28    17 / 25
+//      4 sequences, T = 128,      capacity 32896:  266 / 197  137 / 149   78 / 70    42 / 42
+//      3 sequences, 16 / 4 heads, capacity 20000:   38 / 39    25 / 31    18 / 27    15 / 22
+//     16 sequences, 32 / 8 heads, capacity 32768:  427 / 381  217 / 198  106 / 126   70 / 91
+//     16 sequences, 32 / 8 heads, capacity  4224:   59 / 68    42 / 53    31 / 31    27 / 23
+// With more blocks than pairs the pairs are all busy, longest sequence first, and what the even division gains in a full cache it
+// loses in one that is a quarter full: pairs.  With fewer, the even division is taken where the estimate for a full cache (us
+// per group on a pair and on an SM, start and end) is better by a tenth; such a call on a nearly empty cache pays 7 us.
 static bool pair_kernel_is_better(int T, int G, int B, int Hkv, int Lcap) {
     int n_blk = 1;
     const int ns = attn_pair_plan(T, G, B, Hkv, Lcap, &n_blk);
     const double blocks = (double)B * Hkv * n_blk, groups = (Lcap + AT_BN - 1) / AT_BN;
-    const double sms = sm_count(), rounds = std::max(1.0, blocks / (0.5 * sms)), items = std::max(1.0, blocks / sms);
-    const double pairs = 0.97 * rounds * ceil(groups / ns) + 9.0 + 4.0 * (rounds - 1.0);
-    const double even = 1.55 * blocks * groups / sms + 22.0 + 4.5 * (items - 1.0);
+    if (blocks > 0.5 * sm_count()) return true;
+    const double pairs = 0.97 * ceil(groups / ns) + 9.0, even = 1.55 * blocks * groups / sm_count() + 22.0;
     return pairs <= 1.1 * even;
 }
 
