@@ -400,13 +400,14 @@ int keys_merge_shards(int n, int n_shards, int v_slab, const unsigned long long 
  * stream, i = 0, 1, ... until `capacity` launches have been recorded; later launches
  * are not recorded.  start/stop: host arrays of cudaEvent_t created by the caller and
  * kept alive until the taps are cleared (capacity = 0 or NULL arrays clears them).
+ * Inside a whole step the acceptance and the advance of seq_lens are part of MTV_KERNEL_KV_COMPACT's launch.
  * Not thread-safe; do not use during stream capture.
  */
 #define MTV_KERNEL_HEADS_RESBLOCK 0
 #define MTV_KERNEL_HEADS_VOCAB_TOPK 1
 #define MTV_KERNEL_HEADS_MERGE 2
 #define MTV_KERNEL_ATTN_PARTIAL 3
-#define MTV_KERNEL_ATTN_COMBINE 4
+#define MTV_KERNEL_ATTN_COMBINE 4 /* no longer recorded: the attention merges inside its launch */
 #define MTV_KERNEL_ARGMAX_PARTIAL 5
 #define MTV_KERNEL_ACCEPT_FINISH 6
 #define MTV_KERNEL_KV_COMPACT 7

@@ -50,7 +50,6 @@ static VocabSmem vocab_smem_plan(int NB, int MR, int H, int ctas_per_head) {
         if (fixed + 2 * sb > VT_SMEM_MAX) continue;
         int n = (int)((VT_SMEM_MAX - fixed) / sb);
         if (n > VT_MAX_STAGES) n = VT_MAX_STAGES;
-        // keep at least ~96 KB in flight when the rows are long enough
         s.rows_per_stage = rs; s.n_stages = n; s.stage_bytes = sb;
         break;
     }

@@ -135,7 +135,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
                     const uint32_t base = ring + s * p.stage_bytes;
                     ptx::mbar_arrive_expect_tx(full(s), (uint32_t)(TILES * R + N) * 128u);
                     tma_load_2d(base, &w_map, full(s), kc * LM_KC, row0);                 // rows past V arrive as zeros
-                    if (TILES == 2) tma_load_2d(base + LM_TILE_BYTES, &w_map, full(s), kc * LM_KC, row0 + R);
+                    tma_load_2d(base + LM_TILE_BYTES, &w_map, full(s), kc * LM_KC, row0 + R);
                     tma_load_2d(base + x_off, &x_map, full(s), kc * LM_KC, 0);             // rows past M arrive as zeros
                 }
                 __syncwarp();

@@ -112,17 +112,6 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, bool accumulate) {
-    const uint32_t acc = accumulate ? 1u : 0u;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n"
-        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(acc) : "memory");
-}
 // Shared-memory operand descriptors with 128-byte swizzle and 8-row (8-key) groups 1024 bytes apart, as lower and upper
 // word.  The upper word is the same for all of them; the start address in the lower one counts 16-byte units and never
 // carries (shared-memory addresses stay below 256 KB), so that moving along an operand is one 32-bit add.  lbo_bytes: 16
@@ -153,6 +142,7 @@ __device__ __forceinline__ void tc_commit_elect(uint32_t bar, bool leader) {
         "}\n"
         ::"r"(bar), "r"((uint32_t)leader) : "memory");
 }
+// D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate.
 __device__ __forceinline__ void mma_ss_elect(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t desc_hi, uint32_t idesc,
                                              bool accumulate, bool leader) {
     asm volatile(

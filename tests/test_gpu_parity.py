@@ -372,7 +372,7 @@ def test_full_step_at_the_long_shapes():
 
 
 def test_full_step_from_host_buffers_with_more_layers_than_download_groups():
-    """Twenty layers: the attention outputs leave in groups of two layers (sixteen groups at most)."""
+    """Twenty layers: queries arrive and attention outputs leave in groups of layers, fewer than there are layers."""
     _step_case(2, 256, 2000, 8, 2, 128, 20, "rank_prior", 4, (), 64, [70, 33], seed=9, host=True)
 
 
