@@ -2,53 +2,59 @@
 // attend to the prefix and to their ancestors-or-self among the tree rows of the KV cache, for one layer or for all
 // layers of a step in one launch.
 //
-// Work.  An ITEM is one (layer, sequence, KV head, row block): up to two tiles of 128 query rows — 128 / G whole tree
-// nodes times the G query heads that share the KV head — against all 128-key groups of the sequence.  The grid is
-// persistent, one CTA per SM; the key groups of all items, laid end to end, are divided evenly among the CTAs whatever
-// the sequences' lengths, so that a CTA works on a run of consecutive PIECES: the end of one item, whole items, the
-// beginning of another.  Items with several row blocks go to teams of CTAs that walk the same keys at the same time (the
-// second read of a key group finds it in L2).  Every CTA derives its run from the lengths on the device.
-//   * More items than teams: an item counts its groups plus AT_ITEM_COST (what starting and ending an item costs beside
+// Work.  An ITEM is one (layer, sequence, KV head): the tiles of 128 query rows — 128 / G whole tree nodes times the G query
+// heads that share the KV head — against all 128-key groups of the sequence.  The grid is persistent, one CTA per SM, a row
+// tile per CTA; the CTAs that have the tiles of an item are a TEAM and walk the same keys at the same time.  The key groups of
+// all items, laid end to end, are divided evenly among the teams whatever the sequences' lengths, so that a team works on a run
+// of consecutive PIECES: the end of one item, whole items, the beginning of another.  Every CTA derives its run from the
+// lengths on the device (PieceWalk):
+//   * More items than teams: an item counts its groups plus ITEM_COST (what starting and ending an item costs beside
 //     its groups) and the cuts fall anywhere.
-//   * Fewer: no CTA gets two pieces; the piece length is the smallest for which the pieces of all items fit the teams.
+//   * Fewer: no team gets two pieces; the piece length is the smallest for which the pieces of all items fit the teams.
+//   * Whole items where that makes no run longer by more than MERGE_COST.
 // Pieces that are not whole items leave O / l (fp32: where an item is cut must not show in its precision) and (m, l) in the
-// workspace; at the end of the launch the CTAs that share an item meet at a counter and each combines a slice of its rows.
+// workspace; at the end of the launch the CTAs that share a tile meet at a counter and each combines a slice of its rows.
 // They all do so when the device is this launch's alone (the grid never exceeds one CTA per SM), but nothing depends on it:
 // a warp that has waited for a millisecond leaves its slice to the last one to leave and makes room.
 //
-// One piece.  Two STREAMS of 128 query rows by 128 keys share the tensor core: with two row tiles stream t owns tile t and
-// both see every key group; with one row tile both use it and take alternate groups (merged at the end).  A stream runs
-//     S(0) | PV(0) S(1) | PV(1) S(2) | ...
-// with S of the next group issued right behind O += P V of this one, so that the softmax of one stream runs under the
-// MMAs of the other.  P (bf16) overwrites the scores it came from in tensor memory; the tensor core executes one thread's
-// MMAs in issue order, which is what lets S(j + 1) follow the PV(j) that reads P(j) under it.  Each stream has an issuing
-// warp of its own and they take turns: an issue blocks until the tensor core has nearly caught up and a barrier test costs
-// about a hundred cycles, so with one warp for both the tensor core idled through every test; without turns the streams
-// fall into step and compute their softmax at the same time, with the tensor core idle (4.4 k cycles per pair of ticks
-// against 3.6 k with one warp).
-//   warps 0-7 / 8-15  softmax of stream 0 / 1: two threads own a query row, 64 columns each
-//   warps 16 / 18     issue the MMAs of stream 0 / 1
-//   warp 17           derives the CTA's pieces and requests K and V tiles (TMA) through a ring
-//   warp 19           requests the query tiles (TMA) and clears the V rows past the last key (their P is 0, but 0 * NaN
-//                     would poison O)
-// Tensor memory: S of stream 0 and 1 (128 columns each), O of stream 0 and 1.
+// PAIR (head size 128, more than one row tile): the CTAs of a team are cta_group::2 pairs, whose MMAs (M = 256) read half of
+// a group's K and V from either CTA's shared memory, so that a tile and a group cost an SM 32 KB.  Else a CTA has K and V to
+// itself: at head size 64 that is 32 KB as well, and a single row tile has nobody to share with.
 //
-// What bounds it: per tile pair and key group the tensor core needs 2048 cycles at D = 128 and the special-function unit
-// 1536 (a quarter of the exponentials run as polynomials on the FMA pipes); the dependent chain of one stream, scores
-// visible -> exponentials -> P visible -> PV -> S, sets what is reached of it.  Four softmax warps per scheduler rather than
-// two shorten that chain: a warp's exponentials take 1.2 k cycles for 128 columns, most of it latency.
+// One tile.  A CTA keeps one accumulator O, which leaves room for THREE tiles of scores in tensor memory: S of group j + 3 is
+// issued right behind O += P V of group j, over the P that this one has just read (the tensor core executes one thread's MMAs in
+// issue order),
+//     S(0) S(1) S(2) | PV(0) S(3) | PV(1) S(4) | ...
+// so that a group's softmax has the time of two other groups' MMAs and two groups' softmax run at once.  (The kernel before this
+// one had two row tiles in a CTA, with an accumulator and one tile of scores each: the chain scores -> P -> PV -> scores then took
+// 1.63 k cycles per tile and group, of which the tensor core worked 1024.  Now 1.4 k; what is left of the chain is 1.6 k of
+// softmax and 1.4 k of handing over, shared by three tiles.)
+//   warps 0-7 / 8-15  softmax of groups 2, 4, .. / 1, 3, ..: two threads own a query row, 64 columns each; the first group is
+//                     everybody's, 32 columns a thread.  (All on every group: 4 % slower at 32768 keys, as what a group costs a
+//                     warp beside its exponentials is paid twice as often.)
+//   warp 16           issues the MMAs (odd CTA of a pair: the slot keeper)
+//   warp 17           derives the pieces and requests this CTA's part of K and V groups (TMA) through a ring
+//   warp 18           the slot keeper (odd CTA: tells the even one what has landed, V rows past the last key cleared)
+//   warp 19           requests the query tiles; clears the V rows past the last key (their P is 0, but 0 * NaN would poison O)
+// The slot keeper follows the scores: it gives ring slots back as soon as the MMAs that read them are complete, and puts in its
+// word for a group's PV when V, and K of the scores behind it, are there.  So the issuing warp has one barrier to test per
+// group: a test costs it about a hundred cycles, and the tensor core has only some two MMAs queued.
 //
-// The reference of a row's exponentials is the maximum of its first group, rounded up to a whole number; it moves only when
-// the sum of a thread's P in some later group exceeds 2^32, or one of its exponents 32 where a polynomial would not show it in
-// the sum (from 128 on its result is meaningless).  P and O are floating-point numbers, so a reference that is not the maximum
-// costs range, and the exactness of the largest weights, which a second term of P makes up for (see two_terms); in return no
-// maximum is formed and nothing is exchanged between the two threads of a row in an ordinary group.
+// What bounds it: the tensor core needs 1024 cycles for a tile and group at D = 128 and the special-function unit as many; 8 PV
+// and 8 S MMAs take 1025 with every other unit busy beside them, so the rest of the 1.4 k is the chain.  At 4 x 32768 keys the
+// board's power limit takes 15 to 25 % of the clock on top.
+//
+// The reference of a row's exponentials is common to its four threads: the maximum of the piece's first group, rounded up to a
+// whole number.  It moves only when the sum of a thread's P in some later group exceeds 2^32.  P and O are floating-point
+// numbers, so a reference that is not the maximum costs range, and the exactness of the largest weights, which a second term of
+// P makes up for (see two_terms); in return no maximum is formed and nothing is exchanged between the threads of a row in an
+// ordinary group.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 
-#include "attn_common.cuh"
+#include "attn_work.cuh"
 
 namespace mtv {
 
@@ -60,359 +66,186 @@ int launch_tree_attn_pair(const mtv_tree *tree, int B, int Hq, int Hkv, const __
                           float scale_log2, __nv_bfloat16 *out, int32_t *status, void *ws_o, float *ws_ml, int32_t *ws_order,
                           cudaStream_t stream);
 
-constexpr int AT_BN = 128;            // keys per group
-constexpr int AT_THREADS = 640;
-constexpr int AT_SOFTMAX_WARPS = 16;
-constexpr int AT_MMA_WARP = 16, AT_TMA_WARP = 17, AT_Q_WARP = 19;   // warp 18: MMAs of stream 1
-constexpr int AT_PIECES = 4;          // piece descriptors in flight
-constexpr int AT_ITEM_COST = 1;       // what an item costs beside its key groups, in groups
-// How long a warp waits for the others of an item, in cycles.  In the bounds-checking build it looks once: nearly all slices
-// are then left to the last warp.
-#ifdef MTV_DEBUG_BOUNDS
-constexpr long long AT_MERGE_WAIT = 0;
-#else
-constexpr long long AT_MERGE_WAIT = 2000000;
-#endif
-constexpr int AT_MAX_CTAS = 256;      // merge counters in the tree object: one pair per CTA
-constexpr int AT_MAX_LAYERS = 64;     // layers per launch (two tensor maps each in the kernel's parameters)
-// registers per thread: 96 at launch, moved from the four auxiliary warps to the sixteen softmax warps
-constexpr int AT_LAUNCH_REGS = 96, AT_SOFTMAX_REGS = 104, AT_AUX_REGS = 64;
-static_assert(512 * AT_SOFTMAX_REGS + 128 * AT_AUX_REGS <= AT_THREADS * AT_LAUNCH_REGS, "register split");
-// P goes to the tensor core as bf16, whose rounding is the largest error beside the output's own.  Where a reference that
-// follows the row's maximum made the largest weights exact (they were 1), a fixed reference does not: P then has a second bf16
-// term, what the rounding of the first left.  At head size 64 in every group (O += P V is short there); at 128 in a piece's
-// first group, whose maximum alone used to be the reference.  Rel. error against 64 bits with one term / two / the kernels that
-// this one replaced: D = 64, L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 / .00210; D = 128, L = 512:
-// .00235 / .00204 / .00268.  Cost: eight one-layer calls at head size 64 171 -> 198 us, steps at 128 1 to 2 %.
-template <int D>
-__host__ __device__ constexpr bool two_terms(int group) { return D == 64 || group == 0; }   // of the stream's groups of a piece
-constexpr float AT_SUM_LIMIT = 4294967296.f;   // 2^32: a thread's sum of P over a group beyond it moves the reference
+
+constexpr int ITEM_COST = 2;          // what an item costs beside its key groups, in groups
+constexpr int MERGE_COST = 5;         // what partial results cost: written, met for, read and combined
+constexpr int W_MMA = 16, W_TMA = 17, W_RELAY = 18, W_Q = 19;
+constexpr int NB = 3;                 // tiles of scores
 constexpr float LOG2E = 1.4426950408889634f;
+// P goes to the tensor core as bf16, whose rounding is the largest error beside the output's own.  Where a reference that
+// follows the row's maximum makes the largest weights exact (they are 1), a fixed reference does not: P then has a second bf16
+// term, what the rounding of the first left.  On pairs in a piece's first group, whose maximum is the reference; else in every
+// group (O += P V is short at head size 64, and an item of one row tile is bound by memory).  Rel. error against 64 bits with
+// one term / two / a reference that follows the maximum: D = 64, L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 /
+// .00210; D = 128, L = 512: .00235 / .00204 / .00268.
+template <bool PAIR>
+__host__ __device__ constexpr bool two_terms(int group) { return !PAIR || group == 0; }
+// tensor-memory columns: O, and three tiles of scores; P lies over its scores, each half of the keys over its own: keys 0-63
+// at columns 0-31, keys 64-127 at 64-95; in two terms each quarter over its own: keys 0-31 at columns 0-15, their second
+// terms at 16-31, and so on.
+constexpr uint32_t TM_O = 0, TM_S = 128;
 
-// tensor-memory columns: S of stream t at 128 t, O at 256 + 128 t.  P lies over S, each half of the keys over its own scores:
-// keys 0-63 at columns 0-31, keys 64-127 at 64-95; in two terms each quarter over its own: keys 0-31 at columns 0-15, their
-// second terms at 16-31, and so on.
-constexpr uint32_t TM_S = 0, TM_O = 256;
-
-// Shared memory: two query tiles, the K/V ring, the (m, l) exchange of the two streams, barriers, descriptors.
-template <int D>
+// PAIR: K and V are divided between the two CTAs of a pair
+template <int D, bool PAIR>
 struct AttnSmem {
-    static constexpr uint32_t TILE = 128 * D * 2;          // 128 rows as D / 64 halves of 128-byte rows (128-byte swizzle)
+    static constexpr uint32_t TILE = 128 * D * 2;          // a query tile: 128 rows as D / 64 halves of 128-byte rows (128-byte swizzle)
     static constexpr uint32_t HALF = 128 * 128;
-    static constexpr int STAGES = D == 128 ? 5 : 10;
-    static constexpr uint32_t OFF_RING = 2 * TILE;
-    static constexpr uint32_t OFF_ML = OFF_RING + STAGES * TILE;
-    static constexpr uint32_t OFF_BAR = OFF_ML + 4 * 128 * 4;
-    static constexpr int BAR_KV_FULL = 0;
-    static constexpr int BAR_KV_EMPTY = STAGES;
-    static constexpr int BAR_TAIL = 2 * STAGES;             // a V tile whose last rows must be cleared lands here first
-    static constexpr int BAR_Q_FULL = 3 * STAGES;           // [2 tiles]
-    static constexpr int BAR_Q_EMPTY = BAR_Q_FULL + 2;
-    static constexpr int BAR_S = BAR_Q_EMPTY + 2;           // [2 streams] scores of a tick complete
-    static constexpr int BAR_P = BAR_S + 2;                 // [2] P of a group written
-    static constexpr int BAR_O = BAR_P + 2;                 // [2] the stream's O of the piece complete
-    static constexpr int BAR_PC_FULL = BAR_O + 2;           // [AT_PIECES]
+    static constexpr uint32_t SLOT = TILE / (PAIR ? 2 : 1);    // this CTA's part of a K group (64 keys of a pair) or V group (64 columns)
+    static constexpr uint32_t K_HALF = PAIR ? 64 * 128 : HALF; // the next 64 columns of K
+    static constexpr int STAGES = 10 * 16384 / SLOT;
+    // The slot keeper may wait for K of three groups on: the slot it comes into was given back two groups ago.
+    static constexpr bool K_AHEAD = STAGES >= 2 * NB + 4;
+    static constexpr uint32_t OFF_RING = 2 * TILE;         // two query tiles: the next piece's, and where output rows are staged
+    static constexpr uint32_t OFF_X = OFF_RING + STAGES * SLOT;
+    static constexpr uint32_t OFF_BAR = OFF_X + 4 * 128 * 4;
+    static constexpr int BAR_KV_FULL = 0;                  // of the even CTA of a pair: both parts (its own copy and the odd CTA's word)
+    static constexpr int BAR_KV_EMPTY = BAR_KV_FULL + STAGES;
+    static constexpr int BAR_TAIL = BAR_KV_EMPTY + STAGES; // V whose last rows must be cleared lands here first (odd CTA: not used)
+    static constexpr int BAR_Q_FULL = BAR_TAIL + STAGES;   // [2 tiles] of the even CTA: both CTAs' tiles
+    static constexpr int BAR_Q_EMPTY = BAR_Q_FULL + 2;     // [2]
+    static constexpr int BAR_S = BAR_Q_EMPTY + 2;          // [3] scores of a group complete; behind a piece's last groups but one: their PV is
+    static constexpr int BAR_P = BAR_S + NB;               // [3] even CTA: what PV of a group and the scores behind it wait for
+    static constexpr int BAR_O = BAR_P + NB;               // O of a piece complete
+    static constexpr int BAR_O_FREE = BAR_O + 1;           // even CTA: O of a piece read
+    static constexpr int BAR_PC_FULL = BAR_O_FREE + 1;     // [AT_PIECES]
     static constexpr int BAR_PC_EMPTY = BAR_PC_FULL + AT_PIECES;
-    static constexpr int BAR_XM = BAR_PC_EMPTY + AT_PIECES;    // [2 streams][4] the two warps of a row quarter, references
-    static constexpr int BAR_XO = BAR_XM + 8;                  // [2][4] the two (one row tile: [4], the four) warps, results
-    static constexpr int BAR_STAGED = BAR_XO + 8;              // [STAGES] the output rows staged in a slot have left it
-    static constexpr int BAR_DRAIN = BAR_STAGED + STAGES;
-    static constexpr int BAR_TURN = BAR_DRAIN + 2;          // [2] the stream's turn to issue
-    static constexpr int BAR_COUNT = BAR_TURN + 2;
+    static constexpr int BAR_XM = BAR_PC_EMPTY + AT_PIECES;    // [4] the four warps of a row quarter: references
+    static constexpr int BAR_XO = BAR_XM + 4;                  // [4] results
+    static constexpr int BAR_DRAIN = BAR_XO + 4;
+    static constexpr int BAR_COUNT = BAR_DRAIN + 1;
     static constexpr uint32_t OFF_DESC = OFF_BAR + (BAR_COUNT * 8 + 15) / 16 * 16;
     static constexpr uint32_t OFF_MISC = OFF_DESC + AT_PIECES * 32;
-    static constexpr uint32_t TOTAL = OFF_MISC + 112;
+    static constexpr uint32_t OFF_ASK = OFF_MISC + 64;     // [4] a row quarter is asked to move its reference
+    static constexpr uint32_t OFF_AT = OFF_ASK + 16;       // [4][4] the group that a warp of the quarter is at
+    static constexpr uint32_t TOTAL = OFF_AT + 64;
     static_assert(TOTAL <= 227 * 1024, "shared memory");
+    // bf16 x bf16 -> fp32, M = 256 over a pair, 128 in a CTA; N = 128 keys or D columns; V N-major
+    static constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((PAIR ? 256u : 128u) >> 4) << 24;
+    static constexpr uint32_t IDESC_QK = IDESC | (128u >> 3) << 17, IDESC_PV = IDESC | (uint32_t)(D >> 3) << 17 | 1u << 16;
 };
 
-struct AttnPiece {      // 32 bytes
-    int layer, b, head, gb, cnt, L, flags, first;   // key groups [gb, gb + cnt); cnt = 0: no more pieces;
-                                                    // first: first team that contributes to the item
-};
-constexpr int PIECE_PARTIAL = 1, PIECE_HEAD = 2;   // not a whole item; starts at the item's first group
-struct AttnMerge {      // a partial piece of this CTA, for the merge at the end
-    int first, n, layer, b, head, pad;             // first contributing team, number of them
-};
-
-template <int ML>
-struct __align__(64) AttnMaps {
-    CUtensorMap q, k[ML], v[ML];
-};
-
-struct AttnParams {
-    const int32_t *seq_lens;
-    const uint64_t *anc;     // [T][2]
-    __nv_bfloat16 *out;      // [layers][B][T][Hq][D]
-    uint4 *ws_o;             // [CTA][2 slabs][2 tiles][D / 4 chunks][128 rows] 16-byte chunks of O / l, fp32
-    float2 *ws_ml;           // [CTA][2 slabs][2 tiles][128 rows] (m, l)
-    int32_t *left;           // [CTA][2 slabs][16 warps] 1: the warp's slice of the item is left to the last one
-    int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls; depart counts slices left in its upper half
-    int32_t *status;         // [B] or null
-    int32_t *dev_error;
-    float scale_log2;
-    int B, T, G, Hq, Hkv, Lcap, n_layers;
-    int npc, R;              // tree nodes per tile (128 / G) and the rows they fill
-    unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
-    int n_tiles, n_blk, teams;
-    Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
-};
-
-// Operands: queries and keys K-major; V N-major, its next 64 columns one half tile further.
-// bf16 x bf16 -> fp32, M = 128
-constexpr uint32_t AT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
-constexpr uint32_t AT_B_NMAJOR = 1u << 16;
-
-__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
-__device__ __forceinline__ float trunc_bf16(float x) { return bf16_hi(__float_as_uint(x)); }
-// P = 2^(scale S - m) of 32 scores (two values per instruction where the instruction set has packed forms) and its
-// contribution to the row sum.  Every fourth quadruple runs on the FMA pipes: the special-function unit is the bottleneck of
-// a group.  pk: bf16 pairs; TWO: rest has what their rounding left, as bf16 pairs.  top: the largest exponent among those of
-// the polynomials, which go wrong silently where ex2 gives +inf or NaN.
-template <int DEGREE, bool TWO>
-__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t *pk, uint32_t *rest,
-                                            float &top) {
-#pragma unroll
-    for (int e = 0; e < 16; e += 2) {
-        const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2);
-        const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e + 2]), __uint_as_float(s[2 * e + 3])), sc2, nm2);
-        float2 p01, p23;
-        if (e % 8 == 6) {
-            top = ptx::fmax3_nan(top, x01.x, x01.y);
-            top = ptx::fmax3_nan(top, x23.x, x23.y);
-            p01 = exp2_poly2<DEGREE>(x01);
-            p23 = exp2_poly2<DEGREE>(x23);
-        } else {
-            p01 = make_float2(ex2(x01.x), ex2(x01.y));
-            p23 = make_float2(ex2(x23.x), ex2(x23.y));
-        }
-        la = __fadd2_rn(la, p01);
-        lb = __fadd2_rn(lb, p23);
-        if (TWO) {
-            pk[e] = pack2_bf16(p01.x, p01.y);
-            pk[e + 1] = pack2_bf16(p23.x, p23.y);
-            const float2 r01 = __fadd2_rn(p01, make_float2(-bf16_lo(pk[e]), -bf16_hi(pk[e])));
-            const float2 r23 = __fadd2_rn(p23, make_float2(-bf16_lo(pk[e + 1]), -bf16_hi(pk[e + 1])));
-            rest[e] = pack2_bf16(r01.x, r01.y);
-            rest[e + 1] = pack2_bf16(r23.x, r23.y);
-        } else {
-            pk[e] = pack2_bf16(p01.x, p01.y);
-            pk[e + 1] = pack2_bf16(p23.x, p23.y);
-        }
-    }
+// Positions of half groups in the order in which the tensor core takes them: K0 K1 K2 V0 K3 V1 K4 ... V(cnt-1)
+__device__ __forceinline__ int k_pos(int j) { return j < NB ? j : 2 * j - (NB - 1); }
+__device__ __forceinline__ int v_pos(int j, int cnt) { return min(cnt, NB + j) + j; }
+__device__ __forceinline__ void half_at(int pos, int cnt, bool &is_v, int &j) {
+    const int n0 = min(NB, cnt), r = pos - n0;
+    if (r < 0) { is_v = false; j = pos; return; }
+    is_v = r >= 2 * (cnt - n0) || !(r & 1);
+    j = r >= 2 * (cnt - n0) ? r - (cnt - n0) : is_v ? r >> 1 : (r >> 1) + NB;
 }
-// the largest scale * s of 32 scores; NEG: the scale is negative
-template <bool NEG>
-__device__ __forceinline__ float max_quarter(const uint32_t (&s)[32], float scale) {
-    constexpr uint32_t sign = NEG ? 0x80000000u : 0u;
-    float a = -INFINITY, b = -INFINITY;
+// S phases of a piece beyond whole turns of its barrier: tile b of scores takes one phase per group, and one more where the
+// PV of the last groups but one is told through it.  Bit b: odd number of phases.
+__device__ __forceinline__ uint32_t s_phases(int cnt) {
+    uint32_t odd = 0;
 #pragma unroll
-    for (int e = 0; e < 32; e += 4) {
-        a = ptx::fmax3(a, __uint_as_float(s[e] ^ sign), __uint_as_float(s[e + 1] ^ sign));
-        b = ptx::fmax3(b, __uint_as_float(s[e + 2] ^ sign), __uint_as_float(s[e + 3] ^ sign));
-    }
-    return fmaxf(a, b) * fabsf(scale);
+    for (int b = 0; b < NB; ++b)
+        if (b < cnt) odd |= (uint32_t)(((cnt - b + NB - 1) / NB + (b != (cnt - 1) % NB)) & 1) << b;
+    return odd;
 }
-// Build option -DMTV_TRACE: cycle stamps of one CTA's phases into a buffer given by mtv_trace_set (development aid).
-#ifdef MTV_TRACE
-__device__ long long *g_trace = nullptr;   // [ctas][8 rows][512]
-#define TRACE_INIT(row, cond)                                                                          \
-    int trace_n = 0;                                                                                   \
-    long long *trace_row = g_trace && (cond) ? g_trace + ((size_t)blockIdx.x * 8 + (row)) * 512 : nullptr
-#define TRACE()                                                          \
-    do {                                                                 \
-        if (trace_row && trace_n < 512) trace_row[trace_n++] = clock64(); \
-    } while (0)
-#else
-#define TRACE_INIT(row, cond)
-#define TRACE()
-#endif
-
-// Position of tiles in the order in which a piece of cnt groups consumes them, and back.
-//   two row tiles: K0 V0 K1 V1 ...        one row tile: K0 K1 V0 K2 V1 K3 ... V(cnt-1)
-// Behind them a piece that is a whole item takes a ring slot per row tile to stage its output rows in.
-__device__ __forceinline__ int k_pos(bool one, int i) { return one ? (i == 0 ? 0 : 2 * i - 1) : 2 * i; }
-__device__ __forceinline__ int v_pos(bool one, int i, int cnt) { return one ? min(2 * i + 2, 2 * cnt - 1) : 2 * i + 1; }
-__device__ __forceinline__ void tile_at(bool one, int pos, int cnt, bool &is_v, int &idx) {
-    if (!one) { is_v = pos & 1; idx = pos >> 1; return; }
-    if (pos == 0) { is_v = false; idx = 0; return; }
-    if (pos & 1) { idx = (pos + 1) >> 1; is_v = idx >= cnt; if (is_v) idx = cnt - 1; return; }
-    is_v = true; idx = (pos - 2) >> 1;
+__device__ __forceinline__ uint32_t p_phases(int cnt) {
+    uint32_t odd = 0;
+#pragma unroll
+    for (int b = 0; b < NB; ++b)
+        if (b < cnt) odd |= (uint32_t)(((cnt - b + NB - 1) / NB) & 1) << b;
+    return odd;
 }
 
-__device__ __forceinline__ int ring_slots(const AttnPiece &d, bool one) {
-    return 2 * d.cnt + (d.flags & PIECE_PARTIAL ? 0 : one ? 1 : 2);
+// V rows from the last key on, up to the next multiple of 16: only they take part in O += P V
+template <int HALVES>
+__device__ __forceinline__ void clear_tail(unsigned char *v, int valid, int lane) {
+    for (int e = valid * 8 + lane; e < (valid + 15) / 16 * 16 * 8; e += 32)
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) *reinterpret_cast<uint4 *>(v + h * 16384 + e * 16) = make_uint4(0u, 0u, 0u, 0u);
+    ptx::fence_proxy_async();
 }
 
-// Output row of row r of tile t of a row block (in units of D elements from the item's first row), or -1 if it belongs to nobody.
-// With a group size that does not divide 128 the last 128 - R rows of a tile do (whatever the tile's shared memory held is
-// computed and never written out).
-__device__ __forceinline__ int node_in_tile(const AttnParams &p, int r) { return (int)(((unsigned)r * p.inv_g) >> 16); }
-__device__ __forceinline__ int out_row(const AttnParams &p, int blk, int t, int r) {
-    const int n = node_in_tile(p, r), node = (blk * 2 + t) * p.npc + n;
-    return r < p.R && node < p.T ? node * p.Hq + (r - n * p.G) : -1;
-}
-template <int D>
-__device__ __forceinline__ uint4 *item_out(const AttnParams &p, int layer, int b, int hd) {      // first row of an item's output
-    return reinterpret_cast<uint4 *>(p.out + (((size_t)layer * p.B + b) * p.T * p.Hq + hd * p.G) * D);
-}
-// slabs of the workspace: 16-byte chunk c (4 columns) of row r of tile t; the row's (m, l)
-template <int D>
-__device__ __forceinline__ uint4 *slab_o(const AttnParams &p, int cta, int slab, int t, int r, int c) {
-    return p.ws_o + ((((unsigned)cta * 2 + slab) * 2 + t) * (D / 4) + c) * 128 + r;
-}
-__device__ __forceinline__ float2 *slab_ml(const AttnParams &p, int cta, int slab, int t, int r) {
-    return p.ws_ml + (((unsigned)cta * 2 + slab) * 2 + t) * 128 + r;
-}
-
-// Rows of an item that is shared between CTAs: tile 0's, then tile 1's; contributor c0 combines its share of them, a thread per
-// 16-byte chunk of the output, with the loads of several contributors in flight.  This is warp w's part of it.
-template <int D>
-__device__ __forceinline__ void merge_slice(const AttnParams &p, const AttnMerge &m, int c0, int w, int blk, bool one, int lane) {
-    constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
-    const int rows = one ? p.R : 2 * p.R;
-    const int per = (rows + m.n - 1) / m.n, r_begin = c0 * per;
-    const int n_my = max(0, min(rows, r_begin + per) - r_begin);
-    const unsigned inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;    // e / n_my for e < 4096, n_my <= 256
-    uint4 *dst = item_out<D>(p, m.layer, m.b, m.head);
-#pragma unroll 1
-    for (int e = w * 32 + lane; e < n_my * (D / 8); e += AT_SOFTMAX_WARPS * 32) {
-        const int c = (int)(((unsigned)e * inv_n) >> 20), rr = r_begin + e - c * n_my;
-        const int t = rr >= p.R, r = rr - t * p.R;
-        float acc[8], mm = -INFINITY, wsum = 0.f;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = 0.f;
-#pragma unroll 1
-        for (int s0 = 0; s0 < m.n; s0 += NS) {
-            float2 ml[NS];
-            uint4 v[NS][VC];
-#pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                const int s = min(s0 + k, m.n - 1), cta = (m.first + s) * p.n_blk + blk;
-                const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
-                ml[k] = __ldcg(slab_ml(p, cta, sl, t, r));
-#pragma unroll
-                for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, t, r, c * VC + q));
-                if (s0 + k >= m.n) ml[k] = make_float2(-INFINITY, 0.f);
-            }
-            float mc = mm;
-#pragma unroll
-            for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
-            const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
-            mm = mc;
-            wsum *= resc;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] *= resc;
-#pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
-                wsum += wt;
-#pragma unroll
-                for (int q = 0; q < VC; ++q) {
-                    const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
-                }
-            }
-        }
-        const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
-        const int o = out_row(p, blk, t, r);
-        if (o >= 0)
-            dst[o * (D / 8) + c] =
-                make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
-                           pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
-    }
-}
-// The slices that warps left, of one item, by the softmax warps of the CTA whose warp was the last to leave it.  (Out of the way of the
-// usual case: as part of the merge below it cost the softmax loop, of all things, 4 %.)
-template <int D>
-static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, bool one, int warp, int lane) {
-    for (int u = warp; u < m.n * AT_SOFTMAX_WARPS; u += AT_SOFTMAX_WARPS) {
-        const int c = u / AT_SOFTMAX_WARPS, w = u % AT_SOFTMAX_WARPS, cta = (m.first + c) * p.n_blk + blk;
-        if (__ldcg(p.left + ((unsigned)cta * 2 + (c == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + w)) merge_slice<D>(p, m, c, w, blk, one, lane);
-    }
-}
-
-// NEG: the scale is negative (only taken at head size 64, and kept apart so that the usual case pays nothing for it)
-template <int D, int ML, bool NEG>
+// PAIR: launched in clusters of two.  NEG: the scale is negative (only taken at head size 64, and kept apart so that the usual case
+// pays nothing for it)
+template <int D, bool PAIR, int ML, bool NEG>
 __global__ void __launch_bounds__(AT_THREADS, 1)
 tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constant__ AttnParams p) {
-    using SM = AttnSmem<D>;
-    constexpr int ST = SM::STAGES;
+    using SM = AttnSmem<D, PAIR>;
+    constexpr int STAGES = SM::STAGES;
     extern __shared__ __align__(1024) unsigned char smem[];
-    // Programmatic dependent launch: let the next kernel of the stream be set up while this one runs.
     let_next_start();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0;
     const uint32_t sbase = ptx::smem_u32(smem);
     auto bar = [&](int i) { return sbase + SM::OFF_BAR + (uint32_t)i * 8u; };
+    // the same barrier in the even CTA of a pair
+    auto arrive_lead = [&](int i, uint32_t count = 1) {
+        if (PAIR) ptx::mbar_arrive_remote(ptx::mapa(bar(i), 0), count);
+        else ptx::mbar_arrive(bar(i), count);
+    };
     AttnPiece *desc = reinterpret_cast<AttnPiece *>(smem + SM::OFF_DESC);
-    AttnMerge *merges = reinterpret_cast<AttnMerge *>(smem + SM::OFF_MISC);                 // [2]
-    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + SM::OFF_MISC + 64);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 68);
-    volatile int *n_merge = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 72);     // partial pieces of this CTA
-    int *left_items = reinterpret_cast<int *>(smem + SM::OFF_MISC + 108);                   // of this CTA's: bit i, merges[i]
-    volatile int *beyond = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 76);      // [2 streams][4] a sum beyond AT_SUM_LIMIT
+    AttnMerge *merges = reinterpret_cast<AttnMerge *>(smem + SM::OFF_MISC);                  // [2], 48 bytes
+    volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + SM::OFF_MISC + 48);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 52);
+    volatile int *n_merge = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 56);      // partial pieces of this CTA
+    int *left_items = reinterpret_cast<int *>(smem + SM::OFF_MISC + 60);                     // of this CTA's: bit i, merges[i]
 
+    // CTA blk of the team has row tile blk (blk = 2 block + rank)
     const int team = (int)blockIdx.x / p.n_blk, blk = (int)blockIdx.x % p.n_blk;
-    const bool one = blk * 2 + 1 >= p.n_tiles;      // this CTA's row block has a single row tile
 
-    if (warp == AT_Q_WARP && lane == 0) {
+    if (warp == W_Q && lane == 0) {
         ptx::prefetch_tensormap(&maps.q);
         if (ML == 1) { ptx::prefetch_tensormap(&maps.k[0]); ptx::prefetch_tensormap(&maps.v[0]); }
-        for (int s = 0; s < ST; ++s) {
-            ptx::mbar_init(bar(SM::BAR_KV_FULL + s), 1);
-            ptx::mbar_init(bar(SM::BAR_KV_EMPTY + s), one ? 1 : 2);      // the streams that use the tile
+        for (int s = 0; s < STAGES; ++s) {
+            ptx::mbar_init(bar(SM::BAR_KV_FULL + s), PAIR && rank == 0 ? 2 : 1);
+            ptx::mbar_init(bar(SM::BAR_KV_EMPTY + s), 1);
             ptx::mbar_init(bar(SM::BAR_TAIL + s), 1);
-            ptx::mbar_init(bar(SM::BAR_STAGED + s), one ? 16 : 8);       // the softmax warps of the row tile
         }
         for (int t = 0; t < 2; ++t) {
-            ptx::mbar_init(bar(SM::BAR_Q_FULL + t), 1);
-            ptx::mbar_init(bar(SM::BAR_Q_EMPTY + t), one ? 2 : 1);
-            ptx::mbar_init(bar(SM::BAR_S + t), 1);
-            ptx::mbar_init(bar(SM::BAR_P + t), 8);
-            ptx::mbar_init(bar(SM::BAR_O + t), 1);
+            ptx::mbar_init(bar(SM::BAR_Q_FULL + t), PAIR && rank == 0 ? 2 : 1);
+            ptx::mbar_init(bar(SM::BAR_Q_EMPTY + t), AT_SOFTMAX_WARPS);
         }
+        for (int b = 0; b < NB; ++b) {
+            ptx::mbar_init(bar(SM::BAR_S + b), 1);
+            ptx::mbar_init(bar(SM::BAR_P + b), (PAIR ? 2 : 1) * (16 + 1));      // softmax warps (eight, counted twice, or all) and slot keeper of each CTA
+        }
+        ptx::mbar_init(bar(SM::BAR_O), 1);
+        ptx::mbar_init(bar(SM::BAR_O_FREE), (PAIR ? 2 : 1) * AT_SOFTMAX_WARPS);
         for (int i = 0; i < AT_PIECES; ++i) {
             ptx::mbar_init(bar(SM::BAR_PC_FULL + i), 1);
-            ptx::mbar_init(bar(SM::BAR_PC_EMPTY + i), AT_SOFTMAX_WARPS + 3);   // + issuing and query warps
+            ptx::mbar_init(bar(SM::BAR_PC_EMPTY + i), AT_SOFTMAX_WARPS + 3);   // + warps 16, 18 and 19
         }
-        for (int i = 0; i < 8; ++i) {
-            ptx::mbar_init(bar(SM::BAR_XM + i), 2);
-            ptx::mbar_init(bar(SM::BAR_XO + i), one ? 4 : 2);
-            beyond[i] = 0;
+        for (int i = 0; i < 4; ++i) {
+            ptx::mbar_init(bar(SM::BAR_XM + i), 4);
+            ptx::mbar_init(bar(SM::BAR_XO + i), 4);
+            ptx::sts_u32(sbase + SM::OFF_ASK + i * 4, 0u);
         }
-        for (int t = 0; t < 2; ++t) {
-            ptx::mbar_init(bar(SM::BAR_DRAIN + t), 1);
-            ptx::mbar_init(bar(SM::BAR_TURN + t), 1);
-        }
+        ptx::mbar_init(bar(SM::BAR_DRAIN), 1);
         ptx::fence_mbar_init();
         *abort_flag = 0;
         *n_merge = 0;
         *left_items = 0;
     }
-    if (warp == AT_MMA_WARP) {
-        ptx::tmem_alloc(ptx::smem_u32(const_cast<uint32_t *>(tmem_slot)), 512);
-        ptx::tmem_relinquish();
+    if (warp == W_MMA) {
+        const uint32_t at = ptx::smem_u32(const_cast<uint32_t *>(tmem_slot));
+        if (PAIR) { ptx::tmem_alloc_pair(at, 512); ptx::tmem_relinquish_pair(); }
+        else { ptx::tmem_alloc(at, 512); ptx::tmem_relinquish(); }
     }
-    ptx::tc_fence_before();
-    // Ends the set-up; nothing in front of it touches global memory.  Behind it the previous kernel of the stream is
-    // complete (its outputs may be this kernel's inputs, and it may share the workspace and counters), or what this kernel reads
-    // was written before the gate's call.
+    // Ends the set-up (of both CTAs: nothing goes to the peer before); nothing in front of it touches global memory.  Behind it
+    // the previous kernel of the stream is complete (its outputs may be this kernel's inputs, and it may share the workspace and
+    // counters), or what this kernel reads was written before the gate's call.
     auto begin = [&]() -> uint32_t {
         if (p.gate.word && threadIdx.x == 0) wait_gate(p.gate);
-        asm volatile("bar.sync 0, %0;" ::"n"(AT_THREADS) : "memory");
+        __syncwarp();
+        ptx::tc_fence_before();
+        if (PAIR) { ptx::cluster_arrive(); ptx::cluster_wait(); }
+        else asm volatile("bar.sync 0, %0;" ::"n"(AT_THREADS) : "memory");
         ptx::tc_fence_after();
         if (p.gate.word) ptx::fence_proxy_async_global();      // (for the TMA loads that follow)
         else previous_done();
         return *tmem_slot;                    // tensor-memory base
     };
-
-    // A wait that ran out: everybody stops at the next chance, the sticky error is raised.
+    // A wait that ran out: both CTAs stop at the next chance, the sticky error is raised.
     auto give_up = [&]() {
         *abort_flag = 1;
+        if (PAIR) ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(const_cast<int *>(abort_flag)), rank ^ 1), 1u);
         atomicExch(p.dev_error, MTV_ERR_TIMEOUT);
     };
-    // The pieces in order, for the warps that follow them (whole warp or one thread).
+    // The pieces in order, for the warps that follow them.
     auto read_piece = [&](int pi, AttnPiece &d) -> bool {
         if (!ptx::mbar_wait(bar(SM::BAR_PC_FULL + pi % AT_PIECES), (pi / AT_PIECES) & 1)) { give_up(); return false; }
         d = desc[pi % AT_PIECES];
@@ -422,118 +255,15 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
 
     if (warp >= AT_SOFTMAX_WARPS) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AT_AUX_REGS));
-    if (warp == AT_TMA_WARP) {
-        // ------------------------------------------------------------ this CTA's pieces; K and V tiles
-        const unsigned LH = (unsigned)p.n_layers * (unsigned)p.Hkv, teams = (unsigned)p.teams;
-        int chunk = 0, len = 0, g = 0;        // lengths and group counts of sequences chunk .. chunk + 31, one per lane
-        bool pad = false;
-        unsigned u = 1, pos = 0, hi = 0, off = 0;
-        int layer = 0, b = 0, head = 0;
-        bool real = false;
-        auto load_chunk = [&](int b0) {
-            chunk = b0;
-            const int at = b0 + lane;
-            len = at < p.B && real ? p.seq_lens[at] : 0;
-            g = at < p.B && len + p.T <= p.Lcap ? (len + p.T + AT_BN - 1) / AT_BN : 0;   // 0: does not fit, reported below
-        };
-        auto padded = [&](unsigned gg) { return gg == 0 ? 0u : pad ? (gg + u - 1) / u * u : gg + AT_ITEM_COST; };
+    if (warp == W_TMA) {
+        // ------------------------------------------------------------ the pair's pieces; this CTA's halves of K and V
+        PieceWalk<ITEM_COST, MERGE_COST> walk(p, team, lane);
         // The instructions of a launch come from L2 anew; this stretch runs once without lengths while the set-up goes on.
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 1) { (void)begin(); real = true; }
-            unsigned sum = 0, nz = 0;
-            for (int b0 = 0; b0 < p.B; b0 += 32) {
-                load_chunk(b0);
-                sum += __reduce_add_sync(0xffffffffu, (unsigned)g);
-                nz += __popc(__ballot_sync(0xffffffffu, g > 0));
-                if (real && blockIdx.x == 0 && p.status && b0 + lane < p.B) p.status[b0 + lane] = g > 0 ? MTV_OK : MTV_ERR_CAPACITY;
-            }
-            // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting
-            // anywhere gives most teams two pieces, that is about two groups' worth of extra start and end: whichever is
-            // shorter.
-            const unsigned u_cut = max(1u, (LH * (sum + nz * AT_ITEM_COST) + teams - 1) / teams);
-            unsigned v_head = 0;                  // length of one head's row of all sequences in the CTAs' common address space
-            pad = LH * nz <= teams;
-            u = pad ? max(1u, (LH * sum + teams - 1) / teams) : u_cut;
-            for (;;) {
-                v_head = 0;
-                for (int b0 = 0; b0 < p.B; b0 += 32) {
-                    if (b0 != chunk) load_chunk(b0);
-                    v_head += __reduce_add_sync(0xffffffffu, padded((unsigned)g));
-                }
-                if (!pad || LH * (v_head / u) <= teams) break;
-                if (++u > u_cut + 2) { pad = false; u = u_cut; }
-            }
-            const unsigned v_layer = v_head * (unsigned)p.Hkv;
-            pos = (unsigned)team * u;
-            hi = min(pos + u, v_layer * (unsigned)p.n_layers);
-            // where the run begins
-            if (pos < hi) {
-                layer = (int)(pos / v_layer);
-                unsigned rem = pos % v_layer;
-                for (int b0 = 0;; b0 += 32) {
-                    if (b0 != chunk) load_chunk(b0);
-                    const unsigned mine = padded((unsigned)g) * (unsigned)p.Hkv;
-                    unsigned incl = mine;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (lane >= o) incl += t;
-                    }
-                    const unsigned m = __ballot_sync(0xffffffffu, rem < incl);
-                    if (m) {
-                        const int at = __ffs(m) - 1;
-                        b = b0 + at;
-                        rem -= __shfl_sync(0xffffffffu, incl - mine, at);
-                        break;
-                    }
-                    rem -= __shfl_sync(0xffffffffu, incl, 31);
-                }
-                const unsigned gp = padded((unsigned)__shfl_sync(0xffffffffu, g, b - chunk));
-                head = (int)(rem / gp);
-                off = rem % gp;
-            }
+            if (pass == 1) (void)begin();
+            walk.divide(pass == 1);
         }
-        int n_part = 0;
-        // the next piece of the run (all lanes agree); false at its end
-        auto next_piece = [&](AttnPiece &d) -> bool {
-            while (pos < hi) {
-                const unsigned gg = (unsigned)__shfl_sync(0xffffffffu, g, b - chunk), gp = padded(gg);
-                const int L = __shfl_sync(0xffffffffu, len, b - chunk);
-                const unsigned end = min(gp, off + (hi - pos)), a = pos - off;
-                const unsigned r0 = min(off, gg), r1 = min(end, gg);
-                d.layer = layer; d.b = b; d.head = head; d.gb = (int)r0; d.cnt = (int)(r1 - r0); d.L = L;
-                const bool part = r1 - r0 < gg;
-                d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0);
-                d.first = (int)(a / u);
-                if (r1 > r0 && part && n_part < 2) {
-                    if (lane == 0) {
-                        AttnMerge m;
-                        m.first = d.first; m.n = (int)((a + gg - 1) / u) - m.first + 1;
-                        m.layer = layer; m.b = b; m.head = head; m.pad = 0;
-                        merges[n_part] = m;
-                        *n_merge = n_part + 1;
-                    }
-                    ++n_part;
-                }
-                pos += end - off;
-                off = 0;
-                if (++head == p.Hkv) {        // the next sequence that fits, in this layer or the next
-                    head = 0;
-                    unsigned m = __ballot_sync(0xffffffffu, g > 0) & ~(0xffffffffu >> (31 - (b - chunk)));
-                    while (!m && pos < hi) {
-                        int b0 = chunk + 32;
-                        if (b0 >= p.B) { b0 = 0; ++layer; }
-                        if (b0 != chunk) load_chunk(b0);
-                        m = __ballot_sync(0xffffffffu, g > 0);
-                    }
-                    b = chunk + (m ? __ffs(m) - 1 : 0);
-                }
-                if (r1 > r0) return true;
-            }
-            d.cnt = 0;
-            return false;
-        };
         int n_pub = 0;
         bool ok = true;
         auto publish = [&](const AttnPiece &d) {
@@ -545,127 +275,179 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             __syncwarp();
             ++n_pub;
         };
-        uint32_t seq = 0;                     // ring slots handed out so far: slot seq % ST
-        uint32_t empty_ph = 0, staged_ph = 0, staging = 0;   // bit s: phase of either barrier of slot s; it stages output rows
-        // slots [from, to) of a piece, in the order of their use
+        uint32_t seq = 0;                     // ring slots handed out so far: slot seq % STAGES
+        // halves [from, to) of a piece, in the order of their use
         auto request = [&](const AttnPiece &d, int from, int to) {
             const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
-            for (int pos_t = from; pos_t < to && ok && !*abort_flag; ++pos_t, ++seq) {
-                const uint32_t s = seq % ST;
-                if (seq >= (uint32_t)ST) {
-                    if ((staging >> s) & 1) {
-                        ok = ptx::mbar_wait(bar(SM::BAR_STAGED + s), (staged_ph >> s) & 1);
-                        staged_ph ^= 1u << s;
-                    } else {
-                        ok = ptx::mbar_wait(bar(SM::BAR_KV_EMPTY + s), (empty_ph >> s) & 1);
-                        empty_ph ^= 1u << s;
-                    }
-                    if (!ok) break;
-                }
-                const bool stage = pos_t >= 2 * d.cnt;
-                staging = (staging & ~(1u << s)) | (stage ? 1u << s : 0u);
+            for (int at = from; at < to && ok && !*abort_flag; ++at, ++seq) {
+                const uint32_t s = seq % STAGES, use = seq / STAGES;
+                if (use > 0 && !ptx::mbar_wait(bar(SM::BAR_KV_EMPTY + s), (use - 1) & 1)) { ok = false; break; }
                 if (lane == 0) {
-                    if (stage) {
-                        ptx::mbar_arrive(bar(SM::BAR_KV_FULL + s));        // the slot is the softmax warps'
-                    } else {
-                        bool is_v;
-                        int idx;
-                        tile_at(one, pos_t, d.cnt, is_v, idx);
-                        const bool tail = is_v && d.gb + idx == groups - 1 && (n_keys & 15) != 0;
-                        const uint32_t fb = bar((tail ? SM::BAR_TAIL : SM::BAR_KV_FULL) + s);
-                        ptx::mbar_arrive_expect_tx(fb, SM::TILE);
-                        ptx::tma_load_5d(sbase + SM::OFF_RING + s * SM::TILE, is_v ? &maps.v[ML == 1 ? 0 : d.layer] : &maps.k[ML == 1 ? 0 : d.layer],
-                                         fb, 0, (d.gb + idx) * AT_BN, 0, d.head, d.b);
-                    }
+                    bool is_v;
+                    int j;
+                    half_at(at, d.cnt, is_v, j);
+                    const int key = (d.gb + j) * AT_BN, l = ML == 1 ? 0 : d.layer;
+                    const bool tail = rank == 0 && is_v && d.gb + j == groups - 1 && (n_keys & 15) != 0;
+                    const uint32_t fb = bar((tail ? SM::BAR_TAIL : SM::BAR_KV_FULL) + s), dst = sbase + SM::OFF_RING + s * SM::SLOT;
+                    ptx::mbar_arrive_expect_tx(fb, SM::SLOT);
+                    if (is_v) ptx::tma_load_5d(dst, &maps.v[l], fb, 0, key, (int)rank, d.head, d.b);      // (one CTA: all columns)
+                    else ptx::tma_load_5d(dst, &maps.k[l], fb, 0, key + (int)rank * 64, 0, d.head, d.b);
                 }
                 __syncwarp();
             }
         };
         // A piece is published before the ring can block on the tiles of the one before it: the query warp looks ahead.
         AttnPiece cur, nxt;
-        bool have = next_piece(cur);
+        bool have = walk.next(cur, merges, n_merge);
         publish(cur);
         int done = 0;
-        if (have) { done = min(ring_slots(cur, one), ST); request(cur, 0, done); }
+        if (have) { done = min(2 * cur.cnt, STAGES); request(cur, 0, done); }
         while (have && ok && !*abort_flag) {
-            const bool more = next_piece(nxt);
+            const bool more = walk.next(nxt, merges, n_merge);
             publish(nxt);
-            request(cur, done, ring_slots(cur, one));
+            request(cur, done, 2 * cur.cnt);
             done = 0;
             cur = nxt;
             have = more;
         }
         if (!ok && lane == 0) give_up();
-        if (*abort_flag && lane == 0) {
-            // copies still in flight get a bounded chance to land before the shared memory goes away
-            for (uint32_t t = seq > (uint32_t)ST ? seq - ST : 0; t < seq; ++t)
-                if (!ptx::mbar_wait(bar(SM::BAR_KV_FULL + t % ST), (t / ST) & 1)) break;
+        if (*abort_flag) {
+            // copies still in flight land before the shared memory goes away (their barriers may wait for the peer as well, so
+            // this takes the time that a copy cannot take)
+            const long long t0 = clock64();
+            while (clock64() - t0 < 4000000ll) {}
         }
-    } else if (warp == AT_Q_WARP) {
-        // ------------------------------------------------------------ query tiles; V rows past the last key
-        const int n_q = one ? 1 : 2;
+    } else if (warp == W_Q) {
+        // ------------------------------------------------------------ query tiles; even CTA: V rows past the last key
         (void)begin();
-        uint32_t uses = 0, seq = 0, parity = 0;       // parity: bit s = phase of tail barrier s
+        uint32_t seq = 0, parity = 0;         // parity: bit s = phase of tail barrier s
+        AttnPiece d, e;
+        bool ok = true;
+        auto request_q = [&](int pi, const AttnPiece &x) {
+            const uint32_t t = pi & 1;
+            ok = pi < 2 || ptx::mbar_wait(bar(SM::BAR_Q_EMPTY + t), (pi / 2 - 1) & 1);
+            if (ok && lane == 0) {
+                ptx::mbar_arrive_expect_tx(bar(SM::BAR_Q_FULL + t), (uint32_t)(p.R * D * 2));
+                for (int h = 0; h < D / 64; ++h)
+                    ptx::tma_load_5d(sbase + t * SM::TILE + h * SM::HALF, &maps.q, bar(SM::BAR_Q_FULL + t), 0, x.head * p.G, blk * p.npc, h,
+                                     x.layer * p.B + x.b);
+            }
+            __syncwarp();
+        };
+        // the odd CTA's tile has landed: tell the even one
+        auto tell_q = [&](int pi) {
+            if (!PAIR || rank == 0) return;
+            ok = ok && ptx::mbar_wait(bar(SM::BAR_Q_FULL + (pi & 1)), (pi / 2) & 1);
+            if (ok && lane == 0) arrive_lead(SM::BAR_Q_FULL + (pi & 1));
+            __syncwarp();
+        };
+        bool have = read_piece(0, d) && d.cnt > 0;
+        __syncwarp();
+        if (lane == 0) free_piece(0);
+        if (have) { request_q(0, d); tell_q(0); }
+        for (int pi = 0; have && ok; ++pi) {
+            // the next piece's tile goes to the other place, as soon as the piece before this one has left it
+            if (!read_piece(pi + 1, e)) break;
+            __syncwarp();
+            if (lane == 0) free_piece(pi + 1);
+            have = e.cnt > 0;
+            if (have) { request_q(pi + 1, e); if (!ok) break; tell_q(pi + 1); if (!ok) break; }
+            const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
+            if (rank == 0 && d.gb + d.cnt == groups && (n_keys & 15) != 0) {
+                const uint32_t s = (seq + (uint32_t)v_pos(d.cnt - 1, d.cnt)) % STAGES;
+                ok = ptx::mbar_wait(bar(SM::BAR_TAIL + s), (parity >> s) & 1);
+                if (!ok) break;
+                parity ^= 1u << s;
+                clear_tail<PAIR ? 1 : D / 64>(smem + SM::OFF_RING + s * SM::SLOT, n_keys - (groups - 1) * AT_BN, lane);
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_KV_FULL + s));
+            }
+            seq += 2u * (uint32_t)d.cnt;
+            d = e;
+        }
+        if (!ok && lane == 0) give_up();
+    } else if (PAIR && warp == W_RELAY && rank == 1) {
+        // ------------------------------------------------------------ odd CTA: what has landed, V rows past the last key cleared
+        (void)begin();
+        uint32_t seq = 0;
         AttnPiece d;
         bool ok = true;
-        auto request_q = [&]() {
-            for (int t = 0; t < n_q && ok; ++t) {
-                ok = uses == 0 || ptx::mbar_wait(bar(SM::BAR_Q_EMPTY + t), (uses - 1) & 1);
-                if (ok && lane == 0) {
-                    ptx::mbar_arrive_expect_tx(bar(SM::BAR_Q_FULL + t), (uint32_t)(p.R * D * 2));
-                    for (int h = 0; h < D / 64; ++h)
-                        ptx::tma_load_5d(sbase + t * SM::TILE + h * SM::HALF, &maps.q, bar(SM::BAR_Q_FULL + t), 0, d.head * p.G,
-                                         (blk * 2 + t) * p.npc, h, d.layer * p.B + d.b);
-                }
-                __syncwarp();
-            }
-            ++uses;
-        };
         for (int pi = 0; ok && read_piece(pi, d); ++pi) {
             __syncwarp();
             if (lane == 0) free_piece(pi);
             if (d.cnt == 0) break;
-            request_q();                              // as soon as the piece before no longer needs the tiles
             const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
-            if (ok && d.gb + d.cnt == groups && (n_keys & 15) != 0) {
-                const uint32_t s = (seq + (uint32_t)v_pos(one, d.cnt - 1, d.cnt)) % ST;
-                ok = ptx::mbar_wait(bar(SM::BAR_TAIL + s), (parity >> s) & 1);
+            const bool tail = d.gb + d.cnt == groups && (n_keys & 15) != 0;
+            for (int at = 0; at < 2 * d.cnt && !*abort_flag; ++at, ++seq) {
+                const uint32_t s = seq % STAGES;
+                ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), (seq / STAGES) & 1);
                 if (!ok) break;
-                parity ^= 1u << s;
-                // only the rows up to the next multiple of 16 take part in O += P V
-                const int v0 = n_keys - (groups - 1) * AT_BN, v1 = (v0 + 15) / 16 * 16;
-                unsigned char *vt = smem + SM::OFF_RING + s * SM::TILE;
-                for (int e = v0 * 8 + lane; e < v1 * 8; e += 32)
-#pragma unroll
-                    for (int h = 0; h < D / 64; ++h)
-                        *reinterpret_cast<uint4 *>(vt + h * SM::HALF + e * 16) = make_uint4(0u, 0u, 0u, 0u);
-                ptx::fence_proxy_async();
+                if (tail && at == 2 * d.cnt - 1) {       // (the last half is V of the last group)
+                    clear_tail<PAIR ? 1 : D / 64>(smem + SM::OFF_RING + s * SM::SLOT, n_keys - (groups - 1) * AT_BN, lane);
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive_remote_release(ptx::mapa(bar(SM::BAR_KV_FULL + s), 0));
+                } else if (lane == 0) {
+                    arrive_lead(SM::BAR_KV_FULL + s);
+                }
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_KV_FULL + s));
             }
-            seq += (uint32_t)ring_slots(d, one);
         }
         if (!ok && lane == 0) give_up();
-        __syncwarp();
-        if (*abort_flag && uses > 0)
-            for (int t = 0; t < n_q; ++t) ptx::mbar_wait(bar(SM::BAR_Q_FULL + t), (uses - 1) & 1);
-    } else {
-        // ------------------------------------------------------------ MMA issuer of one stream
-        // The whole warp walks the loop, so that descriptors and addresses stay in uniform registers; one elected lane
-        // issues.  (A lane of a divergent warp has to move every operand of every MMA into uniform registers first:
-        // 85-130 cycles an MMA, more than the 64 it takes.)
-        const bool leader = ptx::elect_one();
-        const int st = warp == AT_MMA_WARP ? 0 : 1, qt = one ? 0 : st;
-        const int first = one ? st : 0, step = one ? 2 : 1;
-        const uint32_t ring_lo = ptx::desc_lo(sbase + SM::OFF_RING, 16), ring_v_lo = ptx::desc_lo(sbase + SM::OFF_RING, SM::HALF);
-        const uint32_t dq = ptx::desc_lo(sbase + qt * SM::TILE, 16);
-        const uint32_t tmem = begin();
-        const uint32_t t_s = tmem + TM_S + st * 128, t_o = tmem + TM_O + st * 128;
+    } else if (warp == W_RELAY || (PAIR && rank == 1)) {
+        // ------------------------------------------------------------ slot keeper
+        // Its word on every group goes into BAR_P, so that it is never more than a phase behind the scores.
+        (void)begin();
+        uint32_t seq = 0, base = 0;           // base: phases of the tiles of scores
+        auto wait_half = [&](int pos) {
+            const uint32_t t = seq + (uint32_t)pos;
+            return ptx::mbar_wait(bar(SM::BAR_KV_FULL + t % STAGES), (t / STAGES) & 1);
+        };
         AttnPiece d;
-        uint32_t slot0 = 0, phase0 = 0;       // ring slot and phase of the piece's first tile
-        uint32_t q_ph = 0, p_ph = 0, turn_ph = st == 0 ? 1 : 0;   // stream 0 begins: a wait for the phase before the first passes
         bool ok = true;
-        TRACE_INIT(0 + 3 * st, lane == 0);
+        auto free_slot = [&](int pos) { ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)pos) % STAGES)); };
+        for (int pi = 0; ok && read_piece(pi, d); ++pi) {
+            __syncwarp();
+            if (lane == 0) free_piece(pi);
+            if (d.cnt == 0) break;
+            int b = 0;
+            uint32_t ph = base;
+            for (int j = 0; j < d.cnt && !*abort_flag; ++j) {
+                ok = ptx::mbar_wait(bar(SM::BAR_S + b), (ph >> b) & 1);
+                if (!ok) break;
+                ph ^= 1u << b;
+                if (lane == 0) {
+                    free_slot(k_pos(j));
+                    if (j >= NB) free_slot(v_pos(j - NB, d.cnt));
+                }
+                __syncwarp();
+                if (rank == 0) {
+                    ok = wait_half(v_pos(j, d.cnt)) && (!SM::K_AHEAD || j + NB >= d.cnt || wait_half(k_pos(j + NB)));
+                    if (!ok) break;
+                }
+                if (lane == 0) arrive_lead(SM::BAR_P + b);
+                __syncwarp();
+                b = b == NB - 1 ? 0 : b + 1;
+            }
+            ok = ok && ptx::mbar_wait(bar(SM::BAR_O), pi & 1);
+            if (!ok) break;
+            if (lane == 0)
+                for (int j = max(0, d.cnt - NB); j < d.cnt; ++j) free_slot(v_pos(j, d.cnt));
+            __syncwarp();
+            base ^= s_phases(d.cnt);
+            seq += 2u * (uint32_t)d.cnt;
+        }
+        if (!ok && lane == 0) give_up();
+    } else {
+        // ------------------------------------------------------------ even CTA: MMA issuer
+        // The whole warp walks the loop, so that descriptors and addresses stay in uniform registers; one elected lane
+        // issues.  Barriers are tested while the tensor core still has MMAs queued.
+        const bool leader = ptx::elect_one();
+        const uint32_t ring_lo = ptx::desc_lo(sbase + SM::OFF_RING, 16), ring_v_lo = ptx::desc_lo(sbase + SM::OFF_RING, SM::HALF);
+        const uint32_t tmem = begin();
+        AttnPiece d;
+        uint32_t slot0 = 0, phase0 = 0;       // ring slot and phase of the piece's first half group
+        uint32_t p_base = 0;
+        bool ok = true;
         for (int pi = 0; ok && read_piece(pi, d); ++pi) {
             __syncwarp();
             if (lane == 0) free_piece(pi);
@@ -673,76 +455,54 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             if (cnt == 0) break;
             const int last_valid = d.L + p.T - (d.gb + cnt - 1) * AT_BN;       // keys of the piece's last group (or more than 128)
             const int last_steps = __shfl_sync(0xffffffffu, min(8, (last_valid + 15) / 16), 0);
-            // ring slot and phase of the tile at a position of the piece
-            auto tile = [&](int pos, uint32_t &s, uint32_t &ph) {
-                const uint32_t t = slot0 + (uint32_t)pos;
-                s = t % ST;
-                ph = (phase0 + t / ST) & 1;
+            const uint32_t dq = ptx::desc_lo(sbase + (pi & 1) * SM::TILE, 16);
+            auto issue_s = [&](int kk, uint32_t s, int b) {
+                const uint32_t oq = (kk / 4) * (SM::HALF >> 4) + (kk % 4) * 2, o_k = (kk / 4) * (SM::K_HALF >> 4) + (kk % 4) * 2;
+                const uint32_t t_d = tmem + TM_S + b * 128, dk = ring_lo + s * (SM::SLOT >> 4) + o_k;
+                if (PAIR) ptx::mma_pair_ss_elect(t_d, dq + oq, dk, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
+                else ptx::mma_ss_elect(t_d, dq + oq, dk, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
             };
-            auto my_turn = [&]() { ok = ok && ptx::mbar_wait(bar(SM::BAR_TURN + st), turn_ph); turn_ph ^= 1; };
-            auto pass_turn = [&]() { if (leader) ptx::mbar_arrive(bar(SM::BAR_TURN + (st ^ 1))); };
-            auto wait_k = [&](int j, uint32_t &s) {
-                uint32_t ph;
-                tile(k_pos(one, j), s, ph);
-                ok = ok && ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph);
+            auto commit = [&](int i) {
+                if (PAIR) ptx::tc_commit_pair_mask_elect(bar(i), 3, leader);
+                else ptx::tc_commit_elect(bar(i), leader);
+            };
+            ok = ptx::mbar_wait(bar(SM::BAR_Q_FULL + (pi & 1)), (pi / 2) & 1);
+            uint32_t s = slot0, ph_kv = phase0;
+            auto next_slot = [&]() { if (++s == STAGES) { s = 0; ph_kv ^= 1; } };
+            for (int j = 0; j < min(NB, cnt) && ok; ++j) {
+                ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph_kv);
                 ptx::tc_fence_after();
-            };
-            // S of group j (its K tile, in slot s, has landed).  The other stream is told shortly before the end: its
-            // first MMA then follows without a gap.
-            auto issue_s = [&](int j, uint32_t s) {
-                const uint32_t dk = ring_lo + s * (SM::TILE >> 4);
-                const uint32_t idesc = AT_IDESC | ((uint32_t)(2 * (j == cnt - 1 ? last_steps : 8)) << 17);   // N = keys rounded up to 16
 #pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) {
-                    constexpr uint32_t half = SM::HALF >> 4;
-                    const uint32_t o = (kk / 4) * half + (kk % 4) * 2;
-                    ptx::mma_ss_elect(t_s, dq + o, dk + o, ptx::DESC_HI, idesc, kk > 0, leader);
-                    if (kk == D / 16 - 3) pass_turn();
-                }
-                ptx::tc_commit_elect(bar(SM::BAR_S + st), leader);
-            };
-            uint32_t ks = 0;
-            ok = ptx::mbar_wait(bar(SM::BAR_Q_FULL + qt), q_ph);
-            q_ph ^= 1;
-            // Both streams take cnt / step + 1 turns (rounded up), whether they have something to issue or not.
-            const int turns = (cnt + step - 1) / step + 1;
-            if (first < cnt) wait_k(first, ks);
-            my_turn();
-            if (ok && first < cnt) issue_s(first, ks);
-            else pass_turn();
-            for (int i = 1; i < turns && ok && !*abort_flag; ++i) {
-                const int j = first + (i - 1) * step;
-                if (j >= cnt) { my_turn(); pass_turn(); continue; }
-                const bool more = j + step < cnt;
-                uint32_t s, ph;
-                tile(v_pos(one, j, cnt), s, ph);
-                TRACE();
-                if (more) wait_k(j + step, ks);
-                ok = ok && ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph);
-                TRACE();
-                ok = ok && ptx::mbar_wait(bar(SM::BAR_P + st), p_ph);
-                TRACE();
-                my_turn();
+                for (int kk = 0; kk < D / 16; ++kk) issue_s(kk, s, j);
+                commit(SM::BAR_S + j);
+                next_slot();
+            }
+            ok = ok && (pi == 0 || ptx::mbar_wait(bar(SM::BAR_O_FREE), (pi - 1) & 1));
+            int b = 0;
+            uint32_t ph_p = p_base;
+            bool go = false;              // all that the group's MMAs wait for is there
+            for (int j = 0; j < cnt; ++j) {
+                if (!go) ok = ok && ptx::mbar_wait(bar(SM::BAR_P + b), (ph_p >> b) & 1);
                 if (!ok) break;
-                TRACE();
+                ph_p ^= 1u << b;
                 ptx::tc_fence_after();
-                const uint32_t dv = ring_v_lo + s * (SM::TILE >> 4);
-                constexpr uint32_t idesc = AT_IDESC | AT_B_NMAJOR | ((uint32_t)(D / 8) << 17);
-                const int steps = j == cnt - 1 ? last_steps : 8;
+                const uint32_t dv = ring_v_lo + s * (SM::SLOT >> 4), t_p = tmem + TM_S + b * 128;
                 // the A operand of sixteen keys: where P lies (see TM_S)
                 auto issue_pv = [&](int kk, uint32_t col, bool accumulate) {
-                    ptx::mma_ts_elect(t_o, t_s + (kk / 4) * 64 + col, dv + kk * 128, ptx::DESC_HI, idesc, accumulate, leader);
+                    const uint32_t t_a = t_p + (kk / 4) * 64 + col;
+                    if (PAIR) ptx::mma_pair_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
+                    else ptx::mma_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
                 };
-                if (two_terms<D>(i - 1)) {
-                    if (steps == 8 && D == 64) {
+                const int steps = j == cnt - 1 ? last_steps : 8;
+                if (two_terms<PAIR>(j)) {
+                    if (!PAIR && steps == 8) {
 #pragma unroll
-                        for (int kk = 0; kk < 16; ++kk)
-                            issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > first || kk > 0);
+                        for (int kk = 0; kk < 16; ++kk) issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > 0 || kk > 0);
                     } else {
 #pragma unroll 1
                         for (int kk = 0; kk < 2 * steps; ++kk) {
                             const int k = kk >> 1;
-                            issue_pv(k, k / 2 % 2 * 32 + k % 2 * 8 + kk % 2 * 16, j > first || kk > 0);
+                            issue_pv(k, k / 2 % 2 * 32 + k % 2 * 8 + kk % 2 * 16, j > 0 || kk > 0);
                         }
                     }
                 } else if (steps == 8) {
@@ -752,110 +512,130 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
 #pragma unroll 1
                     for (int kk = 0; kk < steps; ++kk) issue_pv(kk, kk % 4 * 8, true);
                 }
-                p_ph ^= 1;
-                TRACE();
+                next_slot();
+                const bool more = j + NB < cnt;
+                const int bn = b == NB - 1 ? 0 : b + 1;
+                if (more && !SM::K_AHEAD) ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph_kv);
+                if (!ok) break;
                 if (more) {
-                    issue_s(j + step, ks);
+#pragma unroll
+                    for (int kk = 0; kk < D / 16; ++kk) {
+                        issue_s(kk, s, b);
+                        if (kk == D / 16 - 4) go = __all_sync(0xffffffffu, ptx::mbar_test(bar(SM::BAR_P + bn), (ph_p >> bn) & 1));
+                    }
+                    next_slot();
                 } else {
-                    pass_turn();
-                    ptx::tc_commit_elect(bar(SM::BAR_O + st), leader);
+                    go = false;
                 }
+                commit(j == cnt - 1 ? SM::BAR_O : SM::BAR_S + b);
+                b = bn;
             }
-            const uint32_t t = slot0 + (uint32_t)__shfl_sync(0xffffffffu, ring_slots(d, one), 0);
-            phase0 += t / ST;
-            slot0 = t % ST;
+            p_base ^= p_phases(cnt);
+            slot0 = s;
+            phase0 = ph_kv;
         }
         if (!ok && lane == 0) give_up();
         __syncwarp();
         if (*abort_flag) {                // let what was issued finish
-            ptx::tc_commit_elect(bar(SM::BAR_DRAIN + st), leader);
-            ptx::mbar_wait(bar(SM::BAR_DRAIN + st), 0);
+            if (PAIR) ptx::tc_commit_pair_mask_elect(bar(SM::BAR_DRAIN), 1, leader);
+            else ptx::tc_commit_elect(bar(SM::BAR_DRAIN), leader);
+            ptx::mbar_wait(bar(SM::BAR_DRAIN), 0);
         }
         __syncwarp();
     }
     } else {
         // ------------------------------------------------------------ softmax warps
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(AT_SOFTMAX_REGS));
-        // Thread (row, hf) of stream st: query row `row`, columns [64 hf, 64 hf + 64) of every group of the stream.
-        const int qd = warp & 3, hf = (warp >> 2) & 1, st = warp >> 3;
+        // Thread (row, hf) of set e: query row `row`, columns [64 hf, 64 hf + 64) of groups 1, 3, .. (e = 1) or 2, 4, .. (e = 0).
+        const int qd = warp & 3, hf = (warp >> 2) & 1, e = warp >> 3;
         const int row = qd * 32 + lane;
-        const int tile = one ? 0 : st;
-        const int step = one ? 2 : 1, first = one ? st : 0;
         // 128 bits: the row's node sees tree row i
-        const uint32_t *anc = reinterpret_cast<const uint32_t *>(p.anc + ((blk * 2 + tile) * p.npc + node_in_tile(p, row)) * 2);
-        const bool mine = out_row(p, blk, tile, row) >= 0;
+        const uint32_t *anc = reinterpret_cast<const uint32_t *>(p.anc + (blk * p.npc + node_in_tile(p, row)) * 2);
+        const bool mine = out_row(p, blk, row) >= 0;
         auto anc_word = [&](int w) -> uint32_t {
             if (w < 0) return 0xffffffffu;     // prefix rows are visible to every node
             return w < 4 && mine ? anc[w] : 0u;    // past the tree rows: nothing
         };
         const uint32_t tmem = begin();
         const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16);
-        const uint32_t t_s = lane_base + TM_S + st * 128 + hf * 64, t_o = lane_base + TM_O + st * 128;
-        // (addresses in 32 bits and formed where they are used, phases in one word: the loop below has no register to spare)
-        auto bar_s = [&]() { return bar(SM::BAR_S + st); };
-        auto x_at = [&](int s, int h) { return sbase + SM::OFF_ML + (uint32_t)((s * 2 + h) * 128 + row) * 4u; };   // [stream][half][row]
-        const uint32_t beyond_at = sbase + SM::OFF_MISC + 76u + (uint32_t)(st * 4 + qd) * 4u;
+        const uint32_t t_s0 = lane_base + TM_S + hf * 64;                 // + 128 b: this half of tile b of scores
+        const uint32_t t_o = lane_base + TM_O + (e * 2 + hf) * (D / 4);        // this thread's columns of O
+        auto x_at = [&](int s, int h) { return sbase + SM::OFF_X + (uint32_t)((s * 2 + h) * 128 + row) * 4u; };   // [set][half][row]
+        const uint32_t ask_at = sbase + SM::OFF_ASK + (uint32_t)qd * 4u;
         if (lane < 2) p.left[((unsigned)blockIdx.x * 2 + lane) * AT_SOFTMAX_WARPS + warp] = 0;      // (released with the arrivals)
         constexpr uint32_t hidden = NEG ? 0x7f800000u : 0xff800000u;   // times the scale: -inf
-        uint32_t phases = 0, seq = 0;             // bit 0: scores, 1: O, 2 and 3: the two exchanges
-        auto phase = [&](int i) { return (phases >> i) & 1u; };
+        uint32_t phases = 0;                      // bit 0: exchange of references, 1: of results, 4-6: the tiles of scores
         bool ok = true;
-        TRACE_INIT(1 + st, qd == 0 && hf == 0 && lane == 0);
         float m_used = -INFINITY, l = 0.f;
-        bool begun = false;                    // the stream's O holds something of this piece
-        auto meet = [&]() {                    // the two warps of these rows
+        auto meet = [&]() {                       // the four warps of these rows
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XM + st * 4 + qd));
-            if (!ptx::mbar_wait(bar(SM::BAR_XM + st * 4 + qd), phase(2))) ok = false;
-            phases ^= 4;
+            if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XM + qd));
+            if (!ptx::mbar_wait(bar(SM::BAR_XM + qd), phases & 1)) ok = false;
+            phases ^= 1;
         };
-        // The reference becomes max(both halves' mx) where `is_first` or that exceeds it; O and l (and P, if already written
-        // against the old one) follow.  The two warps of the rows do this together.
-        auto move_reference = [&](float mx, bool is_first, bool p_written) {
-            ptx::sts_f32(x_at(st, hf), mx);
+        auto parity_s = [&](int j, int b) { return ((phases >> (4 + b)) ^ (uint32_t)(j / NB)) & 1u; };   // of the scores of group j
+        // A warp whose exponents do not fit the reference has not written its P of group `at` yet: O += P V waits for it in all
+        // groups from there on, so that all four warps come to wait for scores (or for O) and meet here; next: the group that
+        // this warp is to take next (a warp that asks: at).  What is there then: O with all groups before the earliest one that
+        // is missing (its MMAs are waited for), and P of groups behind that one, which follow the reference like O does.
+        auto move_reference = [&](float mx, int next, bool asks) {
+            meet();                               // (nobody is still at what was exchanged before)
+            ptx::sts_f32(x_at(e, hf), mx);
+            if (lane == 0) ptx::sts_u32(sbase + SM::OFF_AT + (uint32_t)(qd * 4 + e * 2 + hf) * 4u, asks ? (uint32_t)next : 0x7fffffffu);
             meet();
-            const float both = ceilf(fmaxf(mx, ptx::lds_f32(x_at(st, hf ^ 1))));
-            const float m_new = is_first ? both : fmaxf(m_used, both);
-            const bool need = !is_first && m_new != m_used && m_used != -INFINITY;
+            int first = 0x7fffffff;               // (not group 0, which always fits)
+            float m_new = m_used;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                first = min(first, (int)ptx::lds_u32(sbase + SM::OFF_AT + (uint32_t)(qd * 4 + i) * 4u));
+                m_new = fmaxf(m_new, ceilf(ptx::lds_f32(x_at(i >> 1, i & 1))));
+            }
+            const int b_done = (first - 1) % NB;  // O += P V of the group before: the phase behind its scores
+            if (!ptx::mbar_wait(bar(SM::BAR_S + b_done), parity_s(first - 1 + NB, b_done))) ok = false;
+            ptx::tc_fence_after();
+            const bool need = m_new != m_used && m_used != -INFINITY;
             if (__any_sync(0xffffffffu, need)) {
                 const float alpha = need ? ex2(m_used - m_new) : 1.f;
                 uint32_t x[16];
 #pragma unroll 1
-                for (int c = 0; p_written && c < 4; ++c) {       // both terms (a power of two: exact)
-                    ptx::tmem_ld16(t_s + c * 16, x);
-                    ptx::tmem_ld_wait_for16(x);
+                for (int j = next - 4; j < next; j += 2) {    // (a power of two: exact)
+                    if (j < first) continue;
+                    const uint32_t t_p = t_s0 + (uint32_t)(j % NB) * 128;
+#pragma unroll 1
+                    for (int c = 0; c < (PAIR ? 2 : 4); ++c) {        // (both terms)
+                        ptx::tmem_ld16(t_p + c * 16, x);
+                        ptx::tmem_ld_wait_for16(x);
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) x[e] = pack2_bf16(bf16_lo(x[e]) * alpha, bf16_hi(x[e]) * alpha);
-                    ptx::tmem_st16(t_s + c * 16, x);
+                        for (int i = 0; i < 16; ++i) x[i] = pack2_bf16(bf16_lo(x[i]) * alpha, bf16_hi(x[i]) * alpha);
+                        ptx::tmem_st16(t_p + c * 16, x);
+                    }
                 }
 #pragma unroll 1
-                for (int c = 0; begun && c < D / 32; ++c) {      // this half's columns of O; the stream's earlier MMAs are complete
-                    ptx::tmem_ld16(t_o + hf * (D / 2) + c * 16, x);
+                for (int c = 0; c < D / 64; ++c) {
+                    ptx::tmem_ld16(t_o + c * 16, x);
                     ptx::tmem_ld_wait_for16(x);
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) x[e] = __float_as_uint(__uint_as_float(x[e]) * alpha);
-                    ptx::tmem_st16(t_o + hf * (D / 2) + c * 16, x);
+                    for (int i = 0; i < 16; ++i) x[i] = __float_as_uint(__uint_as_float(x[i]) * alpha);
+                    ptx::tmem_st16(t_o + c * 16, x);
                 }
                 ptx::tmem_st_wait();
                 l *= alpha;
             }
             m_used = m_new;
-            if (is_first) return;                  // (the values exchanged are not written again before both warps' P is used)
-            if (lane == 0) ptx::sts_u32(beyond_at, 0u);
+            if (lane == 0) ptx::sts_u32(ask_at, 0u);
             ptx::tc_fence_before();
             meet();
             ptx::tc_fence_after();
         };
-        // Waits for the tensor core; meanwhile the other warp of these rows may ask to move the reference.  If it asks for the
-        // very group that is waited for (complete between the two tests), this warp's P of that group does not exist yet: the
-        // barrier, tested again behind the flag, then says so, the group is taken first, and the question is met at the next
-        // wait.  Otherwise the asked-for group is the one whose P this warp has written, and the barrier cannot complete
-        // before they have met.
-        auto wait_tc = [&](uint32_t b, uint32_t parity) {
+        // Waits for the tensor core; meanwhile another warp of these rows may ask to move the reference.  What is waited for can be
+        // complete all the same: the barrier, tested again behind the question, says so, and the question is met at the next
+        // wait.  (The scores of the group at which a warp asks, and of all before it, are complete when it asks.)
+        auto wait_tc = [&](uint32_t b, uint32_t parity, int next) {
             const long long t0 = clock64();
             while (!ptx::mbar_try_wait(b, parity)) {
-                if (ptx::lds_u32(beyond_at)) {
-                    if (!ptx::mbar_try_wait(b, parity)) move_reference(-INFINITY, false, true);
+                if (ptx::lds_u32(ask_at)) {
+                    if (!ptx::mbar_try_wait(b, parity)) move_reference(-INFINITY, next, false);
+                    else break;
                     continue;
                 }
                 if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { ok = false; return; }
@@ -869,78 +649,54 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             const int a_first = d.gb * AT_BN + hf * 64 - d.L;      // tree row of this half's first column in the first group
             m_used = -INFINITY;
             l = 0.f;
-            begun = false;
-            const bool releases = qd == 0 && hf == 0 && lane == 0;
-            if (first >= cnt && releases) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + tile));
-            // These scores are complete: this stream is done with their K tile and, the MMAs before them being complete too, with
-            // the V tile of its previous group.
-            auto scores_done = [&](int j) {
-                phases ^= 1;
-                TRACE();
-                ptx::tc_fence_after();
-                if (releases) {
-                    ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)k_pos(one, j)) % ST));
-                    if (j >= step) ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)v_pos(one, j - step, cnt)) % ST));
-                    if (j + step >= cnt) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + tile));
-                }
-            };
-            auto p_done = [&]() {
+            if (pi > 0) {                      // (the results of the piece before have been read)
+                if (!ptx::mbar_wait(bar(SM::BAR_XO + qd), (phases >> 1) & 1)) { ok = false; break; }
+                phases ^= 2;
+            }
+            auto p_done = [&](int b, uint32_t count) {
                 ptx::tmem_st_wait();
                 ptx::tc_fence_before();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_P + st));
-                begun = true;
-                TRACE();
+                if (lane == 0) arrive_lead(SM::BAR_P + b, count);
             };
-            constexpr int DEGREE = D == 128 ? 3 : 4;
             const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
-            // ---- the first group: its maximum, then its P in two terms, a quarter at a time (the scores are loaded twice, which
-            //      costs less than the registers of all of them in two terms)
-            if (first < cnt) {
-                if (!ptx::mbar_wait(bar_s(), phase(0))) { ok = false; break; }
-                scores_done(first);
-                const int a0 = a_first + first * AT_BN;      // tree row of this half's first column
-                auto quarter = [&](uint32_t (&q)[32], int c) {
-                    ptx::tmem_ld32(t_s + 32 * c, q);
-                    ptx::tmem_ld_wait_for(q);
-                    if (a0 + 64 > 0) {       // bit e of vis is column e (see below)
-                        const uint32_t vis = __funnelshift_r(anc_word((a0 >> 5) + c), anc_word((a0 >> 5) + c + 1), a0 & 31);
+            // ---- the first group, all four threads of a row on a quarter of it each: its maximum, then its P in two terms
+            {
+                if (!ptx::mbar_wait(bar(SM::BAR_S), parity_s(0, 0))) { ok = false; break; }
+                ptx::tc_fence_after();
+                const uint32_t t_q = t_s0 + e * 32;
+                const int a0 = a_first + e * 32;         // tree row of the quarter's first column
+                uint32_t q[32], pk[32];
+                ptx::tmem_ld32(t_q, q);
+                ptx::tmem_ld_wait_for(q);
+                if (a0 + 32 > 0) {                       // bit i of vis is column i (see below)
+                    const uint32_t vis = __funnelshift_r(anc_word(a0 >> 5), anc_word((a0 >> 5) + 1), a0 & 31);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (!((vis >> e) & 1u)) q[e] = hidden;
-                    }
-                };
-                uint32_t q[32], pk[16], rest[16];
-                float mx = -INFINITY;
-#pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    quarter(q, c);
-                    mx = fmaxf(mx, max_quarter<NEG>(q, p.scale_log2));
+                    for (int i = 0; i < 32; ++i)
+                        if (!((vis >> i) & 1u)) q[i] = hidden;
                 }
-                move_reference(mx, true, false);
+                ptx::sts_f32(x_at(e, hf), max_quarter<NEG>(q, p.scale_log2));
+                meet();
                 if (!ok) break;
+                m_used = ceilf(fmaxf(fmaxf(ptx::lds_f32(x_at(0, 0)), ptx::lds_f32(x_at(0, 1))), fmaxf(ptx::lds_f32(x_at(1, 0)), ptx::lds_f32(x_at(1, 1)))));
                 const float m_eff = m_used == -INFINITY ? 0.f : m_used;
                 float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-                float top = -INFINITY;
-#pragma unroll 1
-                for (int c = 0; c < 2; ++c) {
-                    quarter(q, c);
-                    exp_quarter<DEGREE, true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, rest, top);
-                    ptx::tmem_st16(t_s + 32 * c, pk);
-                    ptx::tmem_st16(t_s + 32 * c + 16, rest);
-                }
-                l = top != top ? top : (la.x + la.y) + (lb.x + lb.y);      // (no exponent is above 0 here)
-                p_done();
+                exp_quarter<true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, pk + 16);
+                ptx::tmem_st32(t_q, pk);
+                l = (la.x + la.y) + (lb.x + lb.y);
+                p_done(0, 1);
             }
-            for (int j = first + step; j < cnt; j += step) {
+            int b = e == 0 ? 2 : 1;
+            for (int j = e == 0 ? 2 : 1; j < cnt; j += 2, b = b == 0 ? NB - 1 : b - 1) {
                 float sum;
                 bool asked = false;
+                const uint32_t t_s = t_s0 + (uint32_t)b * 128;
 #pragma unroll 1
                 for (;;) {
                     if (!asked) {
-                        wait_tc(bar_s(), phase(0));
+                        wait_tc(bar(SM::BAR_S + b), parity_s(j, b), j);
                         if (!ok) break;
-                        scores_done(j);
+                        ptx::tc_fence_after();
                     }
                     uint32_t qa[32], qb[32];
                     ptx::tmem_ld32(t_s, qa);
@@ -949,34 +705,32 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     ptx::tmem_ld_wait_for(qb);
                     const int a0 = a_first + j * AT_BN;      // tree row of this half's first column
                     if (a0 + 64 > 0) {
-                        // the half overlaps the tree rows or the end of the cache: bit e of vis is column e of a quarter
+                        // the half overlaps the tree rows or the end of the cache: bit i of va is column i of a quarter
                         const int w = a0 >> 5, sh = a0 & 31;     // floor division
                         const uint32_t w1 = anc_word(w + 1);
                         const uint32_t va = __funnelshift_r(anc_word(w), w1, sh), vb = __funnelshift_r(w1, anc_word(w + 2), sh);
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            if (!((va >> e) & 1u)) qa[e] = hidden;
-                            if (!((vb >> e) & 1u)) qb[e] = hidden;
+                        for (int i = 0; i < 32; ++i) {
+                            if (!((va >> i) & 1u)) qa[i] = hidden;
+                            if (!((vb >> i) & 1u)) qb[i] = hidden;
                         }
                     }
-                    if (asked) {      // (by a NaN, too, which the row's sum then has to show)
+                    if (asked) {
                         const float mx = fmaxf(max_quarter<NEG>(qa, p.scale_log2), max_quarter<NEG>(qb, p.scale_log2));
-                        move_reference(mx > m_used + 16.f ? mx : -INFINITY, false, false);
+                        move_reference(mx > m_used + 16.f ? mx : -INFINITY, j, true);
                     }
                     const float m_eff = m_used == -INFINITY ? 0.f : m_used;
                     const float2 nm2 = make_float2(-m_eff, -m_eff);
                     float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
-                    float top = -INFINITY;
                     // (rows that belong to nobody may hold anything)
                     auto fits = [&]() {
                         sum = (la.x + la.y) + (lb.x + lb.y);
-                        if (asked && top != top) sum = top;
-                        return asked || !__any_sync(0xffffffffu, mine && (sum > AT_SUM_LIMIT || !(top <= 32.f)));
+                        return asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT);
                     };
-                    if constexpr (two_terms<D>(1)) {
+                    if constexpr (two_terms<PAIR>(1)) {
                         uint32_t pa[16], pb[16], ra[16], rb[16];
-                        exp_quarter<DEGREE, true>(qa, sc2, nm2, la, lb, pa, ra, top);
-                        exp_quarter<DEGREE, true>(qb, sc2, nm2, la, lb, pb, rb, top);
+                        exp_quarter<true>(qa, sc2, nm2, la, lb, pa, ra);
+                        exp_quarter<true>(qb, sc2, nm2, la, lb, pb, rb);
                         if (fits()) {
                             ptx::tmem_st16(t_s, pa);
                             ptx::tmem_st16(t_s + 16, ra);
@@ -985,133 +739,93 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                             break;
                         }
                     } else {
-                        uint32_t pk[32];
-                        exp_quarter<DEGREE, false>(qa, sc2, nm2, la, lb, pk, nullptr, top);
-                        exp_quarter<DEGREE, false>(qb, sc2, nm2, la, lb, pk + 16, nullptr, top);
+                        uint32_t pw[32];
+                        exp_quarter<false>(qa, sc2, nm2, la, lb, pw, nullptr);
+                        exp_quarter<false>(qb, sc2, nm2, la, lb, pw + 16, nullptr);
                         if (fits()) {
-                            ptx::tmem_st32(t_s, pk);
+                            ptx::tmem_st32(t_s, pw);
                             break;
                         }
                     }
-                    // rare: ask the other warp of these rows to come and move the reference, start over
+                    // rare: ask the other warps of these rows to come and move the reference, start over
                     asked = true;
-                    if (lane == 0) ptx::sts_u32(beyond_at, 1u);
+                    if (lane == 0) ptx::sts_u32(ask_at, 1u);
                 }
                 if (!ok) break;
                 l += sum;
-                p_done();
+                p_done(b, 2);
             }
-            // ---- the stream's O of this piece
-            const bool ran = first < cnt;       // (a one-tile piece of a single group has no second stream)
-            if (ok && ran) {
-                wait_tc(bar(SM::BAR_O + st), phase(1));
-                phases ^= 2;
-                if (releases) {
-                    const int jl = one ? cnt - 1 - ((cnt - 1 - st) & 1) : cnt - 1;    // the stream's last group
-                    ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)v_pos(one, jl, cnt)) % ST));
-                }
-                ptx::tc_fence_after();
-            }
+            // ---- O of this piece
+            if (ok) wait_tc(bar(SM::BAR_O), pi & 1, cnt + ((cnt ^ e) & 1));
             if (!ok) break;
+            ptx::tc_fence_after();
+            phases ^= s_phases(cnt) << 4;
             const bool partial = d.flags & PIECE_PARTIAL;
             const int slab = d.flags & PIECE_HEAD ? 1 : 0;
-            // ---- the sums of a row's threads: l of the two halves and, in a one-tile piece, of the two streams:
-            //      O = (w0 O0 + w1 O1) / (w0 l0 + w1 l1) with w_t = exp2(m_t - m)
+            // ---- the row sums of the row's four threads
             auto gather = [&]() {
-                ptx::tc_fence_before();
                 __syncwarp();
-                const uint32_t bar_xo = bar(SM::BAR_XO + (one ? qd : st * 4 + qd));
-                if (lane == 0) ptx::mbar_arrive(bar_xo);
-                if (!ptx::mbar_wait(bar_xo, phase(3))) ok = false;
-                phases ^= 8;
-                ptx::tc_fence_after();
+                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XO + qd));
             };
-            volatile float *x_m = reinterpret_cast<volatile float *>(smem + SM::TILE);   // [stream][row]: the unused query tile
-            ptx::sts_f32(x_at(st, hf), l);
-            if (one && hf == 0) x_m[st * 128 + row] = m_used;
+            ptx::sts_f32(x_at(e, hf), l);
             gather();
-            float l_all = l + ptx::lds_f32(x_at(st, hf ^ 1)), m_all = m_used, w_own = 1.f, w_oth = 0.f;
-            if (one) {
-                const float l_oth = ptx::lds_f32(x_at(st ^ 1, 0)) + ptx::lds_f32(x_at(st ^ 1, 1));
-                const float m_oth = x_m[(st ^ 1) * 128 + row];
-                m_all = fmaxf(m_used, m_oth);
-                w_own = m_used == -INFINITY ? 0.f : ex2(m_used - m_all);
-                w_oth = m_oth == -INFINITY ? 0.f : ex2(m_oth - m_all);
-                l_all = w_own * l_all + w_oth * l_oth;
-            }
+            uint32_t o[D / 4];
+            if constexpr (D == 128) ptx::tmem_ld32(t_o, o);
+            else ptx::tmem_ld16(t_o, o);
+            if (!ptx::mbar_wait(bar(SM::BAR_XO + qd), (phases >> 1) & 1)) ok = false;
+            phases ^= 2;
             if (!ok) break;
+            const float l_all = (ptx::lds_f32(x_at(0, 0)) + ptx::lds_f32(x_at(0, 1))) + (ptx::lds_f32(x_at(1, 0)) + ptx::lds_f32(x_at(1, 1)));
+            gather();                             // the exchanged values have been read: the next piece may overwrite them (and waits)
             const float inv_l = l_all == 0.f ? 0.f : 1.f / l_all;     // (NaN stays NaN)
-            w_own *= inv_l;
-            w_oth *= inv_l;
-            // this thread's columns: a half of them, a quarter in a one-tile piece.  Partial results go to the workspace, whose
-            // layout suits them; output rows are staged in a ring slot (each warp for itself, 16-byte chunks swizzled)
-            // and leave as runs of 64 or 128 bytes: a thread storing its own row straight to memory took 6 k cycles.
-            const bool other_ran = one && (st == 1 || cnt > 1);
-            const int n_col = one ? D / 4 : D / 2, c_begin = one ? (st * 2 + hf) * n_col : hf * n_col;
-            const uint32_t sq = seq + 2u * (uint32_t)cnt + (one ? 0 : st), slot = sq % ST;
-            const uint32_t n_ch = (uint32_t)n_col / 8, rowb = n_ch * 16;          // chunks and bytes of a row's part
-            unsigned char *stage = smem + SM::OFF_RING + slot * SM::TILE + (uint32_t)(one ? warp : warp & 7) * 32u * rowb;
-            if (!partial && !ptx::mbar_wait(bar(SM::BAR_KV_FULL + slot), (sq / ST) & 1)) { ok = false; break; }
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_col; c0 += 16) {
-                uint32_t o[16];
-                float v[16];
+            if constexpr (D == 128) ptx::tmem_ld_wait_for(o);
+            else ptx::tmem_ld_wait_for16(o);
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_lead(SM::BAR_O_FREE);
 #pragma unroll
-                for (int e = 0; e < 16; ++e) v[e] = 0.f;
-                if (ran) {
-                    ptx::tmem_ld16(t_o + c_begin + c0, o);
-                    ptx::tmem_ld_wait_for16(o);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = __uint_as_float(o[e]) * w_own;
-                }
-                if (other_ran) {
-                    ptx::tmem_ld16(lane_base + TM_O + (st ^ 1) * 128 + c_begin + c0, o);
-                    ptx::tmem_ld_wait_for16(o);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = fmaf(__uint_as_float(o[e]), w_oth, v[e]);
-                }
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const uint32_t ch = (uint32_t)c0 / 8 + e;
-                    if (!partial) {
-                        *reinterpret_cast<uint4 *>(stage + lane * rowb + ((ch ^ (lane & (n_ch - 1))) << 4)) =
-                            make_uint4(pack2_bf16(v[8 * e], v[8 * e + 1]), pack2_bf16(v[8 * e + 2], v[8 * e + 3]),
-                                       pack2_bf16(v[8 * e + 4], v[8 * e + 5]), pack2_bf16(v[8 * e + 6], v[8 * e + 7]));
-                    } else if (mine) {
-#pragma unroll
-                        for (int q = 0; q < 2; ++q)
-                            *slab_o<D>(p, blockIdx.x, slab, tile, row, c_begin / 4 + 2 * ch + q) =
-                                make_uint4(__float_as_uint(v[8 * e + 4 * q]), __float_as_uint(v[8 * e + 4 * q + 1]),
-                                           __float_as_uint(v[8 * e + 4 * q + 2]), __float_as_uint(v[8 * e + 4 * q + 3]));
-                    }
-                }
-            }
-            if (!partial) {
-                __syncwarp();
-                const uint32_t sh = n_ch == 8 ? 3 : n_ch == 4 ? 2 : 1, ch = lane & (n_ch - 1);     // n_ch lanes store a row's part
-                uint4 *dst = item_out<D>(p, d.layer, d.b, d.head) + c_begin / 8 + ch;
-#pragma unroll 2
-                for (uint32_t r = lane >> sh; r < 32; r += 32u >> sh) {
-                    const uint4 x = *reinterpret_cast<const uint4 *>(stage + r * rowb + ((ch ^ (r & (n_ch - 1))) << 4));
-                    const int o = out_row(p, blk, tile, qd * 32 + r);
-                    if (o >= 0) dst[o * (D / 8)] = x;
-                }
-                ptx::fence_proxy_async();         // (the next tile comes into the slot through the async proxy)
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_STAGED + slot));
-            }
+            for (int i = 0; i < D / 4; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv_l);
             if (partial) {
-                if (mine && hf == 0 && (!one || st == 0)) *slab_ml(p, blockIdx.x, slab, tile, row) = make_float2(m_all, l_all);
+                // to the workspace, whose layout suits a thread per row
+                if (mine) {
+#pragma unroll
+                    for (int c = 0; c < D / 16; ++c)
+                        *slab_o<D>(p, blockIdx.x, slab, row, (e * 2 + hf) * (D / 16) + c) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+                    if (hf == 0 && e == 0) *slab_ml(p, blockIdx.x, slab, row) = make_float2(m_used, l_all);
+                }
                 // this warp's part is written: tell those that share the item (each warp counts for itself)
                 __syncwarp();
-                if (lane == 0) {
-                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrive + d.first * p.n_blk + blk) : "memory");
+                if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrive + d.first * p.n_blk + blk) : "memory");
+            } else {
+                // Output rows are staged in the piece's query tile (each warp for itself, 16-byte chunks swizzled) and leave as
+                // runs of 32 or 64 bytes.
+                constexpr uint32_t N_CH = D / 32, ROW = N_CH * 16;
+                unsigned char *stage = smem + (uint32_t)(pi & 1) * SM::TILE + (uint32_t)warp * 32u * ROW;
+                auto place = [&](uint32_t r, uint32_t c) { return stage + r * ROW + ((c ^ ((r * N_CH / 8) & (N_CH - 1))) << 4); };
+#pragma unroll
+                for (uint32_t c = 0; c < N_CH; ++c) {
+                    float v[8];
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(o[8 * c + i]);
+                    *reinterpret_cast<uint4 *>(place(lane, c)) =
+                        make_uint4(pack2_bf16(v[0], v[1]), pack2_bf16(v[2], v[3]), pack2_bf16(v[4], v[5]), pack2_bf16(v[6], v[7]));
                 }
+                __syncwarp();
+                const uint32_t c = lane & (N_CH - 1);
+                uint4 *dst = item_out<D>(p, d.layer, d.b, d.head) + (e * 2 + hf) * N_CH + c;
+#pragma unroll
+                for (uint32_t r = lane / N_CH; r < 32; r += 32 / N_CH) {
+                    const uint4 x = *reinterpret_cast<const uint4 *>(place(r, c));
+                    const int at = out_row(p, blk, qd * 32 + r);
+                    if (at >= 0) dst[at * (D / 8)] = x;
+                }
+                ptx::fence_proxy_async();         // (the next query tile comes here through the async proxy)
+                __syncwarp();
             }
-            seq += 2u * (uint32_t)cnt + (partial ? 0u : one ? 1u : 2u);
-            __syncwarp();
-            if (lane == 0) free_piece(pi);
-            gather();                             // O and the exchanged values have been read: the next piece may overwrite them
+            if (lane == 0) {
+                ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + (pi & 1)));
+                free_piece(pi);
+            }
         }
         if (!ok && lane == 0) give_up();
         // ---- merge of the items this CTA shares with others.  Every warp comes here when its own pieces are done.
@@ -1136,7 +850,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     departed = atomicAdd(p.depart + ctr, 0x10001) + 0x10000;
                 }
             }
-            if (__shfl_sync(0xffffffffu, full, 0)) merge_slice<D>(p, m, c0, warp, blk, one, lane);
+            if (__shfl_sync(0xffffffffu, full, 0)) merge_slice<D>(p, m, c0, warp, blk, lane);
             // The last warp to leave: its CTA does what others left, all parts and all marks being complete, and the counters go
             // back to zero (nobody polls them any more; the next call cannot start before this kernel has ended).
             if (lane == 0 && (departed & 0xffff) == all - 1) {
@@ -1150,13 +864,21 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             }
         }
     }
+    __syncwarp();
     ptx::tc_fence_before();
     __syncthreads();
-    ptx::tc_fence_after();
-    if (warp == AT_MMA_WARP) ptx::tmem_dealloc(*tmem_slot, 512);
+    // nobody leaves while the pair's MMAs may still read its shared memory or its barriers may be signalled
+    if (PAIR) ptx::cluster_arrive();
     if (warp < AT_SOFTMAX_WARPS && *left_items)       // (the other warps have too few registers for it)
         for (int i = 0; i < 2; ++i)
-            if ((*left_items >> i) & 1) merge_left<D>(p, merges[i], blk, one, warp, lane);
+            if ((*left_items >> i) & 1) merge_left<D>(p, merges[i], blk, warp, lane);
+    __syncwarp();
+    if (PAIR) ptx::cluster_wait();
+    ptx::tc_fence_after();
+    if (warp == W_MMA) {
+        if (PAIR) ptx::tmem_dealloc_pair(*tmem_slot, 512);
+        else ptx::tmem_dealloc(*tmem_slot, 512);
+    }
     if (p.gate.word) previous_done();
 }
 
@@ -1228,31 +950,33 @@ bool tensor_map_bf16(CUtensorMap *map, const void *base, int rank, const cuuint6
 }
 
 namespace {
-// Row blocks of a problem and the CTAs that work on it.
+// Row tiles of a problem and the CTAs that work on it: at head size 128 items of more than one tile go to CTA pairs.
 struct AttnPlan {
-    int npc, n_tiles, n_blk, teams;
+    int npc, n_tiles, n_blk, teams;      // tree nodes per tile, tiles of an item, CTAs of a team, teams
+    bool pair;
 };
-AttnPlan attn_plan(int T, int G) {
+AttnPlan attn_plan(int T, int G, int D) {
     AttnPlan a;
-    a.npc = 128 / G;                                 // tree nodes per tile
+    a.npc = 128 / G;
     a.n_tiles = (T + a.npc - 1) / a.npc;
-    a.n_blk = (a.n_tiles + 1) / 2;
+    a.pair = D == 128 && a.n_tiles > 1;
+    a.n_blk = a.pair ? (a.n_tiles + 1) / 2 * 2 : a.n_tiles;
     const int sms = sm_count() < AT_MAX_CTAS ? sm_count() : AT_MAX_CTAS;
-    a.teams = sms / a.n_blk;
+    a.teams = (a.pair ? sms / 2 * 2 : sms) / a.n_blk;
     return a;
 }
 }  // namespace
 
-// Workspace: two slabs (a CTA has at most two pieces that are not whole items) of two tiles for every CTA; the kernel on CTA
-// pairs keeps a slab per key split of a query block and the order of the sequences.
+// Workspace: two slabs (a CTA has at most two pieces that are not whole items) for every CTA; the kernel for single layers
+// keeps a slab per key split of a query block and the order of the sequences.
 AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap) {
     AttnWs w;
     w.o_off = w.ml_off = w.left_off = w.total = 0;
     if (Hq / Hkv > 8) return w;          // the call itself refuses such a group; sizes are asked for before that
-    const AttnPlan a = attn_plan(t->T, Hq / Hkv);
+    const AttnPlan a = attn_plan(t->T, Hq / Hkv, D);
     const size_t slabs = (size_t)a.teams * a.n_blk * 2;
-    w.ml_off = align_up(slabs * 2 * 128 * D * sizeof(float), 256);
-    w.left_off = align_up(w.ml_off + slabs * 2 * 128 * sizeof(float2), 256);
+    w.ml_off = align_up(slabs * 128 * D * sizeof(float), 256);
+    w.left_off = align_up(w.ml_off + slabs * 128 * sizeof(float2), 256);
     w.total = align_up(w.left_off + slabs * AT_SOFTMAX_WARPS * sizeof(int32_t), 256);
     if (attn_pair_eligible(D, Hq / Hkv)) {
         int n_blk = 1;
@@ -1266,19 +990,19 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
 }
 
 // Which kernel a call for ONE layer takes at head size 128 (several layers always take the one of this file: 32 layers at
-// L = 512 take 60 us instead of 320, at L = 8192 290 instead of 570).  The kernel on CTA pairs starts and ends faster but
-// leaves pairs idle where blocks and splits do not fill the 74; this one divides the groups evenly.  Only the capacity is known
-// here, not the lengths.  us per call, lengths uniform in [h / 4, h] with h = all, a half, a quarter, an eighth of the
-// capacity (pairs / even division):
-//      7 sequences, 28 / 4 heads, capacity  8112:   72 / 60    41 / 38    26 / 30    18 / 25
-//     12 sequences, 16 / 4 heads, capacity  8192:   71 / 58    40 / 35    25 / 28    17 / 25
-//      4 sequences, T = 128,      capacity 32896:  266 / 197  137 / 149   78 / 70    42 / 42
-//      3 sequences, 16 / 4 heads, capacity 20000:   38 / 39    25 / 31    18 / 27    15 / 22
-//     16 sequences, 32 / 8 heads, capacity 32768:  427 / 381  217 / 198  106 / 126   70 / 91
-//     16 sequences, 32 / 8 heads, capacity  4224:   59 / 68    42 / 53    31 / 31    27 / 23
+// L = 512 take 45 us instead of 320, at L = 8192 260 to 320 instead of 570).  The kernel of attention_pair.cu starts and ends
+// faster but leaves pairs idle where blocks and splits do not fill the 74; this one divides the groups evenly.  Only the capacity
+// is known here, not the lengths.  us per call, lengths uniform in [h / 4, h] with h = all, a half, a quarter, an eighth of the
+// capacity (attention_pair.cu / even division):
+//      7 sequences, 28 / 4 heads, capacity  8112:   72 / 52    41 / 39    26 / 27    18 / 18
+//     12 sequences, 16 / 4 heads, capacity  8192:   70 / 57    40 / 32    24 / 26    17 / 18
+//      4 sequences, T = 128,      capacity 32896:  264 / 180  137 / 119   76 / 59    42 / 45
+//      3 sequences, 16 / 4 heads, capacity 20000:   38 / 33    25 / 27    18 / 22    15 / 19
+//     16 sequences, 32 / 8 heads, capacity 32768:  423 / 350  200 / 209  112 / 112   72 / 83
+//     16 sequences, 32 / 8 heads, capacity  4224:   59 / 62    41 / 52    31 / 40    27 / 37
 // With more blocks than pairs the pairs are all busy, longest sequence first, and what the even division gains in a full cache it
 // loses in one that is a quarter full: pairs.  With fewer, the even division is taken where the estimate for a full cache (us
-// per group on a pair and on an SM, start and end) is better by a tenth; such a call on a nearly empty cache pays 7 us.
+// per group on a pair and on an SM, start and end) is better by a tenth; such a call on a nearly empty cache loses up to 10 us.
 static bool pair_kernel_is_better(int T, int G, int B, int Hkv, int Lcap) {
     int n_blk = 1;
     const int ns = attn_pair_plan(T, G, B, Hkv, Lcap, &n_blk);
@@ -1288,7 +1012,7 @@ static bool pair_kernel_is_better(int T, int G, int B, int Hkv, int Lcap) {
     return pairs <= 1.1 * even;
 }
 
-template <int D, int ML, bool NEG>
+template <int D, bool PAIR, int ML, bool NEG>
 static int launch_attn(const mtv_tree *tree, const AttnPlan &a, AttnParams &p, const __nv_bfloat16 *q, mtv_bf16 *const *k,
                        mtv_bf16 *const *v, int64_t sb, int64_t sh, int64_t st, cudaStream_t stream) {
     AttnMaps<ML> maps;
@@ -1299,26 +1023,27 @@ static int launch_attn(const mtv_tree *tree, const AttnPlan &a, AttnParams &p, c
         const cuuint32_t qb[5] = {64, (cuuint32_t)p.G, (cuuint32_t)p.npc, 1, 1};
         const cuuint64_t cd[5] = {64, (cuuint64_t)p.Lcap, D / 64, (cuuint64_t)p.Hkv, (cuuint64_t)p.B};
         const cuuint64_t cs[4] = {(cuuint64_t)st * 2, 128, (cuuint64_t)sh * 2, (cuuint64_t)sb * 2};
-        const cuuint32_t cb[5] = {64, AT_BN, D / 64, 1, 1};
+        const cuuint32_t kb[5] = {64, PAIR ? AT_BN / 2 : AT_BN, D / 64, 1, 1}, vb[5] = {64, AT_BN, PAIR ? 1 : D / 64, 1, 1};
         if (!tensor_map_bf16(&maps.q, q, 5, qd, qs, qb)) return MTV_ERR_CUDA;
         for (int l = 0; l < p.n_layers; ++l)
-            if (!tensor_map_bf16(&maps.k[l], k[l], 5, cd, cs, cb) || !tensor_map_bf16(&maps.v[l], v[l], 5, cd, cs, cb))
+            if (!tensor_map_bf16(&maps.k[l], k[l], 5, cd, cs, kb) || !tensor_map_bf16(&maps.v[l], v[l], 5, cd, cs, vb))
                 return MTV_ERR_CUDA;
     }
     static PerDeviceOnce once;
     bool *done = once.flag();
     if (!done || !*done) {
         cudaFuncAttributes fa;
-        MTV_CUDA_CHECK(cudaFuncGetAttributes(&fa, tree_attn_kernel<D, ML, NEG>));
+        MTV_CUDA_CHECK(cudaFuncGetAttributes(&fa, tree_attn_kernel<D, PAIR, ML, NEG>));
         if (fa.numRegs < AT_LAUNCH_REGS) {   // the register split would wait for registers that the launch does not own
             set_last_error_text("tree_attn_kernel: compiled with fewer registers than its split needs");
             return MTV_ERR_CUDA;
         }
-        MTV_CUDA_CHECK(cudaFuncSetAttribute(tree_attn_kernel<D, ML, NEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D>::TOTAL));
+        MTV_CUDA_CHECK(cudaFuncSetAttribute(tree_attn_kernel<D, PAIR, ML, NEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnSmem<D, PAIR>::TOTAL));
         if (done) *done = true;
     }
     TapScope tap(MTV_KERNEL_ATTN_PARTIAL, stream);
-    MTV_CUDA_CHECK(launch_dependent(tree_attn_kernel<D, ML, NEG>, dim3(a.teams * a.n_blk), AT_THREADS, AttnSmem<D>::TOTAL, stream, maps, p));
+    MTV_CUDA_CHECK(launch_dependent_clusters(PAIR ? 2 : 1, tree_attn_kernel<D, PAIR, ML, NEG>, dim3(a.teams * a.n_blk), AT_THREADS,
+                                             AttnSmem<D, PAIR>::TOTAL, stream, maps, p));
     return MTV_OK;
 }
 
@@ -1352,7 +1077,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
                                      status, (char *)ws + Lw.o_off, reinterpret_cast<float *>((char *)ws + Lw.pair_ml_off),
                                      reinterpret_cast<int32_t *>((char *)ws + Lw.order_off), (cudaStream_t)stream);
     }
-    const AttnPlan a = attn_plan(tree->T, Hq / Hkv);
+    const AttnPlan a = attn_plan(tree->T, Hq / Hkv, D);
     AttnParams p;
     p.seq_lens = seq_lens; p.anc = tree->d_anc; p.status = status; p.dev_error = tree->d_error;
     p.ws_o = reinterpret_cast<uint4 *>((char *)ws + Lw.o_off);
@@ -1361,7 +1086,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.arrive = tree->d_counters; p.depart = tree->d_counters + AT_MAX_CTAS;
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
-    p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_tiles = a.n_tiles; p.n_blk = a.n_blk; p.teams = a.teams;
+    p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_blk = a.n_blk; p.teams = a.teams;
     p.gate = alongside ? *alongside : Gate{};
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;
@@ -1374,10 +1099,12 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
         p.n_layers = n_layers - l < per_launch ? n_layers - l : per_launch;
         p.out = reinterpret_cast<__nv_bfloat16 *>(out) + l * per_layer;
         const __nv_bfloat16 *ql = reinterpret_cast<const __nv_bfloat16 *>(q) + l * per_layer;
+        constexpr int ML = AT_MAX_LAYERS;
         auto launch = p.n_layers == 1
-                          ? (D == 128 ? launch_attn<128, 1, false> : scale < 0.f ? launch_attn<64, 1, true> : launch_attn<64, 1, false>)
-                          : (D == 128 ? launch_attn<128, AT_MAX_LAYERS, false>
-                                      : scale < 0.f ? launch_attn<64, AT_MAX_LAYERS, true> : launch_attn<64, AT_MAX_LAYERS, false>);
+                          ? (a.pair ? launch_attn<128, true, 1, false> : D == 128 ? launch_attn<128, false, 1, false>
+                             : scale < 0.f ? launch_attn<64, false, 1, true> : launch_attn<64, false, 1, false>)
+                          : (a.pair ? launch_attn<128, true, ML, false> : D == 128 ? launch_attn<128, false, ML, false>
+                             : scale < 0.f ? launch_attn<64, false, ML, true> : launch_attn<64, false, ML, false>);
         const int rc = launch(tree, a, p, ql, k + l, v + l, stride_b, stride_h, stride_t, st);
         if (rc != MTV_OK) return rc;
     }
@@ -1398,9 +1125,3 @@ extern "C" int tree_verify_attention(const mtv_tree_t *tree, int B, int Hq, int 
     return mtv::tree_attention_layers(tree, B, Hq, Hkv, D, 1, q, &k, &v, stride_b, stride_h, stride_t, Lcap, seq_lens, scale,
                                       out, status, ws, ws_bytes, stream);
 }
-
-#ifdef MTV_TRACE
-extern "C" int mtv_trace_set(long long *buf) {
-    return cudaMemcpyToSymbol(mtv::g_trace, &buf, sizeof buf) == cudaSuccess ? 0 : -1;
-}
-#endif

@@ -488,8 +488,8 @@ tree_attn_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
                 const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(sr[2 * e + 2]), __uint_as_float(sr[2 * e + 3])), sc2, nm2);
                 float2 p01, p23;
                 if (e % 8 == 6) {   // every fourth quadruple on the FMA pipes: the special-function unit is the bottleneck of a tile
-                    p01 = exp2_poly2<3>(x01);
-                    p23 = exp2_poly2<3>(x23);
+                    p01 = exp2_poly2(x01);
+                    p23 = exp2_poly2(x23);
                 } else {
                     p01 = make_float2(ex2(x01.x), ex2(x01.y));
                     p23 = make_float2(ex2(x23.x), ex2(x23.y));

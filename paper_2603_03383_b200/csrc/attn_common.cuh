@@ -13,11 +13,9 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 // 2^x for two values on the FMA pipes: x = j + f with j the nearest integer (read off the low mantissa bits of
-// x + 1.5 * 2^23) and f in [-0.5, 0.5]; 2^f by a polynomial with the smallest largest relative error over that interval
-// (degree 3: 7.5e-5, far below the bf16 rounding of P; degree 4: 3.7e-6); 2^j by an add to the exponent field.  x is
-// clamped at -126 (the result then underflows towards zero like ex2's).  From x = 128 on the exponent field overflows (the
-// result may be negative, NaN or small) and a NaN counts as -126: the caller sees to it that neither is used.
-template <int DEGREE>
+// x + 1.5 * 2^23) and f in [-0.5, 0.5]; 2^f by a cubic with the smallest largest relative error over that interval (7.5e-5, far
+// below the bf16 rounding of P); 2^j by an add to the exponent field.  x <= 127; it is clamped at -126 (the result then underflows
+// towards zero like ex2's).
 __device__ __forceinline__ float2 exp2_poly2(float2 x) {
     const float magic = 12582912.f;
     x.x = fmaxf(x.x, -126.f);
@@ -25,17 +23,9 @@ __device__ __forceinline__ float2 exp2_poly2(float2 x) {
     const float2 t = __fadd2_rn(x, make_float2(magic, magic));
     const float2 jf = __fadd2_rn(t, make_float2(-magic, -magic));
     const float2 f = __fadd2_rn(x, make_float2(-jf.x, -jf.y));
-    float2 q;
-    if (DEGREE == 3) {
-        q = __ffma2_rn(make_float2(0.055171650f, 0.055171650f), f, make_float2(0.24261113f, 0.24261113f));
-        q = __ffma2_rn(q, f, make_float2(0.69326097f, 0.69326097f));
-        q = __ffma2_rn(q, f, make_float2(0.99992806f, 0.99992806f));
-    } else {
-        q = __ffma2_rn(make_float2(0.0095701022f, 0.0095701022f), f, make_float2(0.055917859f, 0.055917859f));
-        q = __ffma2_rn(q, f, make_float2(0.24024744f, 0.24024744f));
-        q = __ffma2_rn(q, f, make_float2(0.69312179f, 0.69312179f));
-        q = __ffma2_rn(q, f, make_float2(0.99999928f, 0.99999928f));
-    }
+    float2 q = __ffma2_rn(make_float2(0.055171650f, 0.055171650f), f, make_float2(0.24261113f, 0.24261113f));
+    q = __ffma2_rn(q, f, make_float2(0.69326097f, 0.69326097f));
+    q = __ffma2_rn(q, f, make_float2(0.99992806f, 0.99992806f));
     return make_float2(__int_as_float(__float_as_int(q.x) + (__float_as_int(t.x) << 23)),
                        __int_as_float(__float_as_int(q.y) + (__float_as_int(t.y) << 23)));
 }

@@ -1,0 +1,315 @@
+// How the tree attention divides the key groups of all items among teams of CTAs, the exponentials of a tile, the workspace of
+// partial results and their merge (attention.cu).
+#pragma once
+#include "attn_common.cuh"
+
+namespace mtv {
+
+constexpr int AT_BN = 128;            // keys per group
+constexpr int AT_THREADS = 640;
+constexpr int AT_SOFTMAX_WARPS = 16;
+constexpr int AT_PIECES = 4;          // piece descriptors in flight
+// How long a warp waits for the others of an item, in cycles.  In the bounds-checking build it looks once: nearly all slices
+// are then left to the last warp.
+#ifdef MTV_DEBUG_BOUNDS
+constexpr long long AT_MERGE_WAIT = 0;
+#else
+constexpr long long AT_MERGE_WAIT = 2000000;
+#endif
+constexpr int AT_MAX_CTAS = 256;      // merge counters in the tree object: one pair per CTA
+constexpr int AT_MAX_LAYERS = 64;     // layers per launch (two tensor maps each in the kernel's parameters)
+// registers per thread: 96 at launch, moved from the four auxiliary warps to the sixteen softmax warps
+constexpr int AT_LAUNCH_REGS = 96, AT_SOFTMAX_REGS = 104, AT_AUX_REGS = 64;
+static_assert(512 * AT_SOFTMAX_REGS + 128 * AT_AUX_REGS <= AT_THREADS * AT_LAUNCH_REGS, "register split");
+constexpr float AT_SUM_LIMIT = 4294967296.f;   // 2^32: a thread's sum of P over a group beyond it moves the reference
+
+struct AttnPiece {      // 32 bytes
+    int layer, b, head, gb, cnt, L, flags, first;   // key groups [gb, gb + cnt); cnt = 0: no more pieces;
+                                                    // first: first team that contributes to the item
+};
+constexpr int PIECE_PARTIAL = 1, PIECE_HEAD = 2;   // not a whole item; starts at the item's first group
+struct AttnMerge {      // a partial piece of this CTA, for the merge at the end
+    int first, n, layer, b, head, pad;             // first contributing team, number of them
+};
+
+template <int ML>
+struct __align__(64) AttnMaps {
+    CUtensorMap q, k[ML], v[ML];
+};
+
+struct AttnParams {
+    const int32_t *seq_lens;
+    const uint64_t *anc;     // [T][2]
+    __nv_bfloat16 *out;      // [layers][B][T][Hq][D]
+    uint4 *ws_o;             // [CTA][2 slabs][D / 4 chunks][128 rows] 16-byte chunks of O / l, fp32
+    float2 *ws_ml;           // [CTA][2 slabs][128 rows] (m, l)
+    int32_t *left;           // [CTA][2 slabs][16 warps] 1: the warp's slice of the item is left to the last one
+    int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls; depart counts slices left in its upper half
+    int32_t *status;         // [B] or null
+    int32_t *dev_error;
+    float scale_log2;
+    int B, T, G, Hq, Hkv, Lcap, n_layers;
+    int npc, R;              // tree nodes per tile (128 / G) and the rows they fill
+    unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
+    int n_blk, teams;        // CTAs of a team, teams
+    Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
+};
+
+__device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }
+// P = 2^(scale S - m) of 32 scores (two values per instruction where the instruction set has packed forms) and its
+// contribution to the row sum.  pk: bf16 pairs; TWO: rest has what their rounding left, as bf16 pairs.  All exponentials are the
+// special-function unit's: it needs 1024 cycles for a tile of scores, what the tensor core needs, and with a quarter of them as
+// polynomials on the FMA pipes a step of 4 x 32768 keys takes 4 % longer (867 -> 902 us for four layers), since the board's power
+// limit, not a pipe, sets the pace there.
+template <bool TWO>
+__device__ __forceinline__ void exp_quarter(const uint32_t (&s)[32], float2 sc2, float2 nm2, float2 &la, float2 &lb, uint32_t *pk, uint32_t *rest) {
+#pragma unroll
+    for (int e = 0; e < 16; e += 2) {
+        const float2 x01 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e]), __uint_as_float(s[2 * e + 1])), sc2, nm2);
+        const float2 x23 = __ffma2_rn(make_float2(__uint_as_float(s[2 * e + 2]), __uint_as_float(s[2 * e + 3])), sc2, nm2);
+        const float2 p01 = make_float2(ex2(x01.x), ex2(x01.y)), p23 = make_float2(ex2(x23.x), ex2(x23.y));
+        la = __fadd2_rn(la, p01);
+        lb = __fadd2_rn(lb, p23);
+        pk[e] = pack2_bf16(p01.x, p01.y);
+        pk[e + 1] = pack2_bf16(p23.x, p23.y);
+        if (TWO) {
+            const float2 r01 = __fadd2_rn(p01, make_float2(-bf16_lo(pk[e]), -bf16_hi(pk[e])));
+            const float2 r23 = __fadd2_rn(p23, make_float2(-bf16_lo(pk[e + 1]), -bf16_hi(pk[e + 1])));
+            rest[e] = pack2_bf16(r01.x, r01.y);
+            rest[e + 1] = pack2_bf16(r23.x, r23.y);
+        }
+    }
+}
+// the largest scale * s of 32 scores; NEG: the scale is negative
+template <bool NEG>
+__device__ __forceinline__ float max_quarter(const uint32_t (&s)[32], float scale) {
+    constexpr uint32_t sign = NEG ? 0x80000000u : 0u;
+    float a = -INFINITY, b = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < 32; e += 4) {
+        a = ptx::fmax3(a, __uint_as_float(s[e] ^ sign), __uint_as_float(s[e + 1] ^ sign));
+        b = ptx::fmax3(b, __uint_as_float(s[e + 2] ^ sign), __uint_as_float(s[e + 3] ^ sign));
+    }
+    return fmaxf(a, b) * fabsf(scale);
+}
+// Output row of row r of a CTA's tile (in units of D elements from the item's first row), or -1 if it belongs to nobody: CTA blk of
+// a team has row tile blk.  With a group size that does not divide 128 the last 128 - R rows of a tile do (whatever the tile's
+// shared memory held is computed and never written out).
+__device__ __forceinline__ int node_in_tile(const AttnParams &p, int r) { return (int)(((unsigned)r * p.inv_g) >> 16); }
+__device__ __forceinline__ int out_row(const AttnParams &p, int blk, int r) {
+    const int n = node_in_tile(p, r), node = blk * p.npc + n;
+    return r < p.R && node < p.T ? node * p.Hq + (r - n * p.G) : -1;
+}
+template <int D>
+__device__ __forceinline__ uint4 *item_out(const AttnParams &p, int layer, int b, int hd) {      // first row of an item's output
+    return reinterpret_cast<uint4 *>(p.out + (((size_t)layer * p.B + b) * p.T * p.Hq + hd * p.G) * D);
+}
+// slabs of the workspace: 16-byte chunk c (4 columns) of row r; the row's (m, l)
+template <int D>
+__device__ __forceinline__ uint4 *slab_o(const AttnParams &p, int cta, int slab, int r, int c) {
+    return p.ws_o + (((unsigned)cta * 2 + slab) * (D / 4) + c) * 128 + r;
+}
+__device__ __forceinline__ float2 *slab_ml(const AttnParams &p, int cta, int slab, int r) {
+    return p.ws_ml + ((unsigned)cta * 2 + slab) * 128 + r;
+}
+
+// Rows of a tile that is shared between CTAs: contributor c0 combines its share of them, a thread per 16-byte chunk of the output,
+// with the loads of several contributors in flight.  This is warp w's part of it.
+template <int D>
+__device__ __forceinline__ void merge_slice(const AttnParams &p, const AttnMerge &m, int c0, int w, int blk, int lane) {
+    constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
+    const int per = (p.R + m.n - 1) / m.n, r_begin = c0 * per;
+    const int n_my = max(0, min(p.R, r_begin + per) - r_begin);
+    const unsigned inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;    // e / n_my for e < 2048, n_my <= 128
+    uint4 *dst = item_out<D>(p, m.layer, m.b, m.head);
+#pragma unroll 1
+    for (int e = w * 32 + lane; e < n_my * (D / 8); e += AT_SOFTMAX_WARPS * 32) {
+        const int c = (int)(((unsigned)e * inv_n) >> 20), r = r_begin + e - c * n_my;
+        float acc[8], mm = -INFINITY, wsum = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+#pragma unroll 1
+        for (int s0 = 0; s0 < m.n; s0 += NS) {
+            float2 ml[NS];
+            uint4 v[NS][VC];
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const int s = min(s0 + k, m.n - 1), cta = (m.first + s) * p.n_blk + blk;
+                const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
+                ml[k] = __ldcg(slab_ml(p, cta, sl, r));
+#pragma unroll
+                for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, r, c * VC + q));
+                if (s0 + k >= m.n) ml[k] = make_float2(-INFINITY, 0.f);
+            }
+            float mc = mm;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
+            const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
+            mm = mc;
+            wsum *= resc;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[k] *= resc;
+#pragma unroll
+            for (int k = 0; k < NS; ++k) {
+                const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
+                wsum += wt;
+#pragma unroll
+                for (int q = 0; q < VC; ++q) {
+                    const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
+                }
+            }
+        }
+        const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
+        const int o = out_row(p, blk, r);
+        if (o >= 0)
+            dst[o * (D / 8) + c] =
+                make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
+                           pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
+    }
+}
+// The slices that warps left, of one item, by the softmax warps of the CTA whose warp was the last to leave it.  (Out of the way of the
+// usual case, whose registers it must not touch.)
+template <int D>
+static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, int warp, int lane) {
+    for (int u = warp; u < m.n * AT_SOFTMAX_WARPS; u += AT_SOFTMAX_WARPS) {
+        const int c = u / AT_SOFTMAX_WARPS, w = u % AT_SOFTMAX_WARPS, cta = (m.first + c) * p.n_blk + blk;
+        if (__ldcg(p.left + ((unsigned)cta * 2 + (c == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + w)) merge_slice<D>(p, m, c, w, blk, lane);
+    }
+}
+
+// a / b, b > 0.  A quotient of small numbers is at most one off when it is formed in fp32, and its remainder says which way; the
+// chain of these that a launch starts with takes a third of the time that integer divisions take.
+__device__ __forceinline__ unsigned quotient(unsigned a, unsigned b) {
+    if (a >= 1u << 22) return a / b;
+    unsigned q = (unsigned)__fdividef((float)a, (float)b);
+    const int r = (int)(a - q * b);
+    if (r < 0) --q;
+    else if ((unsigned)r >= b) ++q;
+    return q;
+}
+// The pieces of one team's run, derived by one warp from the lengths on the device (see attention.cu).  COST: what an item costs
+// beside its key groups, MERGE: what writing and combining partial results costs, in groups.
+template <int COST, int MERGE>
+struct PieceWalk {
+    const AttnParams &p;
+    const int lane;
+    const unsigned LH, teams, team;
+    int chunk = 0, len = 0, g = 0;        // lengths and group counts of sequences chunk .. chunk + 31, one per lane
+    bool pad = false;
+    unsigned u = 1, pos = 0, hi = 0, off = 0;
+    int layer = 0, b = 0, head = 0, n_part = 0;
+
+    __device__ __forceinline__ PieceWalk(const AttnParams &p_, int team_, int lane_)
+        : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_) {}
+    __device__ __forceinline__ void load_chunk(int b0, bool real) {
+        chunk = b0;
+        const int at = b0 + lane;
+        len = at < p.B && real ? p.seq_lens[at] : 0;
+        g = at < p.B && len + p.T <= p.Lcap ? (len + p.T + AT_BN - 1) / AT_BN : 0;   // 0: does not fit, reported below
+    }
+    __device__ __forceinline__ unsigned padded(unsigned gg) const { return gg == 0 ? 0u : pad ? quotient(gg + u - 1, u) * u : gg + COST; }
+    // real: false = nothing but going through the code
+    __device__ __forceinline__ void divide(bool real) {
+        unsigned sum = 0, nz = 0, g_max = 0, g_min = 0xffffffffu;
+        for (int b0 = 0; b0 < p.B; b0 += 32) {
+            load_chunk(b0, real);
+            sum += __reduce_add_sync(0xffffffffu, (unsigned)g);
+            nz += __popc(__ballot_sync(0xffffffffu, g > 0));
+            g_max = max(g_max, __reduce_max_sync(0xffffffffu, (unsigned)g));
+            g_min = min(g_min, __reduce_min_sync(0xffffffffu, g > 0 ? (unsigned)g : 0xffffffffu));
+            if (real && blockIdx.x == 0 && p.status && b0 + lane < p.B) p.status[b0 + lane] = g > 0 ? MTV_OK : MTV_ERR_CAPACITY;
+        }
+        // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting
+        // anywhere gives most teams two pieces, that is about two groups' worth of extra start and end: whichever is
+        // shorter.
+        const unsigned u_cut = max(1u, quotient(LH * (sum + nz * COST) + teams - 1, teams));
+        unsigned v_head = 0;                  // length of one head's row of all sequences in the CTAs' common address space
+        pad = LH * nz <= teams;
+        u = pad ? max(1u, quotient(LH * sum + teams - 1, teams)) : u_cut;
+        // Whole items, if that makes no run longer than the division above by more than a merge takes: no team shares one.
+        const unsigned whole = pad ? g_max : quotient(LH * nz + teams - 1, teams) * (g_max + COST);
+        if ((pad || g_min == g_max) && whole <= u + MERGE) u = max(1u, whole);
+        for (;;) {
+            v_head = 0;
+            for (int b0 = 0; b0 < p.B; b0 += 32) {
+                if (b0 != chunk) load_chunk(b0, real);
+                v_head += __reduce_add_sync(0xffffffffu, padded((unsigned)g));
+            }
+            if (!pad || LH * quotient(v_head, u) <= teams) break;
+            if (++u > u_cut + 2) { pad = false; u = u_cut; }
+        }
+        const unsigned v_layer = v_head * (unsigned)p.Hkv;
+        pos = team * u;
+        hi = min(pos + u, v_layer * (unsigned)p.n_layers);
+        // where the run begins
+        if (pos < hi) {
+            layer = (int)quotient(pos, v_layer);
+            unsigned rem = pos - (unsigned)layer * v_layer;
+            for (int b0 = 0;; b0 += 32) {
+                if (b0 != chunk) load_chunk(b0, real);
+                const unsigned mine = padded((unsigned)g) * (unsigned)p.Hkv;
+                unsigned incl = mine;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const unsigned m = __ballot_sync(0xffffffffu, rem < incl);
+                if (m) {
+                    const int at = __ffs(m) - 1;
+                    b = b0 + at;
+                    rem -= __shfl_sync(0xffffffffu, incl - mine, at);
+                    break;
+                }
+                rem -= __shfl_sync(0xffffffffu, incl, 31);
+            }
+            const unsigned gp = padded((unsigned)__shfl_sync(0xffffffffu, g, b - chunk));
+            head = (int)quotient(rem, gp);
+            off = rem - (unsigned)head * gp;
+        }
+    }
+    // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges, too.
+    __device__ __forceinline__ bool next(AttnPiece &d, AttnMerge *merges, volatile int *n_merge) {
+        while (pos < hi) {
+            const unsigned gg = (unsigned)__shfl_sync(0xffffffffu, g, b - chunk), gp = padded(gg);
+            const int L = __shfl_sync(0xffffffffu, len, b - chunk);
+            const unsigned end = min(gp, off + (hi - pos)), a = pos - off;
+            const unsigned r0 = min(off, gg), r1 = min(end, gg);
+            d.layer = layer; d.b = b; d.head = head; d.gb = (int)r0; d.cnt = (int)(r1 - r0); d.L = L;
+            const bool part = r1 - r0 < gg;
+            d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0);
+            d.first = (int)quotient(a, u);
+            if (r1 > r0 && part && n_part < 2) {
+                if (lane == 0) {
+                    AttnMerge m;
+                    m.first = d.first; m.n = (int)quotient(a + gg - 1, u) - m.first + 1;
+                    m.layer = layer; m.b = b; m.head = head; m.pad = 0;
+                    merges[n_part] = m;
+                    *n_merge = n_part + 1;
+                }
+                ++n_part;
+            }
+            pos += end - off;
+            off = 0;
+            if (++head == p.Hkv) {        // the next sequence that fits, in this layer or the next
+                head = 0;
+                unsigned m = __ballot_sync(0xffffffffu, g > 0) & ~(0xffffffffu >> (31 - (b - chunk)));
+                while (!m && pos < hi) {
+                    int b0 = chunk + 32;
+                    if (b0 >= p.B) { b0 = 0; ++layer; }
+                    if (b0 != chunk) load_chunk(b0, true);
+                    m = __ballot_sync(0xffffffffu, g > 0);
+                }
+                b = chunk + (m ? __ffs(m) - 1 : 0);
+            }
+            if (r1 > r0) return true;
+        }
+        d.cnt = 0;
+        return false;
+    }
+};
+
+}  // namespace mtv
