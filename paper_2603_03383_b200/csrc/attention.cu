@@ -258,12 +258,12 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     if (warp == W_TMA) {
         // ------------------------------------------------------------ the pair's pieces; this CTA's halves of K and V
         PieceWalk<ITEM_COST, MERGE_COST> walk(p, team, lane);
-        // The instructions of a launch come from L2 anew; this stretch runs once without lengths while the set-up goes on.
-#pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            if (pass == 1) (void)begin();
-            walk.divide(pass == 1);
-        }
+        // The work is divided while the kernel before this one ends, by the lengths that are there (a call that follows another has
+        // nothing that changes them in between), and looked at again behind it: eight one-layer calls on ragged lengths take 291 us
+        // instead of 314, at head size 64 164 instead of 172.
+        walk.divide(false);
+        (void)begin();
+        if (!walk.still_so()) { walk.divide(true); }
         int n_pub = 0;
         bool ok = true;
         auto publish = [&](const AttnPiece &d) {
@@ -302,6 +302,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         publish(cur);
         int done = 0;
         if (have) { done = min(2 * cur.cnt, STAGES); request(cur, 0, done); }
+        walk.report();
         while (have && ok && !*abort_flag) {
             const bool more = walk.next(nxt, merges, n_merge);
             publish(nxt);

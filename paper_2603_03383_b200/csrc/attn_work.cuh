@@ -204,23 +204,32 @@ struct PieceWalk {
 
     __device__ __forceinline__ PieceWalk(const AttnParams &p_, int team_, int lane_)
         : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_) {}
-    __device__ __forceinline__ void load_chunk(int b0, bool real) {
+    // (through L2: the lengths may be looked at before the kernel that writes them is complete, and again behind it)
+    __device__ __forceinline__ int length(int at) const { return at < p.B ? __ldcg(p.seq_lens + at) : 0; }
+    __device__ __forceinline__ void load_chunk(int b0, bool final) {
         chunk = b0;
-        const int at = b0 + lane;
-        len = at < p.B && real ? p.seq_lens[at] : 0;
-        g = at < p.B && len + p.T <= p.Lcap ? (len + p.T + AT_BN - 1) / AT_BN : 0;   // 0: does not fit, reported below
+        len = final || p.B <= 32 ? length(b0 + lane) : 0;       // (more than 32: read more than once, so not while they may change)
+        if (!final) len = min(max(len, 0), p.Lcap);
+        g = b0 + lane < p.B && len + p.T <= p.Lcap ? (len + p.T + AT_BN - 1) / AT_BN : 0;   // 0: does not fit, see report
+    }
+    // Were the lengths that the work was divided by the ones that are there now?
+    __device__ __forceinline__ bool still_so() const { return p.B <= 32 && __all_sync(0xffffffffu, length(lane) == len); }
+    __device__ __forceinline__ void report() const {
+        if (blockIdx.x == 0 && p.status)
+            for (int b = lane; b < p.B; b += 32) p.status[b] = length(b) + p.T <= p.Lcap ? MTV_OK : MTV_ERR_CAPACITY;
     }
     __device__ __forceinline__ unsigned padded(unsigned gg) const { return gg == 0 ? 0u : pad ? quotient(gg + u - 1, u) * u : gg + COST; }
-    // real: false = nothing but going through the code
-    __device__ __forceinline__ void divide(bool real) {
+    // final: false = with lengths that may still change
+    __device__ __forceinline__ void divide(bool final) {
+        layer = b = head = 0;
+        off = 0;
         unsigned sum = 0, nz = 0, g_max = 0, g_min = 0xffffffffu;
         for (int b0 = 0; b0 < p.B; b0 += 32) {
-            load_chunk(b0, real);
+            load_chunk(b0, final);
             sum += __reduce_add_sync(0xffffffffu, (unsigned)g);
             nz += __popc(__ballot_sync(0xffffffffu, g > 0));
             g_max = max(g_max, __reduce_max_sync(0xffffffffu, (unsigned)g));
             g_min = min(g_min, __reduce_min_sync(0xffffffffu, g > 0 ? (unsigned)g : 0xffffffffu));
-            if (real && blockIdx.x == 0 && p.status && b0 + lane < p.B) p.status[b0 + lane] = g > 0 ? MTV_OK : MTV_ERR_CAPACITY;
         }
         // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting
         // anywhere gives most teams two pieces, that is about two groups' worth of extra start and end: whichever is
@@ -235,7 +244,7 @@ struct PieceWalk {
         for (;;) {
             v_head = 0;
             for (int b0 = 0; b0 < p.B; b0 += 32) {
-                if (b0 != chunk) load_chunk(b0, real);
+                if (b0 != chunk) load_chunk(b0, final);
                 v_head += __reduce_add_sync(0xffffffffu, padded((unsigned)g));
             }
             if (!pad || LH * quotient(v_head, u) <= teams) break;
@@ -249,7 +258,7 @@ struct PieceWalk {
             layer = (int)quotient(pos, v_layer);
             unsigned rem = pos - (unsigned)layer * v_layer;
             for (int b0 = 0;; b0 += 32) {
-                if (b0 != chunk) load_chunk(b0, real);
+                if (b0 != chunk) load_chunk(b0, final);
                 const unsigned mine = padded((unsigned)g) * (unsigned)p.Hkv;
                 unsigned incl = mine;
 #pragma unroll
@@ -271,7 +280,8 @@ struct PieceWalk {
             off = rem - (unsigned)head * gp;
         }
     }
-    // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges, too.
+    // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges (if
+    // there are any), too.
     __device__ __forceinline__ bool next(AttnPiece &d, AttnMerge *merges, volatile int *n_merge) {
         while (pos < hi) {
             const unsigned gg = (unsigned)__shfl_sync(0xffffffffu, g, b - chunk), gp = padded(gg);
@@ -283,7 +293,7 @@ struct PieceWalk {
             d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0);
             d.first = (int)quotient(a, u);
             if (r1 > r0 && part && n_part < 2) {
-                if (lane == 0) {
+                if (lane == 0 && merges) {
                     AttnMerge m;
                     m.first = d.first; m.n = (int)quotient(a + gg - 1, u) - m.first + 1;
                     m.layer = layer; m.b = b; m.head = head; m.pad = 0;
