@@ -74,12 +74,12 @@ constexpr int NB = 3;                 // tiles of scores
 constexpr float LOG2E = 1.4426950408889634f;
 // P goes to the tensor core as bf16, whose rounding is the largest error beside the output's own.  Where a reference that
 // follows the row's maximum makes the largest weights exact (they are 1), a fixed reference does not: P then has a second bf16
-// term, what the rounding of the first left.  On pairs in a piece's first group, whose maximum is the reference; else in every
-// group (O += P V is short at head size 64, and an item of one row tile is bound by memory).  Rel. error against 64 bits with
-// one term / two / a reference that follows the maximum: D = 64, L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 /
-// .00210; D = 128, L = 512: .00235 / .00204 / .00268.
-template <bool PAIR>
-__host__ __device__ constexpr bool two_terms(int group) { return !PAIR || group == 0; }
+// term, what the rounding of the first left.  At head size 64 in every group (O += P V is short there); at 128 in a piece's
+// first group, whose maximum is the reference, and in the second of a single row tile (a kernel with a reference for every other
+// group had two terms in both).  Rel. error against 64 bits with one term / two / a reference that follows the maximum: D = 64,
+// L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 / .00210; D = 128, L = 512: .00235 / .00204 / .00268.
+template <int D, bool PAIR>
+__host__ __device__ constexpr bool two_terms(int group) { return D == 64 || group == 0 || (!PAIR && group == 1); }
 // tensor-memory columns: O, and three tiles of scores; P lies over its scores, each half of the keys over its own: keys 0-63
 // at columns 0-31, keys 64-127 at 64-95; in two terms each quarter over its own: keys 0-31 at columns 0-15, their second
 // terms at 16-31, and so on.
@@ -263,7 +263,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         // instead of 314, at head size 64 164 instead of 172.
         walk.divide(false);
         (void)begin();
-        if (!walk.still_so()) { walk.divide(true); }
+        if (!walk.still_so()) walk.divide(true);
         int n_pub = 0;
         bool ok = true;
         auto publish = [&](const AttnPiece &d) {
@@ -495,8 +495,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     else ptx::mma_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
                 };
                 const int steps = j == cnt - 1 ? last_steps : 8;
-                if (two_terms<PAIR>(j)) {
-                    if (!PAIR && steps == 8) {
+                if (two_terms<D, PAIR>(j)) {
+                    if (D == 64 && steps == 8) {
 #pragma unroll
                         for (int kk = 0; kk < 16; ++kk) issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > 0 || kk > 0);
                     } else {
@@ -728,7 +728,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                         sum = (la.x + la.y) + (lb.x + lb.y);
                         return asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT);
                     };
-                    if constexpr (two_terms<PAIR>(1)) {
+                    if (D == 64 || (!PAIR && j == 1)) {
                         uint32_t pa[16], pb[16], ra[16], rb[16];
                         exp_quarter<true>(qa, sc2, nm2, la, lb, pa, ra);
                         exp_quarter<true>(qb, sc2, nm2, la, lb, pb, rb);

@@ -280,8 +280,7 @@ struct PieceWalk {
             off = rem - (unsigned)head * gp;
         }
     }
-    // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges (if
-    // there are any), too.
+    // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges, too.
     __device__ __forceinline__ bool next(AttnPiece &d, AttnMerge *merges, volatile int *n_merge) {
         while (pos < hi) {
             const unsigned gg = (unsigned)__shfl_sync(0xffffffffu, g, b - chunk), gp = padded(gg);
@@ -293,7 +292,7 @@ struct PieceWalk {
             d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0);
             d.first = (int)quotient(a, u);
             if (r1 > r0 && part && n_part < 2) {
-                if (lane == 0 && merges) {
+                if (lane == 0) {
                     AttnMerge m;
                     m.first = d.first; m.n = (int)quotient(a + gg - 1, u) - m.first + 1;
                     m.layer = layer; m.b = b; m.head = head; m.pad = 0;

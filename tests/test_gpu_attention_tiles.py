@@ -6,8 +6,8 @@ import pytest
 import torch
 
 from oracle import reference as ref
-from paper_2603_03383_b200 import synth
-from tests._cases import assert_close, make_tree
+from paper_2603_03383_b200 import binding, synth
+from tests._cases import assert_close, make_tree, workspace
 from tests.test_gpu_attention_precision import _step_attention
 from tests.test_gpu_attention_range import _run
 
@@ -74,3 +74,27 @@ def test_references_move_in_any_group(T, G, D, step, column):
     out = _run(tree, q, ks, vs, [L] * B, Hkv, D, L + T + 5, step)
     for l in range(n_layers):
         assert_close(out[l], want[l], "layer %d" % l)
+
+
+@pytest.mark.parametrize("D,Hkv,B", [(64, 2, 3), (128, 4, 12), (64, 1, 40)])      # (more than 32 sequences are divided in several turns)
+def test_lengths_that_the_kernel_in_front_advances(D, Hkv, B):
+    """A one-layer call right behind the compaction that advances the lengths, from one number of groups to another."""
+    tb, tree = make_tree("rank_prior", 4, (), 64)
+    T, K, Hq = 64, 4, Hkv * 4
+    lens = [(128 * (2 + b % 5) - T - (b % 4)) for b in range(B)]
+    alen = [b % (K + 1) for b in range(B)]
+    Lcap, top = max(lens) + 8200, max(lens) + K + 1 + T      # (at head size 128 a call with room for long prefixes)
+    k, v = (synth.normal_bf16(T, s, (B, Hkv, Lcap, D), device=DEV) for s in (10, 50))
+    q = synth.normal_bf16(T, 90, (B, T, Hq, D), device=DEV)
+    nodes = torch.tensor([[0] + [j if j <= n else -1 for j in range(1, K + 1)] for n in alen], dtype=torch.int32, device=DEV)   # (rows stay where they are)
+    sl, status = torch.tensor(lens, dtype=torch.int32, device=DEV), torch.zeros(B, dtype=torch.int32, device=DEV)
+    after = [L + n + 1 for L, n in zip(lens, alen)]
+    want = ref.tree_attention(q.cpu(), k[:, :, :top].cpu(), v[:, :, :top].cpu(), torch.tensor(after, dtype=torch.int32), tb["mask"])
+    kp, vp = binding.cache_pointer_array([k], DEV), binding.cache_pointer_array([v], DEV)
+    ws, out = workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap), torch.full_like(q, 9.0)
+    accept = torch.tensor(alen, dtype=torch.int32, device=DEV)
+    binding.kv_compact_accepted(tree, kp, vp, 1, B, Hkv, D, k.stride()[:3], Lcap, sl, accept, nodes, status=status)
+    binding.tree_verify_attention(tree, q, k, v, sl, out, ws, status=status)
+    torch.cuda.synchronize()
+    assert binding.mtv_device_error(tree) == 0 and sl.tolist() == after and status.tolist() == [0] * B
+    assert_close(out, want)
