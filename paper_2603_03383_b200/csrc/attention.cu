@@ -74,12 +74,10 @@ constexpr int NB = 3;                 // tiles of scores
 constexpr float LOG2E = 1.4426950408889634f;
 // P goes to the tensor core as bf16, whose rounding is the largest error beside the output's own.  Where a reference that
 // follows the row's maximum makes the largest weights exact (they are 1), a fixed reference does not: P then has a second bf16
-// term, what the rounding of the first left.  At head size 64 in every group (O += P V is short there); at 128 in a piece's
-// first group, whose maximum is the reference, and in the second of a single row tile (a kernel with a reference for every other
-// group had two terms in both).  Rel. error against 64 bits with one term / two / a reference that follows the maximum: D = 64,
-// L = 128: .00235 / .00166 / .00214, L <= 5003: .00233 / .00166 / .00210; D = 128, L = 512: .00235 / .00204 / .00268.
-template <int D, bool PAIR>
-__host__ __device__ constexpr bool two_terms(int group) { return D == 64 || group == 0 || (!PAIR && group == 1); }
+// term, what the rounding of the first left: at head size 64 in every group (O += P V is short there), at 128 in the first
+// groups of a piece, of which the first has the reference for its maximum.  How many is for PieceWalk to say (two_term_groups).
+template <int D>
+__device__ __forceinline__ bool two_terms(int group, int n_two) { return D == 64 || group < n_two; }
 // tensor-memory columns: O, and three tiles of scores; P lies over its scores, each half of the keys over its own: keys 0-63
 // at columns 0-31, keys 64-127 at 64-95; in two terms each quarter over its own: keys 0-31 at columns 0-15, their second
 // terms at 16-31, and so on.
@@ -257,7 +255,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(AT_AUX_REGS));
     if (warp == W_TMA) {
         // ------------------------------------------------------------ the pair's pieces; this CTA's halves of K and V
-        PieceWalk<ITEM_COST, MERGE_COST> walk(p, team, lane);
+        // (the pair, or CTA, that has the last tile of an odd number of them)
+        PieceWalk<ITEM_COST, MERGE_COST> walk(p, team, lane, (blk | 1) >= p.n_tiles);
         // The work is divided while the kernel before this one ends, by the lengths that are there (a call that follows another has
         // nothing that changes them in between), and looked at again behind it: eight one-layer calls on ragged lengths take 291 us
         // instead of 314, at head size 64 164 instead of 172.
@@ -463,6 +462,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             if (lane == 0) free_piece(pi);
             const int cnt = __shfl_sync(0xffffffffu, d.cnt, 0);
             if (cnt == 0) break;
+            const int n_two = __shfl_sync(0xffffffffu, d.flags >> PIECE_TWO_SHIFT, 0);
             const int last_valid = d.L + p.T - (d.gb + cnt - 1) * AT_BN;       // keys of the piece's last group (or more than 128)
             const int last_steps = __shfl_sync(0xffffffffu, min(8, (last_valid + 15) / 16), 0);
             const uint32_t dq = ptx::desc_lo(sbase + (pi & 1) * SM::TILE, 16);
@@ -504,7 +504,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     else ptx::mma_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
                 };
                 const int steps = j == cnt - 1 ? last_steps : 8;
-                if (two_terms<D, PAIR>(j)) {
+                if (two_terms<D>(j, n_two)) {
                     if (D == 64 && steps == 8) {
 #pragma unroll
                         for (int kk = 0; kk < 16; ++kk) issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > 0 || kk > 0);
@@ -612,7 +612,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     if (j < first) continue;
                     const uint32_t t_p = t_s0 + (uint32_t)(j % NB) * 128;
 #pragma unroll 1
-                    for (int c = 0; c < (PAIR ? 2 : 4); ++c) {        // (both terms)
+                    for (int c = 0; c < 4; ++c) {        // (both terms)
                         ptx::tmem_ld16(t_p + c * 16, x);
                         ptx::tmem_ld_wait_for16(x);
 #pragma unroll
@@ -656,6 +656,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             const volatile AttnPiece &d = desc[pi % AT_PIECES];    // (freed at the end of the piece)
             const int cnt = d.cnt;
             if (cnt == 0 || *abort_flag) break;
+            const int n_two = d.flags >> PIECE_TWO_SHIFT;
             const int a_first = d.gb * AT_BN + hf * 64 - d.L;      // tree row of this half's first column in the first group
             m_used = -INFINITY;
             l = 0.f;
@@ -737,7 +738,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                         sum = (la.x + la.y) + (lb.x + lb.y);
                         return asked || !__any_sync(0xffffffffu, mine && sum > AT_SUM_LIMIT);
                     };
-                    if (D == 64 || (!PAIR && j == 1)) {
+                    if (two_terms<D>(j, n_two)) {
                         uint32_t pa[16], pb[16], ra[16], rb[16];
                         exp_quarter<true>(qa, sc2, nm2, la, lb, pa, ra);
                         exp_quarter<true>(qb, sc2, nm2, la, lb, pb, rb);
@@ -963,6 +964,7 @@ namespace {
 // Row tiles of a problem and the CTAs that work on it: at head size 128 items of more than one tile go to CTA pairs.
 struct AttnPlan {
     int npc, n_tiles, n_blk, teams;      // tree nodes per tile, tiles of an item, CTAs of a team, teams
+    int two_cuts;                        // see two_term_groups
     bool pair;
 };
 AttnPlan attn_plan(int T, int G, int D) {
@@ -973,6 +975,7 @@ AttnPlan attn_plan(int T, int G, int D) {
     a.n_blk = a.pair ? (a.n_tiles + 1) / 2 * 2 : a.n_tiles;
     const int sms = sm_count() < AT_MAX_CTAS ? sm_count() : AT_MAX_CTAS;
     a.teams = (a.pair ? sms / 2 * 2 : sms) / a.n_blk;
+    a.two_cuts = sms / ((a.n_tiles + 1) / 2);
     return a;
 }
 }  // namespace
@@ -1097,6 +1100,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
     p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_blk = a.n_blk; p.teams = a.teams;
+    p.n_tiles = a.n_tiles; p.two_cuts = a.two_cuts;
     p.gate = alongside ? *alongside : Gate{};
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;

@@ -27,7 +27,8 @@ struct AttnPiece {      // 32 bytes
     int layer, b, head, gb, cnt, L, flags, first;   // key groups [gb, gb + cnt); cnt = 0: no more pieces;
                                                     // first: first team that contributes to the item
 };
-constexpr int PIECE_PARTIAL = 1, PIECE_HEAD = 2;   // not a whole item; starts at the item's first group
+// flags: not a whole item; starts at the item's first group; from this bit on, how many groups have their weights in two terms
+constexpr int PIECE_PARTIAL = 1, PIECE_HEAD = 2, PIECE_TWO_SHIFT = 8;
 struct AttnMerge {      // a partial piece of this CTA, for the merge at the end
     int first, n, layer, b, head, pad;             // first contributing team, number of them
 };
@@ -52,6 +53,7 @@ struct AttnParams {
     int npc, R;              // tree nodes per tile (128 / G) and the rows they fill
     unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
     int n_blk, teams;        // CTAs of a team, teams
+    int n_tiles, two_cuts;   // row tiles of an item; see two_term_groups
     Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
 };
 
@@ -197,13 +199,15 @@ struct PieceWalk {
     const AttnParams &p;
     const int lane;
     const unsigned LH, teams, team;
+    const bool lone;                      // one row tile, or the last of an odd number of them
+    float two_rate = 0.f;                 // see two_term_groups
     int chunk = 0, len = 0, g = 0;        // lengths and group counts of sequences chunk .. chunk + 31, one per lane
     bool pad = false;
     unsigned u = 1, pos = 0, hi = 0, off = 0;
     int layer = 0, b = 0, head = 0, n_part = 0;
 
-    __device__ __forceinline__ PieceWalk(const AttnParams &p_, int team_, int lane_)
-        : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_) {}
+    __device__ __forceinline__ PieceWalk(const AttnParams &p_, int team_, int lane_, bool lone_)
+        : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_), lone(lone_) {}
     // (through L2: the lengths may be looked at before the kernel that writes them is complete, and again behind it)
     __device__ __forceinline__ int length(int at) const { return at < p.B ? __ldcg(p.seq_lens + at) : 0; }
     __device__ __forceinline__ void load_chunk(int b0, bool final) {
@@ -250,6 +254,7 @@ struct PieceWalk {
             if (!pad || LH * quotient(v_head, u) <= teams) break;
             if (++u > u_cut + 2) { pad = false; u = u_cut; }
         }
+        two_rate = __fdividef((float)p.two_cuts, (float)max(1u, pad ? LH * sum : LH * v_head));
         const unsigned v_layer = v_head * (unsigned)p.Hkv;
         pos = team * u;
         hi = min(pos + u, v_layer * (unsigned)p.n_layers);
@@ -280,6 +285,21 @@ struct PieceWalk {
             off = rem - (unsigned)head * gp;
         }
     }
+    // How many of a piece's groups have their weights in two terms at head size 128.  The error is that of the output's rounding
+    // and, independent of it and as large, that of the weights' rounding in the groups with one term: .00166 sqrt(1 + their
+    // share).  A division among all SMs, two row tiles to an SM, has more and shorter pieces than one among pairs, or one that
+    // leaves items whole, and has two terms in the first group of each of them (in two groups where an SM has a single row tile):
+    // the error must not show which of the two it is.  So a piece has one such group for each piece that two_cuts teams would
+    // make of it; parts of one are carried from item to item, spread evenly (golden ratio), and a tenth of one is added for what
+    // the spread misses.  (4208 drawn problems replayed: never a larger error than that of the finer division.)  Rel. error
+    // against 64 bits with the finer division / one group of every piece / as it is, 32 / 8 heads: L = 512, 4 layers .00203 /
+    // .00219 / .00166, 32 layers .00215 / .00220 / .00212, 8 layers of a single row tile .00185 / .00203 / .00166; L = 8192, 32
+    // layers .00234 / .00234 / .00234.  It costs 3 % of eight ragged one-layer calls (290 -> 299 us) and
+    // nothing that shows in a step of long or short prefixes.
+    __device__ __forceinline__ int two_term_groups(int cnt, unsigned item) const {
+        const float part = (float)((item * 2654435769u) >> 8) * (1.f / 16777216.f);
+        return min((1 + (int)((float)cnt * two_rate + part + 0.1f)) << (lone ? 1 : 0), cnt);
+    }
     // The next piece of the run (all lanes agree); false at its end.  A piece that is not a whole item goes down in merges, too.
     __device__ __forceinline__ bool next(AttnPiece &d, AttnMerge *merges, volatile int *n_merge) {
         while (pos < hi) {
@@ -289,7 +309,8 @@ struct PieceWalk {
             const unsigned r0 = min(off, gg), r1 = min(end, gg);
             d.layer = layer; d.b = b; d.head = head; d.gb = (int)r0; d.cnt = (int)(r1 - r0); d.L = L;
             const bool part = r1 - r0 < gg;
-            d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0);
+            d.flags = (part ? PIECE_PARTIAL : 0) | (r0 == 0 ? PIECE_HEAD : 0) |
+                      two_term_groups(d.cnt, ((unsigned)layer * (unsigned)p.B + (unsigned)b) * (unsigned)p.Hkv + (unsigned)head) << PIECE_TWO_SHIFT;
             d.first = (int)quotient(a, u);
             if (r1 > r0 && part && n_part < 2) {
                 if (lane == 0) {
