@@ -210,17 +210,20 @@ struct PieceWalk {
         : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_), lone(lone_) {}
     // (through L2: the lengths may be looked at before the kernel that writes them is complete, and again behind it)
     __device__ __forceinline__ int length(int at) const { return at < p.B ? __ldcg(p.seq_lens + at) : 0; }
+    // Key groups of a sequence.  0: it has no room for the tree's rows, or no rows at all (nothing here may wrap or become
+    // negative: the sums below are other sequences' positions); it is passed over, which report() says.
+    __device__ __forceinline__ int groups(int l) const { return l > -p.T && l <= p.Lcap - p.T ? (l + p.T + AT_BN - 1) / AT_BN : 0; }
     __device__ __forceinline__ void load_chunk(int b0, bool final) {
         chunk = b0;
         len = final || p.B <= 32 ? length(b0 + lane) : 0;       // (more than 32: read more than once, so not while they may change)
         if (!final) len = min(max(len, 0), p.Lcap);
-        g = b0 + lane < p.B && len + p.T <= p.Lcap ? (len + p.T + AT_BN - 1) / AT_BN : 0;   // 0: does not fit, see report
+        g = b0 + lane < p.B ? groups(len) : 0;
     }
     // Were the lengths that the work was divided by the ones that are there now?
     __device__ __forceinline__ bool still_so() const { return p.B <= 32 && __all_sync(0xffffffffu, length(lane) == len); }
     __device__ __forceinline__ void report() const {
         if (blockIdx.x == 0 && p.status)
-            for (int b = lane; b < p.B; b += 32) p.status[b] = length(b) + p.T <= p.Lcap ? MTV_OK : MTV_ERR_CAPACITY;
+            for (int b = lane; b < p.B; b += 32) p.status[b] = groups(length(b)) > 0 ? MTV_OK : MTV_ERR_CAPACITY;
     }
     __device__ __forceinline__ unsigned padded(unsigned gg) const { return gg == 0 ? 0u : pad ? quotient(gg + u - 1, u) * u : gg + COST; }
     // final: false = with lengths that may still change

@@ -98,3 +98,29 @@ def test_lengths_that_the_kernel_in_front_advances(D, Hkv, B):
     torch.cuda.synchronize()
     assert binding.mtv_device_error(tree) == 0 and sl.tolist() == after and status.tolist() == [0] * B
     assert_close(out, want)
+
+
+@pytest.mark.parametrize("T,bad,B", [
+    (64, [2**31 - 4, -64, -65, -500, -2**31, 2**31 - 64], 10),     # sums with T that wrap, or leave no key
+    (29, [-29, 3000, 2**31 - 1], 40),                            # more than 32 sequences
+])
+def test_lengths_that_leave_no_keys(T, bad, B):
+    """Such a sequence is reported and passed over, and the others' share of the work does not depend on it."""
+    tb, tree = make_tree("rank_prior", 4, (), T)
+    Hq, Hkv, D, Lcap = 8, 2, 64, 1000
+    lens = [17 * b + 1 for b in range(B)]
+    for i, x in enumerate(bad):
+        lens[(3 * i + 1) % B] = x
+    good = [b for b in range(B) if 0 <= lens[b] <= Lcap - T]
+    k, v = (synth.normal_bf16(T, s, (B, Hkv, Lcap, D), device=DEV) for s in (10, 50))
+    q = synth.normal_bf16(T, 90, (B, T, Hq, D), device=DEV)
+    want = ref.tree_attention(q[good].cpu(), k[good].cpu(), v[good].cpu(), torch.tensor([lens[b] for b in good], dtype=torch.int32), tb["mask"])
+    sl, status = torch.tensor(lens, dtype=torch.int32, device=DEV), torch.full((B,), 7, dtype=torch.int32, device=DEV)
+    out, ws = torch.full_like(q, 9.0), workspace(tree, B, 0, 0, Hq, Hkv, D, Lcap)
+    for _ in range(2):       # (counters are back at zero behind the first call)
+        binding.tree_verify_attention(tree, q, k, v, sl, out, ws, status=status)
+        torch.cuda.synchronize()
+        assert binding.mtv_device_error(tree) == 0
+        assert status.tolist() == [0 if b in good else binding.MTV_ERR_CAPACITY for b in range(B)]
+        assert_close(out[good], want)
+        assert all((out[b] == 9.0).all() for b in range(B) if b not in good)
