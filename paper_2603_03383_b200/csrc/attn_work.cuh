@@ -208,8 +208,8 @@ struct PieceWalk {
 
     __device__ __forceinline__ PieceWalk(const AttnParams &p_, int team_, int lane_, bool lone_)
         : p(p_), lane(lane_), LH((unsigned)p_.n_layers * (unsigned)p_.Hkv), teams((unsigned)p_.teams), team((unsigned)team_), lone(lone_) {}
-    // (through L2: the lengths may be looked at before the kernel that writes them is complete, and again behind it)
-    __device__ __forceinline__ int length(int at) const { return at < p.B ? __ldcg(p.seq_lens + at) : 0; }
+    // (the lengths may be looked at before the kernel that writes them is complete, and again behind it)
+    __device__ __forceinline__ int length(int at) const { return at < p.B ? ld_relaxed(p.seq_lens + at) : 0; }
     // Key groups of a sequence.  0: it has no room for the tree's rows, or no rows at all (nothing here may wrap or become
     // negative: the sums below are other sequences' positions); it is passed over, which report() says.
     __device__ __forceinline__ int groups(int l) const { return l > -p.T && l <= p.Lcap - p.T ? (l + p.T + AT_BN - 1) / AT_BN : 0; }

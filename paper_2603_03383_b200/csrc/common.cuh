@@ -117,7 +117,9 @@ struct PerDeviceOnce {
 // Programmatic dependent launch: the kernel may be set up while the previous kernel of the stream runs, from the moment all
 // of that kernel's blocks have executed let_next_start() or ended.  What is guaranteed is that previous_done() returns when
 // the previous kernel is complete and its writes are visible.  Rules of the kernels launched so:
-//   - whatever the previous kernel (or one before it) writes is touched only behind previous_done();
+//   - whatever the previous kernel (or one before it) writes is touched only behind previous_done().  One exception: the tree
+//     attention looks at the lengths before that, by relaxed loads, to divide its work by them; it bounds what it saw, writes
+//     nothing by it, and compares it behind previous_done() (or the gate) with a second look, dividing anew where they differ;
 //   - every block executes previous_done() before it ends, early or late: a kernel that is complete then implies that
 //     all before it are;
 //   - what was written before the heads (weights, queries, caches, lengths, logits) may be read by the heads' second kernel
