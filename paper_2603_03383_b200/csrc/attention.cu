@@ -961,6 +961,18 @@ bool tensor_map_bf16(CUtensorMap *map, const void *base, int rank, const cuuint6
 }
 
 namespace {
+// Layers of a launch: positions in the common address space of its groups are 32 bits wide (PieceWalk: an item counts its groups
+// and ITEM_COST, or, with fewer items than teams, whole pieces; the last team's run may end a few groups behind the last item).
+// A single layer is not looked at: 2^32 positions are the K and V of far more memory than a device has.
+constexpr double ADDRESS_LIMIT = 4e9;
+constexpr int layers_per_launch(int n_layers, double items, int groups) {
+    int n = n_layers == 1 ? 1 : AT_MAX_LAYERS;
+    while (n > 1 && n * items * (groups + ITEM_COST) > ADDRESS_LIMIT) n /= 2;
+    return n;
+}
+// one group per item: every item takes 1 + ITEM_COST positions, and they stay below 2^32 whatever the number of items
+static_assert(layers_per_launch(AT_MAX_LAYERS, ADDRESS_LIMIT / (AT_MAX_LAYERS * (1 + ITEM_COST)), 1) == AT_MAX_LAYERS &&
+              layers_per_launch(AT_MAX_LAYERS, ADDRESS_LIMIT / (AT_MAX_LAYERS * (1 + ITEM_COST)) * 1.01, 1) == AT_MAX_LAYERS / 2, "address space");
 // Row tiles of a problem and the CTAs that work on it: at head size 128 items of more than one tile go to CTA pairs.
 struct AttnPlan {
     int npc, n_tiles, n_blk, teams;      // tree nodes per tile, tiles of an item, CTAs of a team, teams
@@ -1104,10 +1116,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.gate = alongside ? *alongside : Gate{};
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;
-    // positions in the common address space of a launch's groups are 32 bits wide
-    const double layer_len = (double)B * Hkv * ((Lcap + AT_BN - 1) / AT_BN + 1);
-    int per_launch = n_layers == 1 ? 1 : AT_MAX_LAYERS;
-    while (per_launch > 1 && per_launch * layer_len > 4e9) per_launch /= 2;
+    const int per_launch = layers_per_launch(n_layers, (double)B * Hkv, (Lcap + AT_BN - 1) / AT_BN);
     for (int l = 0; l < n_layers; l += per_launch) {
         if (l > 0) p.gate = Gate{};          // (it shares the counters and the workspace with the launch before)
         p.n_layers = n_layers - l < per_launch ? n_layers - l : per_launch;
