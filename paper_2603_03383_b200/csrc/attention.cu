@@ -91,7 +91,9 @@ struct AttnSmem {
     static constexpr uint32_t SLOT = TILE / (PAIR ? 2 : 1);    // this CTA's part of a K group (64 keys of a pair) or V group (64 columns)
     static constexpr uint32_t K_HALF = PAIR ? 64 * 128 : HALF; // the next 64 columns of K
     static constexpr int STAGES = 10 * 16384 / SLOT;
-    // The slot keeper may wait for K of three groups on: the slot it comes into was given back two groups ago.
+    // The slot keeper's word on a group's PV takes in the K of the scores behind it, three groups on, where the slot that this K
+    // comes into was given back two groups ago.  With five slots it is requested only when the scores of the next group but one
+    // are complete, and PV need not wait for that: the issuing warp waits for it, behind PV.
     static constexpr bool K_AHEAD = STAGES >= 2 * NB + 4;
     static constexpr uint32_t OFF_RING = 2 * TILE;         // two query tiles: the next piece's, and where output rows are staged
     static constexpr uint32_t OFF_X = OFF_RING + STAGES * SLOT;
@@ -1025,9 +1027,11 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
 //      3 sequences, 16 / 4 heads, capacity 20000:   38 / 33    25 / 27    18 / 22    15 / 19
 //     16 sequences, 32 / 8 heads, capacity 32768:  423 / 350  200 / 209  112 / 112   72 / 83
 //     16 sequences, 32 / 8 heads, capacity  4224:   59 / 62    41 / 52    31 / 40    27 / 37
-// With more blocks than pairs the pairs are all busy, longest sequence first, and what the even division gains in a full cache it
-// loses in one that is a quarter full: pairs.  With fewer, the even division is taken where the estimate for a full cache (us
-// per group on a pair and on an SM, start and end) is better by a tenth; such a call on a nearly empty cache loses up to 10 us.
+// With more blocks than pairs the pairs are all busy, longest sequence first: pairs.  With fewer, the even division is taken where
+// the estimate for a full cache (us per group on a pair and on an SM, start and end; fitted to an even division with two row tiles
+// per CTA and not fitted again since) is better by a tenth.  Of the rows above that is the even division for the first three, which
+// loses up to 3 us on a nearly empty cache, and pairs for the others, which lose 5 us in the full cache of the fourth and 73 in
+// that of the fifth, and gain up to 11 elsewhere.  (The rows were taken with one group in two terms per piece: two_term_groups.)
 static bool pair_kernel_is_better(int T, int G, int B, int Hkv, int Lcap) {
     int n_blk = 1;
     const int ns = attn_pair_plan(T, G, B, Hkv, Lcap, &n_blk);

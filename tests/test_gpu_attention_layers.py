@@ -15,7 +15,7 @@ DEV = "cuda"
 @pytest.mark.parametrize("T,Hq,Hkv,D,lens,n_layers", [
     (64, 8, 2, 128, [63], 2),                  # one group and the tree across a group boundary
     (64, 8, 2, 128, [64, 0, 129], 5),          # last group exactly full; an empty prefix; ragged
-    (29, 4, 1, 128, [700], 3),                 # one row tile: both streams on the same rows, pieces of one group
+    (29, 4, 1, 128, [700], 3),                 # one row tile, pieces of one group
     (128, 16, 2, 128, [1000, 1], 2),           # four row blocks
     (64, 7, 1, 128, [300, 517], 9),            # rows that belong to nobody
     (65, 8, 8, 64, [127, 128], 4),

@@ -1,5 +1,4 @@
-"""Scores far above those of a piece's first group, in the columns whose exponentials are polynomials and in the others, and
-scores that are not numbers."""
+"""Scores far above those of a piece's first group, in every part of a group's columns, and scores that are not numbers."""
 import math
 
 import pytest
