@@ -15,7 +15,7 @@
 // Pieces that are not whole items leave O / l (fp32: where an item is cut must not show in its precision) and (m, l) in the
 // workspace; at the end of the launch the CTAs that share a tile meet at a counter and each combines a slice of its rows.
 // They all do so when the device is this launch's alone (the grid never exceeds one CTA per SM), but nothing depends on it:
-// a warp that has waited for a millisecond leaves its slice to the last one to leave and makes room.
+// a CTA that has waited for a millisecond leaves its slice to the last one to leave and makes room.
 //
 // PAIR (head size 128, more than one row tile): the CTAs of a team are cta_group::2 pairs, whose MMAs (M = 256) read half of
 // a group's K and V from either CTA's shared memory, so that a tile and a group cost an SM 32 KB.  Else a CTA has K and V to
@@ -35,7 +35,8 @@
 //   warp 16           issues the MMAs (odd CTA of a pair: the slot keeper)
 //   warp 17           derives the pieces and requests this CTA's part of K and V groups (TMA) through a ring
 //   warp 18           the slot keeper (odd CTA: tells the even one what has landed, V rows past the last key cleared)
-//   warp 19           requests the query tiles; clears the V rows past the last key (their P is 0, but 0 * NaN would poison O)
+//   warp 19           requests the query tiles; clears the V rows past the last key (their P is 0, but 0 * NaN would poison O);
+//                     meets the other contributors of an item
 // The slot keeper follows the scores: it gives ring slots back as soon as the MMAs that read them are complete, and puts in its
 // word for a group's PV when V, and K of the scores behind it, are there.  So the issuing warp has one barrier to test per
 // group: a test costs it about a hundred cycles, and the tensor core has only some two MMAs queued.
@@ -111,7 +112,9 @@ struct AttnSmem {
     static constexpr int BAR_PC_EMPTY = BAR_PC_FULL + AT_PIECES;
     static constexpr int BAR_XM = BAR_PC_EMPTY + AT_PIECES;    // [4] the four warps of a row quarter: references
     static constexpr int BAR_XO = BAR_XM + 4;                  // [4] results
-    static constexpr int BAR_DRAIN = BAR_XO + 4;
+    static constexpr int BAR_OUT = BAR_XO + 4;                 // a partial result is written by the sixteen warps
+    static constexpr int BAR_GO = BAR_OUT + 1;                 // [2] all partial results of an item are there (or the slice is left)
+    static constexpr int BAR_DRAIN = BAR_GO + 2;
     static constexpr int BAR_COUNT = BAR_DRAIN + 1;
     static constexpr uint32_t OFF_DESC = OFF_BAR + (BAR_COUNT * 8 + 15) / 16 * 16;
     static constexpr uint32_t OFF_MISC = OFF_DESC + AT_PIECES * 32;
@@ -182,7 +185,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + SM::OFF_MISC + 48);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 52);
     volatile int *n_merge = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 56);      // partial pieces of this CTA
-    int *left_items = reinterpret_cast<int *>(smem + SM::OFF_MISC + 60);                     // of this CTA's: bit i, merges[i]
+    volatile int *left_items = reinterpret_cast<volatile int *>(smem + SM::OFF_MISC + 60);   // of this CTA's: bit i, merges[i]; bit 2 + i: slice left
 
     // CTA blk of the team has row tile blk (blk = 2 block + rank)
     const int team = (int)blockIdx.x / p.n_blk, blk = (int)blockIdx.x % p.n_blk;
@@ -214,6 +217,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             ptx::mbar_init(bar(SM::BAR_XO + i), 4);
             ptx::sts_u32(sbase + SM::OFF_ASK + i * 4, 0u);
         }
+        ptx::mbar_init(bar(SM::BAR_OUT), AT_SOFTMAX_WARPS);
+        for (int i = 0; i < 2; ++i) ptx::mbar_init(bar(SM::BAR_GO + i), 1);
         ptx::mbar_init(bar(SM::BAR_DRAIN), 1);
         ptx::fence_mbar_init();
         *abort_flag = 0;
@@ -323,6 +328,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         // ------------------------------------------------------------ query tiles; even CTA: V rows past the last key
         (void)begin();
         uint32_t seq = 0, parity = 0;         // parity: bit s = phase of tail barrier s
+        int n_out = 0;                        // partial results
+        if (lane < 2) p.left[blockIdx.x * 2 + lane] = 0;     // (released with the first of them)
         AttnPiece d, e;
         bool ok = true;
         auto request_q = [&](int pi, const AttnPiece &x) {
@@ -364,9 +371,52 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_KV_FULL + s));
             }
+            if (d.flags & PIECE_PARTIAL) {
+                // The softmax warps have written their parts: one fence and one word for all of them.  (A release by every
+                // warp: 16 fences one after the other, and 16 times the polls and additions at the counters.)
+                ok = ptx::mbar_wait(bar(SM::BAR_OUT), n_out & 1);
+                if (!ok) break;
+                ++n_out;
+                if (lane == 0) {
+                    __threadfence();
+                    asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(merge_counter(p, d.first, blk)) : "memory");
+                }
+            }
             seq += 2u * (uint32_t)d.cnt;
             d = e;
         }
+        // The items that this CTA shares with others: a look at the counter until all parts are there, then the softmax warps
+        // combine this CTA's slice.
+        if (ok && !*abort_flag && lane == 0) {
+            const int n_m = *n_merge;
+            for (int i = 0; i < n_m; ++i) {
+                const int n = merges[i].n, first = merges[i].first;
+                int32_t *c = merge_counter(p, first, blk);
+                const long long t0 = clock64();
+                bool full;
+                while (!(full = ld_acquire(c) >= n))
+                    if (clock64() - t0 > AT_MERGE_WAIT) break;
+                if (!full) {
+                    p.left[blockIdx.x * 2 + (team == first ? 1 : 0)] = 1;
+                    *left_items |= 4 << i;
+                    __threadfence();
+                }
+                ptx::mbar_arrive(bar(SM::BAR_GO + i));
+                const int before = atomicAdd(c + AT_DEPART, full ? 1 : 0x10001), marked = (before >> 16) + (full ? 0 : 1);
+                // The last one to leave: its CTA does what others left, all parts and all marks being complete, and the counters go
+                // back to zero (nobody looks at them any more; the next call cannot start before this kernel has ended).
+                if ((before & 0xffff) == n - 1) {
+                    if (marked) {
+                        (void)ld_acquire(c);
+                        (void)ld_acquire(c + AT_DEPART);
+                        *left_items |= 1 << i;
+                    }
+                    c[0] = 0;
+                    c[AT_DEPART] = 0;
+                }
+            }
+        }
+        __syncwarp();
         if (!ok && lane == 0) give_up();
     } else if (PAIR && warp == W_RELAY && rank == 1) {
         // ------------------------------------------------------------ odd CTA: what has landed, V rows past the last key cleared
@@ -574,10 +624,10 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         const uint32_t t_o = lane_base + TM_O + (e * 2 + hf) * (D / 4);        // this thread's columns of O
         auto x_at = [&](int s, int h) { return sbase + SM::OFF_X + (uint32_t)((s * 2 + h) * 128 + row) * 4u; };   // [set][half][row]
         const uint32_t ask_at = sbase + SM::OFF_ASK + (uint32_t)qd * 4u;
-        if (lane < 2) p.left[((unsigned)blockIdx.x * 2 + lane) * AT_SOFTMAX_WARPS + warp] = 0;      // (released with the arrivals)
         constexpr uint32_t hidden = NEG ? 0x7f800000u : 0xff800000u;   // times the scale: -inf
         uint32_t phases = 0;                      // bit 0: exchange of references, 1: of results, 4-6: the tiles of scores
         bool ok = true;
+        int n_part = 0;                           // partial results written
         float m_used = -INFINITY, l = 0.f;
         auto meet = [&]() {                       // the four warps of these rows
             __syncwarp();
@@ -806,9 +856,9 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                         *slab_o<D>(p, blockIdx.x, slab, row, (e * 2 + hf) * (D / 16) + c) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
                     if (hf == 0 && e == 0) *slab_ml(p, blockIdx.x, slab, row) = make_float2(m_used, l_all);
                 }
-                // this warp's part is written: tell those that share the item (each warp counts for itself)
+                ++n_part;
                 __syncwarp();
-                if (lane == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(p.arrive + d.first * p.n_blk + blk) : "memory");
+                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_OUT));
             } else {
                 // Output rows are staged in the piece's query tile (each warp for itself, 16-byte chunks swizzled) and leave as
                 // runs of 32 or 64 bytes.
@@ -841,40 +891,12 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             }
         }
         if (!ok && lane == 0) give_up();
-        // ---- merge of the items this CTA shares with others.  Every warp comes here when its own pieces are done.
-        const int n_m = *n_merge;
+        // ---- the items that this CTA shares with others
 #pragma unroll 1
-        for (int i = 0; i < n_m; ++i) {
-            const AttnMerge m = merges[i];
-            const int ctr = m.first * p.n_blk + blk, all = m.n * AT_SOFTMAX_WARPS, c0 = team - m.first;
-            int departed = 0, full = 0;
-            if (lane == 0) {
-                // relaxed polls (a round trip to L2 each), one acquire when the counter is full
-                int32_t *c = p.arrive + ctr;
-                const long long t0 = clock64();
-                while (!(full = *reinterpret_cast<volatile int32_t *>(c) >= all))
-                    if (clock64() - t0 > AT_MERGE_WAIT) break;
-                if (full) {
-                    (void)ld_acquire(c);
-                    departed = atomicAdd(p.depart + ctr, 1);         // (its round trip overlaps the merge)
-                } else {
-                    p.left[((unsigned)blockIdx.x * 2 + (c0 == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + warp] = 1;
-                    __threadfence();
-                    departed = atomicAdd(p.depart + ctr, 0x10001) + 0x10000;
-                }
-            }
-            if (__shfl_sync(0xffffffffu, full, 0)) merge_slice<D>(p, m, c0, warp, blk, lane);
-            // The last warp to leave: its CTA does what others left, all parts and all marks being complete, and the counters go
-            // back to zero (nobody polls them any more; the next call cannot start before this kernel has ended).
-            if (lane == 0 && (departed & 0xffff) == all - 1) {
-                if (departed >> 16) {
-                    (void)ld_acquire(p.arrive + ctr);
-                    (void)ld_acquire(p.depart + ctr);
-                    atomicOr(left_items, 1 << i);
-                }
-                p.arrive[ctr] = 0;
-                p.depart[ctr] = 0;
-            }
+        for (int i = 0; i < n_part && ok; ++i) {
+            const MergeSlice<D> slice(p, merges[i], team - merges[i].first);
+            if (!ptx::mbar_wait(bar(SM::BAR_GO + i), 0)) { give_up(); break; }
+            if (!((*left_items >> (2 + i)) & 1)) slice.run(p, merges[i], warp * 32 + lane, blk);
         }
     }
     __syncwarp();
@@ -884,7 +906,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     if (PAIR) ptx::cluster_arrive();
     if (warp < AT_SOFTMAX_WARPS && *left_items)       // (the other warps have too few registers for it)
         for (int i = 0; i < 2; ++i)
-            if ((*left_items >> i) & 1) merge_left<D>(p, merges[i], blk, warp, lane);
+            if ((*left_items >> i) & 1) merge_left<D>(p, merges[i], blk, warp * 32 + lane);
     __syncwarp();
     if (PAIR) ptx::cluster_wait();
     ptx::tc_fence_after();
@@ -1004,7 +1026,7 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
     const size_t slabs = (size_t)a.teams * a.n_blk * 2;
     w.ml_off = align_up(slabs * 128 * D * sizeof(float), 256);
     w.left_off = align_up(w.ml_off + slabs * 128 * sizeof(float2), 256);
-    w.total = align_up(w.left_off + slabs * AT_SOFTMAX_WARPS * sizeof(int32_t), 256);
+    w.total = align_up(w.left_off + slabs * sizeof(int32_t), 256);
     if (attn_pair_eligible(D, Hq / Hkv)) {
         int n_blk = 1;
         const int ns = attn_pair_plan(t->T, Hq / Hkv, B, Hkv, Lcap, &n_blk);
@@ -1112,7 +1134,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.ws_o = reinterpret_cast<uint4 *>((char *)ws + Lw.o_off);
     p.ws_ml = reinterpret_cast<float2 *>((char *)ws + Lw.ml_off);
     p.left = reinterpret_cast<int32_t *>((char *)ws + Lw.left_off);
-    p.arrive = tree->d_counters; p.depart = tree->d_counters + AT_MAX_CTAS;
+    p.counters = tree->d_counters;
     p.scale_log2 = (scale == 0.f ? 1.f / sqrtf((float)D) : scale) * LOG2E;
     p.B = B; p.T = tree->T; p.G = Hq / Hkv; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
     p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_blk = a.n_blk; p.teams = a.teams;

@@ -66,7 +66,7 @@ constexpr uint32_t TC_SMEM_BYTES = 1024 + TC_OFF_ML + TC_ML_BYTES;
 static_assert(TC_SMEM_BYTES <= 227 * 1024, "shared memory budget");
 constexpr float TC_RESCALE_THRESHOLD = 8.f;
 constexpr int TC_MAX_SPLITS = 32;
-constexpr int TC_MAX_COUNTERS = 256;   // merge counters in the tree object: one per (query block, CTA rank)
+constexpr int TC_MAX_COUNTERS = MERGE_COUNTERS;   // one per (query block, CTA rank)
 
 // tensor-memory columns: S buffer b of stream t at 128 b + 64 t (P over its first 32 columns), O of stream t at 256 + 128 t
 constexpr uint32_t TM_S = 0, TM_O = 256;
@@ -102,7 +102,7 @@ struct TcParams {
     __nv_bfloat16 *out;    // [B][T][Hq][128]
     __nv_bfloat16 *ws_o;   // [query blocks][nsplit][256 rows][128] partial O / l (only when nsplit > 1)
     float2 *ws_ml;         // [query blocks][nsplit][256] partial (m, l)
-    int32_t *arrive, *depart;   // [query blocks][2] merge counters, zero between calls
+    int32_t *counters;     // [query blocks][2] merge counters, zero between calls
     int32_t *status;       // [B] or null
     const int32_t *order;  // [B] sequences by descending length, or null: grid index z -> sequence
     int32_t *dev_error;
@@ -598,7 +598,7 @@ tree_attn_pair_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_co
             // ---- publish this split's rows, then combine a slice of the rows of all splits
             if (st == 0) __stcg(p.ws_ml + (slab0 + split) * 256 + slab_row0 + row, make_float2(m_all, l_all));
             softmax_sync();   // every softmax thread's stores precede the release below
-            int32_t *arrive = p.arrive + grp * 2 + rank, *depart = p.depart + grp * 2 + rank;
+            int32_t *arrive = p.counters + (grp * 2 + rank) * MERGE_STRIDE, *depart = arrive + MERGE_STRIDE / 2;
             if (threadIdx.x == 0) {
                 __threadfence();
                 asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(arrive) : "memory");
@@ -750,7 +750,7 @@ int launch_tree_attn_pair(const mtv_tree *tree, int B, int Hq, int Hkv, const __
     TcParams p;
     p.seq_lens = seq_lens; p.anc = tree->d_anc; p.out = out; p.status = status; p.dev_error = tree->d_error;
     p.ws_o = reinterpret_cast<__nv_bfloat16 *>(ws_o); p.ws_ml = reinterpret_cast<float2 *>(ws_ml);
-    p.arrive = tree->d_counters; p.depart = tree->d_counters + TC_MAX_COUNTERS;
+    p.counters = tree->d_counters;
     p.scale_log2 = scale_log2;
     p.T = T; p.G = G; p.Hq = Hq; p.Hkv = Hkv; p.Lcap = Lcap;
     p.nsplit = attn_pair_plan(T, G, B, Hkv, Lcap, &p.n_blk);

@@ -9,14 +9,15 @@ constexpr int AT_BN = 128;            // keys per group
 constexpr int AT_THREADS = 640;
 constexpr int AT_SOFTMAX_WARPS = 16;
 constexpr int AT_PIECES = 4;          // piece descriptors in flight
-// How long a warp waits for the others of an item, in cycles.  In the bounds-checking build it looks once: nearly all slices
-// are then left to the last warp.
+// How long a CTA waits for the others of an item, in cycles.  In the bounds-checking build it looks once: nearly all slices
+// are then left to the last one.
 #ifdef MTV_DEBUG_BOUNDS
 constexpr long long AT_MERGE_WAIT = 0;
 #else
 constexpr long long AT_MERGE_WAIT = 2000000;
 #endif
-constexpr int AT_MAX_CTAS = 256;      // merge counters in the tree object: one pair per CTA
+constexpr int AT_MAX_CTAS = MERGE_COUNTERS;   // a pair of merge counters per CTA (the first of a team's, for the item it begins)
+constexpr int AT_DEPART = 16;         // ints from a CTA's first counter to its second
 constexpr int AT_MAX_LAYERS = 64;     // layers per launch (two tensor maps each in the kernel's parameters)
 // registers per thread: 96 at launch, moved from the four auxiliary warps to the sixteen softmax warps
 constexpr int AT_LAUNCH_REGS = 96, AT_SOFTMAX_REGS = 104, AT_AUX_REGS = 64;
@@ -44,8 +45,8 @@ struct AttnParams {
     __nv_bfloat16 *out;      // [layers][B][T][Hq][D]
     uint4 *ws_o;             // [CTA][2 slabs][D / 4 chunks][128 rows] 16-byte chunks of O / l, fp32
     float2 *ws_ml;           // [CTA][2 slabs][128 rows] (m, l)
-    int32_t *left;           // [CTA][2 slabs][16 warps] 1: the warp's slice of the item is left to the last one
-    int32_t *arrive, *depart;   // [CTA] merge counters, zero between calls; depart counts slices left in its upper half
+    int32_t *left;           // [CTA][2 slabs] 1: the CTA's slice of the item is left to the last one
+    int32_t *counters;       // merge counters, zero between calls; the second one counts slices left in its upper half
     int32_t *status;         // [B] or null
     int32_t *dev_error;
     float scale_log2;
@@ -116,70 +117,85 @@ __device__ __forceinline__ float2 *slab_ml(const AttnParams &p, int cta, int sla
     return p.ws_ml + ((unsigned)cta * 2 + slab) * 128 + r;
 }
 
-// Rows of a tile that is shared between CTAs: contributor c0 combines its share of them, a thread per 16-byte chunk of the output,
-// with the loads of several contributors in flight.  This is warp w's part of it.
+// The counters that the contributors of an item meet at: of its first contributor, for row tile blk.
+__device__ __forceinline__ int32_t *merge_counter(const AttnParams &p, int first, int blk) {
+    return p.counters + (first * p.n_blk + blk) * MERGE_STRIDE;
+}
+// Rows of a tile that is shared between CTAs: contributor c0 combines its share of them, a thread per VC 16-byte chunks of a row, with
+// the loads of NS contributors in flight.  All CTAs do this at the same time, and L2 gives some 20 bytes per cycle and SM then, so the
+// bytes count more than the round trips: with five contributors or a single chunk at a time (its (m, l) are a third of the
+// bytes) eight one-layer calls on ragged lengths take 306 and 343 us instead of 285.
 template <int D>
-__device__ __forceinline__ void merge_slice(const AttnParams &p, const AttnMerge &m, int c0, int w, int blk, int lane) {
-    constexpr int VC = 2, NS = 3;                        // chunks per thread and contributor; contributors at a time
-    const int per = (p.R + m.n - 1) / m.n, r_begin = c0 * per;
-    const int n_my = max(0, min(p.R, r_begin + per) - r_begin);
-    const unsigned inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;    // e / n_my for e < 2048, n_my <= 128
-    uint4 *dst = item_out<D>(p, m.layer, m.b, m.head);
+struct MergeSlice {
+    static constexpr int VC = 2, NS = 3, NT = D / 4 / VC;    // (VC = 2: 16 bytes of output)
+    int r_begin, n_my;
+    unsigned inv_n;                                      // e / n_my = (e * inv_n) >> 20 for e < 2048, n_my <= 64
+    __device__ __forceinline__ MergeSlice(const AttnParams &p, const AttnMerge &m, int c0) {
+        const int per = (p.R + m.n - 1) / m.n;           // (m.n >= 2)
+        r_begin = c0 * per;
+        n_my = max(0, min(p.R, r_begin + per) - r_begin);
+        inv_n = n_my > 0 ? ((1u << 20) + n_my - 1) / n_my : 0;
+    }
+    __device__ __forceinline__ void run(const AttnParams &p, const AttnMerge &m, int thread, int blk) const {
+        uint4 *dst = item_out<D>(p, m.layer, m.b, m.head);
 #pragma unroll 1
-    for (int e = w * 32 + lane; e < n_my * (D / 8); e += AT_SOFTMAX_WARPS * 32) {
-        const int c = (int)(((unsigned)e * inv_n) >> 20), r = r_begin + e - c * n_my;
-        float acc[8], mm = -INFINITY, wsum = 0.f;
+        for (int e = thread; e < n_my * NT; e += AT_SOFTMAX_WARPS * 32) {
+            const int c = (int)(((unsigned)e * inv_n) >> 20), r = r_begin + e - c * n_my;
+            float acc[4 * VC], mm = -INFINITY, wsum = 0.f;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+            for (int k = 0; k < 4 * VC; ++k) acc[k] = 0.f;
 #pragma unroll 1
-        for (int s0 = 0; s0 < m.n; s0 += NS) {
-            float2 ml[NS];
-            uint4 v[NS][VC];
+            for (int s0 = 0; s0 < m.n; s0 += NS) {
+                float2 ml[NS];
+                uint4 v[NS][VC];
 #pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                const int s = min(s0 + k, m.n - 1), cta = (m.first + s) * p.n_blk + blk;
-                const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
-                ml[k] = __ldcg(slab_ml(p, cta, sl, r));
+                for (int k = 0; k < NS; ++k) {
+                    const int s = s0 + k, cta = (m.first + s) * p.n_blk + blk;
+                    const int sl = s == 0 ? 1 : 0;       // the first contributor's piece begins the item
+                    ml[k] = make_float2(-INFINITY, 0.f);
 #pragma unroll
-                for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, r, c * VC + q));
-                if (s0 + k >= m.n) ml[k] = make_float2(-INFINITY, 0.f);
-            }
-            float mc = mm;
+                    for (int q = 0; q < VC; ++q) v[k][q] = make_uint4(0u, 0u, 0u, 0u);
+                    if (s < m.n) {
+                        ml[k] = __ldcg(slab_ml(p, cta, sl, r));
 #pragma unroll
-            for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
-            const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
-            mm = mc;
-            wsum *= resc;
+                        for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, r, c * VC + q));
+                    }
+                }
+                float mc = mm;
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[k] *= resc;
+                for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
+                const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
+                mm = mc;
+                wsum *= resc;
 #pragma unroll
-            for (int k = 0; k < NS; ++k) {
-                const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
-                wsum += wt;
+                for (int k = 0; k < 4 * VC; ++k) acc[k] *= resc;
 #pragma unroll
-                for (int q = 0; q < VC; ++q) {
-                    const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
+                for (int k = 0; k < NS; ++k) {
+                    const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
+                    wsum += wt;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
+                    for (int q = 0; q < VC; ++q) {
+                        const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
+                    }
                 }
             }
+            const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
+            const int o = out_row(p, blk, r);
+            if (o >= 0)
+                dst[o * (D / 8) + c] =
+                    make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
+                               pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
         }
-        const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
-        const int o = out_row(p, blk, r);
-        if (o >= 0)
-            dst[o * (D / 8) + c] =
-                make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
-                           pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
     }
-}
-// The slices that warps left, of one item, by the softmax warps of the CTA whose warp was the last to leave it.  (Out of the way of the
+};
+// The slices that CTAs left, of one item, by the softmax warps of the CTA that was the last to leave it.  (Out of the way of the
 // usual case, whose registers it must not touch.)
 template <int D>
-static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, int warp, int lane) {
-    for (int u = warp; u < m.n * AT_SOFTMAX_WARPS; u += AT_SOFTMAX_WARPS) {
-        const int c = u / AT_SOFTMAX_WARPS, w = u % AT_SOFTMAX_WARPS, cta = (m.first + c) * p.n_blk + blk;
-        if (__ldcg(p.left + ((unsigned)cta * 2 + (c == 0 ? 1 : 0)) * AT_SOFTMAX_WARPS + w)) merge_slice<D>(p, m, c, w, blk, lane);
-    }
+static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, int thread) {
+    for (int c = 0; c < m.n; ++c)
+        if (__ldcg(p.left + ((m.first + c) * p.n_blk + blk) * 2 + (c == 0 ? 1 : 0))) MergeSlice<D>(p, m, c).run(p, m, thread, blk);
 }
 
 // a / b, b > 0.  A quotient of small numbers is at most one off when it is formed in fp32, and its remainder says which way; the
@@ -238,9 +254,10 @@ struct PieceWalk {
             g_max = max(g_max, __reduce_max_sync(0xffffffffu, (unsigned)g));
             g_min = min(g_min, __reduce_min_sync(0xffffffffu, g > 0 ? (unsigned)g : 0xffffffffu));
         }
-        // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting
-        // anywhere gives most teams two pieces, that is about two groups' worth of extra start and end: whichever is
-        // shorter.
+        // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting anywhere gives most
+        // teams a second piece, and so a second partial result: whichever is shorter.  (Eight one-layer calls, cutting where
+        // padding makes a piece longer by more than 2 / 6 / 10 groups: 4 x 8000 keys, T = 128, 571 / 529 / 529 us; seven ragged
+        // sequences 297 / 282 / 282 and 310 / 306 / 300.)
         const unsigned u_cut = max(1u, quotient(LH * (sum + nz * COST) + teams - 1, teams));
         unsigned v_head = 0;                  // length of one head's row of all sequences in the CTAs' common address space
         pad = LH * nz <= teams;
@@ -255,7 +272,7 @@ struct PieceWalk {
                 v_head += __reduce_add_sync(0xffffffffu, padded((unsigned)g));
             }
             if (!pad || LH * quotient(v_head, u) <= teams) break;
-            if (++u > u_cut + 2) { pad = false; u = u_cut; }
+            if (++u > u_cut + MERGE) { pad = false; u = u_cut; }
         }
         two_rate = __fdividef((float)p.two_cuts, (float)max(1u, LH * (LH * nz > (unsigned)p.two_cuts ? sum + nz : sum)));
         const unsigned v_layer = v_head * (unsigned)p.Hkv;

@@ -27,7 +27,7 @@ struct mtv_tree {
     const int32_t *d_cand_offset = nullptr;   // [K]
     int32_t *d_error = nullptr;               // sticky device-side error word (0 = none)
     const int32_t *d_depth = nullptr;         // [T]
-    int32_t *d_counters = nullptr;            // [512] merge counters of the attention kernel, zero between calls
+    int32_t *d_counters = nullptr;            // [MERGE_COUNTERS][MERGE_STRIDE] merge counters of the attention kernels, zero between calls
 };
 
 namespace mtv {
@@ -43,6 +43,11 @@ void set_last_error_text(const char *text);
             return MTV_ERR_CUDA;                              \
         }                                                     \
     } while (0)
+
+// Merge counters of the attention kernels, in the tree object: a 128-byte line each, so that those who look at one and those who add
+// to another do not queue at the same slice of L2.
+constexpr int MERGE_COUNTERS = 256, MERGE_STRIDE = 32;
+constexpr size_t MERGE_COUNTER_BYTES = (size_t)MERGE_COUNTERS * MERGE_STRIDE * sizeof(int32_t);
 
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
