@@ -222,7 +222,6 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         ptx::mbar_init(bar(SM::BAR_DRAIN), 1);
         ptx::fence_mbar_init();
         *abort_flag = 0;
-        *n_merge = 0;
         *left_items = 0;
     }
     if (warp == W_MMA) {
@@ -267,9 +266,22 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         // The work is divided while the kernel before this one ends, by the lengths that are there (a call that follows another has
         // nothing that changes them in between), and looked at again behind it: eight one-layer calls on ragged lengths take 291 us
         // instead of 314, at head size 64 164 instead of 172.
-        walk.divide(false);
+        AttnPiece cur, nxt;
+        bool have = false;
+        const bool early = walk.early();
+        if (lane == 0) *n_merge = 0;
+        __syncwarp();
+        if (early) {
+            walk.divide();
+            have = walk.next(cur, merges, n_merge);
+        }
         (void)begin();
-        if (!walk.still_so()) walk.divide(true);
+        if (!early || !walk.still_so()) {
+            if (lane == 0) *n_merge = 0;
+            __syncwarp();
+            walk.divide();
+            have = walk.next(cur, merges, n_merge);
+        }
         int n_pub = 0;
         bool ok = true;
         auto publish = [&](const AttnPiece &d) {
@@ -303,8 +315,6 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             }
         };
         // A piece is published before the ring can block on the tiles of the one before it: the query warp looks ahead.
-        AttnPiece cur, nxt;
-        bool have = walk.next(cur, merges, n_merge);
         publish(cur);
         int done = 0;
         if (have) { done = min(2 * cur.cnt, STAGES); request(cur, 0, done); }

@@ -229,26 +229,26 @@ struct PieceWalk {
     // Key groups of a sequence.  0: it has no room for the tree's rows, or no rows at all (nothing here may wrap or become
     // negative: the sums below are other sequences' positions); it is passed over, which report() says.
     __device__ __forceinline__ int groups(int l) const { return l > -p.T && l <= p.Lcap - p.T ? (l + p.T + AT_BN - 1) / AT_BN : 0; }
-    __device__ __forceinline__ void load_chunk(int b0, bool final) {
+    __device__ __forceinline__ void load_chunk(int b0) {
         chunk = b0;
-        len = final || p.B <= 32 ? length(b0 + lane) : 0;       // (more than 32: read more than once, so not while they may change)
-        if (!final) len = min(max(len, 0), p.Lcap);
+        len = length(b0 + lane);
         g = b0 + lane < p.B ? groups(len) : 0;
     }
-    // Were the lengths that the work was divided by the ones that are there now?
-    __device__ __forceinline__ bool still_so() const { return p.B <= 32 && __all_sync(0xffffffffu, length(lane) == len); }
+    // May the work be divided by lengths that may still change?  (More than 32 are read more than once, which must agree.)
+    __device__ __forceinline__ bool early() const { return p.B <= 32; }
+    // Were they the ones that are there now?
+    __device__ __forceinline__ bool still_so() const { return __all_sync(0xffffffffu, length(lane) == len); }
     __device__ __forceinline__ void report() const {
         if (blockIdx.x == 0 && p.status)
             for (int b = lane; b < p.B; b += 32) p.status[b] = groups(length(b)) > 0 ? MTV_OK : MTV_ERR_CAPACITY;
     }
     __device__ __forceinline__ unsigned padded(unsigned gg) const { return gg == 0 ? 0u : pad ? quotient(gg + u - 1, u) * u : gg + COST; }
-    // final: false = with lengths that may still change
-    __device__ __forceinline__ void divide(bool final) {
-        layer = b = head = 0;
+    __device__ __forceinline__ void divide() {
+        layer = b = head = n_part = 0;
         off = 0;
         unsigned sum = 0, nz = 0, g_max = 0, g_min = 0xffffffffu;
         for (int b0 = 0; b0 < p.B; b0 += 32) {
-            load_chunk(b0, final);
+            load_chunk(b0);
             sum += __reduce_add_sync(0xffffffffu, (unsigned)g);
             nz += __popc(__ballot_sync(0xffffffffu, g > 0));
             g_max = max(g_max, __reduce_max_sync(0xffffffffu, (unsigned)g));
@@ -259,20 +259,37 @@ struct PieceWalk {
         // padding makes a piece longer by more than 2 / 6 / 10 groups: 4 x 8000 keys, T = 128, 571 / 529 / 529 us; seven ragged
         // sequences 297 / 282 / 282 and 310 / 306 / 300.)
         const unsigned u_cut = max(1u, quotient(LH * (sum + nz * COST) + teams - 1, teams));
-        unsigned v_head = 0;                  // length of one head's row of all sequences in the CTAs' common address space
         pad = LH * nz <= teams;
         u = pad ? max(1u, quotient(LH * sum + teams - 1, teams)) : u_cut;
         // Whole items, if that makes no run longer than the division above by more than a merge takes: no team shares one.
         const unsigned whole = pad ? g_max : quotient(LH * nz + teams - 1, teams) * (g_max + COST);
-        if ((pad || g_min == g_max) && whole <= u + MERGE) u = max(1u, whole);
-        for (;;) {
-            v_head = 0;
+        unsigned v_head;                      // length of one head's row of all sequences in the CTAs' common address space
+        if ((pad || g_min == g_max) && whole <= u + MERGE) {
+            u = max(1u, whole);
+            v_head = pad ? nz * u : sum + nz * COST;
+        } else if (pad) {
+            // the smallest u for which the pieces fit the teams: sixteen candidates at once, two lanes each
+            const unsigned mine = u + (lane & 15);
+            unsigned n = 0;
             for (int b0 = 0; b0 < p.B; b0 += 32) {
-                if (b0 != chunk) load_chunk(b0, final);
-                v_head += __reduce_add_sync(0xffffffffu, padded((unsigned)g));
+                if (b0 != chunk) load_chunk(b0);
+                for (int i = lane >> 4, e = min(32, p.B - b0); i < (e + 1) / 2 * 2; i += 2) {
+                    const unsigned gi = (unsigned)__shfl_sync(0xffffffffu, g, i & 31);
+                    n += quotient(gi + mine - 1, mine);
+                }
             }
-            if (!pad || LH * quotient(v_head, u) <= teams) break;
-            if (++u > u_cut + MERGE) { pad = false; u = u_cut; }
+            n += __shfl_xor_sync(0xffffffffu, n, 16);
+            const unsigned fit = __ballot_sync(0xffffffffu, LH * n <= teams && mine <= u_cut + MERGE) & 0xffffu;
+            if (fit) {
+                u = __shfl_sync(0xffffffffu, mine, __ffs(fit) - 1);
+                v_head = u * __shfl_sync(0xffffffffu, n, __ffs(fit) - 1);
+            } else {
+                pad = false;
+                u = u_cut;
+                v_head = sum + nz * COST;
+            }
+        } else {
+            v_head = sum + nz * COST;
         }
         two_rate = __fdividef((float)p.two_cuts, (float)max(1u, LH * (LH * nz > (unsigned)p.two_cuts ? sum + nz : sum)));
         const unsigned v_layer = v_head * (unsigned)p.Hkv;
@@ -280,10 +297,10 @@ struct PieceWalk {
         hi = min(pos + u, v_layer * (unsigned)p.n_layers);
         // where the run begins
         if (pos < hi) {
-            layer = (int)quotient(pos, v_layer);
+            layer = p.n_layers == 1 ? 0 : (int)quotient(pos, v_layer);
             unsigned rem = pos - (unsigned)layer * v_layer;
             for (int b0 = 0;; b0 += 32) {
-                if (b0 != chunk) load_chunk(b0, final);
+                if (b0 != chunk) load_chunk(b0);
                 const unsigned mine = padded((unsigned)g) * (unsigned)p.Hkv;
                 unsigned incl = mine;
 #pragma unroll
@@ -352,7 +369,7 @@ struct PieceWalk {
                 while (!m && pos < hi) {
                     int b0 = chunk + 32;
                     if (b0 >= p.B) { b0 = 0; ++layer; }
-                    if (b0 != chunk) load_chunk(b0, true);
+                    if (b0 != chunk) load_chunk(b0);
                     m = __ballot_sync(0xffffffffu, g > 0);
                 }
                 b = chunk + (m ? __ffs(m) - 1 : 0);
