@@ -82,6 +82,7 @@ struct VocabParams {
     int gate_clear;      // the last CTA of all clears it
     int expand;          // the last head to finish expands all heads' candidates into the tree tokens
     int tile_rows;       // (tensor cores) vocabulary rows per tile
+    int x_rows;          // (tensor cores) rows of the activation operand
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, xs_off, lists_off, zbuf_off, bars_off;
 };

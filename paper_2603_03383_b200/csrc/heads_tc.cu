@@ -3,13 +3,13 @@
 // per weight element), the tensor cores can; what has to be kept is the precision of the single-row
 // path, where activations stay fp32 and the candidate ids must match a double-precision checker:
 //   * the fp32 activations h' are split into three bf16 terms hi + mid + lo (24 bits of mantissa, exact
-//     to 2^-25); the three terms of up to 16 batch rows are the 48 rows of the MMA's N operand, and their
+//     to 2^-25); the three terms of up to 16 batch rows are the rows (16, 32 or 48) of the MMA's N operand, and their
 //     products with the bf16 weights are exact;
 //   * the tensor core's fp32 accumulator truncates: over H = 4096 the sums drift by ~3e-6 of the largest
 //     logit.  The K chunks therefore take turns over four accumulators that are added in the epilogue
 //     with ordinary fp32 additions, which divides the drift by four.
 // Layout of the work as in the fused LM head: persistent CTAs (a contiguous slab of one head's vocabulary
-// rows each), TMA producer warp -> ring of stages (64 columns of 128 weight rows + the 48 activation
+// rows each), TMA producer warp -> ring of stages (64 columns of 128 weight rows + the activation
 // rows) -> MMA issuer, accumulators double-buffered in tensor memory -> four epilogue warps, one thread
 // per vocabulary row, that keep per-warp sorted candidate lists (a logit is looked at only if it beats
 // the last entry of the warp's list and those of the CTA's other warps).  What follows the projection is shared with the single-row kernel.
@@ -26,7 +26,7 @@ namespace mtv {
 
 constexpr int HT_THREADS = 192;            // warps 0-3 epilogue, warp 4 MMA issuer, warp 5 TMA producer
 constexpr int HT_EPI_WARPS = 4;
-constexpr int HT_N = 3 * HT_NB;            // hi | mid | lo rows of the activation operand
+constexpr int HT_N = 3 * HT_NB;            // rows of the activation operand for 16 batch rows: hi | mid | lo, B of each
 constexpr int HT_NACC = 4;                 // accumulators that take turns over the K chunks
 constexpr int HT_ACC_COLS = 64;            // tensor-memory columns reserved per accumulator (48 used)
 constexpr uint32_t HT_W_BYTES = 128 * 128; // 128 weight rows x 64 columns
@@ -39,7 +39,10 @@ static_assert(HT_STAGE_BYTES % 1024 == 0, "stages must keep the 1024-byte alignm
 static_assert(2 * HT_NACC * HT_ACC_COLS <= 512, "tensor memory");
 static_assert(HT_SMEM_BYTES <= 220 * 1024, "shared memory");
 
-constexpr uint32_t HT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(HT_N >> 3) << 17) | ((128u >> 4) << 24);
+// Rows that the MMA multiplies: 3 B rounded up to the 16 that M = 128 asks for.  Five batch rows need 16 of the 48, and every
+// column chunk of the weights (16 KB) is accompanied by 2 KB of activations instead of 6.
+static inline int ht_n(int B) { return (3 * B + 15) / 16 * 16; }
+constexpr uint32_t HT_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);     // | N / 8 << 17
 
 __device__ __forceinline__ void ht_tma_2d(uint32_t dst, const void *map, uint32_t bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -51,8 +54,9 @@ __device__ __forceinline__ void ht_tma_2d(uint32_t dst, const void *map, uint32_
 // The same pipeline with the K H rows of W1 as the MMA's M side (tiles of 128 rows, persistent CTAs) and the
 // bf16 hidden states of up to 16 batch rows as its N side (exact: they are bf16 to begin with).  The epilogue
 // (thread = output row) adds the four accumulators, the bias and the residual in fp32 and writes h' as the
-// three bf16 terms the vocabulary projection multiplies: xsplit[k][part][b][o], part = 0 (hi), 1 (mid),
-// 2 (lo), h' = hi + mid + lo up to 2^-25.  Batch rows b >= B hold finite values nobody reads.
+// three bf16 terms the vocabulary projection multiplies: xsplit[k][part B + b][o], part = 0 (hi), 1 (mid),
+// 2 (lo), h' = hi + mid + lo up to 2^-25.  A head has 48 rows there; those from 3 B on hold anything (each feeds a column of its
+// own in the accumulators, which nobody reads).
 constexpr int RT_STAGES = 8;
 constexpr uint32_t RT_X_BYTES = HT_NB * 128;
 constexpr uint32_t RT_STAGE_BYTES = HT_W_BYTES + RT_X_BYTES;   // 18 KB
@@ -194,17 +198,17 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
                 const float bias = p.b1 ? __bfloat162float(p.b1[(size_t)k * p.H + o]) : 0.f;
 #pragma unroll
                 for (int b = 0; b < HT_NB; ++b) {
+                    if (b >= p.B) break;
                     const float yy = y[b] + bias;
-                    const float h = b < p.B ? __bfloat162float(p.hidden[(size_t)b * p.H + o]) : 0.f;
-                    float x = h + yy / (1.f + expf(-yy));
+                    float x = __bfloat162float(p.hidden[(size_t)b * p.H + o]) + yy / (1.f + expf(-yy));
                     const __nv_bfloat16 hi = __float2bfloat16_rn(x);
                     x -= __bfloat162float(hi);                         // exact
                     const __nv_bfloat16 mid = __float2bfloat16_rn(x);
                     x -= __bfloat162float(mid);                        // exact
                     __nv_bfloat16 *dst = p.xsplit + ((size_t)k * HT_N + b) * p.H + o;
                     dst[0] = hi;
-                    dst[(size_t)HT_NB * p.H] = mid;
-                    dst[(size_t)2 * HT_NB * p.H] = __float2bfloat16_rn(x);
+                    dst[(size_t)p.B * p.H] = mid;
+                    dst[(size_t)2 * p.B * p.H] = __float2bfloat16_rn(x);
                 }
             }
         }
@@ -231,7 +235,7 @@ heads_resblock_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid
     }
 }
 
-// grid = (ctas_per_head, K).  w_map: [K V][H] weights, box 64 x 128; x_map: [K 48][H] split activations, box 64 x 48.
+// grid = (ctas_per_head, K).  w_map: [K V][H] weights, box 64 x 128; x_map: [K 48][H] split activations, box 64 x N.
 __global__ void __launch_bounds__(HT_THREADS, 1)
 heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map,
                            const VocabParams p) {
@@ -290,6 +294,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     const int v_end = kd > 0 ? min(p.V, v_begin + rows_per) : v_begin;
     const int n_tiles = (v_end - v_begin + R - 1) / R;
     const int n_kc = p.H / 64;
+    const uint32_t idesc = HT_IDESC | (uint32_t)(p.x_rows >> 3) << 17;
 
     if (warp == 5) {
         // ---------------------------------------------------------------- TMA producer
@@ -299,7 +304,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             wait_gate(p.gate);
             ptx::fence_proxy_async_global();
             for (int t = 0; t < n_early; ++t) {
-                ptx::mbar_arrive_expect_tx(full(t), (uint32_t)R * 128u + HT_X_BYTES);
+                ptx::mbar_arrive_expect_tx(full(t), (uint32_t)(R + p.x_rows) * 128u);
                 ht_tma_2d(ring + t * HT_STAGE_BYTES, &w_map, full(t), t % n_kc * 64, k * p.V + v_begin + t / n_kc * R);
             }
         }
@@ -314,7 +319,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 if (lane == 0) {
                     const uint32_t base = ring + s * HT_STAGE_BYTES;
                     if (it >= n_early) {
-                        ptx::mbar_arrive_expect_tx(full(s), (uint32_t)R * 128u + HT_X_BYTES);
+                        ptx::mbar_arrive_expect_tx(full(s), (uint32_t)(R + p.x_rows) * 128u);
                         ht_tma_2d(base, &w_map, full(s), kc * 64, row0);
                     }
                     ht_tma_2d(base + HT_W_BYTES, &x_map, full(s), kc * 64, k * HT_N);
@@ -345,7 +350,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 const uint32_t d = tmem + (u * HT_NACC + kc % HT_NACC) * HT_ACC_COLS;
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)
-                    ptx::mma_ss_elect(d, w + kk * 2, w + (HT_W_BYTES >> 4) + kk * 2, ptx::DESC_HI, HT_IDESC, kc >= HT_NACC || kk > 0, leader);
+                    ptx::mma_ss_elect(d, w + kk * 2, w + (HT_W_BYTES >> 4) + kk * 2, ptx::DESC_HI, idesc, kc >= HT_NACC || kk > 0, leader);
                 ptx::tc_commit_elect(empty(s), leader);
                 if (kc == n_kc - 1) ptx::tc_commit_elect(acc_full(u), leader);
             }
@@ -370,8 +375,8 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 uint32_t hi[16], mid[16], lo[16];
                 const uint32_t col = tmem + ((uint32_t)(warp * 32) << 16) + (u * HT_NACC + a) * HT_ACC_COLS;
                 ptx::tmem_ld16(col, hi);
-                ptx::tmem_ld16(col + 16, mid);
-                ptx::tmem_ld16(col + 32, lo);
+                ptx::tmem_ld16(col + p.B, mid);
+                ptx::tmem_ld16(col + 2 * p.B, lo);
                 ptx::tmem_ld_wait();
 #pragma unroll
                 for (int b = 0; b < HT_NB; ++b)
@@ -441,7 +446,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     const int slab = (V + L.ctas_per_head - 1) / L.ctas_per_head, slab_tiles = (slab + 127) / 128;
     const int w2_R = (slab + slab_tiles - 1) / slab_tiles;
     if (!tma_map_2d_bf16(&w1_map, W1, w1_rows, H, w1_R) || !tma_map_2d_bf16(&h_map, hidden, B, H, HT_NB) ||
-        !tma_map_2d_bf16(&w2_map, W2, range.n * V, H, w2_R) || !tma_map_2d_bf16(&x_map, xsplit, range.n * HT_N, H, HT_N))
+        !tma_map_2d_bf16(&w2_map, W2, range.n * V, H, w2_R) || !tma_map_2d_bf16(&x_map, xsplit, range.n * HT_N, H, ht_n(B)))
         return MTV_ERR_CUDA;
     {
         ResblockTcParams r;
@@ -464,7 +469,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     p.counters = reinterpret_cast<int32_t *>(ws + L.counters_off);
     p.cand = cand; p.cand_logit = cand_logit; p.tree_tok = tree_tok;
     p.dev_error = t->d_error;
-    p.tile_rows = w2_R;
+    p.tile_rows = w2_R; p.x_rows = ht_n(B);
     p.rows_per_stage = 0; p.n_stages = 0; p.n_it = 0;
     p.stage_bytes = 0; p.xs_off = 0; p.lists_off = 0; p.zbuf_off = 0; p.bars_off = 0;
     TapScope tap(MTV_KERNEL_HEADS_VOCAB_TOPK, st);
