@@ -64,11 +64,10 @@ struct Gate {
     int32_t *word = nullptr;
     int32_t number = 0;
 };
-// Heads [k0, k0 + n) of a call; expand: the tree's tokens follow (the other heads' candidates are already there).
+// Heads [k0, k0 + n) of a call.
 // gate_stays: later kernels of the step wait at the gate, too, and the last of them clears it (null: the heads do).
 struct HeadsRange {
     int k0, n;
-    bool expand;
     Gate *gate_stays = nullptr;
 };
 // MTV_OK, or what such a call is refused with

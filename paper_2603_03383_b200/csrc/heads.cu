@@ -35,13 +35,12 @@ struct VocabSmem {
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, ring_bytes, xs_off, lists_off, zbuf_off, bars_off, total;
 };
-static VocabSmem vocab_smem_plan(int NB, int MR, int H, int ctas_per_head) {
+static VocabSmem vocab_smem_plan(int NB, int MR, int H) {
     VocabSmem s;
     s.n_it = (H / 8 + 31) / 32;                       // 16-byte chunks per lane and row
     const uint32_t row_bytes = (uint32_t)H * 2;
     const uint32_t xs_bytes = (uint32_t)NB * s.n_it * 64 * 16;
     const uint32_t lists_bytes = (uint32_t)VT_CONS_WARPS * NB * MTV_MAX_TOPK * 8;
-    const uint32_t merge_bytes = (uint32_t)ctas_per_head * MTV_MAX_TOPK * 8;   // final merge reuses the ring
     const uint32_t zbuf_bytes = NB > 1 ? VT_GROUPS * 2 * VT_GROUP_WARPS * 32 * 4 : 0;   // partial logits of the column parts
     const uint32_t fixed = xs_bytes + lists_bytes + zbuf_bytes + 256;
     s.rows_per_stage = 0;
@@ -55,7 +54,7 @@ static VocabSmem vocab_smem_plan(int NB, int MR, int H, int ctas_per_head) {
     }
     if (s.rows_per_stage == 0) { s.total = 0; return s; }
     s.ring_bytes = s.n_stages * s.stage_bytes;
-    if (s.ring_bytes < merge_bytes) s.ring_bytes = (merge_bytes + 127) / 128 * 128;
+    if (s.ring_bytes < MERGE_SCRATCH) s.ring_bytes = MERGE_SCRATCH;      // (merging the lists reuses the ring)
     s.xs_off = (s.ring_bytes + 127) / 128 * 128;
     s.lists_off = s.xs_off + xs_bytes;
     s.zbuf_off = s.lists_off + lists_bytes;
@@ -205,7 +204,7 @@ heads_resblock_kernel(int B, int H, int K, const __nv_bfloat16 *__restrict__ hid
 // 16-byte reads are conflict-free) and inserts a logit into its private sorted list only
 // when it beats the list's last entry.  Afterwards the warps' lists are merged per CTA;
 // the last CTA of a head (atomic ticket, no waiting) merges the CTAs' lists into the
-// candidate buffer, and the last head to finish expands the candidates into tree tokens.
+// candidate buffer and expands them into the tokens of the tree nodes that stand for them.
 // MR: (one batch row) weight rows per warp and stage, so that short rows, too, come in stages of tens of kilobytes and pay
 // for waits, activation reads and reductions together: H = 1152, V = 91936, two heads took 124 us.
 template <int NB, int MR>
@@ -442,7 +441,7 @@ heads_vocab_topk_kernel(const VocabParams p) {
         return;
     }
 
-    vocab_tail(p, NB, VT_CONS_WARPS, lval, lidx, smem, k, bz, b0, per, kd, p.xs_off);
+    vocab_tail(p, NB, VT_CONS_WARPS, lval, lidx, smem, k, bz, b0, per, kd);
 }
 
 template <int NB, int MR>
@@ -453,7 +452,7 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     float *hprime = reinterpret_cast<float *>(ws + L.hprime_off);
     const int btiles = (B + NB - 1) / NB;
     const size_t sm1 = (size_t)NB * H * sizeof(float);
-    const VocabSmem S = vocab_smem_plan(NB, MR, H, L.ctas_per_head);
+    const VocabSmem S = vocab_smem_plan(NB, MR, H);
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
@@ -473,7 +472,7 @@ static int launch_heads(const mtv_tree *t, const HeadsRange &r, int B, int H, in
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = r.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = hprime;
-    p.kd_arr = t->d_kd + r.k0; p.off_arr = t->d_cand_offset + r.k0; p.expand = r.expand;
+    p.kd_arr = t->d_kd + r.k0; p.off_arr = t->d_cand_offset + r.k0;
     p.gate = btiles == 1 ? gate : Gate{}; p.gate_clear = btiles == 1 && !r.gate_stays;   // (a second batch tile would meet it cleared)
     p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
@@ -509,7 +508,7 @@ int heads_check(const mtv_tree *tree, int n_heads, int B, int H, int V, const mt
     if (ws_bytes < L.total) return MTV_ERR_WORKSPACE;
     if (!L.use_tc) {
         const int NB = nb_for(B);
-        const VocabSmem S = vocab_smem_plan(NB, B == 1 ? rows_per_warp(H, V, L) : 1, H, L.ctas_per_head);
+        const VocabSmem S = vocab_smem_plan(NB, B == 1 ? rows_per_warp(H, V, L) : 1, H);
         if ((size_t)NB * H * sizeof(float) > VT_SMEM_MAX || S.total == 0) return MTV_ERR_UNSUPPORTED_SHAPE;
         if (NB > 1 && S.rows_per_stage < (NB >= 4 ? 4 : 2)) return MTV_ERR_UNSUPPORTED_SHAPE;   // rows too long for a block of rows per stage
     }
@@ -550,6 +549,6 @@ extern "C" int medusa_heads_topk(const mtv_tree_t *tree, int B, int H, int V,
                                  void *ws, size_t ws_bytes, void *stream) {
     MTV_RANGE("medusa_heads_topk");
     if (!tree) return MTV_ERR_INVALID_ARG;
-    return mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true, nullptr}, B, H, V, hidden, W1, b1, W2, root_tok, cand, cand_logit,
+    return mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, nullptr}, B, H, V, hidden, W1, b1, W2, root_tok, cand, cand_logit,
                                  tree_tok, ws, ws_bytes, stream);
 }

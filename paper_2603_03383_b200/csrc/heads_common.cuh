@@ -1,7 +1,7 @@
 // Pieces shared by the two vocabulary-projection kernels of the Medusa heads (Section 3.1): the
 // parameter block, the ordering of candidates, and everything that follows the projection itself —
 // merging the warps' candidate lists per CTA, the merge across the CTAs of a head by the last one to
-// finish (atomic ticket, nobody waits), and the expansion into tree tokens by the last head (Section 3.2).
+// finish (atomic ticket, nobody waits), and the expansion of the head's candidates into tree tokens (Section 3.2).
 #pragma once
 #include "common.cuh"
 
@@ -30,32 +30,45 @@ __device__ __forceinline__ void cand_exchange(float &v, int &i, int o, bool down
     const bool lower = (lane & o) == 0, mine_better = cand_before(v, i, ov, oi);
     if ((lower == down) != mine_better) { v = ov; i = oi; }
 }
-// One candidate per lane (cand: it has one) against a list of kd <= 16 entries in shared memory.  A few are inserted one
-// after the other (about 100 cycles each); many, as when a list is still empty, are sorted over the lanes and merged (about
-// 900 cycles).  s_thr: the best kd-th entry of any list of this batch row in the CTA, as an order-preserving integer.
-static __device__ __noinline__ void list_update(float z, int v, bool cand, float *lv, int32_t *li, int kd, int *s_thr, int lane) {
+// Two sorted lists of sixteen, a half warp each has one of either: the sixteen best of both, sorted.  (The better of entry s and the
+// other list's entry 15 - s are those sixteen, as a bitonic sequence.)  About 200 cycles.
+__device__ __forceinline__ void list_merge(float &v, int &i, float ov, int oi, int lane) {
+    const int src = (lane & 16) | (15 - (lane & 15));
+    const float rv = __shfl_sync(0xffffffffu, ov, src);
+    const int ri = __shfl_sync(0xffffffffu, oi, src);
+    if (cand_before(rv, ri, v, i)) { v = rv; i = ri; }
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) cand_exchange(v, i, o, true, lane);
+}
+// One candidate per lane (cand: it has one; their ids ascend with the lanes) against a list of kd <= 16 entries in shared memory.  A
+// few are inserted one after the other (about 100 cycles each); many, as when a list is still empty, are ranked, each lane counting
+// those before its own, and merged: a quarter of the time that sorting them over the lanes took, and the first tile of a
+// CTA has all lists of up to sixteen batch rows to fill.  s_thr: the best kd-th entry of any list of this batch row in the CTA, as an
+// order-preserving integer.  ranked: sixteen places of this warp.
+static __device__ __noinline__ void list_update(float z, int v, bool cand, float *lv, int32_t *li, int kd, int *s_thr, int lane, float2 *ranked) {
     unsigned m = __ballot_sync(0xffffffffu, cand);
     float ev = lane < kd ? lv[lane] : -INFINITY;
     int ei = lane < kd ? li[lane] : 0x7fffffff;
-    if (__popc(m) < 8) {
+    if (__popc(m) < 6) {
         while (m) {
             const int src = __ffs(m) - 1;
             m &= m - 1;
             list_insert(ev, ei, __shfl_sync(0xffffffffu, z, src), __shfl_sync(0xffffffffu, v, src), kd, lane);
         }
     } else {
-        float x = cand ? z : -INFINITY;
-        int xi = cand ? v : 0x7fffffff;
-#pragma unroll 1
-        for (int k = 2; k <= 32; k <<= 1)          // bitonic sort, best first
-#pragma unroll 1
-            for (int o = k >> 1; o > 0; o >>= 1) cand_exchange(x, xi, o, (lane & k) == 0, lane);
-        // the better of entry s and candidate 15 - s: the sixteen best of both, bitonic
-        const float rv = __shfl_sync(0xffffffffu, x, 15 - (lane & 15));
-        const int ri = __shfl_sync(0xffffffffu, xi, 15 - (lane & 15));
-        if (!cand_before(ev, ei, rv, ri)) { ev = rv; ei = ri; }
-#pragma unroll 1
-        for (int o = 8; o > 0; o >>= 1) cand_exchange(ev, ei, o, true, lane);
+        const int bits = __float_as_int(z + 0.f);              // (-0.0 and 0.0 are equal)
+        const int key = cand ? bits ^ ((bits >> 31) & 0x7fffffff) : (int)0x80000000;      // (no number has this key)
+        int before = 0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const int other = __shfl_sync(0xffffffffu, key, j);
+            before += (other > key) | ((other == key) & (j < lane));
+        }
+        if (before < 16) ranked[before] = make_float2(cand ? z : -INFINITY, __int_as_float(cand ? v : 0x7fffffff));
+        __syncwarp();
+        const float2 c = ranked[lane & 15];
+        list_merge(ev, ei, c.x, __float_as_int(c.y), lane);
+        __syncwarp();
     }
     if (lane < kd) { lv[lane] = ev; li[lane] = ei; }
     if (lane == kd - 1) {
@@ -80,43 +93,99 @@ struct VocabParams {
     int32_t *dev_error;
     Gate gate;           // the weights are complete behind it (no word: behind the previous kernel)
     int gate_clear;      // the last CTA of all clears it
-    int expand;          // the last head to finish expands all heads' candidates into the tree tokens
     int tile_rows;       // (tensor cores) vocabulary rows per tile
     int x_rows;          // (tensor cores) rows of the activation operand
     int rows_per_stage, n_stages, n_it;
     uint32_t stage_bytes, xs_off, lists_off, zbuf_off, bars_off;
 };
 
-// lval / lidx: [n_warps][NB][MTV_MAX_TOPK] sorted candidate lists in shared memory (unused slots hold
-// (-inf, 0x7fffffff)); smem / scratch_bytes: shared memory free for the cross-CTA merge (at least
-// per * MTV_MAX_TOPK * 8 bytes: one warp's staging area; more lets more warps merge batch rows side by side).
-// Every thread of the CTA calls this.
-__device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, const int n_warps, const float *lval,
-                                           const int32_t *lidx, unsigned char *smem, const int k, const int bz,
-                                           const int b0, const int per, const int kd, const uint32_t scratch_bytes) {
-    __shared__ int s_flag;
-    // ---- merge the warps' lists: rank each entry among all CONS_WARPS*kd entries of its batch row
-    for (int e = threadIdx.x; e < NB * n_warps * MTV_MAX_TOPK; e += (int)blockDim.x) {
-        const int b = e / (n_warps * MTV_MAX_TOPK);
-        const int w = (e / MTV_MAX_TOPK) % n_warps, sl = e % MTV_MAX_TOPK;
-        if (sl >= kd || b0 + b >= p.B) continue;
-        const float zz = lval[(w * NB + b) * MTV_MAX_TOPK + sl];
-        const int id = lidx[(w * NB + b) * MTV_MAX_TOPK + sl];
-        int rank = 0;
-        for (int w2 = 0; w2 < n_warps; ++w2)
-            for (int s2 = 0; s2 < kd; ++s2) {
-                const float z2 = lval[(w2 * NB + b) * MTV_MAX_TOPK + s2];
-                const int id2 = lidx[(w2 * NB + b) * MTV_MAX_TOPK + s2];
-                // unused slots all carry the same sentinel: order them by position
-                if (cand_before(z2, id2, zz, id) || (z2 == zz && id2 == id && (w2 * MTV_MAX_TOPK + s2) < (w * MTV_MAX_TOPK + sl)))
-                    ++rank;
+// The best sixteen of n sorted lists for each of `rows` rows, by all warps of the CTA.  src(row, list, slot, v, i) reads an entry,
+// dst(row, slot, v, i) takes one of the result.  A row's lists are divided among up to four units, a half warp of a unit merges every
+// other list of its share, and a warp has three units side by side, whose chains of shuffles overlap, with the next lists on their
+// way; a second pass merges what the units of a row leave in scratch ([rows][<= 4][16]: with at most 17 warps 4 KB).  (A tournament of
+// kd rounds over the lists' heads, a warp per row, took 26 us for 16 rows of 37 lists at the end of a call, 9 us for two rows.)
+constexpr uint32_t MERGE_SCRATCH = 4096 + 1024;      // and the candidates of 16 rows
+template <typename Src, typename Dst>
+__device__ __forceinline__ void merge_lists(int rows, int n, float2 *scratch, const Src &src, const Dst &dst) {
+    constexpr int R = 3;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, half = lane >> 4, s = lane & 15, n_warps = (int)blockDim.x / 32;
+    const int parts = max(1, min(min(4, R * n_warps / rows), n / 4)), units = rows * parts, turns = (n + 2 * parts - 1) / (2 * parts);
+#pragma unroll 1
+    for (int unit0 = warp; unit0 < units; unit0 += R * n_warps) {
+        float v[R], v0[R], v1[R];
+        int i[R], i0[R], i1[R], row[R], list[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int unit = min(unit0 + r * n_warps, units - 1);      // (past the end: once more, and not kept)
+            row[r] = unit / parts;
+            list[r] = (unit - row[r] * parts) * 2 + half;
+            v[r] = -INFINITY;
+            i[r] = 0x7fffffff;
+        }
+        auto load = [&](int t, float (&lv)[R], int (&li)[R]) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int at = list[r] + t * 2 * parts;
+                lv[r] = -INFINITY;
+                li[r] = 0x7fffffff;
+                if (at < n) src(row[r], at, s, lv[r], li[r]);
             }
-        if (rank < kd) {
-            const size_t o = (((size_t)k * p.B + b0 + b) * per + blockIdx.x) * MTV_MAX_TOPK + rank;
-            p.part_val[o] = zz;
-            p.part_idx[o] = id;
+        };
+        load(0, v0, i0);
+        load(1, v1, i1);
+#pragma unroll 1
+        for (int t = 0; t < turns; ++t) {      // (rolled: this code is met cold)
+            float v2[R];
+            int i2[R];
+            load(t + 2, v2, i2);
+#pragma unroll
+            for (int r = 0; r < R; ++r) list_merge(v[r], i[r], v0[r], i0[r], lane);
+#pragma unroll
+            for (int r = 0; r < R; ++r) { v0[r] = v1[r]; i0[r] = i1[r]; v1[r] = v2[r]; i1[r] = i2[r]; }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            list_merge(v[r], i[r], __shfl_xor_sync(0xffffffffu, v[r], 16), __shfl_xor_sync(0xffffffffu, i[r], 16), lane);
+            const int unit = unit0 + r * n_warps;
+            if (half != 0 || unit >= units) continue;
+            if (parts == 1) dst(row[r], s, v[r], i[r]);
+            else scratch[unit * 16 + s] = make_float2(v[r], __int_as_float(i[r]));
         }
     }
+    if (parts == 1) return;
+    __syncthreads();
+#pragma unroll 1
+    for (int row = warp; row < rows; row += n_warps) {
+        const auto entry = [&](int c) { return c < parts ? scratch[(row * parts + c) * 16 + s] : make_float2(-INFINITY, __int_as_float(0x7fffffff)); };
+        const float2 e0 = entry(half), e1 = entry(half + 2);
+        float v = e0.x;
+        int i = __float_as_int(e0.y);
+        if (parts > 2) list_merge(v, i, e1.x, __float_as_int(e1.y), lane);
+        list_merge(v, i, __shfl_xor_sync(0xffffffffu, v, 16), __shfl_xor_sync(0xffffffffu, i, 16), lane);
+        if (half == 0) dst(row, s, v, i);
+    }
+}
+
+// lval / lidx: [n_warps][NB][MTV_MAX_TOPK] sorted candidate lists in shared memory (unused slots hold
+// (-inf, 0x7fffffff)); smem: MERGE_SCRATCH bytes, free by now.  Every thread of the CTA calls this.
+__device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, const int n_warps, const float *lval,
+                                           const int32_t *lidx, unsigned char *smem, const int k, const int bz,
+                                           const int b0, const int per, const int kd) {
+    __shared__ int s_flag;
+    float2 *scratch = reinterpret_cast<float2 *>(smem);
+    const int rows = min(NB, p.B - b0);
+    const size_t list0 = ((size_t)k * p.B + b0) * per;        // lists of all CTAs: [head][batch row][CTA][16]
+    // ---- the warps' lists
+    merge_lists(rows, n_warps, scratch,
+                [&](int b, int w, int s, float &v, int &i) {
+                    v = lval[(w * NB + b) * MTV_MAX_TOPK + s];
+                    i = lidx[(w * NB + b) * MTV_MAX_TOPK + s];
+                },
+                [&](int b, int s, float v, int i) {
+                    const size_t o = (list0 + (size_t)b * per + blockIdx.x) * MTV_MAX_TOPK + s;
+                    p.part_val[o] = v;
+                    p.part_idx[o] = i;
+                });
     // ---- last CTA of this head merges the CTAs' lists (ticket: nobody waits)
     int32_t *counters = p.counters + (size_t)bz * (p.K + 1);
     __threadfence();
@@ -125,100 +194,31 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     __syncthreads();
     if (!s_flag) return;
     __threadfence();
-    {
-        // The CTAs' lists are sorted, so the best kd of all of them come out of a kd-round tournament over
-        // the lists' heads.  Each warp takes one batch row at a time: it stages the row's lists in shared
-        // memory, lane l plays for lists l, l + 32, ...
-        const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-        const int off = p.off_arr[k];
-        const uint32_t per_warp = (uint32_t)per * MTV_MAX_TOPK * 8;
-        int n_w = (int)(scratch_bytes / per_warp);
-        if (n_w > (int)blockDim.x / 32) n_w = (int)blockDim.x / 32;
-        constexpr int MAXL = 8;                               // lists per lane: up to 256 CTAs per head
-        if (warp < n_w) {
-            float *mval = reinterpret_cast<float *>(smem + (size_t)warp * per_warp);   // [per][MTV_MAX_TOPK]
-            int32_t *midx = reinterpret_cast<int32_t *>(mval + per * MTV_MAX_TOPK);
-            for (int b = warp; b < NB && b0 + b < p.B; b += n_w) {
-                const size_t base = ((size_t)k * p.B + b0 + b) * per * MTV_MAX_TOPK;
-                __syncwarp();
-                // the kd entries of each list, many loads in flight (all sixteen slots of every list, one round trip to L2
-                // at a time, took 8 us at the end of every call)
-                const unsigned n_e = (unsigned)(per * kd), inv = (1u << 20) / (unsigned)kd + 1u;   // e / kd for e < 4096
-#pragma unroll 1
-                for (unsigned e0 = lane; e0 < n_e; e0 += 32 * 8) {
-                    float v[8];
-                    int id[8];
-                    unsigned at[8];
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) {
-                        const unsigned e = min(e0 + 32 * q, n_e - 1), c = (e * inv) >> 20;
-                        at[q] = c * MTV_MAX_TOPK + (e - c * (unsigned)kd);
-                        v[q] = __ldcg(p.part_val + base + at[q]);
-                        id[q] = __ldcg(p.part_idx + base + at[q]);
-                    }
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) { mval[at[q]] = v[q]; midx[at[q]] = id[q]; }
-                }
-                __syncwarp();
-                int head[MAXL];
-#pragma unroll
-                for (int q = 0; q < MAXL; ++q) head[q] = 0;
-                for (int r = 0; r < kd; ++r) {
-                    // this lane's best head
-                    float bv = -INFINITY;
-                    int bi = 0x7fffffff, bq = -1;
-#pragma unroll
-                    for (int q = 0; q < MAXL; ++q) {
-                        const int c = lane + 32 * q;
-                        if (c < per && head[q] < kd) {
-                            const float v = mval[c * MTV_MAX_TOPK + head[q]];
-                            const int id = midx[c * MTV_MAX_TOPK + head[q]];
-                            if (bq < 0 || cand_before(v, id, bv, bi)) { bv = v; bi = id; bq = q; }
-                        }
-                    }
-                    // the warp's best: value first, then id, then lane (equal sentinels)
-                    float wv = bv;
-                    int wi = bi, wl = bq < 0 ? 64 : lane;
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const float ov = __shfl_xor_sync(0xffffffffu, wv, o);
-                        const int oi = __shfl_xor_sync(0xffffffffu, wi, o);
-                        const int ol = __shfl_xor_sync(0xffffffffu, wl, o);
-                        const bool other = ol < 64 && (wl >= 64 || cand_before(ov, oi, wv, wi) || (ov == wv && oi == wi && ol < wl));
-                        if (other) { wv = ov; wi = oi; wl = ol; }
-                    }
-                    if (lane == 0) {
-                        p.cand[(size_t)(b0 + b) * p.C + off + r] = wi;
-                        if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + r] = wv;
-                    }
-                    if (lane == wl) {
-#pragma unroll
-                        for (int q = 0; q < MAXL; ++q)
-                            if (q == bq) ++head[q];
-                    }
-                }
-            }
-        }
-    }
-    // ---- last head of this batch tile expands the candidates into the tree tokens
-    __threadfence();
+    static_assert(MTV_MAX_T <= 192, "a thread per tree node");
+    const int off = p.off_arr[k], node = threadIdx.x, slot = node < p.T ? p.tree_indices[node] : -1;
+    int32_t *tok = reinterpret_cast<int32_t *>(smem + MERGE_SCRATCH - 1024);      // [rows][16]
+    merge_lists(rows, per, scratch,
+                [&](int b, int c, int s, float &v, int &i) {
+                    const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
+                    v = __ldcg(p.part_val + o);
+                    i = __ldcg(p.part_idx + o);
+                },
+                [&](int b, int s, float v, int i) {
+                    tok[b * 16 + s] = i;
+                    if (s >= kd) return;
+                    p.cand[(size_t)(b0 + b) * p.C + off + s] = i;
+                    if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + s] = v;
+                });
     __syncthreads();
-    if (threadIdx.x == 0) {
-        s_flag = atomicAdd(&counters[p.K], 1) == p.K - 1;
-        if (s_flag && p.gate_clear) *p.gate.word = 0;
+    // ---- the tokens of the tree nodes that are this head's candidates (the first head: and the root's)
+    if (slot >= off && slot < off + kd)
+        for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = tok[b * 16 + slot - off];
+    if (off == 1 && node < p.T) {
+        if (MTV_INDEX_OK(slot, p.C, p.dev_error) && slot == 0)
+            for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = p.root_tok[b0 + b];
+        if (node < rows) p.cand[(size_t)(b0 + node) * p.C] = p.root_tok[b0 + node];
     }
-    __syncthreads();
-    if (!s_flag || !p.expand) return;
-    __threadfence();
-    for (int e = threadIdx.x; e < NB * p.T; e += (int)blockDim.x) {
-        const int b = b0 + e / p.T, i = e % p.T;
-        if (b >= p.B) break;
-        const int slot = p.tree_indices[i];
-        if (!MTV_INDEX_OK(slot, p.C, p.dev_error)) continue;
-        const int32_t root = p.root_tok[b];
-        if (i == 0) p.cand[(size_t)b * p.C] = root;
-        p.tree_tok[(size_t)b * p.T + i] = slot == 0 ? root : __ldcg(p.cand + (size_t)b * p.C + slot);
-    }
+    if (p.gate_clear && threadIdx.x == 0 && atomicAdd(&counters[p.K], 1) == p.K - 1) *p.gate.word = 0;     // (all have read it)
 }
 
 }  // namespace mtv

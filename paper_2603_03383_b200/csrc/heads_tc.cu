@@ -244,6 +244,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
     __shared__ int abort_flag_s;
     __shared__ int issued_s;
     __shared__ int s_thr[HT_NB];
+    __shared__ float2 ranked[HT_EPI_WARPS][16];
     __shared__ __align__(8) unsigned long long bar_mem[2 * HT_STAGES + 5];
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const uint32_t raw = ptx::smem_u32(smem_raw);
@@ -393,7 +394,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 int32_t *bi = my_idx + b * MTV_MAX_TOPK;
                 // not behind this warp's list nor behind any list of the CTA
                 const bool cand = valid && z[b] >= thr_value(s_thr[b]) && cand_before(z[b], v, bv[kd - 1], bi[kd - 1]);
-                if (__any_sync(0xffffffffu, cand)) list_update(z[b], v, cand, bv, bi, kd, &s_thr[b], lane);
+                if (__any_sync(0xffffffffu, cand)) list_update(z[b], v, cand, bv, bi, kd, &s_thr[b], lane, ranked[warp]);
             }
         }
         if (!ok) *abort_flag = 1;
@@ -419,7 +420,7 @@ heads_vocab_topk_tc_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
             }
         return;
     }
-    vocab_tail(p, HT_NB, HT_EPI_WARPS, lval, lidx, ring_gen, k, 0, 0, per, kd, HT_STAGES * HT_STAGE_BYTES);
+    vocab_tail(p, HT_NB, HT_EPI_WARPS, lval, lidx, ring_gen, k, 0, 0, per, kd);
 }
 
 bool heads_tc_eligible(int B, int H) { return B >= 2 && B <= HT_NB && H >= 64 && H % 64 == 0; }
@@ -462,7 +463,7 @@ int launch_heads_tc(const mtv_tree *t, const HeadsRange &range, int B, int H, in
     VocabParams p;
     p.B = B; p.H = H; p.V = V; p.K = range.n; p.T = t->T; p.C = t->C;
     p.W2 = W2; p.hprime = nullptr;
-    p.kd_arr = t->d_kd + range.k0; p.off_arr = t->d_cand_offset + range.k0; p.expand = range.expand;
+    p.kd_arr = t->d_kd + range.k0; p.off_arr = t->d_cand_offset + range.k0;
     p.gate = gate; p.gate_clear = !range.gate_stays; p.tree_indices = t->d_tree_indices; p.root_tok = root_tok;
     p.part_val = reinterpret_cast<float *>(ws + L.part_val_off);
     p.part_idx = reinterpret_cast<int32_t *>(ws + L.part_idx_off);

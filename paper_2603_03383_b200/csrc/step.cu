@@ -80,7 +80,7 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
         if (rc != MTV_OK) return rc;
     }
     mtv::Gate gate;
-    rc = mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, true, w.apart ? &gate : nullptr}, a->B, a->H, a->V, a->hidden, a->W1, a->b1,
+    rc = mtv::heads_topk_range(tree, mtv::HeadsRange{0, tree->K, w.apart ? &gate : nullptr}, a->B, a->H, a->V, a->hidden, a->W1, a->b1,
                                a->W2, root_tok, a->cand, a->cand_logit, a->tree_tok, a->ws, a->ws_bytes, stream);
     if (rc != MTV_OK) return rc;
     rc = mtv::tree_attention_layers(tree, a->B, a->Hq, a->Hkv, a->D, a->n_layers, a->q_layers, a->k_caches_host, a->v_caches_host,
@@ -232,13 +232,13 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
         MTV_CUDA_CHECK(cudaEventRecord(g_aux.q_up[g], up));
         return MTV_OK;
     };
-    auto heads = [&](int k0, int n, bool expand) {
-        return mtv::heads_topk_range(tree, mtv::HeadsRange{k0, n, expand, nullptr}, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok,
+    auto heads = [&](int k0, int n) {
+        return mtv::heads_topk_range(tree, mtv::HeadsRange{k0, n, nullptr}, d->B, d->H, d->V, d->hidden, d->W1, d->b1, d->W2, d->root_tok,
                                      d->cand, d->cand_logit, d->tree_tok, d->ws, d->ws_bytes, stream);
     };
     const int before = tree->K / 2;
     int rc = upload_q(0);
-    if (rc == MTV_OK && before > 0) rc = heads(0, before, false);   // (enqueued before the other copies: each costs the host 4 us)
+    if (rc == MTV_OK && before > 0) rc = heads(0, before);   // (enqueued before the other copies: each costs the host 4 us)
     for (int g = 1; g < groups && rc == MTV_OK; ++g) rc = upload_q(g);
     if (rc != MTV_OK) return rc;
     if (d->x_final && d->W_lm)
@@ -260,7 +260,7 @@ extern "C" int mtv_verify_step_host(const mtv_tree_t *tree, const mtv_step_args 
         MTV_CUDA_CHECK(cudaMemcpyAsync(h->out_layers + l0 * per_layer, d->out_layers + l0 * per_layer, n * per_layer * 2,
                                        cudaMemcpyDeviceToHost, down));
     }
-    rc = heads(before, tree->K - before, true);
+    rc = heads(before, tree->K - before);
     if (rc != MTV_OK) return rc;
     // acceptance and compaction
     MTV_CUDA_CHECK(cudaStreamWaitEvent(st, g_aux.logits_up, 0));
