@@ -47,7 +47,7 @@ __device__ __forceinline__ int ld_acquire(const int32_t *p) {
     return v;
 }
 
-// Tensor map over bf16 data (rank 4 or 5) with a 128-byte-swizzled box whose innermost extent is 64 elements, from a table
+// Tensor map over bf16 data (rank 2 to 5) with a 128-byte-swizzled box whose innermost extent is 64 elements, from a table
 // of those already encoded.
 bool tensor_map_bf16(CUtensorMap *map, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides_bytes,
                      const cuuint32_t *box);

@@ -39,6 +39,11 @@ struct __align__(64) AttnMaps {
     CUtensorMap q, k[ML], v[ML];
 };
 
+// Where a (layer, sequence, head) is in the one tensor map of all layers: dimension 3 at head + head_b * sequence, dimension 4 at
+// b * sequence + layer * layer.
+struct CacheFold {
+    int head_b, b, layer;
+};
 struct AttnParams {
     const int32_t *seq_lens;
     const uint64_t *anc;     // [T][2]
@@ -55,6 +60,7 @@ struct AttnParams {
     unsigned inv_g;          // 65536 / G rounded up: row r of a tile is node (r * inv_g) >> 16 (exact for r < 256, G <= 8)
     int n_blk, teams;        // CTAs of a team, teams
     int n_tiles, two_cuts;   // row tiles of an item; see two_term_groups
+    CacheFold fold;
     Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
 };
 
