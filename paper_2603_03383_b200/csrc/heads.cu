@@ -54,7 +54,7 @@ static VocabSmem vocab_smem_plan(int NB, int MR, int H) {
     }
     if (s.rows_per_stage == 0) { s.total = 0; return s; }
     s.ring_bytes = s.n_stages * s.stage_bytes;
-    if (s.ring_bytes < MERGE_SCRATCH) s.ring_bytes = MERGE_SCRATCH;      // (merging the lists reuses the ring)
+    if (s.ring_bytes < sizeof(MergeSmem)) s.ring_bytes = sizeof(MergeSmem);      // (merging the lists reuses the ring)
     s.xs_off = (s.ring_bytes + 127) / 128 * 128;
     s.lists_off = s.xs_off + xs_bytes;
     s.zbuf_off = s.lists_off + lists_bytes;

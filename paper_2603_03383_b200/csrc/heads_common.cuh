@@ -99,17 +99,13 @@ struct VocabParams {
     uint32_t stage_bytes, xs_off, lists_off, zbuf_off, bars_off;
 };
 
-// The best sixteen of n sorted lists for each of `rows` rows, by all warps of the CTA.  src(row, list, slot, v, i) reads an entry,
-// dst(row, slot, v, i) takes one of the result.  A row's lists are divided among up to four units, a half warp of a unit merges every
-// other list of its share, and a warp has three units side by side, whose chains of shuffles overlap, with the next lists on their
-// way; a second pass merges what the units of a row leave in scratch ([rows][<= 4][16]: with at most 17 warps 4 KB).  (A tournament of
-// kd rounds over the lists' heads, a warp per row, took 26 us for 16 rows of 37 lists at the end of a call, 9 us for two rows.)
-constexpr uint32_t MERGE_SCRATCH = 4096 + 1024;      // and the candidates of 16 rows
-template <typename Src, typename Dst>
-__device__ __forceinline__ void merge_lists(int rows, int n, float2 *scratch, const Src &src, const Dst &dst) {
-    constexpr int R = 3;
+// One pass over n sorted lists of sixteen of each of `rows` rows, by all warps of the CTA: `parts` units per row, each of which leaves the
+// best sixteen of its share.  The two half warps of a unit merge every other list of it, with the next lists on their way; a warp has
+// R units side by side, whose chains of shuffles overlap.  src(row, list, slot, v, i) reads an entry, dst(row, part, slot, v, i) takes one.
+template <int R, typename Src, typename Dst>
+__device__ __forceinline__ void merge_pass(int rows, int n, int parts, const Src &src, const Dst &dst) {
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, half = lane >> 4, s = lane & 15, n_warps = (int)blockDim.x / 32;
-    const int parts = max(1, min(min(4, R * n_warps / rows), n / 4)), units = rows * parts, turns = (n + 2 * parts - 1) / (2 * parts);
+    const int units = rows * parts, turns = (n + 2 * parts - 1) / (2 * parts);
 #pragma unroll 1
     for (int unit0 = warp; unit0 < units; unit0 += R * n_warps) {
         float v[R], v0[R], v1[R];
@@ -119,8 +115,6 @@ __device__ __forceinline__ void merge_lists(int rows, int n, float2 *scratch, co
             const int unit = min(unit0 + r * n_warps, units - 1);      // (past the end: once more, and not kept)
             row[r] = unit / parts;
             list[r] = (unit - row[r] * parts) * 2 + half;
-            v[r] = -INFINITY;
-            i[r] = 0x7fffffff;
         }
         auto load = [&](int t, float (&lv)[R], int (&li)[R]) {
 #pragma unroll
@@ -131,10 +125,11 @@ __device__ __forceinline__ void merge_lists(int rows, int n, float2 *scratch, co
                 if (at < n) src(row[r], at, s, lv[r], li[r]);
             }
         };
-        load(0, v0, i0);
-        load(1, v1, i1);
+        load(0, v, i);
+        load(1, v0, i0);
+        load(2, v1, i1);
 #pragma unroll 1
-        for (int t = 0; t < turns; ++t) {      // (rolled: this code is met cold)
+        for (int t = 1; t < turns; ++t) {      // (rolled: this code is met cold)
             float v2[R];
             int i2[R];
             load(t + 2, v2, i2);
@@ -147,36 +142,66 @@ __device__ __forceinline__ void merge_lists(int rows, int n, float2 *scratch, co
         for (int r = 0; r < R; ++r) {
             list_merge(v[r], i[r], __shfl_xor_sync(0xffffffffu, v[r], 16), __shfl_xor_sync(0xffffffffu, i[r], 16), lane);
             const int unit = unit0 + r * n_warps;
-            if (half != 0 || unit >= units) continue;
-            if (parts == 1) dst(row[r], s, v[r], i[r]);
-            else scratch[unit * 16 + s] = make_float2(v[r], __int_as_float(i[r]));
+            if (half == 0 && unit < units) dst(row[r], list[r] / 2, s, v[r], i[r]);
         }
     }
-    if (parts == 1) return;
-    __syncthreads();
-#pragma unroll 1
-    for (int row = warp; row < rows; row += n_warps) {
-        const auto entry = [&](int c) { return c < parts ? scratch[(row * parts + c) * 16 + s] : make_float2(-INFINITY, __int_as_float(0x7fffffff)); };
-        const float2 e0 = entry(half), e1 = entry(half + 2);
-        float v = e0.x;
-        int i = __float_as_int(e0.y);
-        if (parts > 2) list_merge(v, i, e1.x, __float_as_int(e1.y), lane);
-        list_merge(v, i, __shfl_xor_sync(0xffffffffu, v, 16), __shfl_xor_sync(0xffffffffu, i, 16), lane);
-        if (half == 0) dst(row, s, v, i);
+}
+// The best sixteen of n sorted lists for each row: passes that take at least four lists into one until one is left.  (A tournament of
+// kd rounds over the lists' heads, a warp per row, took 26 us for 16 rows of 37 lists at the end of a call, 9 us for two rows.)
+struct MergeSmem {
+    float2 a[52][16], b[26][16];      // what passes leave
+    int32_t tok[16][16];              // candidates of a head
+};
+template <typename Src, typename Dst>
+__device__ __forceinline__ void merge_lists(int rows, int n, MergeSmem *sm, const Src &src, const Dst &dst) {
+    constexpr int R = 3;
+    const int n_warps = (int)blockDim.x / 32;
+    int parts = max(1, min((n + 3) / 4, R * n_warps / rows));
+    if (parts == 1) {
+        const auto to = [&](int row, int, int s, float v, int i) { dst(row, s, v, i); };
+        if (rows <= n_warps) merge_pass<1>(rows, n, 1, src, to);
+        else merge_pass<R>(rows, n, 1, src, to);
+        return;
     }
+    float2 (*from)[16] = sm->a, (*to)[16] = sm->b;
+    {
+        const auto leave = [&](int row, int part, int s, float v, int i) { from[row * parts + part][s] = make_float2(v, __int_as_float(i)); };
+        if (rows * parts <= n_warps) merge_pass<1>(rows, n, parts, src, leave);
+        else merge_pass<R>(rows, n, parts, src, leave);
+    }
+#pragma unroll 1
+    do {
+        __syncthreads();
+        n = parts;
+        parts = max(1, min((n + 3) / 4, n_warps / rows));
+        merge_pass<1>(
+            rows, n, parts,
+            [&](int row, int l, int s, float &v, int &i) {
+                const float2 e = from[row * n + l][s];
+                v = e.x;
+                i = __float_as_int(e.y);
+            },
+            [&](int row, int part, int s, float v, int i) {
+                if (parts == 1) dst(row, s, v, i);
+                else to[row * parts + part][s] = make_float2(v, __int_as_float(i));
+            });
+        float2 (*const t)[16] = from;
+        from = to;
+        to = t;
+    } while (parts > 1);
 }
 
 // lval / lidx: [n_warps][NB][MTV_MAX_TOPK] sorted candidate lists in shared memory (unused slots hold
-// (-inf, 0x7fffffff)); smem: MERGE_SCRATCH bytes, free by now.  Every thread of the CTA calls this.
+// (-inf, 0x7fffffff)); smem: sizeof(MergeSmem), free by now.  Every thread of the CTA calls this.
 __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, const int n_warps, const float *lval,
                                            const int32_t *lidx, unsigned char *smem, const int k, const int bz,
                                            const int b0, const int per, const int kd) {
     __shared__ int s_flag;
-    float2 *scratch = reinterpret_cast<float2 *>(smem);
+    MergeSmem *sm = reinterpret_cast<MergeSmem *>(smem);
     const int rows = min(NB, p.B - b0);
     const size_t list0 = ((size_t)k * p.B + b0) * per;        // lists of all CTAs: [head][batch row][CTA][16]
     // ---- the warps' lists
-    merge_lists(rows, n_warps, scratch,
+    merge_lists(rows, n_warps, sm,
                 [&](int b, int w, int s, float &v, int &i) {
                     v = lval[(w * NB + b) * MTV_MAX_TOPK + s];
                     i = lidx[(w * NB + b) * MTV_MAX_TOPK + s];
@@ -188,23 +213,24 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
                 });
     // ---- last CTA of this head merges the CTAs' lists (ticket: nobody waits)
     int32_t *counters = p.counters + (size_t)bz * (p.K + 1);
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_flag = atomicAdd(&counters[k], 1) == per - 1;
+    if (threadIdx.x == 0) {            // (one fence for the CTA: the barriers order the others' accesses against it)
+        __threadfence();
+        s_flag = atomicAdd(&counters[k], 1) == per - 1;
+        __threadfence();
+    }
     __syncthreads();
     if (!s_flag) return;
-    __threadfence();
     static_assert(MTV_MAX_T <= 192, "a thread per tree node");
     const int off = p.off_arr[k], node = threadIdx.x, slot = node < p.T ? p.tree_indices[node] : -1;
-    int32_t *tok = reinterpret_cast<int32_t *>(smem + MERGE_SCRATCH - 1024);      // [rows][16]
-    merge_lists(rows, per, scratch,
+    merge_lists(rows, per, sm,
                 [&](int b, int c, int s, float &v, int &i) {
                     const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
                     v = __ldcg(p.part_val + o);
                     i = __ldcg(p.part_idx + o);
                 },
                 [&](int b, int s, float v, int i) {
-                    tok[b * 16 + s] = i;
+                    sm->tok[b][s] = i;
                     if (s >= kd) return;
                     p.cand[(size_t)(b0 + b) * p.C + off + s] = i;
                     if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + s] = v;
@@ -212,7 +238,7 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     __syncthreads();
     // ---- the tokens of the tree nodes that are this head's candidates (the first head: and the root's)
     if (slot >= off && slot < off + kd)
-        for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = tok[b * 16 + slot - off];
+        for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = sm->tok[b][slot - off];
     if (off == 1 && node < p.T) {
         if (MTV_INDEX_OK(slot, p.C, p.dev_error) && slot == 0)
             for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = p.root_tok[b0 + b];
