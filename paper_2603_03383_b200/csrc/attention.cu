@@ -28,7 +28,10 @@
 // so that a group's softmax has the time of two other groups' MMAs and two groups' softmax run at once.  (The kernel before this
 // one had two row tiles in a CTA, with an accumulator and one tile of scores each: the chain scores -> P -> PV -> scores then took
 // 1.63 k cycles per tile and group, of which the tensor core worked 1024.  Now 1.4 k; what is left of the chain is 1.6 k of
-// softmax and 1.4 k of handing over, shared by three tiles.)
+// softmax and 1.4 k of handing over, shared by three tiles.)  The pieces follow one another in the same way: the last PV of a piece
+// has the first scores of the next one behind it, and the softmax warps take that one's first group before they read and write
+// the finished O.  (With pieces one after the other eight one-layer calls on ragged lengths took 281 us, now 256; 21 layers of eight
+// sequences of two or three groups 161 and 151, at head size 64 145 and 134; of one group 125 and 108.)
 //   warps 0-7 / 8-15  softmax of groups 2, 4, .. / 1, 3, ..: two threads own a query row, 64 columns each; the first group is
 //                     everybody's, 32 columns a thread.  (All on every group: 4 % slower at 32768 keys, as what a group costs a
 //                     warp beside its exponentials is paid twice as often.)
@@ -104,15 +107,17 @@ struct AttnSmem {
     static constexpr int BAR_TAIL = BAR_KV_EMPTY + STAGES; // V whose last rows must be cleared lands here first (odd CTA: not used)
     static constexpr int BAR_Q_FULL = BAR_TAIL + STAGES;   // [2 tiles] of the even CTA: both CTAs' tiles
     static constexpr int BAR_Q_EMPTY = BAR_Q_FULL + 2;     // [2]
-    static constexpr int BAR_S = BAR_Q_EMPTY + 2;          // [3] scores of a group complete; behind a piece's last groups but one: their PV is
+    static constexpr int BAR_S = BAR_Q_EMPTY + 2;          // [3] scores of a group complete, and the PV in front of them
     static constexpr int BAR_P = BAR_S + NB;               // [3] even CTA: what PV of a group and the scores behind it wait for
-    static constexpr int BAR_O = BAR_P + NB;               // O of a piece complete
+    static constexpr int BAR_PV = BAR_P + NB;              // [2] PV of a piece's last group but two / but one, where no scores follow it
+    static constexpr int BAR_O = BAR_PV + 2;               // O of a piece complete
     static constexpr int BAR_O_FREE = BAR_O + 1;           // even CTA: O of a piece read
     static constexpr int BAR_PC_FULL = BAR_O_FREE + 1;     // [AT_PIECES]
     static constexpr int BAR_PC_EMPTY = BAR_PC_FULL + AT_PIECES;
-    static constexpr int BAR_XM = BAR_PC_EMPTY + AT_PIECES;    // [4] the four warps of a row quarter: references
-    static constexpr int BAR_XO = BAR_XM + 4;                  // [4] results
-    static constexpr int BAR_OUT = BAR_XO + 4;                 // a partial result is written by the sixteen warps
+    static constexpr int BAR_XM = BAR_PC_EMPTY + AT_PIECES;    // [4] the four warps of a row quarter: meet
+    static constexpr int BAR_XO = BAR_XM + 4;                  // [4] have read what they exchanged
+    static constexpr int BAR_XG = BAR_XO + 4;                  // [4] have written all P of a piece
+    static constexpr int BAR_OUT = BAR_XG + 4;                 // a partial result is written by the sixteen warps
     static constexpr int BAR_GO = BAR_OUT + 1;                 // [2] all partial results of an item are there (or the slice is left)
     static constexpr int BAR_DRAIN = BAR_GO + 2;
     static constexpr int BAR_COUNT = BAR_DRAIN + 1;
@@ -127,31 +132,12 @@ struct AttnSmem {
     static constexpr uint32_t IDESC_QK = IDESC | (128u >> 3) << 17, IDESC_PV = IDESC | (uint32_t)(D >> 3) << 17 | 1u << 16;
 };
 
-// Positions of half groups in the order in which the tensor core takes them: K0 K1 K2 V0 K3 V1 K4 ... V(cnt-1)
-__device__ __forceinline__ int k_pos(int j) { return j < NB ? j : 2 * j - (NB - 1); }
-__device__ __forceinline__ int v_pos(int j, int cnt) { return min(cnt, NB + j) + j; }
-__device__ __forceinline__ void half_at(int pos, int cnt, bool &is_v, int &j) {
-    const int n0 = min(NB, cnt), r = pos - n0;
-    if (r < 0) { is_v = false; j = pos; return; }
-    is_v = r >= 2 * (cnt - n0) || !(r & 1);
-    j = r >= 2 * (cnt - n0) ? r - (cnt - n0) : is_v ? r >> 1 : (r >> 1) + NB;
-}
-// S phases of a piece beyond whole turns of its barrier: tile b of scores takes one phase per group, and one more where the
-// PV of the last groups but one is told through it.  Bit b: odd number of phases.
-__device__ __forceinline__ uint32_t s_phases(int cnt) {
-    uint32_t odd = 0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-        if (b < cnt) odd |= (uint32_t)(((cnt - b + NB - 1) / NB + (b != (cnt - 1) % NB)) & 1) << b;
-    return odd;
-}
-__device__ __forceinline__ uint32_t p_phases(int cnt) {
-    uint32_t odd = 0;
-#pragma unroll
-    for (int b = 0; b < NB; ++b)
-        if (b < cnt) odd |= (uint32_t)(((cnt - b + NB - 1) / NB) & 1) << b;
-    return odd;
-}
+// The half groups of all pieces of a CTA, in the order in which the tensor core takes them and the ring has them: K of three groups, then
+// V(0) K(3) V(1) K(4) ..; groups count on from piece to piece, but K runs ahead into the next piece only, whose query tile is there.
+// K of group k, `before` being the first group of the piece before its own:
+__device__ __forceinline__ int k_pos(int k, int before) { return k + max(k - (NB - 1), before); }
+// V of group j of a piece that begins with group `first` and has cnt groups, nxt in the next one:
+__device__ __forceinline__ int v_pos(int first, int j, int cnt, int nxt) { return 2 * (first + j) + min(NB, cnt + nxt - j); }
 
 // V rows from the last key on, up to the next multiple of 16: only they take part in O += P V
 template <int HALVES>
@@ -201,7 +187,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         }
         for (int t = 0; t < 2; ++t) {
             ptx::mbar_init(bar(SM::BAR_Q_FULL + t), PAIR && rank == 0 ? 2 : 1);
-            ptx::mbar_init(bar(SM::BAR_Q_EMPTY + t), AT_SOFTMAX_WARPS);
+            ptx::mbar_init(bar(SM::BAR_Q_EMPTY + t), 1);
+            ptx::mbar_init(bar(SM::BAR_PV + t), 1);
         }
         for (int b = 0; b < NB; ++b) {
             ptx::mbar_init(bar(SM::BAR_S + b), 1);
@@ -216,6 +203,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         for (int i = 0; i < 4; ++i) {
             ptx::mbar_init(bar(SM::BAR_XM + i), 4);
             ptx::mbar_init(bar(SM::BAR_XO + i), 4);
+            ptx::mbar_init(bar(SM::BAR_XG + i), 4);
             ptx::sts_u32(sbase + SM::OFF_ASK + i * 4, 0u);
         }
         ptx::mbar_init(bar(SM::BAR_OUT), AT_SOFTMAX_WARPS);
@@ -294,41 +282,49 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             __syncwarp();
             ++n_pub;
         };
-        uint32_t seq = 0;                     // ring slots handed out so far: slot seq % STAGES
-        // halves [from, to) of a piece, in the order of their use
-        auto request = [&](const AttnPiece &d, int from, int to) {
-            const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
-            for (int at = from; at < to && ok && !*abort_flag; ++at, ++seq) {
-                const uint32_t s = seq % STAGES, use = seq / STAGES;
-                if (use > 0 && !ptx::mbar_wait(bar(SM::BAR_KV_EMPTY + s), (use - 1) & 1)) { ok = false; break; }
-                if (lane == 0) {
-                    bool is_v;
-                    int j;
-                    half_at(at, d.cnt, is_v, j);
-                    const int key = (d.gb + j) * AT_BN, l = ML == 1 ? 0 : d.layer;
-                    const int c3 = ML == 1 ? d.head + p.fold.head_b * d.b : d.head, c4 = ML == 1 ? p.fold.b * d.b + p.fold.layer * d.layer : d.b;
-                    const bool tail = rank == 0 && is_v && d.gb + j == groups - 1 && (n_keys & 15) != 0;
-                    const uint32_t fb = bar((tail ? SM::BAR_TAIL : SM::BAR_KV_FULL) + s), dst = sbase + SM::OFF_RING + s * SM::SLOT;
-                    ptx::mbar_arrive_expect_tx(fb, SM::SLOT);
-                    if (is_v) ptx::tma_load_5d(dst, &maps.v[l], fb, 0, key, (int)rank, c3, c4);      // (one CTA: all columns)
-                    else ptx::tma_load_5d(dst, &maps.k[l], fb, 0, key + (int)rank * 64, 0, c3, c4);
-                }
-                __syncwarp();
+        uint32_t slot = 0, use = 0;           // the next ring slot, and how often all have been handed out
+        // a half of group j of a piece
+        auto request = [&](const AttnPiece &d, bool is_v, int j) {
+            if (use > 0 && !ptx::mbar_wait(bar(SM::BAR_KV_EMPTY + slot), (use - 1) & 1)) { ok = false; return; }
+            if (lane == 0) {
+                const int n_keys = d.L + p.T, key = (d.gb + j) * AT_BN, l = ML == 1 ? 0 : d.layer;
+                const int c3 = ML == 1 ? d.head + p.fold.head_b * d.b : d.head, c4 = ML == 1 ? p.fold.b * d.b + p.fold.layer * d.layer : d.b;
+                const bool tail = rank == 0 && is_v && key + AT_BN >= n_keys && (n_keys & 15) != 0;
+                const uint32_t fb = bar((tail ? SM::BAR_TAIL : SM::BAR_KV_FULL) + slot), dst = sbase + SM::OFF_RING + slot * SM::SLOT;
+                ptx::mbar_arrive_expect_tx(fb, SM::SLOT);
+                if (is_v) ptx::tma_load_5d(dst, &maps.v[l], fb, 0, key, (int)rank, c3, c4);      // (one CTA: all columns)
+                else ptx::tma_load_5d(dst, &maps.k[l], fb, 0, key + (int)rank * 64, 0, c3, c4);
             }
+            __syncwarp();
+            if (++slot == STAGES) { slot = 0; ++use; }
         };
-        // A piece is published before the ring can block on the tiles of the one before it: the query warp looks ahead.
+        // A piece is published when the one before it begins; the first copies do not wait for that.
         publish(cur);
-        int done = 0;
-        if (have) { done = min(2 * cur.cnt, STAGES); request(cur, 0, done); }
-        walk.report();
+        int a = 0;                            // groups whose K is requested ahead of V
+        if (have)
+            for (; a < min(NB - 1, cur.cnt); ++a) request(cur, false, a);
         while (have && ok && !*abort_flag) {
             const bool more = walk.next(nxt, merges, n_merge);
             publish(nxt);
-            request(cur, done, 2 * cur.cnt);
-            done = 0;
+            for (int j = 0; j < cur.cnt && ok && !*abort_flag;) {
+                const int g = j + a;
+                if (a < NB && g < cur.cnt + nxt.cnt) {
+                    const bool n = g >= cur.cnt;
+                    AttnPiece d;
+                    d.layer = n ? nxt.layer : cur.layer; d.b = n ? nxt.b : cur.b; d.head = n ? nxt.head : cur.head;
+                    d.gb = n ? nxt.gb : cur.gb; d.L = n ? nxt.L : cur.L;
+                    request(d, false, n ? g - cur.cnt : g);
+                    ++a;
+                } else {
+                    request(cur, true, j);
+                    ++j;
+                    --a;
+                }
+            }
             cur = nxt;
             have = more;
         }
+        walk.report();
         if (!ok && lane == 0) give_up();
         if (*abort_flag) {
             // copies still in flight land before the shared memory goes away (their barriers may wait for the peer as well, so
@@ -339,8 +335,8 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     } else if (warp == W_Q) {
         // ------------------------------------------------------------ query tiles; even CTA: V rows past the last key
         (void)begin();
-        uint32_t seq = 0, parity = 0;         // parity: bit s = phase of tail barrier s
-        int n_out = 0;                        // partial results
+        uint32_t parity = 0;                  // bit s: phase of tail barrier s
+        int first = 0, n_out = 0;             // groups of the pieces before; partial results
         if (lane < 2) p.left[blockIdx.x * 2 + lane] = 0;     // (released with the first of them)
         AttnPiece d, e;
         bool ok = true;
@@ -367,7 +363,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         if (lane == 0) free_piece(0);
         if (have) { request_q(0, d); tell_q(0); }
         for (int pi = 0; have && ok; ++pi) {
-            // the next piece's tile goes to the other place, as soon as the piece before this one has left it
+            // the next piece's tile goes to the other place, as soon as the scores of the piece before this one are complete
             if (!read_piece(pi + 1, e)) break;
             __syncwarp();
             if (lane == 0) free_piece(pi + 1);
@@ -375,7 +371,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
             if (have) { request_q(pi + 1, e); if (!ok) break; tell_q(pi + 1); if (!ok) break; }
             const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
             if (rank == 0 && d.gb + d.cnt == groups && (n_keys & 15) != 0) {
-                const uint32_t s = (seq + (uint32_t)v_pos(d.cnt - 1, d.cnt)) % STAGES;
+                const uint32_t s = (uint32_t)v_pos(first, d.cnt - 1, d.cnt, e.cnt) % STAGES;
                 ok = ptx::mbar_wait(bar(SM::BAR_TAIL + s), (parity >> s) & 1);
                 if (!ok) break;
                 parity ^= 1u << s;
@@ -394,7 +390,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(merge_counter(p, d.first, blk)) : "memory");
                 }
             }
-            seq += 2u * (uint32_t)d.cnt;
+            first += d.cnt;
             d = e;
         }
         // The items that this CTA shares with others: a look at the counter until all parts are there, then the softmax warps
@@ -433,21 +429,16 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     } else if (PAIR && warp == W_RELAY && rank == 1) {
         // ------------------------------------------------------------ odd CTA: what has landed, V rows past the last key cleared
         (void)begin();
-        uint32_t seq = 0;
-        AttnPiece d;
+        int at = 0, first = 0;
+        AttnPiece d, e;
         bool ok = true;
-        for (int pi = 0; ok && read_piece(pi, d); ++pi) {
-            __syncwarp();
-            if (lane == 0) free_piece(pi);
-            if (d.cnt == 0) break;
-            const int n_keys = d.L + p.T, groups = (n_keys + AT_BN - 1) / AT_BN;
-            const bool tail = d.gb + d.cnt == groups && (n_keys & 15) != 0;
-            for (int at = 0; at < 2 * d.cnt && !*abort_flag; ++at, ++seq) {
-                const uint32_t s = seq % STAGES;
-                ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), (seq / STAGES) & 1);
+        auto pass = [&](int until, bool tail, int n_keys) {       // tail: the last of them has rows to clear
+            for (; ok && at < until && !*abort_flag; ++at) {
+                const uint32_t s = (uint32_t)at % STAGES;
+                ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ((uint32_t)at / STAGES) & 1);
                 if (!ok) break;
-                if (tail && at == 2 * d.cnt - 1) {       // (the last half is V of the last group)
-                    clear_tail<PAIR ? 1 : D / 64>(smem + SM::OFF_RING + s * SM::SLOT, n_keys - (groups - 1) * AT_BN, lane);
+                if (tail && at == until - 1) {
+                    clear_tail<PAIR ? 1 : D / 64>(smem + SM::OFF_RING + s * SM::SLOT, n_keys - (n_keys - 1) / AT_BN * AT_BN, lane);
                     __syncwarp();
                     if (lane == 0) ptx::mbar_arrive_remote_release(ptx::mapa(bar(SM::BAR_KV_FULL + s), 0));
                 } else if (lane == 0) {
@@ -455,61 +446,74 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                 }
                 __syncwarp();
             }
+        };
+        bool have = read_piece(0, d) && d.cnt > 0;
+        __syncwarp();
+        if (lane == 0) free_piece(0);
+        if (have) pass(min(NB, d.cnt), false, 0);     // (whatever the next piece has)
+        for (int pi = 0; have && ok; ++pi) {
+            if (!read_piece(pi + 1, e)) break;
+            __syncwarp();
+            if (lane == 0) free_piece(pi + 1);
+            const int n_keys = d.L + p.T;
+            pass(v_pos(first, d.cnt - 1, d.cnt, e.cnt) + 1, (d.gb + d.cnt) * AT_BN >= n_keys && (n_keys & 15) != 0, n_keys);
+            first += d.cnt;
+            d = e;
+            have = d.cnt > 0;
         }
         if (!ok && lane == 0) give_up();
     } else if (warp == W_RELAY || (PAIR && rank == 1)) {
         // ------------------------------------------------------------ slot keeper
-        // Two things go their own ways here, so it looks at their barriers in turns: slots whose scores (and PV in front of them)
-        // are complete, and groups whose V, and K of the scores behind it, are there.  (With a wait for either in order a slot of K
+        // Two things go their own ways here, so it looks at their barriers in turns: slots whose scores (and PV in front of them) are
+        // complete, and groups whose V, and K of the scores behind it, are there.  (With a wait for either in order a slot of K
         // came back three half groups late: 32 layers of a single row tile, with its five slots, took 169 us instead of 148 at 4096
         // keys, 130 instead of 110 at 8192 of four heads.)  Its word on every group goes into BAR_P, behind its scores, so that it is
-        // never more than a phase behind them.
+        // never more than a phase behind them.  When scores are complete, everything in front of them in the ring is done with.
         (void)begin();
-        uint32_t seq = 0, base = 0;           // base: phases of the tiles of scores
-        auto there = [&](int pos) {
-            const uint32_t t = seq + (uint32_t)pos;
-            return ptx::mbar_test(bar(SM::BAR_KV_FULL + t % STAGES), (t / STAGES) & 1);
-        };
-        AttnPiece d;
-        bool ok = true;
-        auto free_slot = [&](int pos) { ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + (seq + (uint32_t)pos) % STAGES)); };
-        for (int pi = 0; ok && read_piece(pi, d); ++pi) {
-            __syncwarp();
-            if (lane == 0) free_piece(pi);
-            if (d.cnt == 0) break;
-            if (lane == 0) {
-                int scored = 0, told = 0, b = 0, b_told = 0;     // groups whose scores are complete; groups told of
-                uint32_t ph = base;
-                long long t0 = clock64();
-                while (told < d.cnt && !*abort_flag) {
-                    if (scored < d.cnt && ptx::mbar_test(bar(SM::BAR_S + b), (ph >> b) & 1)) {
-                        ph ^= 1u << b;
-                        free_slot(k_pos(scored));
-                        if (scored >= NB) free_slot(v_pos(scored - NB, d.cnt));
-                        ++scored;
-                        b = b == NB - 1 ? 0 : b + 1;
-                        t0 = clock64();
-                    }
-                    if (told < scored && (rank == 1 || (there(v_pos(told, d.cnt)) &&
-                                                        (!SM::K_AHEAD || told + NB >= d.cnt || there(k_pos(told + NB)))))) {
-                        arrive_lead(SM::BAR_P + b_told);
-                        ++told;
-                        b_told = b_told == NB - 1 ? 0 : b_told + 1;
-                        t0 = clock64();
-                    }
-                    if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { ok = false; break; }
+        if (lane == 0) {
+            int pi = 0, before = 0, first = 0;            // first groups of the piece before and of the piece of the next word
+            int cnt = 0, nxt = 0, scored = 0, told = 0;   // their groups; scores complete and words given, from `first` on
+            uint32_t freed = 0;                           // half groups given back
+            AttnPiece d;
+            bool known = false;                           // nxt
+            if (read_piece(0, d)) cnt = d.cnt;
+            auto there = [&](int at) { return ptx::mbar_test(bar(SM::BAR_KV_FULL + (uint32_t)at % STAGES), ((uint32_t)at / STAGES) & 1); };
+            long long t0 = clock64();
+            while (cnt > 0 && !*abort_flag) {
+                if (!known && ptx::mbar_test(bar(SM::BAR_PC_FULL + (pi + 1) % AT_PIECES), ((pi + 1) / AT_PIECES) & 1)) {
+                    nxt = reinterpret_cast<const volatile AttnPiece *>(desc)[(pi + 1) % AT_PIECES].cnt;
+                    known = true;
                 }
+                const uint32_t k = (uint32_t)(first + scored);
+                if (scored < cnt + nxt && ptx::mbar_test(bar(SM::BAR_S + k % NB), (k / NB) & 1)) {
+                    for (const uint32_t to = (uint32_t)k_pos((int)k, scored < cnt ? before : first); freed <= to; ++freed)
+                        ptx::mbar_arrive(bar(SM::BAR_KV_EMPTY + freed % STAGES));
+                    ++scored;
+                    if (scored == cnt) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + (pi & 1)));
+                    else if (scored == cnt + nxt) ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + ((pi + 1) & 1)));
+                    t0 = clock64();
+                }
+                if (known && told < scored) {
+                    const int at = v_pos(first, told, cnt, nxt);
+                    if (rank == 1 || (there(at) && (!SM::K_AHEAD || told + NB >= cnt + nxt || there(at + 1)))) {
+                        arrive_lead(SM::BAR_P + (first + told) % NB);
+                        if (++told == cnt) {
+                            free_piece(pi++);
+                            before = first;
+                            first += cnt;
+                            scored -= cnt;
+                            told = 0;
+                            cnt = nxt;
+                            nxt = 0;
+                            known = false;
+                        }
+                        t0 = clock64();
+                    }
+                }
+                if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { give_up(); break; }
             }
-            ok = __all_sync(0xffffffffu, ok);
-            ok = ok && ptx::mbar_wait(bar(SM::BAR_O), pi & 1);
-            if (!ok) break;
-            if (lane == 0)
-                for (int j = max(0, d.cnt - NB); j < d.cnt; ++j) free_slot(v_pos(j, d.cnt));
-            __syncwarp();
-            base ^= s_phases(d.cnt);
-            seq += 2u * (uint32_t)d.cnt;
         }
-        if (!ok && lane == 0) give_up();
+        __syncwarp();
     } else {
         // ------------------------------------------------------------ even CTA: MMA issuer
         // The whole warp walks the loop, so that descriptors and addresses stay in uniform registers; one elected lane
@@ -517,96 +521,112 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         const bool leader = ptx::elect_one();
         const uint32_t ring_lo = ptx::desc_lo(sbase + SM::OFF_RING, 16), ring_v_lo = ptx::desc_lo(sbase + SM::OFF_RING, SM::HALF);
         const uint32_t tmem = begin();
-        AttnPiece d;
-        uint32_t slot0 = 0, phase0 = 0;       // ring slot and phase of the piece's first half group
-        uint32_t p_base = 0;
+        // what it has to know of a piece: groups, how many of them in two terms, steps of sixteen keys of the last
+        struct Part { int cnt, n_two, last_steps; };
         bool ok = true;
-        for (int pi = 0; ok && read_piece(pi, d); ++pi) {
-            __syncwarp();
-            if (lane == 0) free_piece(pi);
-            const int cnt = __shfl_sync(0xffffffffu, d.cnt, 0);
-            if (cnt == 0) break;
-            const int n_two = __shfl_sync(0xffffffffu, d.flags >> PIECE_TWO_SHIFT, 0);
-            const int last_valid = d.L + p.T - (d.gb + cnt - 1) * AT_BN;       // keys of the piece's last group (or more than 128)
-            const int last_steps = __shfl_sync(0xffffffffu, min(8, (last_valid + 15) / 16), 0);
-            const uint32_t dq = ptx::desc_lo(sbase + (pi & 1) * SM::TILE, 16);
-            auto issue_s = [&](int kk, uint32_t s, int b) {
-                const uint32_t oq = (kk / 4) * (SM::HALF >> 4) + (kk % 4) * 2, o_k = (kk / 4) * (SM::K_HALF >> 4) + (kk % 4) * 2;
-                const uint32_t t_d = tmem + TM_S + b * 128, dk = ring_lo + s * (SM::SLOT >> 4) + o_k;
-                if (PAIR) ptx::mma_pair_ss_elect(t_d, dq + oq, dk, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
-                else ptx::mma_ss_elect(t_d, dq + oq, dk, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
-            };
-            auto commit = [&](int i) {
-                if (PAIR) ptx::tc_commit_pair_mask_elect(bar(i), 3, leader);
-                else ptx::tc_commit_elect(bar(i), leader);
-            };
-            ok = ptx::mbar_wait(bar(SM::BAR_Q_FULL + (pi & 1)), (pi / 2) & 1);
-            uint32_t s = slot0, ph_kv = phase0;
-            auto next_slot = [&]() { if (++s == STAGES) { s = 0; ph_kv ^= 1; } };
-            for (int j = 0; j < min(NB, cnt) && ok; ++j) {
-                ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph_kv);
-                ptx::tc_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < D / 16; ++kk) issue_s(kk, s, j);
-                commit(SM::BAR_S + j);
-                next_slot();
-            }
-            ok = ok && (pi == 0 || ptx::mbar_wait(bar(SM::BAR_O_FREE), (pi - 1) & 1));
-            int b = 0;
-            uint32_t ph_p = p_base;
-            bool go = false;              // all that the group's MMAs wait for is there
-            for (int j = 0; j < cnt; ++j) {
-                if (!go) ok = ok && ptx::mbar_wait(bar(SM::BAR_P + b), (ph_p >> b) & 1);
+        auto look = [&](int pi) {
+            Part x = {0, 0, 0};
+            AttnPiece d;
+            if (!read_piece(pi, d)) { ok = false; return x; }
+            const int last_valid = d.L + p.T - (d.gb + d.cnt - 1) * AT_BN;         // keys of the piece's last group (or more than 128)
+            x.cnt = __shfl_sync(0xffffffffu, d.cnt, 0);
+            x.n_two = __shfl_sync(0xffffffffu, d.flags >> PIECE_TWO_SHIFT, 0);
+            x.last_steps = __shfl_sync(0xffffffffu, min(8, (last_valid + 15) / 16), 0);
+            return x;
+        };
+        auto commit = [&](int i) {
+            if (PAIR) ptx::tc_commit_pair_mask_elect(bar(i), 3, leader);
+            else ptx::tc_commit_elect(bar(i), leader);
+        };
+        uint32_t s = 0, ph_kv = 0;                // ring slot and its phase
+        auto next_slot = [&]() { if (++s == STAGES) { s = 0; ph_kv ^= 1; } };
+        auto next_group = [](int t) { return t == 2 * NB - 1 ? 0 : t + 1; };
+        // t_s, t_v: the next scores and the next PV as group number modulo 6: tile of scores, and from 3 on its barriers' odd phases
+        int pi = 0, j = 0, ahead = 0, t_s = 0, t_v = 0, q_there = -1;      // next PV: group j of piece pi; groups that scores are ahead
+        bool known = false, go = false, k_there = false;      // the next piece is; all that PV waits for, K of the scores behind it are there
+        Part cur = look(0), nxt = {0, 0, 0};
+        while (ok && cur.cnt > 0) {
+            // scores as far ahead as there are tiles for them, into the next piece at most
+            while (ahead < NB && j + ahead < cur.cnt + nxt.cnt) {
+                const int q = j + ahead < cur.cnt ? pi : pi + 1;
+                if (q != q_there) {
+                    ok = ptx::mbar_wait(bar(SM::BAR_Q_FULL + (q & 1)), (q / 2) & 1);
+                    q_there = q;
+                }
+                if (!k_there) ok = ok && ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph_kv);
                 if (!ok) break;
-                ph_p ^= 1u << b;
                 ptx::tc_fence_after();
-                const uint32_t dv = ring_v_lo + s * (SM::SLOT >> 4), t_p = tmem + TM_S + b * 128;
-                // the A operand of sixteen keys: where P lies (see TM_S)
-                auto issue_pv = [&](int kk, uint32_t col, bool accumulate) {
-                    const uint32_t t_a = t_p + (kk / 4) * 64 + col;
-                    if (PAIR) ptx::mma_pair_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
-                    else ptx::mma_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
-                };
-                const int steps = j == cnt - 1 ? last_steps : 8;
-                if (two_terms<D>(j, n_two)) {
-                    if (D == 64 && steps == 8) {
+                const int b = t_s >= NB ? t_s - NB : t_s;
+                const uint32_t dq = ptx::desc_lo(sbase + (q & 1) * SM::TILE, 16), t_d = tmem + TM_S + b * 128, dk = ring_lo + s * (SM::SLOT >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < 16; ++kk) issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > 0 || kk > 0);
-                    } else {
-#pragma unroll 1
-                        for (int kk = 0; kk < 2 * steps; ++kk) {
-                            const int k = kk >> 1;
-                            issue_pv(k, k / 2 % 2 * 32 + k % 2 * 8 + kk % 2 * 16, j > 0 || kk > 0);
-                        }
-                    }
-                } else if (steps == 8) {
+                for (int kk = 0; kk < D / 16; ++kk) {
+                    const uint32_t oq = (kk / 4) * (SM::HALF >> 4) + (kk % 4) * 2, o_k = (kk / 4) * (SM::K_HALF >> 4) + (kk % 4) * 2;
+                    if (PAIR) ptx::mma_pair_ss_elect(t_d, dq + oq, dk + o_k, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
+                    else ptx::mma_ss_elect(t_d, dq + oq, dk + o_k, ptx::DESC_HI, SM::IDESC_QK, kk > 0, leader);
+                    if (kk == D / 16 - 4) go = __all_sync(0xffffffffu, ptx::mbar_test(bar(SM::BAR_P + (t_v >= NB ? t_v - NB : t_v)), t_v >= NB));
+                }
+                commit(SM::BAR_S + b);
+                next_slot();
+                t_s = next_group(t_s);
+                ++ahead;
+                k_there = false;
+            }
+            if (!ok) break;
+            if (j == cur.cnt) {                   // on to the next piece
+                __syncwarp();
+                if (lane == 0) free_piece(pi);
+                ++pi;
+                j = 0;
+                cur = nxt;
+                nxt = {0, 0, 0};
+                known = false;
+                continue;
+            }
+            if (!known) {
+                nxt = look(pi + 1);
+                known = true;
+                continue;
+            }
+            if (j == 0 && pi > 0) ok = ptx::mbar_wait(bar(SM::BAR_O_FREE), (pi - 1) & 1);
+            const int b = t_v >= NB ? t_v - NB : t_v;
+            if (!go) ok = ok && ptx::mbar_wait(bar(SM::BAR_P + b), t_v >= NB);
+            if (!ok) break;
+            go = false;
+            ptx::tc_fence_after();
+            const uint32_t dv = ring_v_lo + s * (SM::SLOT >> 4), t_p = tmem + TM_S + b * 128;
+            // the A operand of sixteen keys: where P lies (see TM_S)
+            auto issue_pv = [&](int kk, uint32_t col, bool accumulate) {
+                const uint32_t t_a = t_p + (kk / 4) * 64 + col;
+                if (PAIR) ptx::mma_pair_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
+                else ptx::mma_ts_elect(tmem + TM_O, t_a, dv + kk * 128, ptx::DESC_HI, SM::IDESC_PV, accumulate, leader);
+            };
+            const int steps = j == cur.cnt - 1 ? cur.last_steps : 8;
+            if (two_terms<D>(j, cur.n_two)) {
+                if (D == 64 && steps == 8) {
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) issue_pv(kk, kk % 4 * 8, true);
+                    for (int kk = 0; kk < 16; ++kk) issue_pv(kk & 7, kk / 2 % 2 * 32 + kk % 2 * 8 + kk / 8 * 16, j > 0 || kk > 0);
                 } else {
 #pragma unroll 1
-                    for (int kk = 0; kk < steps; ++kk) issue_pv(kk, kk % 4 * 8, true);
-                }
-                next_slot();
-                const bool more = j + NB < cnt;
-                const int bn = b == NB - 1 ? 0 : b + 1;
-                if (more && !SM::K_AHEAD) ok = ptx::mbar_wait(bar(SM::BAR_KV_FULL + s), ph_kv);
-                if (!ok) break;
-                if (more) {
-#pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk) {
-                        issue_s(kk, s, b);
-                        if (kk == D / 16 - 4) go = __all_sync(0xffffffffu, ptx::mbar_test(bar(SM::BAR_P + bn), (ph_p >> bn) & 1));
+                    for (int kk = 0; kk < 2 * steps; ++kk) {
+                        const int k = kk >> 1;
+                        issue_pv(k, k / 2 % 2 * 32 + k % 2 * 8 + kk % 2 * 16, j > 0 || kk > 0);
                     }
-                    next_slot();
-                } else {
-                    go = false;
                 }
-                commit(j == cnt - 1 ? SM::BAR_O : SM::BAR_S + b);
-                b = bn;
+            } else if (steps == 8) {
+#pragma unroll
+                for (int kk = 0; kk < 8; ++kk) issue_pv(kk, kk % 4 * 8, true);
+            } else {
+#pragma unroll 1
+                for (int kk = 0; kk < steps; ++kk) issue_pv(kk, kk % 4 * 8, true);
             }
-            p_base ^= p_phases(cnt);
-            slot0 = s;
-            phase0 = ph_kv;
+            next_slot();
+            t_v = next_group(t_v);
+            const bool more = j + NB < cur.cnt + nxt.cnt;      // scores follow, and their K is there
+            if (j == cur.cnt - 1) commit(SM::BAR_O);
+            else if (!more) commit(SM::BAR_PV + (j == cur.cnt - 2 ? 1 : 0));
+            k_there = more && SM::K_AHEAD;
+            ++j;
+            --ahead;
         }
         if (!ok && lane == 0) give_up();
         __syncwarp();
@@ -637,21 +657,29 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         auto x_at = [&](int s, int h) { return sbase + SM::OFF_X + (uint32_t)((s * 2 + h) * 128 + row) * 4u; };   // [set][half][row]
         const uint32_t ask_at = sbase + SM::OFF_ASK + (uint32_t)qd * 4u;
         constexpr uint32_t hidden = NEG ? 0x7f800000u : 0xff800000u;   // times the scale: -inf
-        uint32_t phases = 0;                      // bit 0: exchange of references, 1: of results, 4-6: the tiles of scores
+        // Phases: bit 0: meetings, 1: what was exchanged has been read, 2: all P of a piece written, 3: BAR_PV + 1.
+        uint32_t phases = 0;
+        // The piece: its number, its groups, and its first group's number modulo 6 (tile of scores, and from 3 on its barriers' odd phases)
+        int piece = 0, cnt = 0, t0 = 0;
         bool ok = true;
         int n_part = 0;                           // partial results written
         float m_used = -INFINITY, l = 0.f;
-        auto meet = [&]() {                       // the four warps of these rows
+        auto arrive_x = [&](int i) {
             __syncwarp();
-            if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XM + qd));
-            if (!ptx::mbar_wait(bar(SM::BAR_XM + qd), phases & 1)) ok = false;
-            phases ^= 1;
+            if (lane == 0) ptx::mbar_arrive(bar(i + qd));
         };
-        auto parity_s = [&](int j, int b) { return ((phases >> (4 + b)) ^ (uint32_t)(j / NB)) & 1u; };   // of the scores of group j
+        auto wait_x = [&](int i, uint32_t bit) {
+            if (!ptx::mbar_wait(bar(i + qd), (phases >> bit) & 1)) ok = false;
+            phases ^= 1u << bit;
+        };
+        auto meet = [&]() {                       // the four warps of these rows
+            arrive_x(SM::BAR_XM);
+            wait_x(SM::BAR_XM, 0);
+        };
         // A warp whose exponents do not fit the reference has not written its P of group `at` yet: O += P V waits for it in all
-        // groups from there on, so that all four warps come to wait for scores (or for O) and meet here; next: the group that
-        // this warp is to take next (a warp that asks: at).  What is there then: O with all groups before the earliest one that
-        // is missing (its MMAs are waited for), and P of groups behind that one, which follow the reference like O does.
+        // groups from there on, so that all four warps come to wait for scores (or for the others' P) and meet here; next: the
+        // group that this warp is to take next (a warp that asks: at).  What is there then: O with all groups before the earliest
+        // one that is missing (its MMAs are waited for), and P of groups behind that one, which follow the reference like O does.
         auto move_reference = [&](float mx, int next, bool asks) {
             meet();                               // (nobody is still at what was exchanged before)
             ptx::sts_f32(x_at(e, hf), mx);
@@ -664,8 +692,13 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                 first = min(first, (int)ptx::lds_u32(sbase + SM::OFF_AT + (uint32_t)(qd * 4 + i) * 4u));
                 m_new = fmaxf(m_new, ceilf(ptx::lds_f32(x_at(i >> 1, i & 1))));
             }
-            const int b_done = (first - 1) % NB;  // O += P V of the group before: the phase behind its scores
-            if (!ptx::mbar_wait(bar(SM::BAR_S + b_done), parity_s(first - 1 + NB, b_done))) ok = false;
+            // O += P V of the group before: told with the scores behind it, or by itself
+            if (!ptx::mbar_wait(bar(SM::BAR_PC_FULL + (piece + 1) % AT_PIECES), ((piece + 1) / AT_PIECES) & 1)) ok = false;
+            const int done = first - 1, nxt = ok ? reinterpret_cast<const volatile AttnPiece *>(desc)[(piece + 1) % AT_PIECES].cnt : 0;
+            const uint32_t k = (uint32_t)(t0 + done + NB);
+            if (done + NB < cnt + nxt) ok = ok && ptx::mbar_wait(bar(SM::BAR_S + k % NB), (k / NB) & 1);
+            else if (done == cnt - 2) ok = ok && ptx::mbar_wait(bar(SM::BAR_PV + 1), (phases >> 3) & 1);
+            else ok = ok && ptx::mbar_wait(bar(SM::BAR_PV), 0);      // (of the last piece only)
             ptx::tc_fence_after();
             const bool need = m_new != m_used && m_used != -INFINITY;
             if (__any_sync(0xffffffffu, need)) {
@@ -674,7 +707,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
 #pragma unroll 1
                 for (int j = next - 4; j < next; j += 2) {    // (a power of two: exact)
                     if (j < first) continue;
-                    const uint32_t t_p = t_s0 + (uint32_t)(j % NB) * 128;
+                    const uint32_t t_p = t_s0 + (uint32_t)(t0 + j) % NB * 128;
 #pragma unroll 1
                     for (int c = 0; c < 4; ++c) {        // (both terms)
                         ptx::tmem_ld16(t_p + c * 16, x);
@@ -705,41 +738,43 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         // complete all the same: the barrier, tested again behind the question, says so, and the question is met at the next
         // wait.  (The scores of the group at which a warp asks, and of all before it, are complete when it asks.)
         auto wait_tc = [&](uint32_t b, uint32_t parity, int next) {
-            const long long t0 = clock64();
+            const long long since = clock64();
             while (!ptx::mbar_try_wait(b, parity)) {
                 if (ptx::lds_u32(ask_at)) {
                     if (!ptx::mbar_try_wait(b, parity)) move_reference(-INFINITY, next, false);
                     else break;
                     continue;
                 }
-                if (clock64() - t0 > ptx::WAIT_CYCLE_LIMIT) { ok = false; return; }
+                if (clock64() - since > ptx::WAIT_CYCLE_LIMIT) { ok = false; return; }
             }
         };
-        for (int pi = 0; ok; ++pi) {
-            if (!ptx::mbar_wait(bar(SM::BAR_PC_FULL + pi % AT_PIECES), (pi / AT_PIECES) & 1)) { ok = false; break; }
-            const volatile AttnPiece &d = desc[pi % AT_PIECES];    // (freed at the end of the piece)
-            const int cnt = d.cnt;
-            if (cnt == 0 || *abort_flag) break;
-            const int n_two = d.flags >> PIECE_TWO_SHIFT;
-            const int a_first = d.gb * AT_BN + hf * 64 - d.L;      // tree row of this half's first column in the first group
-            m_used = -INFINITY;
-            l = 0.f;
-            if (pi > 0) {                      // (the results of the piece before have been read)
-                if (!ptx::mbar_wait(bar(SM::BAR_XO + qd), (phases >> 1) & 1)) { ok = false; break; }
-                phases ^= 2;
+        auto p_done = [&](int b, uint32_t count) {
+            ptx::tmem_st_wait();
+            ptx::tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_lead(SM::BAR_P + b, count);
+        };
+        const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
+        // The first group of a piece comes before the end of the piece before it: the tensor core has its PV, and the scores behind,
+        // to do while O is read and written out.
+        for (int pi = 0;; ++pi) {
+            if (pi > 0) {                         // all P of the piece before are written: nobody asks to move its reference any more
+                arrive_x(SM::BAR_XG);
+                wait_tc(bar(SM::BAR_XG + qd), (phases >> 2) & 1, cnt + ((cnt ^ e) & 1));
+                phases ^= 4;
             }
-            auto p_done = [&](int b, uint32_t count) {
-                ptx::tmem_st_wait();
-                ptx::tc_fence_before();
-                __syncwarp();
-                if (lane == 0) arrive_lead(SM::BAR_P + b, count);
-            };
-            const float2 sc2 = make_float2(p.scale_log2, p.scale_log2);
-            // ---- the first group, all four threads of a row on a quarter of it each: its maximum, then its P in two terms
-            {
-                if (!ptx::mbar_wait(bar(SM::BAR_S), parity_s(0, 0))) { ok = false; break; }
+            ok = ok && ptx::mbar_wait(bar(SM::BAR_PC_FULL + pi % AT_PIECES), (pi / AT_PIECES) & 1);
+            if (!ok || *abort_flag) break;
+            const volatile AttnPiece &d = desc[pi % AT_PIECES];    // (freed at the end of the piece)
+            const int cnt_new = d.cnt, a_first = d.gb * AT_BN + hf * 64 - d.L;      // tree row of this half's first column in the first group
+            const int t_new = (int)((unsigned)(t0 + cnt) % (2 * NB));
+            float m_new = -INFINITY, l_new = 0.f;
+            if (cnt_new > 0) {
+                // ---- the first group, all four threads of a row on a quarter of it each: its maximum, then its P in two terms
+                const int b = t_new >= NB ? t_new - NB : t_new;
+                if (!ptx::mbar_wait(bar(SM::BAR_S + b), t_new >= NB)) { ok = false; break; }
                 ptx::tc_fence_after();
-                const uint32_t t_q = t_s0 + e * 32;
+                const uint32_t t_q = t_s0 + (uint32_t)b * 128 + e * 32;
                 const int a0 = a_first + e * 32;         // tree row of the quarter's first column
                 uint32_t q[32], pk[32];
                 ptx::tmem_ld32(t_q, q);
@@ -750,26 +785,93 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                     for (int i = 0; i < 32; ++i)
                         if (!((vis >> i) & 1u)) q[i] = hidden;
                 }
-                ptx::sts_f32(x_at(e, hf), max_quarter<NEG>(q, p.scale_log2));
+                const float mx = max_quarter<NEG>(q, p.scale_log2);
+                if (pi > 0) wait_x(SM::BAR_XO, 1);
+                ptx::sts_f32(x_at(e, hf), mx);
                 meet();
                 if (!ok) break;
-                m_used = ceilf(fmaxf(fmaxf(ptx::lds_f32(x_at(0, 0)), ptx::lds_f32(x_at(0, 1))), fmaxf(ptx::lds_f32(x_at(1, 0)), ptx::lds_f32(x_at(1, 1)))));
-                const float m_eff = m_used == -INFINITY ? 0.f : m_used;
+                m_new = ceilf(fmaxf(fmaxf(ptx::lds_f32(x_at(0, 0)), ptx::lds_f32(x_at(0, 1))), fmaxf(ptx::lds_f32(x_at(1, 0)), ptx::lds_f32(x_at(1, 1)))));
+                arrive_x(SM::BAR_XO);
+                const float m_eff = m_new == -INFINITY ? 0.f : m_new;
                 float2 la = make_float2(0.f, 0.f), lb = make_float2(0.f, 0.f);
                 exp_quarter<true>(q, sc2, make_float2(-m_eff, -m_eff), la, lb, pk, pk + 16);
                 ptx::tmem_st32(t_q, pk);
-                l = (la.x + la.y) + (lb.x + lb.y);
-                p_done(0, 1);
+                l_new = (la.x + la.y) + (lb.x + lb.y);
+                p_done(b, 1);
             }
-            int b = e == 0 ? 2 : 1;
-            for (int j = e == 0 ? 2 : 1; j < cnt; j += 2, b = b == 0 ? NB - 1 : b - 1) {
+            if (pi > 0) {
+                // ---- O of the piece before
+                const volatile AttnPiece &o_d = desc[(pi - 1) % AT_PIECES];
+                if (!ptx::mbar_wait(bar(SM::BAR_O), (pi - 1) & 1)) { ok = false; break; }
+                ptx::tc_fence_after();
+                // ---- the row sums of the row's four threads
+                wait_x(SM::BAR_XO, 1);
+                ptx::sts_f32(x_at(e, hf), l);
+                arrive_x(SM::BAR_XM);
+                uint32_t o[D / 4];
+                if constexpr (D == 128) ptx::tmem_ld32(t_o, o);
+                else ptx::tmem_ld16(t_o, o);
+                wait_x(SM::BAR_XM, 0);
+                if (!ok) break;
+                const float l_all = (ptx::lds_f32(x_at(0, 0)) + ptx::lds_f32(x_at(0, 1))) + (ptx::lds_f32(x_at(1, 0)) + ptx::lds_f32(x_at(1, 1)));
+                arrive_x(SM::BAR_XO);
+                const float inv_l = l_all == 0.f ? 0.f : 1.f / l_all;     // (NaN stays NaN)
+                if constexpr (D == 128) ptx::tmem_ld_wait_for(o);
+                else ptx::tmem_ld_wait_for16(o);
+                ptx::tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_lead(SM::BAR_O_FREE);
+#pragma unroll
+                for (int i = 0; i < D / 4; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv_l);
+                if (o_d.flags & PIECE_PARTIAL) {
+                    // to the workspace, whose layout suits a thread per row
+                    const int slab = o_d.flags & PIECE_HEAD ? 1 : 0;
+                    if (mine) {
+#pragma unroll
+                        for (int c = 0; c < D / 16; ++c)
+                            *slab_o<D>(p, blockIdx.x, slab, row, (e * 2 + hf) * (D / 16) + c) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
+                        if (hf == 0 && e == 0) *slab_ml(p, blockIdx.x, slab, row) = make_float2(m_used, l_all);
+                    }
+                    ++n_part;
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_OUT));
+                } else if (mine) {
+                    // a thread's columns are 32 or 64 bytes of its row
+                    uint4 *dst = item_out<D>(p, o_d.layer, o_d.b, o_d.head) + out_row(p, blk, row) * (D / 8) + (e * 2 + hf) * (D / 32);
+#pragma unroll
+                    for (int c = 0; c < D / 64; ++c) {
+                        uint32_t w[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) w[i] = pack2_bf16(__uint_as_float(o[16 * c + 2 * i]), __uint_as_float(o[16 * c + 2 * i + 1]));
+                        if (p.out32) ptx::st_global_32(dst + 2 * c, w);
+                        else {
+                            dst[2 * c] = make_uint4(w[0], w[1], w[2], w[3]);
+                            dst[2 * c + 1] = make_uint4(w[4], w[5], w[6], w[7]);
+                        }
+                    }
+                }
+                __syncwarp();
+                if (lane == 0) free_piece(pi - 1);
+            }
+            if (cnt_new <= 1 && cnt >= 2) phases ^= 8;     // (the PV of the piece's last group but one was told by itself)
+            piece = pi;
+            cnt = cnt_new;
+            t0 = t_new;
+            m_used = m_new;
+            l = l_new;
+            if (cnt == 0) break;
+            const int n_two = d.flags >> PIECE_TWO_SHIFT;
+            int t = t0 + (e == 0 ? 2 : 1);
+            for (int j = e == 0 ? 2 : 1; j < cnt; j += 2, t += 2) {
+                if (t >= 2 * NB) t -= 2 * NB;
+                const int b = t >= NB ? t - NB : t;
                 float sum;
                 bool asked = false;
                 const uint32_t t_s = t_s0 + (uint32_t)b * 128;
 #pragma unroll 1
                 for (;;) {
                     if (!asked) {
-                        wait_tc(bar(SM::BAR_S + b), parity_s(j, b), j);
+                        wait_tc(bar(SM::BAR_S + b), t >= NB, j);
                         if (!ok) break;
                         ptx::tc_fence_after();
                     }
@@ -830,77 +932,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
                 l += sum;
                 p_done(b, 2);
             }
-            // ---- O of this piece
-            if (ok) wait_tc(bar(SM::BAR_O), pi & 1, cnt + ((cnt ^ e) & 1));
             if (!ok) break;
-            ptx::tc_fence_after();
-            phases ^= s_phases(cnt) << 4;
-            const bool partial = d.flags & PIECE_PARTIAL;
-            const int slab = d.flags & PIECE_HEAD ? 1 : 0;
-            // ---- the row sums of the row's four threads
-            auto gather = [&]() {
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_XO + qd));
-            };
-            ptx::sts_f32(x_at(e, hf), l);
-            gather();
-            uint32_t o[D / 4];
-            if constexpr (D == 128) ptx::tmem_ld32(t_o, o);
-            else ptx::tmem_ld16(t_o, o);
-            if (!ptx::mbar_wait(bar(SM::BAR_XO + qd), (phases >> 1) & 1)) ok = false;
-            phases ^= 2;
-            if (!ok) break;
-            const float l_all = (ptx::lds_f32(x_at(0, 0)) + ptx::lds_f32(x_at(0, 1))) + (ptx::lds_f32(x_at(1, 0)) + ptx::lds_f32(x_at(1, 1)));
-            gather();                             // the exchanged values have been read: the next piece may overwrite them (and waits)
-            const float inv_l = l_all == 0.f ? 0.f : 1.f / l_all;     // (NaN stays NaN)
-            if constexpr (D == 128) ptx::tmem_ld_wait_for(o);
-            else ptx::tmem_ld_wait_for16(o);
-            ptx::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) arrive_lead(SM::BAR_O_FREE);
-#pragma unroll
-            for (int i = 0; i < D / 4; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * inv_l);
-            if (partial) {
-                // to the workspace, whose layout suits a thread per row
-                if (mine) {
-#pragma unroll
-                    for (int c = 0; c < D / 16; ++c)
-                        *slab_o<D>(p, blockIdx.x, slab, row, (e * 2 + hf) * (D / 16) + c) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
-                    if (hf == 0 && e == 0) *slab_ml(p, blockIdx.x, slab, row) = make_float2(m_used, l_all);
-                }
-                ++n_part;
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar(SM::BAR_OUT));
-            } else {
-                // Output rows are staged in the piece's query tile (each warp for itself, 16-byte chunks swizzled) and leave as
-                // runs of 32 or 64 bytes.
-                constexpr uint32_t N_CH = D / 32, ROW = N_CH * 16;
-                unsigned char *stage = smem + (uint32_t)(pi & 1) * SM::TILE + (uint32_t)warp * 32u * ROW;
-                auto place = [&](uint32_t r, uint32_t c) { return stage + r * ROW + ((c ^ ((r * N_CH / 8) & (N_CH - 1))) << 4); };
-#pragma unroll
-                for (uint32_t c = 0; c < N_CH; ++c) {
-                    float v[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(o[8 * c + i]);
-                    *reinterpret_cast<uint4 *>(place(lane, c)) =
-                        make_uint4(pack2_bf16(v[0], v[1]), pack2_bf16(v[2], v[3]), pack2_bf16(v[4], v[5]), pack2_bf16(v[6], v[7]));
-                }
-                __syncwarp();
-                const uint32_t c = lane & (N_CH - 1);
-                uint4 *dst = item_out<D>(p, d.layer, d.b, d.head) + (e * 2 + hf) * N_CH + c;
-#pragma unroll
-                for (uint32_t r = lane / N_CH; r < 32; r += 32 / N_CH) {
-                    const uint4 x = *reinterpret_cast<const uint4 *>(place(r, c));
-                    const int at = out_row(p, blk, qd * 32 + r);
-                    if (at >= 0) dst[at * (D / 8)] = x;
-                }
-                ptx::fence_proxy_async();         // (the next query tile comes here through the async proxy)
-                __syncwarp();
-            }
-            if (lane == 0) {
-                ptx::mbar_arrive(bar(SM::BAR_Q_EMPTY + (pi & 1)));
-                free_piece(pi);
-            }
         }
         if (!ok && lane == 0) give_up();
         // ---- the items that this CTA shares with others
@@ -1190,6 +1222,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     p.npc = a.npc; p.R = a.npc * p.G; p.inv_g = (65536u + p.G - 1) / p.G; p.n_blk = a.n_blk; p.teams = a.teams;
     p.n_tiles = a.n_tiles; p.two_cuts = a.two_cuts;
     p.gate = alongside ? *alongside : Gate{};
+    p.out32 = ((uintptr_t)out & 31) == 0;
     const size_t per_layer = (size_t)B * tree->T * Hq * D;
     cudaStream_t st = (cudaStream_t)stream;
     const int per_launch = layers_per_launch(n_layers, (double)B * Hkv, (Lcap + AT_BN - 1) / AT_BN);

@@ -61,6 +61,7 @@ struct AttnParams {
     int n_blk, teams;        // CTAs of a team, teams
     int n_tiles, two_cuts;   // row tiles of an item; see two_term_groups
     CacheFold fold;
+    int out32;               // out begins at a multiple of 32 bytes
     Gate gate;               // with a word: the inputs are complete behind it, the previous kernel is waited for at the end
 };
 
