@@ -103,6 +103,10 @@ AcceptWs accept_ws_layout(const mtv_tree *t, int B, int V);
 int argmax_keys_partial(const mtv_tree *tree, int B, int V, const mtv_bf16 *logits, unsigned long long *part, const Gate &alongside,
                         cudaStream_t stream);
 
+// lm_head_argmax; alongside: the weights and the final hidden states are complete at this gate (as above).
+int lm_head_keys(const mtv_tree *tree, int B, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W, int32_t *am, float *am_val,
+                 unsigned long long *keys, const Gate &alongside, cudaStream_t stream);
+
 int sm_count();   // of the current device
 
 // Set-up that has to happen once per device (kernel attributes, symbol addresses): one flag per device ordinal.

@@ -45,11 +45,24 @@ struct LmParams {
     int n_pairs;                // units of two weight tiles over the vocabulary
     int n_stages;
     uint32_t stage_bytes;
+    Gate gate;                  // with a word: W and x are complete behind it; else behind the previous kernel
 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void *map, uint32_t bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
+}
+// The weights and the nodes' states are there (a warp; TMA loads follow).
+__device__ __forceinline__ void lm_inputs_there(const Gate &gate, int lane) {
+    if (!gate.word) {
+        previous_done();
+        return;
+    }
+    if (lane == 0) {
+        wait_gate(gate);
+        ptx::fence_proxy_async_global();
+    }
+    __syncwarp();
 }
 // Best key of 32 columns over the warp's 32 rows (row of lane l: v0 + l), acc[e] = this lane's row in column e: lane l gets
 // the key of column l — the order-preserving image of the value in the high word, 0xffffffff - row in the low one, so that a
@@ -97,6 +110,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
     constexpr uint32_t W_BYTES = TILES * LM_TILE_BYTES;
     constexpr uint32_t TMEM_COLS = 2 * TILES * N;   // 2 buffers x TILES x N columns
 
+    let_next_start();
     for (int i = threadIdx.x; i < N; i += LM_THREADS) best[i] = 0ull;
     if (threadIdx.x == 0) {
         for (int s = 0; s < NST; ++s) { ptx::mbar_init(full(s), 1); ptx::mbar_init(empty(s), 1); }
@@ -125,6 +139,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
 
     if (warp == 5) {
         // ---------------------------------------------------------------- TMA producer
+        lm_inputs_there(p.gate, lane);
         int it = 0;
         for (int q = 0; q < my_pairs && !*abort_flag; ++q) {
             const int row0 = (cta + q * n_cta) * TILES * R;
@@ -217,6 +232,7 @@ lm_head_argmax_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_co
         }
         __syncthreads();
     }
+    previous_done();            // (the keys are zero)
     for (int n = threadIdx.x; n < N; n += LM_THREADS) {
         if (n < p.M && best[n] != 0ull) atomicMax(p.keys + n, best[n]);
     }
@@ -267,6 +283,7 @@ lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
         ptx::st_cluster_u32(ptx::mapa(ptx::smem_u32(&abort_flag_s), rank ^ 1), 1u);
     };
 
+    let_next_start();
     for (int i = threadIdx.x; i < p.passes * p.N; i += LP_THREADS) best[i] = 0ull;
     if (threadIdx.x == 0) {
         for (int s = 0; s < LP_STAGES; ++s) { ptx::mbar_init(full(s), 1); ptx::mbar_init(empty(s), 1); ptx::mbar_init(ready(s), 1); }
@@ -296,6 +313,7 @@ lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
 
     if (warp == 5) {
         // ---------------------------------------------------------------- TMA producer
+        lm_inputs_there(p.gate, lane);
         int it = 0;
         for (int q = 0; q < my_items && !*abort_flag; ++q) {
             const int item = pair + q * n_pairs;
@@ -393,6 +411,7 @@ lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
                 if (issued_s > s) ptx::mbar_wait(full(s), (uses - 1) & 1);
             }
     }
+    previous_done();            // (the keys are zero)
     for (int n = threadIdx.x; n < p.passes * p.N; n += LP_THREADS)
         if (n < p.M && best[n] != 0ull) atomicMax(p.keys + n, best[n]);
     // nobody leaves while the pair's MMAs may still read its shared memory or its barriers may be signalled
@@ -403,12 +422,12 @@ lm_head_argmax_pair_kernel(const __grid_constant__ CUtensorMap w_map, const __gr
 }
 
 static int launch_lm_head_pair(const mtv_tree_t *tree, int M, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W,
-                               unsigned long long *keys, cudaStream_t st) {
+                               unsigned long long *keys, const Gate &gate, cudaStream_t st) {
     for (int m0 = 0; m0 < M; m0 += LP_MAX_NODES) {
         const int m = M - m0 < LP_MAX_NODES ? M - m0 : LP_MAX_NODES;
         CUtensorMap w_map, x_map;
         LmParams p;
-        p.keys = keys + m0; p.dev_error = tree->d_error; p.M = m; p.H = H; p.V = V;
+        p.keys = keys + m0; p.dev_error = tree->d_error; p.M = m; p.H = H; p.V = V; p.gate = gate;
         p.passes = (m + 255) / 256;
         p.N = ((m + p.passes - 1) / p.passes + 31) / 32 * 32;       // passes of equal width: no columns of an MMA for nothing
         const int pairs = sm_count() / 2;
@@ -423,15 +442,23 @@ static int launch_lm_head_pair(const mtv_tree_t *tree, int M, int H, int V, cons
         if (!tma_map_2d_bf16(&w_map, W, V, H, p.R) || !tma_map_2d_bf16(&x_map, x + (size_t)m0 * H, m, H, p.N / 2)) return MTV_ERR_CUDA;
         const long items = (long)p.n_pairs * p.passes;
         const int grid = 2 * (int)(items < pairs ? items : pairs);
-        lm_head_argmax_pair_kernel<<<grid, LP_THREADS, LP_SMEM_BYTES, st>>>(w_map, x_map, p);
+        MTV_CUDA_CHECK(launch_dependent(lm_head_argmax_pair_kernel, dim3(grid), LP_THREADS, LP_SMEM_BYTES, st, w_map, x_map, p));
     }
     return MTV_OK;
 }
 
+__global__ void __launch_bounds__(256) lm_head_clear_kernel(int M, unsigned long long *keys) {
+    let_next_start();           // (the projection starts beside this: only its last step needs the keys)
+    previous_done();
+    const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    if (m < M) keys[m] = 0ull;
+}
 // keys -> (argmax, value)
-__global__ void lm_head_finish_kernel(int M, const unsigned long long *__restrict__ keys, int32_t *__restrict__ am,
+__global__ void lm_head_finish_kernel(int M, const unsigned long long *keys, int32_t *__restrict__ am,
                                       float *__restrict__ am_val) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
+    let_next_start();
+    previous_done();
     if (m >= M) return;
     const unsigned long long k = keys[m];
     am[m] = (int32_t)(0xffffffffu - (uint32_t)(k & 0xffffffffu));
@@ -441,17 +468,14 @@ __global__ void lm_head_finish_kernel(int M, const unsigned long long *__restric
     }
 }
 
-}  // namespace mtv
-
-extern "C" int lm_head_argmax(const mtv_tree_t *tree, int B, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W,
-                              int32_t *am, float *am_val, unsigned long long *keys, void *stream) {
-    using namespace mtv;
-    MTV_RANGE("lm_head_argmax");
+// The keys of all nodes.  The launches are programmatic dependents of one another: with a memset and ordinary launches the
+// projection started 5 us behind whatever was in front of it.
+int lm_head_keys(const mtv_tree_t *tree, int B, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W, int32_t *am, float *am_val,
+                 unsigned long long *keys, const Gate &gate, cudaStream_t st) {
     if (!tree || !tree->on_device || !x || !W || !keys || B < 1 || V < 1 || (am_val && !am)) return MTV_ERR_INVALID_ARG;
     if (H < 64 || H % 64 != 0) return MTV_ERR_UNSUPPORTED_SHAPE;
     if (((uintptr_t)x | (uintptr_t)W) & 15) return MTV_ERR_INVALID_ARG;
     const int M = B * tree->T;
-    cudaStream_t st = (cudaStream_t)stream;
     static PerDeviceOnce attr_once;
     bool *attr_done = attr_once.flag();
     if (!attr_done || !*attr_done) {
@@ -460,16 +484,16 @@ extern "C" int lm_head_argmax(const mtv_tree_t *tree, int B, int H, int V, const
         MTV_CUDA_CHECK(cudaFuncSetAttribute(lm_head_argmax_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, LP_SMEM_BYTES));
         if (attr_done) *attr_done = true;
     }
-    MTV_CUDA_CHECK(cudaMemsetAsync(keys, 0, (size_t)M * 8, st));
+    MTV_CUDA_CHECK(launch_dependent(lm_head_clear_kernel, dim3((M + 255) / 256), 256, 0, st, M, keys));
     if (M > 128) {
-        const int rc = launch_lm_head_pair(tree, M, H, V, x, W, keys, st);
+        const int rc = launch_lm_head_pair(tree, M, H, V, x, W, keys, gate, st);
         if (rc != MTV_OK) return rc;
     } else {
         const int N = M <= 64 ? 64 : 128;
         constexpr int tiles = 2;                             // weight tiles per stage (see the kernel)
         CUtensorMap w_map, x_map;
         LmParams p;
-        p.keys = keys; p.dev_error = tree->d_error; p.M = M; p.H = H; p.V = V; p.N = N; p.passes = 1;
+        p.keys = keys; p.dev_error = tree->d_error; p.M = M; p.H = H; p.V = V; p.N = N; p.passes = 1; p.gate = gate;
         p.stage_bytes = tiles * LM_TILE_BYTES + N * 128;
         p.n_stages = (int)((LM_SMEM_MAX - 1024) / p.stage_bytes);
         if (p.n_stages > LM_MAX_STAGES) p.n_stages = LM_MAX_STAGES;
@@ -483,10 +507,17 @@ extern "C" int lm_head_argmax(const mtv_tree_t *tree, int B, int H, int V, const
         p.n_pairs = ctas * rounds;
         p.R = ((V + tiles * p.n_pairs - 1) / (tiles * p.n_pairs) + 7) / 8 * 8;
         if (!tma_map_2d_bf16(&w_map, W, V, H, p.R) || !tma_map_2d_bf16(&x_map, x, M, H, N)) return MTV_ERR_CUDA;
-        if (N == 64) lm_head_argmax_kernel<64><<<ctas, LM_THREADS, smem, st>>>(w_map, x_map, p);
-        else lm_head_argmax_kernel<128><<<ctas, LM_THREADS, smem, st>>>(w_map, x_map, p);
+        if (N == 64) MTV_CUDA_CHECK(launch_dependent(lm_head_argmax_kernel<64>, dim3(ctas), LM_THREADS, smem, st, w_map, x_map, p));
+        else MTV_CUDA_CHECK(launch_dependent(lm_head_argmax_kernel<128>, dim3(ctas), LM_THREADS, smem, st, w_map, x_map, p));
     }
-    if (am) lm_head_finish_kernel<<<(M + 127) / 128, 128, 0, st>>>(M, keys, am, am_val);
-    MTV_CUDA_CHECK(cudaGetLastError());
+    if (am) MTV_CUDA_CHECK(launch_dependent(lm_head_finish_kernel, dim3((M + 127) / 128), 128, 0, st, M, keys, am, am_val));
     return MTV_OK;
+}
+
+}  // namespace mtv
+
+extern "C" int lm_head_argmax(const mtv_tree_t *tree, int B, int H, int V, const mtv_bf16 *x, const mtv_bf16 *W,
+                              int32_t *am, float *am_val, unsigned long long *keys, void *stream) {
+    MTV_RANGE("lm_head_argmax");
+    return mtv::lm_head_keys(tree, B, H, V, x, W, am, am_val, keys, mtv::Gate{}, (cudaStream_t)stream);
 }

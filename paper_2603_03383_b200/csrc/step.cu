@@ -92,7 +92,7 @@ static int verify_step(const mtv_tree_t *tree, const mtv_step_args *a, const int
         int ns = 1;
         if (a->x_final && a->W_lm) {
             keys = static_cast<unsigned long long *>(a->ws);     // where a caller may look for them; the heads are done, their tickets lie behind
-            rc = lm_head_argmax(tree, a->B, a->H, a->V, a->x_final, a->W_lm, nullptr, nullptr, keys, stream);
+            rc = mtv::lm_head_keys(tree, a->B, a->H, a->V, a->x_final, a->W_lm, nullptr, nullptr, keys, gate, (cudaStream_t)stream);
         } else {
             ns = mtv::accept_ws_layout(tree, a->B, a->V).nsplit;
             rc = mtv::argmax_keys_partial(tree, a->B, a->V, a->logits, keys, gate, (cudaStream_t)stream);
