@@ -239,10 +239,10 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     // ---- the tokens of the tree nodes that are this head's candidates (the first head: and the root's)
     if (slot >= off && slot < off + kd)
         for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = sm->tok[b][slot - off];
-    if (off == 1 && node < p.T) {
-        if (MTV_INDEX_OK(slot, p.C, p.dev_error) && slot == 0)
+    if (off == 1) {
+        if (node < p.T && MTV_INDEX_OK(slot, p.C, p.dev_error) && slot == 0)
             for (int b = 0; b < rows; ++b) p.tree_tok[(size_t)(b0 + b) * p.T + node] = p.root_tok[b0 + b];
-        if (node < rows) p.cand[(size_t)(b0 + node) * p.C] = p.root_tok[b0 + node];
+        if ((int)threadIdx.x < rows) p.cand[(size_t)(b0 + threadIdx.x) * p.C] = p.root_tok[b0 + threadIdx.x];     // (more rows than nodes, maybe)
     }
     if (p.gate_clear && threadIdx.x == 0 && atomicAdd(&counters[p.K], 1) == p.K - 1) *p.gate.word = 0;     // (all have read it)
 }

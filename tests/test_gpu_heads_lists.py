@@ -58,3 +58,20 @@ def test_stage_heights(H, V):
     assert binding.mtv_device_error(tree) == 0
     assert torch.equal(cand.cpu(), cand_ref) and torch.equal(tt.cpu(), tt_ref)
     assert (cl.double().cpu() - cl_ref).abs().max().item() <= 2e-5 * cl_ref.abs().max().item()
+
+
+@pytest.mark.parametrize("B,H", [(1, 64), (13, 64), (16, 64), (16, 72)])
+@pytest.mark.parametrize("topk", [(2,), (1, 1), (3, 2)])
+def test_more_rows_than_nodes(B, H, topk):
+    """The root's token in every row's candidates and tree, also where a tree has fewer nodes than there are rows."""
+    V, K = 900, len(topk)
+    tb, tree = make_tree("cartesian", K, topk)
+    from tests._cases import oracle_heads_with_margin
+    _, inp, _, cand_ref, _, tt_ref = oracle_heads_with_margin(B, H, V, K, tb, 70 + B)
+    hidden, W1, b1, W2, root = [t.to(DEV) for t in inp]
+    cand = torch.full((B, tree.C), -7, dtype=torch.int32, device=DEV)
+    tt = torch.full((B, tree.T), -7, dtype=torch.int32, device=DEV)
+    binding.medusa_heads_topk(tree, hidden, W1, b1, W2, root, cand, None, tt, workspace(tree, B, H, V, 0, 0, 0, 0))
+    torch.cuda.synchronize()
+    assert binding.mtv_device_error(tree) == 0
+    assert torch.equal(cand.cpu(), cand_ref) and torch.equal(tt.cpu(), tt_ref)
