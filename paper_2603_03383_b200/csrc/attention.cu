@@ -940,7 +940,12 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
         for (int i = 0; i < n_part && ok; ++i) {
             const MergeSlice<D> slice(p, merges[i], team - merges[i].first);
             if (!ptx::mbar_wait(bar(SM::BAR_GO + i), 0)) { give_up(); break; }
-            if (!((*left_items >> (2 + i)) & 1)) slice.run(p, merges[i], warp * 32 + lane, blk);
+            if ((*left_items >> (2 + i)) & 1) continue;
+            if (merges[i].n > MERGE_MANY) {
+                if (slice.n_my > 0) merge_few_rows<D>(p, merges[i], slice.r_begin, slice.n_my, warp * 32 + lane, blk);
+            } else {
+                slice.run(p, merges[i], warp * 32 + lane, blk);
+            }
         }
     }
     __syncwarp();

@@ -197,6 +197,75 @@ struct MergeSlice {
         }
     }
 };
+// The same for many contributors, whose slices have few rows: `split` lanes of a warp share the contributors of a chunk, that many fewer
+// round trips to L2.  (One sequence of 9284 keys and a single head, cut into 73 pieces: 30 -> 17 us a call.  Apart from run(), whose code is
+// slower for being both: ragged calls 256 -> 272 us; and for fewer contributors the way here costs more than it saves: head size
+// 64 with four 158 -> 166 us.)
+constexpr int MERGE_MANY = 24;
+template <int D>
+static __device__ __noinline__ void merge_few_rows(const AttnParams &p, const AttnMerge &m, int r_begin, int n_my, int thread, int blk) {
+    constexpr int VC = 2, NS = 3, NT = D / 4 / VC;
+    // (more than 24 contributors: at most six rows each, 96 chunks)
+    static_assert((128 / (MERGE_MANY + 1) + 1) * NT * 4 <= AT_SOFTMAX_WARPS * 32, "a thread per chunk and share");
+    const int all = n_my * NT, split = all * 8 <= AT_SOFTMAX_WARPS * 32 ? 8 : 4, each = 32 / split, sub = (thread & 31) / each;
+    const int e = (thread >> 5) * each + (thread & 31) % each, e_in = min(e, all - 1), c = e_in / n_my, r = r_begin + e_in - c * n_my;
+    float acc[4 * VC], mm = -INFINITY, wsum = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4 * VC; ++k) acc[k] = 0.f;
+    auto join = [&](float mc) {                      // another reference
+        const float resc = mm == -INFINITY ? 0.f : ex2(mm - mc);
+        mm = mc;
+        wsum *= resc;
+#pragma unroll
+        for (int k = 0; k < 4 * VC; ++k) acc[k] *= resc;
+    };
+#pragma unroll 1
+    for (int s0 = sub; s0 < m.n; s0 += split * NS) {
+        float2 ml[NS];
+        uint4 v[NS][VC];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const int s = s0 + k * split, cta = (m.first + s) * p.n_blk + blk;
+            const int sl = s == 0 ? 1 : 0;
+            ml[k] = make_float2(-INFINITY, 0.f);
+#pragma unroll
+            for (int q = 0; q < VC; ++q) v[k][q] = make_uint4(0u, 0u, 0u, 0u);
+            if (s < m.n) {
+                ml[k] = __ldcg(slab_ml(p, cta, sl, r));
+#pragma unroll
+                for (int q = 0; q < VC; ++q) v[k][q] = __ldcg(slab_o<D>(p, cta, sl, r, c * VC + q));
+            }
+        }
+        float mc = mm;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) mc = fmaxf(mc, ml[k].x);
+        join(mc);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const float wt = ml[k].x == -INFINITY ? 0.f : ex2(ml[k].x - mc) * ml[k].y;
+            wsum += wt;
+#pragma unroll
+            for (int q = 0; q < VC; ++q) {
+                const uint32_t vw[4] = {v[k][q].x, v[k][q].y, v[k][q].z, v[k][q].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[4 * q + i] = fmaf(wt, __uint_as_float(vw[i]), acc[4 * q + i]);
+            }
+        }
+    }
+#pragma unroll 1
+    for (int o = each; o < 32; o <<= 1) {
+        join(fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o)));
+        wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
+#pragma unroll
+        for (int k = 0; k < 4 * VC; ++k) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    }
+    const float inv = wsum == 0.f ? 0.f : 1.f / wsum;
+    const int o = out_row(p, blk, r);
+    if (o >= 0 && sub == 0 && e < all)
+        item_out<D>(p, m.layer, m.b, m.head)[o * (D / 8) + c] =
+            make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
+                       pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
+}
 // The slices that CTAs left, of one item, by the softmax warps of the CTA that was the last to leave it.  (Out of the way of the
 // usual case, whose registers it must not touch.)
 template <int D>

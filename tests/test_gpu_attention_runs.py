@@ -1,5 +1,5 @@
 """Runs of many short items on one CTA: pieces of one to five groups follow one another, so that scores, weights and outputs of
-neighbouring items are in flight together.  Against plain PyTorch in 64 bits; the bound is that of all attention tests."""
+neighbouring items are in flight together; and few long items, cut into many pieces.  Against plain PyTorch in 64 bits; the bound is that of all attention tests."""
 import pytest
 import torch
 
@@ -25,14 +25,9 @@ def _reference(q, k, v, lens, mask):
     return out
 
 
-@pytest.mark.parametrize("lens", LENS)
-@pytest.mark.parametrize("T,Hq,Hkv,D", [(64, 32, 8, 128), (29, 16, 8, 128), (117, 32, 8, 128), (64, 32, 8, 64), (22, 24, 8, 64)])
-@pytest.mark.parametrize("growing", [False, True])
-def test_runs_of_short_items(T, Hq, Hkv, D, lens, growing):
+def _check(T, Hq, Hkv, D, lens, n_layers, growing=False):
     """growing: keys of later groups are longer, so that their weights do not fit the first group's reference."""
-    K, H, V, n_layers = 4, 64, 600, 12
-    lens = LENS[lens]
-    B = len(lens)
+    K, H, V, B = 4, 64, 600, len(lens)
     tb, tree = make_tree("rank_prior", K, (), T)
     mask = torch.as_tensor(tb["mask"], device=DEV).bool().view(T, T)
     Lcap = max(lens) + T + 3
@@ -62,3 +57,22 @@ def test_runs_of_short_items(T, Hq, Hkv, D, lens, growing):
     assert binding.mtv_device_error(tree) == 0
     for l in range(n_layers):
         assert_close(out[l], want[l], "layer %d" % l)
+
+
+@pytest.mark.parametrize("lens", LENS)
+@pytest.mark.parametrize("T,Hq,Hkv,D", [(64, 32, 8, 128), (29, 16, 8, 128), (117, 32, 8, 128), (64, 32, 8, 64), (22, 24, 8, 64)])
+@pytest.mark.parametrize("growing", [False, True])
+def test_runs_of_short_items(T, Hq, Hkv, D, lens, growing):
+    _check(T, Hq, Hkv, D, LENS[lens], 12, growing)
+
+
+@pytest.mark.parametrize("T,Hq,Hkv,D,lens,n_layers", [
+    (47, 1, 1, 128, [9284], 2),        # 73 contributors with two rows each
+    (100, 4, 1, 128, [4500], 1),       # pairs, 36 contributors
+    (97, 4, 1, 128, [3100], 1),        # 25 contributors: the fewest that take this way
+    (61, 2, 1, 64, [12000, 6000], 1),
+    (128, 1, 1, 64, [18900], 1),       # 149 groups on 148 CTAs
+])
+@pytest.mark.parametrize("growing", [False, True])
+def test_many_contributors(T, Hq, Hkv, D, lens, n_layers, growing):
+    _check(T, Hq, Hkv, D, lens, n_layers, growing)
