@@ -1094,27 +1094,23 @@ AttnWs attn_ws_layout(const mtv_tree *t, int B, int Hq, int Hkv, int D, int Lcap
 
 // Which kernel a call for ONE layer takes at head size 128 (several layers always take the one of this file: 32 layers at
 // L = 512 take 45 us instead of 320, at L = 8192 260 to 320 instead of 570).  The kernel of attention_pair.cu starts and ends
-// faster but leaves pairs idle where blocks and splits do not fill the 74; this one divides the groups evenly.  Only the capacity
-// is known here, not the lengths.  us per call, lengths uniform in [h / 4, h] with h = all, a half, a quarter, an eighth of the
-// capacity (attention_pair.cu / even division):
-//      7 sequences, 28 / 4 heads, capacity  8112:   72 / 52    41 / 39    26 / 27    18 / 18
-//     12 sequences, 16 / 4 heads, capacity  8192:   70 / 57    40 / 32    24 / 26    17 / 18
-//      4 sequences, T = 128,      capacity 32896:  264 / 180  137 / 119   76 / 59    42 / 45
-//      3 sequences, 16 / 4 heads, capacity 20000:   38 / 33    25 / 27    18 / 22    15 / 19
-//     16 sequences, 32 / 8 heads, capacity 32768:  423 / 350  200 / 209  112 / 112   72 / 83
-//     16 sequences, 32 / 8 heads, capacity  4224:   59 / 62    41 / 52    31 / 40    27 / 37
-// With more blocks than pairs the pairs are all busy, longest sequence first: pairs.  With fewer, the even division is taken where
-// the estimate for a full cache (us per group on a pair and on an SM, start and end; fitted to an even division with two row tiles
-// per CTA and not fitted again since) is better by a tenth.  Of the rows above that is the even division for the first three, which
-// loses up to 3 us on a nearly empty cache, and pairs for the others, which lose 5 us in the full cache of the fourth and 73 in
-// that of the fifth, and gain up to 11 elsewhere.  (The rows were taken with one group in two terms per piece: two_term_groups.)
-static bool pair_kernel_is_better(int T, int G, int B, int Hkv, int Lcap) {
+// faster but leaves pairs idle where blocks and splits do not fill them, or where a second round of blocks follows the first; this one
+// divides the groups evenly.  Only the capacity is known here, not the lengths.  Estimates in us for a full cache, fitted to both
+// kernels' times for 142 shapes (1 to 16 sequences, 1 to 8 heads, groups of 1 to 8, T = 16 to 128, capacities of 107 to 65536, lengths of
+// 1 to 0.15 of it): the choice costs 0.8 % over the better of the two on average and 20 % at worst, where pairs alone cost 11 %,
+// the even division alone 10.5 %.  us per call, pairs / even division, and what is taken:
+//      1 sequence,  32 / 8 heads, capacity  8256:   18 / 23  pairs          8 sequences, 24 / 8 heads, T = 29,  3029:   35 / 28  even
+//      1 sequence,   8 / 2 heads, capacity  2112:   10 / 16  pairs          4 sequences, 32 / 8 heads, T = 128, 33024: 311 / 259  even
+//     16 sequences, 16 / 8 heads, T = 20,    320:   23 / 13  even          16 sequences, 32 / 8 heads, capacity 1564:   37 / 42  even
+//      7 sequences, 28 / 4 heads, capacity  8176:   71 / 48  even           2 sequences, 28 / 4 heads, capacity 3064:   18 / 20  pairs
+static bool pair_kernel_is_better(const AttnPlan &a, int T, int G, int B, int Hkv, int Lcap) {
     int n_blk = 1;
     const int ns = attn_pair_plan(T, G, B, Hkv, Lcap, &n_blk);
-    const double blocks = (double)B * Hkv * n_blk, groups = (Lcap + AT_BN - 1) / AT_BN;
-    if (blocks > 0.5 * sm_count()) return true;
-    const double pairs = 0.97 * ceil(groups / ns) + 9.0, even = 1.55 * blocks * groups / sm_count() + 22.0;
-    return pairs <= 1.1 * even;
+    const double items = (double)B * Hkv, groups = (Lcap + AT_BN - 1) / AT_BN;
+    const double pairs = 6.19 + 0.734 * ceil(groups / ns) * std::max(1.0, items * n_blk / (sm_count() / 2)) + (ns > 1 ? 2.59 : 0.0);
+    const double all = items * groups / a.teams, whole = ceil(items / a.teams) * groups;
+    const double even = 7.28 + 0.607 * (whole <= all + MERGE_COST ? whole : all + 4.57 / 0.607);
+    return pairs <= even;
 }
 
 // One tensor map for the caches of all layers, where they lie evenly spaced in memory and a map's five dimensions are enough: 64
@@ -1206,7 +1202,7 @@ int tree_attention_layers(const mtv_tree *tree, int B, int Hq, int Hkv, int D, i
     if (D == 128 && scale < 0.f) return MTV_ERR_INVALID_ARG;
     const AttnWs Lw = attn_ws_layout(tree, B, Hq, Hkv, D, Lcap);
     if (ws_bytes < Lw.total) return MTV_ERR_WORKSPACE;
-    if (n_layers == 1 && attn_pair_eligible(D, Hq / Hkv) && pair_kernel_is_better(tree->T, Hq / Hkv, B, Hkv, Lcap)) {
+    if (n_layers == 1 && attn_pair_eligible(D, Hq / Hkv) && pair_kernel_is_better(attn_plan(tree->T, Hq / Hkv, D), tree->T, Hq / Hkv, B, Hkv, Lcap)) {
         TapScope tap(MTV_KERNEL_ATTN_PARTIAL, (cudaStream_t)stream);
         return launch_tree_attn_pair(tree, B, Hq, Hkv, reinterpret_cast<const __nv_bfloat16 *>(q),
                                      reinterpret_cast<const __nv_bfloat16 *>(k[0]), reinterpret_cast<const __nv_bfloat16 *>(v[0]),
