@@ -332,8 +332,8 @@ struct PieceWalk {
         }
         // Piece length u of either way to divide.  Padding to whole pieces wastes the teams it leaves idle, cutting anywhere gives most
         // teams a second piece, and so a second partial result: whichever is shorter.  (Eight one-layer calls, cutting where
-        // padding makes a piece longer by more than 2 / 6 / 10 groups: 4 x 8000 keys, T = 128, 571 / 529 / 529 us; seven ragged
-        // sequences 297 / 282 / 282 and 310 / 306 / 300.)
+        // padding makes a piece longer by more than 5 / 7 groups: 4 x 8000 keys, T = 128, 531 / 491 us; seven ragged sequences
+        // 281 / 272.)
         const unsigned u_cut = max(1u, quotient(LH * (sum + nz * COST) + teams - 1, teams));
         pad = LH * nz <= teams;
         u = pad ? max(1u, quotient(LH * sum + teams - 1, teams)) : u_cut;
