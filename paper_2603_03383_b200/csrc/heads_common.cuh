@@ -146,6 +146,75 @@ __device__ __forceinline__ void merge_pass(int rows, int n, int parts, const Src
         }
     }
 }
+// The same for many lists of which few can matter: the kd-th largest of the lists' first entries bounds what is looked for, so that only
+// lists that begin at or above it are merged (kd of them, more where first entries are equal).  A warp per row; lists [row][n][16] in
+// global memory, n <= 160.  (Apart: few calls come here, and the others' code is better off without it.)
+static __device__ __noinline__ void merge_leading(int rows, int n, int kd, const float *part_val, const int32_t *part_idx, float2 (*result)[16]) {
+    constexpr int Q = 5;
+    const auto src = [&](int row, int l, int s, float &v, int &i) {
+        v = __ldcg(part_val + (row * n + l) * 16 + s);
+        i = __ldcg(part_idx + (row * n + l) * 16 + s);
+    };
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, half = lane >> 4, s = lane & 15, n_warps = (int)blockDim.x / 32;
+#pragma unroll 1
+    for (int row = warp; row < rows; row += n_warps) {
+        int key[Q], rest[Q];               // order-preserving images of the first entries
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            float v = -INFINITY;
+            int i;
+            if (lane + 32 * q < n) src(row, lane + 32 * q, 0, v, i);
+            const int bits = __float_as_int(v + 0.f);          // (-0.0 and 0.0 are equal)
+            rest[q] = key[q] = lane + 32 * q < n ? bits ^ ((bits >> 31) & 0x7fffffff) : (int)0x80000000;
+        }
+        int bound = (int)0x80000000;
+#pragma unroll 1
+        for (int r = 0; r < kd; ++r) {
+            int best = rest[0];
+#pragma unroll
+            for (int q = 1; q < Q; ++q) best = max(best, rest[q]);
+            bound = __reduce_max_sync(0xffffffffu, best);
+            bool take = lane == __ffs(__ballot_sync(0xffffffffu, best == bound)) - 1;          // one of them
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (take && rest[q] == bound) { rest[q] = (int)0x80000000; take = false; }
+        }
+        unsigned in[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) in[q] = __ballot_sync(0xffffffffu, lane + 32 * q < n && key[q] >= bound);
+        auto pop = [&]() {                 // the next list, or n
+            int c = n;
+#pragma unroll
+            for (int q = Q - 1; q >= 0; --q)
+                if (in[q]) c = 32 * q + __ffs(in[q]) - 1;
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (c >> 5 == q && c < n) in[q] &= in[q] - 1;
+            return c;
+        };
+        auto load = [&](float &v, int &i) {          // a list for each half warp; false: there was none for either
+            const int c0 = pop(), c1 = pop(), c = half ? c1 : c0;
+            v = -INFINITY;
+            i = 0x7fffffff;
+            if (c < n) src(row, c, s, v, i);
+            return c0 < n;
+        };
+        float v, nv;
+        int i, ni;
+        load(v, i);
+        bool more = load(nv, ni);
+#pragma unroll 1
+        while (more) {
+            const float ov = nv;
+            const int oi = ni;
+            more = load(nv, ni);
+            list_merge(v, i, ov, oi, lane);
+        }
+        list_merge(v, i, __shfl_xor_sync(0xffffffffu, v, 16), __shfl_xor_sync(0xffffffffu, i, 16), lane);
+        if (half == 0) result[row][s] = make_float2(v, __int_as_float(i));
+    }
+    __syncthreads();
+}
 // The best sixteen of n sorted lists for each row: passes that take at least four lists into one until one is left.  (A tournament of
 // kd rounds over the lists' heads, a warp per row, took 26 us for 16 rows of 37 lists at the end of a call, 9 us for two rows.)
 struct MergeSmem {
@@ -223,18 +292,28 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     if (!s_flag) return;
     static_assert(MTV_MAX_T <= 192, "a thread per tree node");
     const int off = p.off_arr[k], node = threadIdx.x, slot = node < p.T ? p.tree_indices[node] : -1;
-    merge_lists(rows, per, sm,
-                [&](int b, int c, int s, float &v, int &i) {
-                    const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
-                    v = __ldcg(p.part_val + o);
-                    i = __ldcg(p.part_idx + o);
-                },
-                [&](int b, int s, float v, int i) {
-                    sm->tok[b][s] = i;
-                    if (s >= kd) return;
-                    p.cand[(size_t)(b0 + b) * p.C + off + s] = i;
-                    if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + s] = v;
-                });
+    const auto take = [&](int b, int s, float v, int i) {
+        sm->tok[b][s] = i;
+        if (s >= kd) return;
+        p.cand[(size_t)(b0 + b) * p.C + off + s] = i;
+        if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + s] = v;
+    };
+    // Rough cycles of either way: 500 for a turn of merges, 1500 for the passes behind the first; 3500 and 350 per candidate for a row by its
+    // leading lists.  (13 rows of 148 lists with three candidates wanted: 58 -> 40 us a call; with 37 lists or less merging all is faster.)
+    const int warps = (int)blockDim.x / 32, parts = max(1, min((per + 3) / 4, 3 * warps / rows));
+    const int all = (rows * parts + 3 * warps - 1) / (3 * warps) * ((per + 2 * parts - 1) / (2 * parts)) * 500 + (parts > 1 ? 1500 : 0);
+    if (per > 64 && per <= 160 && (rows + warps - 1) / warps * (3500 + 350 * kd) < all) {
+        merge_leading(rows, per, kd, p.part_val + list0 * MTV_MAX_TOPK, p.part_idx + list0 * MTV_MAX_TOPK, sm->a);
+        for (int e = threadIdx.x; e < rows * 16; e += (int)blockDim.x) take(e / 16, e % 16, sm->a[e / 16][e % 16].x, __float_as_int(sm->a[e / 16][e % 16].y));
+    } else {
+        merge_lists(rows, per, sm,
+                    [&](int b, int c, int s, float &v, int &i) {
+                        const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
+                        v = __ldcg(p.part_val + o);
+                        i = __ldcg(p.part_idx + o);
+                    },
+                    take);
+    }
     __syncthreads();
     // ---- the tokens of the tree nodes that are this head's candidates (the first head: and the root's)
     if (slot >= off && slot < off + kd)
