@@ -226,6 +226,7 @@ __device__ __forceinline__ void merge_lists(int rows, int n, MergeSmem *sm, cons
     constexpr int R = 3;
     const int n_warps = (int)blockDim.x / 32;
     int parts = max(1, min((n + 3) / 4, R * n_warps / rows));
+    if (rows * parts > n_warps && rows * parts < 2 * n_warps) parts = max(1, n_warps / rows);     // (a unit per warp, rather than two for some)
     if (parts == 1) {
         const auto to = [&](int row, int, int s, float v, int i) { dst(row, s, v, i); };
         if (rows <= n_warps) merge_pass<1>(rows, n, 1, src, to);
@@ -242,7 +243,7 @@ __device__ __forceinline__ void merge_lists(int rows, int n, MergeSmem *sm, cons
     do {
         __syncthreads();
         n = parts;
-        parts = max(1, min((n + 3) / 4, n_warps / rows));
+        parts = n <= 8 ? 1 : max(1, min((n + 3) / 4, n_warps / rows));
         merge_pass<1>(
             rows, n, parts,
             [&](int row, int l, int s, float &v, int &i) {
@@ -299,10 +300,10 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
         if (p.cand_logit) p.cand_logit[(size_t)(b0 + b) * (p.C - 1) + off - 1 + s] = v;
     };
     // Rough cycles of either way: 500 for a turn of merges, 1500 for the passes behind the first; 3500 and 350 per candidate for a row by its
-    // leading lists.  (13 rows of 148 lists with three candidates wanted: 58 -> 40 us a call; with 37 lists or less merging all is faster.)
+    // leading lists.  (13 rows of 148 lists with three candidates wanted: 58 -> 40 us a call; 16 rows of 29 lists are faster by merging all.)
     const int warps = (int)blockDim.x / 32, parts = max(1, min((per + 3) / 4, 3 * warps / rows));
     const int all = (rows * parts + 3 * warps - 1) / (3 * warps) * ((per + 2 * parts - 1) / (2 * parts)) * 500 + (parts > 1 ? 1500 : 0);
-    if (per > 64 && per <= 160 && (rows + warps - 1) / warps * (3500 + 350 * kd) < all) {
+    if (per <= 160 && (rows + warps - 1) / warps * (3500 + 350 * kd) < all) {
         merge_leading(rows, per, kd, p.part_val + list0 * MTV_MAX_TOPK, p.part_idx + list0 * MTV_MAX_TOPK, sm->a);
         for (int e = threadIdx.x; e < rows * 16; e += (int)blockDim.x) take(e / 16, e % 16, sm->a[e / 16][e % 16].x, __float_as_int(sm->a[e / 16][e % 16].y));
     } else {
