@@ -11,7 +11,7 @@
 //   * More items than teams: an item counts its groups plus ITEM_COST (what starting and ending an item costs beside
 //     its groups) and the cuts fall anywhere.
 //   * Fewer: no team gets two pieces; the piece length is the smallest for which the pieces of all items fit the teams.
-//   * Whole items where that makes no run longer by more than MERGE_COST.
+//   * Whole items where that makes no run longer by more than WHOLE_COST.
 // Pieces that are not whole items leave O / l (fp32: where an item is cut must not show in its precision) and (m, l) in the
 // workspace; at the end of the launch the CTAs that share a tile meet at a counter and each combines a slice of its rows.
 // They all do so when the device is this launch's alone (the grid never exceeds one CTA per SM), but nothing depends on it:
@@ -72,8 +72,13 @@ int launch_tree_attn_pair(const mtv_tree *tree, int B, int Hq, int Hkv, const __
 
 
 constexpr int ITEM_COST = 2;          // what an item costs beside its key groups, in groups
-constexpr int MERGE_COST = 7;         // what partial results cost: written, met for, read and combined (5: ragged calls up to 3 % slower, four
-                                      // sequences of 8000 keys, T = 128, 531 us instead of 491)
+// What partial results cost (written, met for, read and combined), in groups, as a limit to how much longer runs are made so that a team has
+// one piece.  (5: ragged calls up to 3 % slower, four sequences of 8000 keys, T = 128, 531 us instead of 491.)
+constexpr int MERGE_COST = 7;
+// The same for items that stay whole, so that there are no partial results.  (5: 26 steps of 4 to 28 layers that differ in this 2.8 % slower on
+// average, 86 instead of 75 us for 23 layers of 12 / 2 heads, two sequences of 1470 keys, T = 82; one-layer calls of ten to twelve groups,
+// which have all their groups in two terms then, 2 to 8 % faster: 17.2 us instead of 18.0.)
+constexpr int WHOLE_COST = 7;
 constexpr int W_MMA = 16, W_TMA = 17, W_RELAY = 18, W_Q = 19;
 constexpr int NB = 3;                 // tiles of scores
 constexpr float LOG2E = 1.4426950408889634f;
@@ -252,7 +257,7 @@ tree_attn_kernel(const __grid_constant__ AttnMaps<ML> maps, const __grid_constan
     if (warp == W_TMA) {
         // ------------------------------------------------------------ the pair's pieces; this CTA's halves of K and V
         // (the pair, or CTA, that has the last tile of an odd number of them)
-        PieceWalk<ITEM_COST, MERGE_COST> walk(p, team, lane, (blk | 1) >= p.n_tiles);
+        PieceWalk<ITEM_COST, WHOLE_COST, MERGE_COST> walk(p, team, lane, (blk | 1) >= p.n_tiles);
         // The work is divided while the kernel before this one ends, by the lengths that are there (a call that follows another has
         // nothing that changes them in between), and looked at again behind it: eight one-layer calls on ragged lengths take 291 us
         // instead of 314, at head size 64 164 instead of 172.
