@@ -215,7 +215,7 @@ static __device__ __noinline__ void merge_leading(int rows, int n, int kd, const
     }
     __syncthreads();
 }
-// The best sixteen of n sorted lists for each row: passes that take at least four lists into one until one is left.  (A tournament of
+// The best sixteen of n sorted lists for each row: passes that take about four lists into one, the last one up to eight, until one is left.  (A tournament of
 // kd rounds over the lists' heads, a warp per row, took 26 us for 16 rows of 37 lists at the end of a call, 9 us for two rows.)
 struct MergeSmem {
     float2 a[52][16], b[26][16];      // what passes leave
@@ -261,6 +261,49 @@ __device__ __forceinline__ void merge_lists(int rows, int n, MergeSmem *sm, cons
     } while (parts > 1);
 }
 
+// One or two candidates of n <= 160 sorted lists for each row: a warp per row has the first kd entries of all lists in registers and takes
+// the best of them kd times: one round trip to L2 and no barrier, where merging lists of sixteen costs the same whatever is wanted.  us a call
+// of one row and one / two candidates a head (H = 512, V = 16000), merged -> so: one head (148 lists) 19.4 -> 14.4 / 19.4 -> 14.8, four heads
+// (37) 22.6 -> 19.6 / 22.7 -> 20.3; 16 rows, one candidate 33.9 -> 31.4 and 47.2 -> 42.1.  From three candidates on merging is faster than
+// what went before it (one row of 148 lists 20.6 -> 19.5), with one it was not (16.2 -> 19.4).
+constexpr int FEW = 2, FEW_LISTS = 160;
+template <typename Src, typename Dst>
+__device__ __forceinline__ void best_few(int rows, int n, int kd, const Src &src, const Dst &dst) {
+    constexpr int Q = FEW_LISTS / 32;
+    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, n_warps = (int)blockDim.x / 32;
+#pragma unroll 1
+    for (int row = warp; row < rows; row += n_warps) {
+        float v[Q][FEW];
+        int i[Q][FEW];
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+#pragma unroll
+            for (int s = 0; s < FEW; ++s) {
+                v[q][s] = -INFINITY;
+                i[q][s] = 0x7fffffff;
+                if (lane + 32 * q < n && s < kd) src(row, lane + 32 * q, s, v[q][s], i[q][s]);
+            }
+#pragma unroll 1
+        for (int r = 0; r < kd; ++r) {
+            float bv = v[0][0];
+            int bi = i[0][0];
+#pragma unroll
+            for (int q = 1; q < Q; ++q)
+                if (cand_before(v[q][0], i[q][0], bv, bi)) { bv = v[q][0]; bi = i[q][0]; }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+                if (cand_before(ov, oi, bv, bi)) { bv = ov; bi = oi; }
+            }
+            if (lane == 0) dst(row, r, bv, bi);
+#pragma unroll
+            for (int q = 0; q < Q; ++q)        // the list that it came from goes on (those that have ended all begin alike)
+                if (i[q][0] == bi) { v[q][0] = v[q][1]; i[q][0] = i[q][1]; }
+        }
+    }
+}
+
 // lval / lidx: [n_warps][NB][MTV_MAX_TOPK] sorted candidate lists in shared memory (unused slots hold
 // (-inf, 0x7fffffff)); smem: sizeof(MergeSmem), free by now.  Every thread of the CTA calls this.
 __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, const int n_warps, const float *lval,
@@ -271,16 +314,18 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     const int rows = min(NB, p.B - b0);
     const size_t list0 = ((size_t)k * p.B + b0) * per;        // lists of all CTAs: [head][batch row][CTA][16]
     // ---- the warps' lists
-    merge_lists(rows, n_warps, sm,
-                [&](int b, int w, int s, float &v, int &i) {
-                    v = lval[(w * NB + b) * MTV_MAX_TOPK + s];
-                    i = lidx[(w * NB + b) * MTV_MAX_TOPK + s];
-                },
-                [&](int b, int s, float v, int i) {
-                    const size_t o = (list0 + (size_t)b * per + blockIdx.x) * MTV_MAX_TOPK + s;
-                    p.part_val[o] = v;
-                    p.part_idx[o] = i;
-                });
+    const bool few = kd <= FEW && per <= FEW_LISTS;       // (the other entries of the CTAs' lists are then neither written nor read)
+    const auto of_warp = [&](int b, int w, int s, float &v, int &i) {
+        v = lval[(w * NB + b) * MTV_MAX_TOPK + s];
+        i = lidx[(w * NB + b) * MTV_MAX_TOPK + s];
+    };
+    const auto leave = [&](int b, int s, float v, int i) {
+        const size_t o = (list0 + (size_t)b * per + blockIdx.x) * MTV_MAX_TOPK + s;
+        p.part_val[o] = v;
+        p.part_idx[o] = i;
+    };
+    if (few) best_few(rows, n_warps, kd, of_warp, leave);
+    else merge_lists(rows, n_warps, sm, of_warp, leave);
     // ---- last CTA of this head merges the CTAs' lists (ticket: nobody waits)
     int32_t *counters = p.counters + (size_t)bz * (p.K + 1);
     __syncthreads();
@@ -303,17 +348,18 @@ __device__ __forceinline__ void vocab_tail(const VocabParams &p, const int NB, c
     // leading lists.  (13 rows of 148 lists with three candidates wanted: 58 -> 40 us a call; 16 rows of 29 lists are faster by merging all.)
     const int warps = (int)blockDim.x / 32, parts = max(1, min((per + 3) / 4, 3 * warps / rows));
     const int all = (rows * parts + 3 * warps - 1) / (3 * warps) * ((per + 2 * parts - 1) / (2 * parts)) * 500 + (parts > 1 ? 1500 : 0);
-    if (per <= 160 && (rows + warps - 1) / warps * (3500 + 350 * kd) < all) {
+    const auto of_cta = [&](int b, int c, int s, float &v, int &i) {
+        const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
+        v = __ldcg(p.part_val + o);
+        i = __ldcg(p.part_idx + o);
+    };
+    if (few) {
+        best_few(rows, per, kd, of_cta, take);
+    } else if (per <= 160 && (rows + warps - 1) / warps * (3500 + 350 * kd) < all) {
         merge_leading(rows, per, kd, p.part_val + list0 * MTV_MAX_TOPK, p.part_idx + list0 * MTV_MAX_TOPK, sm->a);
         for (int e = threadIdx.x; e < rows * 16; e += (int)blockDim.x) take(e / 16, e % 16, sm->a[e / 16][e % 16].x, __float_as_int(sm->a[e / 16][e % 16].y));
     } else {
-        merge_lists(rows, per, sm,
-                    [&](int b, int c, int s, float &v, int &i) {
-                        const size_t o = (list0 + (size_t)b * per + c) * MTV_MAX_TOPK + s;
-                        v = __ldcg(p.part_val + o);
-                        i = __ldcg(p.part_idx + o);
-                    },
-                    take);
+        merge_lists(rows, per, sm, of_cta, take);
     }
     __syncthreads();
     // ---- the tokens of the tree nodes that are this head's candidates (the first head: and the root's)
