@@ -203,7 +203,7 @@ struct MergeSlice {
 // 64 with four 158 -> 166 us.)
 constexpr int MERGE_MANY = 24;
 template <int D>
-static __device__ __noinline__ void merge_few_rows(const AttnParams &p, const AttnMerge &m, int r_begin, int n_my, int thread, int blk) {
+__device__ __forceinline__ void few_rows(const AttnParams &p, const AttnMerge &m, int r_begin, int n_my, int thread, int blk) {
     constexpr int VC = 2, NS = 3, NT = D / 4 / VC;
     // (more than 24 contributors: at most six rows each, 96 chunks)
     static_assert((128 / (MERGE_MANY + 1) + 1) * NT * 4 <= AT_SOFTMAX_WARPS * 32, "a thread per chunk and share");
@@ -266,19 +266,23 @@ static __device__ __noinline__ void merge_few_rows(const AttnParams &p, const At
             make_uint4(pack2_bf16(acc[0] * inv, acc[1] * inv), pack2_bf16(acc[2] * inv, acc[3] * inv),
                        pack2_bf16(acc[4] * inv, acc[5] * inv), pack2_bf16(acc[6] * inv, acc[7] * inv));
 }
-// Slice c of an item, by the softmax warps of a CTA.  Whoever does it, and whenever, it is summed in the same order.
 template <int D>
-__device__ __forceinline__ void merge_slice(const AttnParams &p, const AttnMerge &m, int c, int thread, int blk) {
-    const MergeSlice<D> slice(p, m, c);
-    if (m.n <= MERGE_MANY) slice.run(p, m, thread, blk);
-    else if (slice.n_my > 0) merge_few_rows<D>(p, m, slice.r_begin, slice.n_my, thread, blk);
+static __device__ __noinline__ void merge_few_rows(const AttnParams &p, const AttnMerge &m, int r_begin, int n_my, int thread, int blk) {
+    few_rows<D>(p, m, r_begin, n_my, thread, blk);
 }
-// The slices that CTAs left, of one item, by the softmax warps of the CTA that was the last to leave it.  (Out of the way of the
-// usual case, whose registers it must not touch.)
+// The slices that CTAs left, of one item, by the softmax warps of the CTA that was the last to leave it: summed as their own CTAs would
+// have, since bits must not depend on who is late.  (Out of the way of the usual case, whose registers it must not touch, and calling nothing:
+// with calls of merge_few_rows from here, or a choice between the two in the kernel, the compiler's registers for the kernel change, and eight
+// one-layer calls with twenty contributors take 136 to 139 us instead of 124, or at ragged lengths 269 instead of 256.)
 template <int D>
 static __device__ __noinline__ void merge_left(const AttnParams &p, const AttnMerge &m, int blk, int thread) {
-    for (int c = 0; c < m.n; ++c)
-        if (__ldcg(p.left + ((m.first + c) * p.n_blk + blk) * 2 + (c == 0 ? 1 : 0))) merge_slice<D>(p, m, c, thread, blk);
+#pragma unroll 1
+    for (int c = 0; c < m.n; ++c) {
+        if (!__ldcg(p.left + ((m.first + c) * p.n_blk + blk) * 2 + (c == 0 ? 1 : 0))) continue;
+        const MergeSlice<D> slice(p, m, c);
+        if (m.n <= MERGE_MANY) slice.run(p, m, thread, blk);
+        else if (slice.n_my > 0) few_rows<D>(p, m, slice.r_begin, slice.n_my, thread, blk);
+    }
 }
 
 // a / b, b > 0.  A quotient of small numbers is at most one off when it is formed in fp32, and its remainder says which way; the
