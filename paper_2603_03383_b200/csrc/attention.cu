@@ -27,8 +27,8 @@
 //     S(0) S(1) S(2) | PV(0) S(3) | PV(1) S(4) | ...
 // so that a group's softmax has the time of two other groups' MMAs and two groups' softmax run at once.  (The kernel before this
 // one had two row tiles in a CTA, with an accumulator and one tile of scores each: the chain scores -> P -> PV -> scores then took
-// 1.63 k cycles per tile and group, of which the tensor core worked 1024.  Now 1.4 k; what is left of the chain is 1.6 k of
-// softmax and 1.4 k of handing over, shared by three tiles.)  The pieces follow one another in the same way: the last PV of a piece
+// 1.63 k cycles per tile and group, of which the tensor core worked 1024.  Now 1.25 k in pieces of hundreds of groups, 1.4 k in those of
+// sixty, 1.6 k in those of twenty; what is left of the chain is 1.6 k of softmax and 1.4 k of handing over, shared by three tiles.)  The pieces follow one another in the same way: the last PV of a piece
 // has the first scores of the next one behind it, and the softmax warps take that one's first group before they read and write
 // the finished O.  (With pieces one after the other eight one-layer calls on ragged lengths took 281 us, now 256; 21 layers of eight
 // sequences of two or three groups 161 and 151, at head size 64 145 and 134; of one group 125 and 108.)
@@ -45,8 +45,8 @@
 // group: a test costs it about a hundred cycles, and the tensor core has only some two MMAs queued.
 //
 // What bounds it: the tensor core needs 1024 cycles for a tile and group at D = 128 and the special-function unit as many; 8 PV
-// and 8 S MMAs take 1025 with every other unit busy beside them, so the rest of the 1.4 k is the chain.  At 4 x 32768 keys the
-// board's power limit takes 15 to 25 % of the clock on top.
+// and 8 S MMAs take 1025 with every other unit busy beside them, so the rest is the chain.  At 4 x 32768 keys, T = 128, the
+// board's power limit takes the clock down to 1.1 GHz of 1.97 (at 16 x 1024 to 4096 keys, T = 64, to 1.18): 7112 groups x 1253 cycles are 8.1 ms.
 //
 // The reference of a row's exponentials is common to its four threads: the maximum of the piece's first group, rounded up to a
 // whole number.  It moves only when the sum of a thread's P in some later group exceeds 2^32.  P and O are floating-point
@@ -105,7 +105,7 @@ struct AttnSmem {
     // comes into was given back two groups ago.  With five slots it is requested only when the scores of the next group but one
     // are complete, and PV need not wait for that: the issuing warp waits for it, behind PV.
     static constexpr bool K_AHEAD = STAGES >= 2 * NB + 4;
-    static constexpr uint32_t OFF_RING = 2 * TILE;         // two query tiles: the next piece's, and where output rows are staged
+    static constexpr uint32_t OFF_RING = 2 * TILE;         // two query tiles: this piece's and the next one's; a place is free once its last scores are complete
     static constexpr uint32_t OFF_X = OFF_RING + STAGES * SLOT;
     static constexpr uint32_t OFF_BAR = OFF_X + 4 * 128 * 4;
     static constexpr int BAR_KV_FULL = 0;                  // of the even CTA of a pair: both parts (its own copy and the odd CTA's word)
